@@ -176,12 +176,13 @@ typedef struct {
     int64_t n_nodes, n_elems, nnz;
     int32_t n_colors, max_row, precision, scatter;
     int64_t device_bytes;   /* device memory owned by the handle */
-    int32_t rows_per_block; /* row-gather launch shape in use: rows per block of the per-row
-                               star kernel, -1 for the edge-fan kernel, 0 if unavailable */
+    int32_t rows_per_block; /* row-gather launch shape in use: 32, 64, 96 or 128 for the per-row
+                               star kernel (its warps per block: that many rows' worth, at most
+                               four), -1 for the edge-fan kernel, 0 if unavailable */
     int32_t n_plans;        /* row-gather launch shapes available */
-    int32_t persistent;     /* 1: the row gather runs as a persistent grid (a CTA's next block of
-                               rows copies its column indices and walk while the current one
-                               writes out), 0: one CTA per block of rows */
+    int32_t persistent;     /* 1: the row gather runs as a persistent grid of warps (a warp's next
+                               group of rows is fetched while the current one is merged and
+                               written out), 0: the edge-fan kernel, one CTA per block of rows */
     int32_t exact_rows;     /* mixed modes: rows of the nodes of badly shaped elements
                                (|d1||d2||d3| > 16 |det| from any node); after every assembly or
                                time step these rows are recomputed in double from the coordinates

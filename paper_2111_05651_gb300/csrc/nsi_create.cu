@@ -283,6 +283,66 @@ static bool encode_walk(const uint16_t* tri, int m, int dp, std::vector<uint8_t>
   return true;
 }
 
+// A row's walk cut into nsub sub-walks of about equal element counts, one per
+// lane of the row gather: the row's bytes are nsub lengths, then each
+// sub-walk's bytes.  A sub-walk is a list of segments (a walk's path, or a
+// piece of one): two filling bytes, the window nodes p and q before the
+// segment's first element, whose upper three bits hold the segment's element
+// count (low three bits in the first, high three in the second byte), then the
+// path's element bytes.  Positions become slots (the row's entries without the
+// diagonal dp).  Returns false if a sub-walk needs more than 255 bytes.
+static bool split_walk(const uint8_t* steps, int nsteps, int dp, int nsub, std::vector<uint8_t>& out) {
+  constexpr int SEG_MAX = 63;
+  int m = 0;
+  for (int s = 0; s < nsteps; ++s) m += (steps[s] & WALK_ELEM) != 0;
+  if (m == 0) return true;
+  auto slot = [&](int pos) { return (unsigned)(pos - (pos > dp ? 1 : 0)); };
+  const size_t head = out.size();
+  out.insert(out.end(), nsub, (uint8_t)0);
+  size_t sub_start = out.size(), seg = 0;
+  int wp = dp, wq = dp, e = 0, sub = 0, cnt = 0;
+  bool open = false;  // a segment is being written
+  auto close = [&]() {
+    if (!open) return;
+    out[seg] |= (uint8_t)((cnt & 7) << 5);
+    out[seg + 1] |= (uint8_t)((cnt >> 3) << 5);
+    open = false;
+  };
+  for (int s = 0; s < nsteps; ++s) {
+    const int pos = steps[s] & WALK_POS;
+    if (!(steps[s] & WALK_ELEM)) {  // a new path fills the window
+      close();
+      wp = wq;
+      wq = pos;
+      continue;
+    }
+    while (sub + 1 < nsub && (int64_t)e * nsub >= (int64_t)m * (sub + 1)) {  // the next sub-walk starts here
+      close();
+      if (out.size() - sub_start > 255) return false;
+      out[head + sub] = (uint8_t)(out.size() - sub_start);
+      sub_start = out.size();
+      ++sub;
+    }
+    if (open && cnt == SEG_MAX) close();
+    if (!open) {
+      seg = out.size();
+      out.push_back((uint8_t)slot(wp));
+      out.push_back((uint8_t)slot(wq));
+      cnt = 0;
+      open = true;
+    }
+    out.push_back((uint8_t)(slot(pos) | (steps[s] & (WALK_ELEM | WALK_NEG | WALK_EVQ))));
+    ++cnt;
+    ++e;
+    if (!(steps[s] & WALK_EVQ)) wp = wq;
+    wq = pos;
+  }
+  close();
+  if (out.size() - sub_start > 255) return false;
+  out[head + sub] = (uint8_t)(out.size() - sub_start);
+  return true;
+}
+
 static nsi_status build(NsiHandle* h, const NsiMesh* m, cudaStream_t s) {
   const int64_t n = h->n, E = h->E;
   std::vector<int32_t> ln(4 * E);
@@ -427,7 +487,9 @@ static nsi_status build(NsiHandle* h, const NsiMesh* m, cudaStream_t s) {
     });
   }
 
-  // 4a. every row's element walk (the order and steps of the kernel's element loop)
+  // 4a. every row's sub-walks (the order and steps of the kernel's element
+  // loops), one per lane of the row
+  h->nsub = n >= SMALL_MESH_ROWS ? 2 : 4;
   std::vector<int32_t> walk_ptr;
   std::vector<uint8_t> walk;
   if (h->gather_ok) {
@@ -436,11 +498,14 @@ static nsi_status build(NsiHandle* h, const NsiMesh* m, cudaStream_t s) {
     std::mutex mu;
     std::atomic<bool> bad{false};
     parallel_for(n, [&](int64_t lo, int64_t hi) {
-      std::vector<uint8_t> buf;
+      std::vector<uint8_t> buf, steps;
       WalkWork ws;
       for (int64_t i = lo; i < hi && !bad.load(std::memory_order_relaxed); ++i) {
         const size_t before = buf.size();
-        if (!is_long[i] && !encode_walk(&star[inc_ptr[i]], (int)(inc_ptr[i + 1] - inc_ptr[i]), diag[i], buf, ws)) {
+        steps.clear();
+        if (!is_long[i] &&
+            !(encode_walk(&star[inc_ptr[i]], (int)(inc_ptr[i + 1] - inc_ptr[i]), diag[i], steps, ws) &&
+              split_walk(steps.data(), (int)steps.size(), diag[i], h->nsub, buf))) {
           // a star the encoder cannot walk: the row becomes a long row
           buf.resize(before);
           is_long[i] = 1;
@@ -603,53 +668,49 @@ static nsi_status build(NsiHandle* h, const NsiMesh* m, cudaStream_t s) {
     }
   }
 
-  // 7. gather launch plan: largest rows-per-block whose entries fit the budget
+  // 7. gather launch plans: warps per block by the plan's name, chosen for the
+  // most resident warps per SM (shared memory of the groups, the kernel's
+  // registers); on a tie the smallest block
   {
-    // rows per block chosen for the most resident warps per SM (shared memory
-    // of the block's layout, the kernel's registers, 2048 threads per SM); on
-    // a tie the smallest block, whose barriers hold fewer warps
-    const size_t smem_sm = 228 * 1024, smem_max = 200 * 1024;
+    const size_t smem_sm = 228 * 1024;
     const int regs = std::max(32, gather_kernel_regs(h->precision));
-    int64_t short_max = 0;
+    const int RW = 32 / h->nsub;
+    int64_t slots = 1, mL = 0, mS = 0;
     for (int64_t i = 0; i < n; ++i)
-      if (!is_long[i]) short_max = std::max(short_max, row_len[i]);
-    int chosen = 0, best_warps = 0;
-    for (int R : {32, 64, 96, 128}) {
-      if (!h->gather_ok) break;
-      int64_t mL = 0, mS = 0;
-      for (int64_t r0 = 0; r0 < n; r0 += R) {
-        const int64_t r1 = std::min(n, r0 + R);
+      if (!is_long[i]) slots = std::max(slots, row_len[i] - 1);
+    if (h->gather_ok)
+      for (int64_t r0 = 0; r0 < n; r0 += RW) {
+        const int64_t r1 = std::min(n, r0 + RW);
         mL = std::max<int64_t>(mL, rp64[r1] - rp64[r0]);
         mS = std::max<int64_t>(mS, walk_ptr[r1] - walk_ptr[r0]);
       }
-      // slots per row: the longest row the kernel takes, or more where a
-      // block's long rows would not leave room for its entries in R * w
-      const int W = (int)std::max<int64_t>({1, short_max, (mL + R - 1) / R});
-      const GatherSmem g = gather_smem(h->precision, R, W, (int)mL, (int)mS);
-      const size_t sm = g.total();
-      if (sm > smem_max || !g.stage_fits()) continue;
-      int blocks = (int)std::min<size_t>({smem_sm / (sm + 1024), (size_t)32, (size_t)(2048 / R),
-                                          (size_t)(65536 / (R * regs))});
-      const int warps = blocks * R / 32;
+    // slots per row: the longest row the kernel takes, or more where a group's
+    // entries (long rows' among them) would not fit the bytes of nb0 and nb1
+    int W = (int)slots;
+    GatherSmem g = gather_smem(h->precision, RW, W, (int)mL, (int)mS);
+    g.H = h->nsub;
+    while (!g.group_fits()) g.W = ++W;
+    int chosen = -1, best_warps = 0;
+    for (int R : {32, 64, 96, 128}) {
+      if (!h->gather_ok || g.total() > (size_t)SMEM_MAX) break;
+      int warps = std::min(R / RW, 4);
+      while (g.total() * warps > (size_t)SMEM_MAX) --warps;
+      const int blocks = (int)std::min<size_t>({smem_sm / (g.total() * warps + 1024), (size_t)32,
+                                                (size_t)(65536 / (32 * warps * regs))});
       GatherPlan cand;
       cand.rows_per_block = R;
+      cand.warps = warps;
       cand.max_block_entries = (int)mL;
       cand.max_block_steps = (int)mS;
       cand.w = W;
-      cand.n_blocks = (n + R - 1) / R;
       h->plans[h->n_plans++] = cand;
-      if (warps > best_warps) {
-        best_warps = warps;
+      if (blocks * warps > best_warps) {
+        best_warps = blocks * warps;
         chosen = h->n_plans - 1;
       }
     }
-    if (best_warps == 0) h->gather_ok = false;
+    if (chosen < 0) h->gather_ok = false;
     else h->plan = h->plans[chosen];
-    // the persistent grid (next block's phase 0 under the current block's
-    // write-out) measured faster for the mixed modes: mixed64 0.280 against
-    // 0.302 ms, mixed32 0.228 against 0.239 ms at the 100^3 cube; it slowed
-    // FP64 (4.23 against 3.29 ms, on an earlier kernel)
-    h->persistent = h->precision != NSI_FP64;
   }
 
   // 7b. badly shaped elements (mixed modes): a float determinant of an
@@ -727,7 +788,8 @@ static nsi_status build(NsiHandle* h, const NsiMesh* m, cudaStream_t s) {
     if ((st = dev_upload(h, &h->walk, walk.data(), walk.size(), s))) return st;
   }
   if (pos_ok || h->gather_ok) {
-    if ((st = dev_upload(h, &h->diag_pos, diag.data(), n, s))) return st;
+    diag.resize(n + 32, 0);  // the row gather copies whole groups
+    if ((st = dev_upload(h, &h->diag_pos, diag.data(), diag.size(), s))) return st;
   }
   if (pos_ok) {
     if ((st = dev_upload(h, &h->elem_pos, elem_pos.data(), E, s))) return st;
@@ -880,7 +942,7 @@ nsi_status nsi_info(const NsiHandle* h, NsiInfo* info) {
   info->device_bytes = h->device_bytes;
   info->rows_per_block = h->use_fan ? -1 : h->plan.rows_per_block;
   info->n_plans = h->n_plans;
-  info->persistent = h->persistent && !h->use_fan ? 1 : 0;
+  info->persistent = h->use_fan ? 0 : 1;
   info->exact_rows = (int32_t)std::min<int64_t>(h->exact_rows, INT32_MAX);
   info->long_rows = (int32_t)std::min<int64_t>(h->long_rows, INT32_MAX);
   info->fan_ok = h->fan_ok ? 1 : 0;

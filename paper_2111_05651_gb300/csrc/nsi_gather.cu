@@ -1,0 +1,1096 @@
+// The row gather: the assembly (A, G, rhs), the time step with cached
+// geometry (A = A_static + C(u), rhs) and the paper's per-node outputs, for
+// one mesh or a batch of meshes.
+//
+//   pack_kernel, batched_pack_kernel  the call's node records
+//   gather_persistent_kernel          one mesh, a persistent grid of warps
+//   batched_kernel                    many meshes in one persistent launch
+//
+// A warp takes groups of 32 / H consecutive CSR rows, H lanes per row.  The
+// elements around a row's node (its star) are ordered at create along walks of
+// neighbouring elements and cut into `nsub` sub-walks; each of the row's lanes
+// follows its own and adds into its own accumulators, and the lanes' sums are
+// merged in a fixed order, so results do not depend on timing.  Every output
+// is written once, in memory order; there are no atomics and no zeroing.
+//
+// What bounds it, and why H lanes per row: a walk is a serial chain of element
+// evaluations, and the slots it works on (edge vectors, velocities and
+// accumulators of a row's neighbours) are in shared memory, which limits the
+// resident warps.  One lane per row kept 32 rows of slots per warp (20 KB, 11
+// warps per SM) behind chains of 24 elements; two lanes per row keep 16 rows
+// and a second set of accumulators (13 KB, 16 warps) behind chains of 12, and
+// the neighbours' records come as one 256-bit load each, in registers under the
+// previous group's write-out, instead of two 16-byte copies through shared
+// memory (100^3 cube, us, one lane per row -> two: mixed64 277 -> 271 in random
+// and 269 -> 235 in natural node order, mixed32 228 -> 226, time step 275 ->
+// 229, nodal outputs 216 -> 126; 47x61x38 mixed32 39.6 -> 31.4).  The records
+// bypass L1 (allocating there cost 439 us: 115 KB of sectors in flight per SM
+// through the 28 KB that shared memory leaves).  What is left in random order is
+// the rate of scattered 32-byte requests (40 us against natural order; loading
+// still earlier changes nothing), then issue: 67 M warp instructions at the
+// 70^3 cube, 53% of the slots used.  FP64 is bound by the FP64 pipe.
+//
+// A small mesh has four lanes per row: its groups do not fill the chip, so the
+// chain is the time (8^3 cube in FP64: 66 us with one lane, 29 with four; 20^3
+// mixed64 13.8 with one, 12.5 with two, 10.9 with four; at 30 000 rows two and
+// four are equal, and at 100^3 four cost 374 us).
+#include <algorithm>
+#include <mutex>
+
+#include "nsi_device.cuh"
+
+namespace nsi {
+
+namespace {
+
+enum { ASSEMBLE = 0, STEP = 1, NODAL = 2 };
+constexpr int MAX_WARPS = 4;  // warps per block
+
+// --------------------------------------------------------------- copies ---
+__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+
+// A node's record in registers: 32 bytes (mixed) or 64 (FP64) by 256-bit loads
+// (records are 32-byte aligned and written by an earlier launch).
+template <int P>
+struct NodeRec {
+  uint4 a, b;
+  __device__ __forceinline__ void load(const void* rec, int64_t j) {
+    const unsigned* r = static_cast<const unsigned*>(rec) + 8 * j;
+    asm("ld.global.nc.L1::no_allocate.v8.u32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
+        : "l"(r));
+  }
+  // edge vector from node o to this one
+  __device__ __forceinline__ V3<float> minus(const NodeRec& o) const {
+    const V3<float> h{__uint_as_float(a.x) - __uint_as_float(o.a.x), __uint_as_float(a.y) - __uint_as_float(o.a.y),
+                      __uint_as_float(a.z) - __uint_as_float(o.a.z)};
+    return add(h, sub(record_lo(__uint_as_float(b.z), __uint_as_float(b.w)),
+                      record_lo(__uint_as_float(o.b.z), __uint_as_float(o.b.w))));
+  }
+  __device__ __forceinline__ V3<float> vel() const {
+    return {__uint_as_float(a.w), __uint_as_float(b.x), __uint_as_float(b.y)};
+  }
+};
+template <>
+struct NodeRec<NSI_FP64> {
+  double x, y, z, ux, uy, uz;
+  __device__ __forceinline__ void load(const void* rec, int64_t j) {
+    const double* r = static_cast<const double*>(rec) + 8 * j;
+    [[maybe_unused]] double pad;
+    asm("ld.global.nc.L1::no_allocate.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(x), "=d"(y), "=d"(z), "=d"(pad) : "l"(r));
+    asm("ld.global.nc.L1::no_allocate.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(ux), "=d"(uy), "=d"(uz), "=d"(pad) : "l"(r + 4));
+  }
+  __device__ __forceinline__ V3<double> minus(const NodeRec& o) const { return {x - o.x, y - o.y, z - o.z}; }
+  __device__ __forceinline__ V3<double> vel() const { return {ux, uy, uz}; }
+};
+
+// -------------------------------------------------------------- kernel I/O ---
+// the layout of a warp's shared memory (GatherSmem) as the kernels take it:
+// byte offsets of its regions, the bytes of one accumulator plane, R * W, and
+// the limits that the bounds checks compare with.  Kernel parameters are
+// operands of the instructions that use them and take no registers.
+struct GroupLay {
+  int nb1, acc, plane, walk, info, cols, total, N, W, L, S;
+  explicit GroupLay(const GatherSmem& g)
+      : nb1((int)g.nb1()), acc((int)g.acc()), plane((int)(g.ab * g.N())), walk((int)g.walk()), info((int)g.info()),
+        cols((int)g.cols()), total((int)g.total()), N((int)g.N()), W(g.W),
+        L(g.L), S(g.S) {}
+};
+// what the kernels read of a mesh
+struct WalkMesh {
+  int64_t n, nnz;
+  const int32_t* row_ptr;
+  const int32_t* col_idx;
+  const int32_t* walk_ptr;
+  const uint8_t* walk;
+  const uint8_t* diag_pos;
+  const D4* xyz64;
+  const float4* xyz_hi;
+  const float4* xyz_lo;
+  void* rec;
+  unsigned* err;
+};
+// outputs by mode (kmr = rho/24, the density mass per det)
+template <int MODE>
+struct WalkOut;
+template <>
+struct WalkOut<ASSEMBLE> {
+  void *A, *G, *rhs;
+};
+template <>
+struct WalkOut<STEP> {
+  void *A, *rhs;
+  const void* A_static;
+};
+template <>
+struct WalkOut<NODAL> {
+  void *rhs, *dt_rho, *mass_rho;
+  double kmr;
+  float kmrf;
+};
+template <int MODE>
+struct WalkItem {
+  WalkMesh m;
+  FieldView f;
+  WalkOut<MODE> o;
+  int group0;  // the first of the mesh's row groups in the launch
+};
+
+// ------------------------------------------------------------ the sub-walk ---
+// Products that are rounded, and cross and dot products with their
+// multiply-adds spelt out: the single-mesh and the batched kernel are compiled
+// apart and give the same bits.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+template <typename T>
+__device__ __forceinline__ V3<T> cross_fma(const V3<T>& a, const V3<T>& b) {
+  return {fma(a.y, b.z, -mul_rn(a.z, b.y)), fma(a.z, b.x, -mul_rn(a.x, b.z)), fma(a.x, b.y, -mul_rn(a.y, b.x))};
+}
+template <typename T>
+__device__ __forceinline__ T dot_fma(const V3<T>& a, const V3<T>& b) {
+  return fma(a.z, b.z, fma(a.y, b.y, mul_rn(a.x, b.x)));
+}
+
+// Accumulators of a row's slots in shared memory, one plane per lane of the
+// row: the sums of A and of the pressure gradient (-c_i / 24) of each entry
+// (mixed: a float4 (G_x, G_y, G_z, A); FP64 two planes (A, G_x), (G_y, G_z));
+// the time step only A.  A slot is touched by one lane until the merge.
+template <int P, int MODE>
+struct Slots;
+// paired float arithmetic: one instruction for two lanes of a float2
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+
+template <int P>
+struct Slots<P, ASSEMBLE> {
+  float4* a;
+  struct V {
+    float2 g, r;  // (G_x, G_y), (G_z, A)
+  };
+  __device__ __forceinline__ Slots(unsigned char* p, size_t) : a(reinterpret_cast<float4*>(p)) {}
+  static __device__ __forceinline__ V zero_value() { return {make_float2(0.f, 0.f), make_float2(0.f, 0.f)}; }
+  __device__ __forceinline__ V load(int k) const {
+    const float4 v = a[k];
+    return {make_float2(v.x, v.y), make_float2(v.z, v.w)};
+  }
+  __device__ __forceinline__ void store(int k, const V& v) { a[k] = make_float4(v.g.x, v.g.y, v.r.x, v.r.y); }
+  static __device__ __forceinline__ V sum(const V& x, const V& y) { return {add2(x.g, y.g), add2(x.r, y.r)}; }
+  static __device__ __forceinline__ V pick(bool c, const V& x, const V& y) {
+    return {make_float2(c ? x.g.x : y.g.x, c ? x.g.y : y.g.y), make_float2(c ? x.r.x : y.r.x, c ? x.r.y : y.r.y)};
+  }
+};
+template <>
+struct Slots<NSI_FP64, ASSEMBLE> {
+  T2<double>*a0, *a1;
+  struct V {
+    T2<double> x, y;  // (A, G_x), (G_y, G_z)
+  };
+  __device__ __forceinline__ Slots(unsigned char* p, size_t N)
+      : a0(reinterpret_cast<T2<double>*>(p)), a1(reinterpret_cast<T2<double>*>(p) + N) {}
+  static __device__ __forceinline__ V zero_value() { return {{0.0, 0.0}, {0.0, 0.0}}; }
+  __device__ __forceinline__ V load(int k) const { return {a0[k], a1[k]}; }
+  __device__ __forceinline__ void store(int k, const V& v) {
+    a0[k] = v.x;
+    a1[k] = v.y;
+  }
+  static __device__ __forceinline__ V sum(const V& x, const V& y) {
+    return {{x.x.x + y.x.x, x.x.y + y.x.y}, {x.y.x + y.y.x, x.y.y + y.y.y}};
+  }
+  static __device__ __forceinline__ V pick(bool c, const V& x, const V& y) {
+    return {{c ? x.x.x : y.x.x, c ? x.x.y : y.x.y}, {c ? x.y.x : y.y.x, c ? x.y.y : y.y.y}};
+  }
+};
+template <int P>
+struct Slots<P, STEP> {
+  using V = typename Prec<P>::T;
+  V* a;
+  __device__ __forceinline__ Slots(unsigned char* p, size_t) : a(reinterpret_cast<V*>(p)) {}
+  static __device__ __forceinline__ V zero_value() { return V(0); }
+  __device__ __forceinline__ V load(int k) const { return a[k]; }
+  __device__ __forceinline__ void store(int k, V v) { a[k] = v; }
+  static __device__ __forceinline__ V sum(V x, V y) { return x + y; }
+  static __device__ __forceinline__ V pick(bool c, V x, V y) { return c ? x : y; }
+};
+template <int P>
+struct Slots<P, NODAL> {
+  struct V {};
+  __device__ __forceinline__ Slots(unsigned char*, size_t) {}
+  static __device__ __forceinline__ V zero_value() { return {}; }
+  __device__ __forceinline__ V load(int) const { return {}; }
+  __device__ __forceinline__ void store(int, V) {}
+  static __device__ __forceinline__ V sum(V, V) { return {}; }
+  static __device__ __forceinline__ V pick(bool, V, V) { return {}; }
+};
+
+// One lane's sub-walk of one row, node i as the origin: segments of
+// neighbouring elements.  A window of two neighbours (p, q) stays in registers
+// with their edge vectors, velocities and accumulators; every step brings one
+// node c in from shared memory, evaluates the element (i, p, q, c), then
+// writes back the accumulator of the node that leaves the window; c always
+// becomes q, and p keeps its node or takes q's.  With
+// c_p = d_q x d_c, c_q = d_c x d_p, c_c = d_p x d_q (cofactors of the
+// Jacobian, calculate_cartesian_derivatives, for the order (p, q, c)),
+// det = d_p . c_p and c_i = -(c_p + c_q + c_c), the element adds
+//   A(i,x) += w . c_x  (x = p, q, c),  w = rho/120 (2 u_i + u_p + u_q + u_c) + mu/(6 det) c_i
+// (the staged velocities carry the factor rho/120, p's also the 2 u_i; the time
+// step has no viscous part),
+// -c_i / 24 (= -|T| grad N_i / 4, the element's G(i, x)) to the three
+// pressure-gradient sums and det to the lumped mass sum (scaled after the
+// walk).  For the order (p, q, c) an odd permutation of the element's own, det
+// and every cofactor change sign, w does not, so every contribution is
+// multiplied by -1.  M = -c_c is carried from the previous step: after q
+// leaves, the window (p, c) has d_p x d_c = -c_q; after p leaves, (q, c) has
+// d_q x d_c = c_p.
+template <int P, int MODE>
+struct WalkNode {
+  int k;  // slot (in rows of the group)
+  V3<typename Prec<P>::T> d, v;
+  typename Slots<P, MODE>::V a;
+};
+
+template <int P, int RW, int MODE>
+__device__ __forceinline__ void walk_lane(const uint8_t* __restrict__ st, int nbytes,
+                                          const T4<typename Prec<P>::T>* nb0, const T2<typename Prec<P>::T>* nb1,
+                                          Slots<P, MODE>& acc, const V3<typename Prec<P>::T>& u2i,
+                                          typename Prec<P>::T kmu, Acc<P>& detsum) {
+  using T = typename Prec<P>::T;
+  using Node = WalkNode<P, MODE>;
+  constexpr T kg = T(-1.0 / 24.0);  // the pressure-gradient sums are accumulated scaled
+  auto load = [&](unsigned w) {
+    Node nd;
+    nd.k = (int)(w & WALK_POS) * RW;
+    const T4<T> x = nb0[nd.k];
+    nd.d = V3<T>{x.x, x.y, x.z};
+    if constexpr (MODE != NODAL) {
+      const T2<T> y = nb1[nd.k];
+      nd.v = V3<T>{x.w, y.x, y.y};
+      nd.a = acc.load(nd.k);
+    }
+    return nd;
+  };
+  for (int s = 0; s < nbytes;) {
+    // a segment: two filling bytes with the element count in their upper
+    // bits, then one byte per element
+    const unsigned f1 = st[s], f2 = st[s + 1];
+    const int cnt = (int)((f1 >> 5) | ((f2 >> 5) << 3));
+    const uint8_t* e = st + s + 2;
+    s += 2 + cnt;
+    Node p = load(f1), n0 = load(f2);
+    V3<T> M{};
+    if constexpr (MODE != NODAL) {
+      M = cross_fma(n0.d, p.d);
+      p.v = add(u2i, p.v);
+    }
+    unsigned w = e[0];
+    Node n1 = load(w), n2;
+    // The next step's node is loaded while this element is evaluated (never
+    // one of p, q, c: the walk is encoded that way; the last step reloads its
+    // own node, unused).
+    auto step = [&](Node& q, Node& c, Node& nx, int i) {
+      const unsigned wn = e[i + 1 < cnt ? i + 1 : i];
+      nx = load(wn);
+      const bool neg = (w & WALK_NEG) != 0u, evq = (w & WALK_EVQ) != 0u;
+      const T f = neg ? T(-1) : T(1);
+      const V3<T> cp = cross_fma(q.d, c.d);
+      const T det = dot_fma(p.d, cp);
+      if constexpr (P == NSI_MIXED_F32_ACC64) detsum.add(f * det);
+      else detsum.v = fma(f, det, detsum.v);
+      if constexpr (MODE != NODAL) {
+        const V3<T> cq = cross_fma(c.d, p.d);
+        V3<T> w3{p.v.x + q.v.x + c.v.x, p.v.y + q.v.y + c.v.y, p.v.z + q.v.z + c.v.z};
+        if constexpr (MODE == ASSEMBLE) {
+          const V3<T> ci{M.x - (cp.x + cq.x), M.y - (cp.y + cq.y), M.z - (cp.z + cq.z)};
+          const T kv = mul_rn(kmu, rcp_fast(det));
+          w3 = V3<T>{fma(kv, ci.x, w3.x), fma(kv, ci.y, w3.y), fma(kv, ci.z, w3.z)};
+          const T fg = neg ? -kg : kg;
+          const T ap = dot_fma(w3, cp), aq = dot_fma(w3, cq), ac = dot_fma(w3, M);
+          if constexpr (P == NSI_FP64) {
+            auto upd = [&](typename Slots<P, MODE>::V& a, T fs, T v) {
+              a.x.x = fma(fs, v, a.x.x);
+              a.x.y = fma(fg, ci.x, a.x.y);
+              a.y.x = fma(fg, ci.y, a.y.x);
+              a.y.y = fma(fg, ci.z, a.y.y);
+            };
+            upd(p.a, f, ap);
+            upd(q.a, f, aq);
+            upd(c.a, neg ? T(1) : T(-1), ac);
+          } else {
+            const float2 gg = make_float2(fg, fg), cxy = make_float2(ci.x, ci.y);
+            auto upd = [&](typename Slots<P, MODE>::V& a, float fs, float v) {
+              a.g = fma2(gg, cxy, a.g);
+              a.r = fma2(make_float2(fg, fs), make_float2(ci.z, v), a.r);
+            };
+            upd(p.a, f, ap);
+            upd(q.a, f, aq);
+            upd(c.a, -f, ac);
+          }
+        } else {
+          p.a = fma(f, dot_fma(w3, cp), p.a);
+          q.a = fma(f, dot_fma(w3, cq), q.a);
+          c.a = fma(neg ? T(1) : T(-1), dot_fma(w3, M), c.a);
+        }
+        M = V3<T>{evq ? cq.x : -cp.x, evq ? cq.y : -cp.y, evq ? cq.z : -cp.z};
+        acc.store(evq ? q.k : p.k, Slots<P, MODE>::pick(evq, q.a, p.a));
+      }
+      if (!evq) {
+        p = q;
+        if constexpr (MODE != NODAL) p.v = add(u2i, q.v);
+      }
+      w = wn;
+    };
+    // q, c and the node in flight rotate through n0, n1, n2: three steps per
+    // iteration bring them back to their places, so the newest node never
+    // moves between registers (only p's update depends on the walk)
+    int i = 0;
+    for (; i + 3 <= cnt; i += 3) {
+      step(n0, n1, n2, i);
+      step(n1, n2, n0, i + 1);
+      step(n2, n0, n1, i + 2);
+    }
+    if (i < cnt) {
+      step(n0, n1, n2, i);
+      if (i + 1 < cnt) {
+        step(n1, n2, n0, i + 1);
+        acc.store(n2.k, n2.a);
+      } else {
+        acc.store(n1.k, n1.a);
+      }
+    } else {
+      acc.store(n0.k, n0.a);
+    }
+    acc.store(p.k, p.a);
+  }
+}
+
+// every byte of a row's sub-walks within the row's bytes and its slots (debug)
+__device__ __forceinline__ bool walk_ok(const uint8_t* st, int nbytes, int nsub, int slots) {
+  if (nbytes == 0) return true;
+  if (nbytes < nsub) return false;
+  int at = nsub;
+  for (int k = 0; k < nsub; ++k) {
+    const int end = at + st[k];
+    if (end > nbytes) return false;
+    while (at < end) {
+      if (at + 2 >= end) return false;
+      const int cnt = (st[at] >> 5) | ((st[at + 1] >> 5) << 3);
+      if (cnt < 1 || at + 2 + cnt > end) return false;
+      for (int b = 0; b < 2 + cnt; ++b)
+        if ((int)(st[at + b] & WALK_POS) >= slots) return false;
+      at += 2 + cnt;
+    }
+  }
+  return at == nbytes;
+}
+
+// ---------------------------------------------------------------- groups ---
+// One row of a group, as each of its lanes sees it.
+struct GroupRow {
+  int32_t rs, re, w0, w1;  // CSR and walk bounds
+  int dp;
+};
+// the bounds and diagonal positions of rows [r0, r0 + RW) into shared memory
+// (rows past the mesh's end get its last bound)
+template <int RW>
+__device__ __forceinline__ void copy_rows(const WalkMesh& m, unsigned char* info, int64_t r0, int lane) {
+  int32_t* b = reinterpret_cast<int32_t*>(info);
+  if (lane <= RW) {
+    const int64_t i = min(r0 + lane, m.n);
+    cp_async4(b + lane, m.row_ptr + i);
+    cp_async4(b + RW + 1 + lane, m.walk_ptr + i);
+  }
+  if (lane < RW / 4) cp_async4(b + 2 * (RW + 1) + lane, m.diag_pos + r0 + 4 * lane);  // (padded past n)
+}
+template <int RW>
+__device__ __forceinline__ GroupRow read_row(const unsigned char* info, int t) {
+  const int32_t* b = reinterpret_cast<const int32_t*>(info);
+  GroupRow r;
+  r.rs = b[t];
+  r.re = b[t + 1];
+  r.w0 = b[RW + 1 + t];
+  r.w1 = b[RW + 2 + t];
+  r.dp = info[8 * (RW + 1) + t];
+  return r;
+}
+// slots of a row: its off-diagonal entries (none for a long row, which
+// long_rows_kernel computes)
+__device__ __forceinline__ int row_slots(const GroupRow& r) {
+  return r.dp == DIAG_LONG ? 0 : max(0, r.re - r.rs - 1);
+}
+// row position of slot s (the diagonal has none)
+__device__ __forceinline__ int slot_pos(int s, int dp) { return s + (s >= dp ? 1 : 0); }
+
+// the walk bytes of the group's rows into shared memory, as aligned words
+__device__ __forceinline__ void copy_walk(const WalkMesh& m, unsigned char* dst, int32_t w0, int32_t w1, int lane) {
+  const int off = w0 & 3;
+  const uint32_t* src = reinterpret_cast<const uint32_t*>(m.walk + (w0 - off));
+  const int words = (w1 - w0 + off + 3) >> 2;
+  for (int k = lane; k < words; k += 32) cp_async4(reinterpret_cast<uint32_t*>(dst) + k, src + k);
+}
+
+template <int P>
+__device__ __forceinline__ Acc<P> scaled(const Acc<P>& s, typename Prec<P>::T c) {
+  Acc<P> r;
+  if constexpr (P == NSI_MIXED_F32_ACC64) {
+    const float p = __fmul_rn(s.hi, c);  // c * (hi + lo), product error kept
+    r.hi = p;
+    r.lo = fmaf(s.lo, c, fmaf(s.hi, c, -p));
+  } else {
+    r.v = s.v * c;
+  }
+  return r;
+}
+// a + (the same accumulator of the lane `off` away): the error terms first (a
+// commutative sum), so that both lanes of a pair hold bitwise the same value
+template <int P>
+__device__ __forceinline__ void merge_lanes(Acc<P>& a, int off) {
+  if constexpr (P == NSI_MIXED_F32_ACC64) {
+    const float hi = __shfl_xor_sync(0xffffffffu, a.hi, off), lo = __shfl_xor_sync(0xffffffffu, a.lo, off);
+    a.lo += lo;
+    a.add(hi);
+  } else {
+    a.v += __shfl_xor_sync(0xffffffffu, a.v, off);
+  }
+}
+
+// The group loop of one warp: groups g, g + stride, ... below g_end; `src`
+// gives a group's mesh.  H lanes per row: lane = h * RW + t works on row t.
+// The next group's row bounds are copied under the current walk, its walk
+// bytes and column indices under the merge, and its records are loaded under
+// the write-out.
+template <int P, int H, int MODE, bool DEBUG, typename Source>
+__device__ __forceinline__ void group_loop(const Source& src, int g, int stride, int g_end, unsigned char* smem,
+                                           const GroupLay& lay) {
+  using T = typename Prec<P>::T;
+  using Out = typename Prec<P>::Out;
+  constexpr unsigned FULL = 0xffffffffu;
+  constexpr int RW = 32 / H;
+  int lane = threadIdx.x & 31, t = lane & (RW - 1), h = lane / RW;
+  if (g >= g_end) return;  // warp-uniform
+  // The lane's place, made opaque between the phases of a group: otherwise the
+  // compiler keeps every phase's addresses in registers over the whole loop.
+  auto refresh = [&]() { asm volatile("" : "+r"(lane), "+r"(t), "+r"(h)); };
+  auto nb0 = [&]() { return reinterpret_cast<T4<T>*>(smem) + t; };
+  auto nb1 = [&]() { return reinterpret_cast<T2<T>*>(smem + lay.nb1) + t; };
+  // one lane's accumulators
+  auto slots = [&](int p) { return Slots<P, MODE>(smem + lay.acc + p * lay.plane, lay.N); };
+
+  constexpr int UT = P == NSI_FP64 ? 4 : 16 / H;  // records of a lane in flight
+
+  auto copy_cols = [&](const WalkMesh& m, int32_t c0, int32_t c1) {
+    if (DEBUG && c1 - c0 > lay.L) return;  // reported below
+    for (int k = lane; k < c1 - c0; k += 32) cp_async4(reinterpret_cast<int32_t*>(smem + lay.cols) + k, m.col_idx + c0 + k);
+  };
+  // a row's record and its first UT slots' per lane, col its column indices
+  struct Recs {
+    NodeRec<P> me, r[UT];
+  };
+  auto load_recs = [&](Recs& v, const WalkMesh& m, const GroupRow& r, const int32_t* col, int64_t i, int s0) {
+    const int ns = row_slots(r);
+    const int64_t self = min(i, m.n - 1);
+    if (s0 == h) v.me.load(m.rec, self);
+#pragma unroll
+    for (int c = 0; c < UT; ++c) {
+      const int s = s0 + c * H;
+      int64_t k = s < ns ? (int64_t)col[slot_pos(s, r.dp)] : self;  // (past the row: its own, unused)
+      if (DEBUG && (k < 0 || k >= m.n)) {
+        atomicOr(m.err, ERR_BAD_INDEX);
+        k = self;
+      }
+      v.r[c].load(m.rec, k);
+    }
+  };
+  // the group's slots: edge vectors from the row's node, velocities, zeroed
+  // sums; 2 rho/120 u_i of the row's own node
+  V3<T> u2i;
+  auto put = [&](Recs& v, const WalkMesh& m, const FieldView& f, const GroupRow& r, int64_t i) {
+    const T kc = kc_of<T>(f), kc2 = kc + kc;
+    const V3<T> ui = v.me.vel();
+    u2i = V3<T>{mul_rn(kc2, ui.x), mul_rn(kc2, ui.y), mul_rn(kc2, ui.z)};
+    const int ns = DEBUG ? min(row_slots(r), lay.W) : row_slots(r);
+#pragma unroll 1
+    for (int s0 = h; s0 < ns; s0 += UT * H) {
+      if (s0 != h) load_recs(v, m, r, m.col_idx + r.rs, i, s0);
+#pragma unroll
+      for (int c = 0; c < UT; ++c) {
+        if (s0 + c * H >= ns) break;
+        const int k = (s0 + c * H) * RW;
+        const V3<T> d = v.r[c].minus(v.me);
+        if constexpr (MODE == NODAL) {
+          nb0()[k] = T4<T>{d.x, d.y, d.z, T(0)};
+        } else {
+          const V3<T> u = v.r[c].vel();
+          nb0()[k] = T4<T>{d.x, d.y, d.z, mul_rn(kc, u.x)};
+          nb1()[k] = T2<T>{mul_rn(kc, u.y), mul_rn(kc, u.z)};
+        }
+      }
+    }
+    if constexpr (MODE != NODAL)
+      for (int b = 16 * lane; b < H * lay.plane; b += 16 * 32)
+        *reinterpret_cast<float4*>(smem + lay.acc + b) = make_float4(0.f, 0.f, 0.f, 0.f);
+    __syncwarp();
+  };
+  // a group's column indices in shared memory, or in memory where they do not fit (debug)
+  auto cols_of = [&](const WalkMesh& m, const GroupRow& r, int32_t c0, int32_t c1) {
+    return DEBUG && c1 - c0 > lay.L ? m.col_idx + r.rs
+                                    : reinterpret_cast<const int32_t*>(smem + lay.cols) + (r.rs - c0);
+  };
+
+  // the first group
+  int at = src.find(g);
+  GroupRow row;
+  int32_t wb, we, base, end;
+  {
+    const WalkMesh& m = src.item(at).m;
+    const int64_t r0 = (int64_t)(g - src.item(at).group0) * RW;
+    copy_rows<RW>(m, smem + lay.info, r0, lane);
+    cp_async_wait_all();
+    __syncwarp();
+    row = read_row<RW>(smem + lay.info, t);
+    base = __shfl_sync(FULL, row.rs, 0), end = __shfl_sync(FULL, row.re, RW - 1);
+    wb = __shfl_sync(FULL, row.w0, 0), we = __shfl_sync(FULL, row.w1, RW - 1);
+    if (!DEBUG || we - wb <= lay.S) copy_walk(m, smem + lay.walk, wb, we, lane);
+    copy_cols(m, base, end);
+    cp_async_wait_all();
+    __syncwarp();
+    Recs v;
+    load_recs(v, m, row, cols_of(m, row, base, end), r0 + t, h);
+    __syncwarp();
+    put(v, m, src.item(at).f, row, r0 + t);
+  }
+  while (true) {
+    const WalkMesh& m = src.item(at).m;
+    const FieldView& f = src.item(at).f;
+    const WalkOut<MODE>& o = src.item(at).o;
+    const int64_t i = (int64_t)(g - src.item(at).group0) * RW + t;
+    const bool valid = i < m.n;
+    const int ns = row_slots(row);
+    const int L = end - base, lb = row.rs - base;
+    bool fits = true;
+    if (DEBUG) {
+      fits = L <= lay.L && we - wb <= lay.S && !__any_sync(FULL, ns > lay.W || (ns > 0 && row.dp > ns));
+      if (!fits && lane == 0) atomicOr(m.err, ERR_STAR);
+    }
+    const T kmass = kmass_of<T>(f);
+    refresh();
+
+    // the next group's row bounds, in flight during the walk
+    const int gn = g + stride;
+    const bool more = gn < g_end;  // warp-uniform
+    const int atn = more ? src.find(gn) : at;
+    if (more) copy_rows<RW>(src.item(atn).m, smem + lay.info, (int64_t)(gn - src.item(atn).group0) * RW, lane);
+
+    // 1. the row's sub-walk h
+    refresh();
+    Acc<P> detsum;
+    detsum.zero();
+    if (fits && ns > 0) {
+      Slots<P, MODE> acc = slots(h);
+      if constexpr (MODE == ASSEMBLE && P == NSI_FP64) {
+        acc.a0 += t;
+        acc.a1 += t;
+      } else if constexpr (MODE != NODAL) {
+        acc.a += t;
+      }
+      const uint8_t* st = (smem + lay.walk) + (row.w0 - wb) + (wb & 3);
+      const int nb = row.w1 - row.w0;
+      if (DEBUG && !walk_ok(st, nb, H, ns)) {
+        atomicOr(m.err, ERR_STAR);
+      } else if (nb > 0) {
+        // (each lane finds its bytes first: the row's lanes walk together)
+        int b = H;
+        for (int k = 0; k < h; ++k) b += st[k];
+        walk_lane<P, RW, MODE>(st + b, st[h], nb0(), nb1(), acc, u2i, kmu_of<T>(f), detsum);
+      }
+    }
+    __syncwarp();
+
+    // the next group's walk bytes and column indices
+    refresh();
+    GroupRow rown = row;
+    int32_t wbn = 0, wen = 0, basen = 0, endn = 0;
+    if (more) {
+      cp_async_wait_all();
+      __syncwarp();
+      const WalkMesh& mn = src.item(atn).m;
+      rown = read_row<RW>(smem + lay.info, t);
+      basen = __shfl_sync(FULL, rown.rs, 0), endn = __shfl_sync(FULL, rown.re, RW - 1);
+      wbn = __shfl_sync(FULL, rown.w0, 0), wen = __shfl_sync(FULL, rown.w1, RW - 1);
+      if (!DEBUG || wen - wbn <= lay.S) copy_walk(mn, smem + lay.walk, wbn, wen, lane);
+      copy_cols(mn, basen, endn);
+    }
+    V3<T> un{T(0), T(0), T(0)};
+    if (valid) un = load_vec<T>(f.un, i);
+    // the time step's A_static: the lane's first entries and the diagonal,
+    // read before the slice is written (A may be A_static)
+    constexpr int NS = 8;
+    [[maybe_unused]] Out as[NS], sd = Out(0);
+    if constexpr (MODE == STEP) {
+      const Out* As = static_cast<const Out*>(o.A_static) + base;
+#pragma unroll
+      for (int c = 0; c < NS; ++c)
+        if (lane + 32 * c < L) as[c] = As[lane + 32 * c];
+      if (h == 0 && ns > 0) sd = As[lb + row.dp];
+    }
+#pragma unroll
+    for (int off = RW; off < 32; off <<= 1) merge_lanes<P>(detsum, off);
+
+    // 2. the lanes' sums merged, the diagonal from the partition of unity
+    // (sum_b grad N_b = 0):
+    //   A(i,i) = lumped mass - sum_{j != i} A(i,j)   (convection + viscous parts)
+    //   G(i,i) = 1/3 sum_{j != i} G(i,j)             (each element adds c_i to three
+    //                                                 off-diagonal entries and the diagonal)
+    // and the row moved into CSR order for the write-out (over the slots' edge
+    // vectors and velocities, which are no longer needed)
+    [[maybe_unused]] float dlo = 0.f;  // mixed64: the error term of the diagonal's leading part dhi
+    [[maybe_unused]] float dhi = 0.f;
+    const int len = !fits || row.dp == DIAG_LONG ? 0 : row.re - row.rs;
+    const int zl = fits && row.dp == DIAG_LONG ? row.re - row.rs : 0;  // a long row's entries
+    if constexpr (MODE == ASSEMBLE) {
+      using S = Slots<P, ASSEMBLE>;
+      Acc<P> ra;
+      ra.zero();
+      T4<T>* stage = reinterpret_cast<T4<T>*>(smem);
+      // the planes' sums of the lane's slots and their entries
+      auto each = [&](auto&& use) {
+#pragma unroll 1
+        for (int s = h; s < (fits ? ns : 0); s += H) {
+          typename S::V v = slots(0).load(s * RW + t);
+#pragma unroll
+          for (int p = 1; p < H; ++p) v = S::sum(v, slots(p).load(s * RW + t));
+          use(v, lb + slot_pos(s, row.dp));
+        }
+      };
+      if constexpr (P == NSI_FP64) {
+        double gx = 0.0, gy = 0.0, gz = 0.0;
+        each([&](const typename S::V& v, int e) {
+          ra.add(v.x.x);
+          gx += v.x.y;
+          gy += v.y.x;
+          gz += v.y.y;
+          stage[e] = T4<T>{v.x.x, v.x.y, v.y.x, v.y.y};
+        });
+#pragma unroll
+        for (int off = RW; off < 32; off <<= 1) {
+          merge_lanes<P>(ra, off);
+          gx += __shfl_xor_sync(FULL, gx, off);
+          gy += __shfl_xor_sync(FULL, gy, off);
+          gz += __shfl_xor_sync(FULL, gz, off);
+        }
+        if (h == 0 && len > 0)
+          stage[lb + row.dp] = T4<T>{fma(kmass, detsum.v, -ra.v), gx * (1.0 / 3.0), gy * (1.0 / 3.0), gz * (1.0 / 3.0)};
+      } else {
+        float2 g = make_float2(0.f, 0.f);
+        float gz = 0.f;
+        each([&](const typename S::V& v, int e) {
+          ra.add(v.r.y);
+          g = add2(g, v.g);
+          gz += v.r.x;
+          stage[e] = T4<T>{v.r.y, v.g.x, v.g.y, v.r.x};
+        });
+#pragma unroll
+        for (int off = RW; off < 32; off <<= 1) {
+          merge_lanes<P>(ra, off);
+          g.x += __shfl_xor_sync(FULL, g.x, off);
+          g.y += __shfl_xor_sync(FULL, g.y, off);
+          gz += __shfl_xor_sync(FULL, gz, off);
+        }
+        float ad;
+        if constexpr (P == NSI_MIXED_F32_ACC64) {
+          Acc<P> d = scaled<P>(detsum, kmass);
+          d.add(-ra.hi);
+          d.lo -= ra.lo;
+          dhi = ad = d.hi;
+          dlo = d.lo;
+        } else {
+          ad = fmaf(kmass, detsum.v, -ra.v);
+        }
+        if (h == 0 && len > 0)
+          stage[lb + row.dp] = T4<T>{ad, g.x * (1.0f / 3.0f), g.y * (1.0f / 3.0f), gz * (1.0f / 3.0f)};
+      }
+      for (int q = h; q < zl; q += H) stage[lb + q] = T4<T>{T(0), T(0), T(0), T(0)};  // a long row, computed later
+    } else if constexpr (MODE == STEP) {
+      using S = Slots<P, STEP>;
+      Acc<P> ra;
+      ra.zero();
+      T* stage = reinterpret_cast<T*>(smem);
+#pragma unroll 2
+      for (int s = h; s < (fits ? ns : 0); s += H) {
+        const int k = s * RW + t;
+        T v = slots(0).load(k);
+#pragma unroll
+        for (int p = 1; p < H; ++p) v += slots(p).load(k);
+        ra.add(v);
+        stage[lb + slot_pos(s, row.dp)] = v;
+      }
+#pragma unroll
+      for (int off = RW; off < 32; off <<= 1) merge_lanes<P>(ra, off);
+      T ad;
+      if constexpr (P == NSI_MIXED_F32_ACC64) {
+        dhi = ad = -ra.hi;
+        dlo = -ra.lo;
+      } else {
+        ad = -ra.v;
+      }
+      if (h == 0 && len > 0) stage[lb + row.dp] = ad;
+      for (int q = h; q < zl; q += H) stage[lb + q] = T(0);  // a long row: A_static kept, C added later
+    }
+    // lumped RHS: (sum_e rho |T_e| / (4 dt)) u^n_i, spread over the row's lanes
+    if (valid) {
+      Out* Rh = static_cast<Out*>(o.rhs);
+      const T unk[3] = {mul_rn(kmass, un.x), mul_rn(kmass, un.y), mul_rn(kmass, un.z)};
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+        if (k % H == h) store_acc(Rh + k * m.n + i, scaled<P>(detsum, unk[k]));
+      if constexpr (MODE == NODAL) {
+        if (h == 0) store_acc(static_cast<Out*>(o.dt_rho) + i, scaled<P>(detsum, kmass));
+        if (h == H - 1) {
+          T kmr;
+          if constexpr (sizeof(T) == 8) kmr = o.kmr;
+          else kmr = o.kmrf;
+          store_acc(static_cast<Out*>(o.mass_rho) + i, scaled<P>(detsum, kmr));
+        }
+      }
+    }
+    cp_async_wait_all();
+    __syncwarp();
+    // the next group's records, in flight during the write-out
+    Recs v{};
+    if (more) {
+      const WalkMesh& mn = src.item(atn).m;
+      load_recs(v, mn, rown, cols_of(mn, rown, basen, endn), (int64_t)(gn - src.item(atn).group0) * RW + t, h);
+    }
+
+    // 3. the group's contiguous slice of the outputs
+    refresh();
+    if constexpr (MODE == ASSEMBLE) {
+      const T4<T>* stage = reinterpret_cast<const T4<T>*>(smem);
+      Out* A = static_cast<Out*>(o.A) + base;
+      Out *G = static_cast<Out*>(o.G) + base, *G1 = G + m.nnz, *G2 = G1 + m.nnz;
+      // (streaming stores: the outputs leave L2 before the records do)
+      auto write = [&](auto&& put) {
+#pragma unroll 1
+        for (int k = lane; k < (fits ? L : 0); k += 32) put(k, stage[k]);
+      };
+      if constexpr (P == NSI_MIXED_F32_ACC64) {
+        // converted to double exactly from the bits; an infinite, NaN or
+        // subnormal A again by a rare second pass, then every diagonal by the
+        // double nearest its compensated pair
+        bool slow = false;
+        write([&](int k, const T4<T>& v) {
+          slow |= special_float(v.x);
+          __stcs(A + k, float_double(v.x));
+          __stcs(G + k, float_double(v.y));
+          __stcs(G1 + k, float_double(v.z));
+          __stcs(G2 + k, float_double(v.w));
+        });
+        if (__any_sync(FULL, slow)) {
+          for (int k = lane; k < L; k += 32) {
+            const float a = stage[k].x;
+            if (special_float(a)) A[k] = nonfinite_bits(a) ? nonfinite_double(a) : (double)a;
+          }
+        }
+        __syncwarp();
+        if (fits && h == 0 && len > 0)
+          A[lb + row.dp] = nonfinite_bits(dhi) ? nonfinite_double(dhi) : pair_double(dhi, dlo);
+      } else {
+        write([&](int k, const T4<T>& v) {
+          __stcs(A + k, v.x);
+          __stcs(G + k, v.y);
+          __stcs(G1 + k, v.z);
+          __stcs(G2 + k, v.w);
+        });
+      }
+    } else if constexpr (MODE == STEP) {
+      const T* stage = reinterpret_cast<const T*>(smem);
+      const Out* As = static_cast<const Out*>(o.A_static) + base;
+      Out* A = static_cast<Out*>(o.A) + base;
+      auto value = [&](int k) -> Out {  // C(u) of entry k in the output type
+        const T c = stage[k];
+        if constexpr (P == NSI_MIXED_F32_ACC64)
+          return special_float(c) ? (nonfinite_bits(c) ? nonfinite_double(c) : (double)c) : float_double(c);
+        else
+          return c;
+      };
+      if (fits) {
+#pragma unroll
+        for (int c = 0; c < NS; ++c)
+          if (lane + 32 * c < L) A[lane + 32 * c] = as[c] + value(lane + 32 * c);
+        for (int k = lane + 32 * NS; k < L; k += 32) A[k] = As[k] + value(k);
+      }
+      if constexpr (P == NSI_MIXED_F32_ACC64) {  // the diagonal's sum is a compensated pair
+        __syncwarp();
+        if (fits && h == 0 && ns > 0)
+          A[lb + row.dp] = sd + (nonfinite_bits(dhi) ? nonfinite_double(dhi) : pair_double(dhi, dlo));
+      }
+    }
+    if (!more) return;
+    __syncwarp();  // the next group reuses the staging
+    refresh();
+    put(v, src.item(atn).m, src.item(atn).f, rown, (int64_t)(gn - src.item(atn).group0) * RW + t);
+    g = gn;
+    at = atn;
+    row = rown;
+    wb = wbn;
+    we = wen;
+    base = basen;
+    end = endn;
+  }
+}
+
+
+// where a group's mesh comes from: the one mesh of a launch, or a batch's
+template <int MODE>
+struct OneMesh {
+  const WalkItem<MODE>& one;
+  __device__ __forceinline__ int find(int) const { return 0; }
+  __device__ __forceinline__ const WalkItem<MODE>& item(int) const { return one; }
+};
+
+template <int P, int H, int MODE, bool DEBUG>
+__global__ void __launch_bounds__(32 * MAX_WARPS, P == NSI_FP64 ? 2 : 4)
+    gather_persistent_kernel(const __grid_constant__ WalkItem<MODE> item, GroupLay lay, int g0, int g_end) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  const int warps = blockDim.x >> 5, w = threadIdx.x >> 5;
+  group_loop<P, H, MODE, DEBUG>(OneMesh<MODE>{item}, g0 + (int)blockIdx.x * warps + w, (int)gridDim.x * warps, g_end,
+                                smem_raw + w * lay.total, lay);
+}
+
+// ------------------------------------------------------ batched kernel ---
+// The meshes with two lanes per row first, then those with four: a warp takes
+// its share of the first's groups, then of the second's, so that every mesh is
+// assembled as by its own launch.
+struct BatchArgs {
+  int32_t count[2];  // meshes
+  int32_t total[2];  // row groups
+  WalkItem<ASSEMBLE> item[NSI_MAX_BATCH];
+};
+static_assert(sizeof(BatchArgs) + 2 * sizeof(GroupLay) <= 32764, "kernel parameters");
+
+struct BatchMesh {
+  const BatchArgs& args;
+  int first, count;
+  // the mesh of group g: the last item with group0 <= g
+  __device__ __forceinline__ int find(int g) const {
+    int lo = first, hi = first + count - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (args.item[mid].group0 <= g) lo = mid;
+      else hi = mid - 1;
+    }
+    return lo;
+  }
+  __device__ __forceinline__ const WalkItem<ASSEMBLE>& item(int k) const { return args.item[k]; }
+};
+
+template <int P>
+__global__ void __launch_bounds__(32 * MAX_WARPS, P == NSI_FP64 ? 2 : 4)
+    batched_kernel(const __grid_constant__ BatchArgs args, GroupLay lay2, GroupLay lay4) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  const int warps = blockDim.x >> 5, w = threadIdx.x >> 5;
+  const int all = (int)gridDim.x * warps, me = (int)blockIdx.x * warps + w;
+  unsigned char* smem = smem_raw + w * max(lay2.total, lay4.total);
+  group_loop<P, 2, ASSEMBLE, false>(BatchMesh{args, 0, args.count[0]}, me, all, args.total[0], smem, lay2);
+  __syncwarp();
+  // (the warps with one group less of the first kind begin the second)
+  const int start = me - args.total[0] % all;
+  group_loop<P, 4, ASSEMBLE, false>(BatchMesh{args, args.count[0], args.count[1]}, start < 0 ? start + all : start, all,
+                                    args.total[1], smem, lay4);
+}
+
+template <int P>
+__global__ void __launch_bounds__(256) pack_kernel(WalkMesh m, FieldView f) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i < m.n) pack_node<P>(m, f, m.rec, i);
+}
+
+// the node records of every mesh of a batch in one launch: a block packs the
+// rows of 8 consecutive groups of 16, or of 16 of 8
+template <int P>
+__global__ void __launch_bounds__(128) batched_pack_kernel(const __grid_constant__ BatchArgs args) {
+  const int blocks2 = (args.total[0] + 7) / 8;
+  const int kind = (int)blockIdx.x < blocks2 ? 0 : 1;
+  const int rw = kind ? 8 : 16;
+  const int g = ((int)blockIdx.x - kind * blocks2) * (128 / rw) + (int)threadIdx.x / rw;
+  if (g >= args.total[kind]) return;
+  const BatchMesh src{args, kind * args.count[0], args.count[kind]};
+  const WalkItem<ASSEMBLE>& it = src.item(src.find(g));
+  const int64_t i = (int64_t)(g - it.group0) * rw + threadIdx.x % rw;
+  if (i < it.m.n) pack_node<P>(it.m, it.f, it.m.rec, i);
+}
+
+// ----------------------------------------------------------- launchers ---
+WalkMesh walk_mesh(const NsiHandle* h, void* rec) {
+  WalkMesh m;
+  m.n = h->n;
+  m.nnz = h->nnz;
+  m.row_ptr = h->row_ptr;
+  m.col_idx = h->col_idx;
+  m.walk_ptr = h->walk_ptr;
+  m.walk = h->walk;
+  m.diag_pos = h->diag_pos;
+  m.xyz64 = h->xyz64;
+  m.xyz_hi = h->xyz_hi;
+  m.xyz_lo = h->xyz_lo;
+  m.rec = rec ? rec : h->rec;
+  m.err = h->err;
+  return m;
+}
+
+// the shared memory of one warp's group of 32 / H rows
+GatherSmem group_smem(int precision, int mode, int H, int W, int L, int S) {
+  GatherSmem g = gather_smem(precision, 32 / H, W, L, S, mode != ASSEMBLE);
+  g.H = H;
+  g.xs = 0;  // A_static is read in the write-out
+  if (mode != ASSEMBLE) g.ab = mode == STEP ? g.tb : 0;
+  return g;
+}
+
+template <typename K>
+nsi_status allow_smem(K kernel, std::once_flag& once, cudaError_t& err) {
+  std::call_once(once, [&] { err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX); });
+  return err == cudaSuccess ? NSI_OK : cuda_fail(err, "cudaFuncSetAttribute(row gather)");
+}
+
+// blocks of a persistent launch: as many as are resident at once, no more
+// than the groups need
+template <typename K>
+nsi_status resident_grid(K kernel, int warps, size_t smem, int64_t groups, int64_t* grid) {
+  int per_sm = 0, sms = 0, dev = 0;
+  NSI_CUDA(cudaGetDevice(&dev));
+  NSI_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  NSI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 32 * warps, smem));
+  *grid = std::max<int64_t>(1, std::min<int64_t>((groups + warps - 1) / warps, (int64_t)std::max(1, per_sm) * sms));
+  return NSI_OK;
+}
+
+template <int P, int H, int MODE, bool DEBUG>
+nsi_status run_groups(NsiHandle* h, const WalkItem<MODE>& item, int64_t row0, int64_t row1, cudaStream_t s) {
+  static std::once_flag once;
+  static cudaError_t err = cudaSuccess;
+  const auto kernel = gather_persistent_kernel<P, H, MODE, DEBUG>;
+  nsi_status st = allow_smem(kernel, once, err);
+  if (st) return st;
+  constexpr int RW = 32 / H;
+  const GatherPlan& pl = h->plan;
+  const GatherSmem lay = group_smem(P, MODE, H, pl.w, pl.max_block_entries, pl.max_block_steps);
+  const size_t smem = lay.total() * pl.warps;
+  const int64_t g0 = row0 / RW, g1 = (row1 + RW - 1) / RW;
+  int64_t grid = 0;
+  if ((st = resident_grid(kernel, pl.warps, smem, g1 - g0, &grid))) return st;
+  if (h->ev_start) NSI_CUDA(cudaEventRecord(h->ev_start, s));
+  kernel<<<grid, 32 * pl.warps, smem, s>>>(item, GroupLay(lay), (int)g0, (int)g1);
+  if (h->ev_stop) NSI_CUDA(cudaEventRecord(h->ev_stop, s));
+  return check_launch("gather_persistent_kernel");
+}
+
+template <int P, int MODE>
+nsi_status run_lanes(NsiHandle* h, const WalkItem<MODE>& item, int64_t row0, int64_t row1, cudaStream_t s) {
+  switch (h->nsub) {
+    case 2:
+      return h->debug ? run_groups<P, 2, MODE, true>(h, item, row0, row1, s)
+                      : run_groups<P, 2, MODE, false>(h, item, row0, row1, s);
+    default:
+      return h->debug ? run_groups<P, 4, MODE, true>(h, item, row0, row1, s)
+                      : run_groups<P, 4, MODE, false>(h, item, row0, row1, s);
+  }
+}
+
+}  // namespace
+
+template <int P>
+nsi_status launch_pack(NsiHandle* h, const FieldView& f, void* rec, cudaStream_t s) {
+  pack_kernel<P><<<(h->n + 255) / 256, 256, 0, s>>>(walk_mesh(h, rec), f);
+  return check_launch("pack_kernel");
+}
+
+template <int P>
+nsi_status launch_gather(NsiHandle* h, const FieldView& f, const OutView& o, int64_t row0, int64_t row1, void* rec,
+                         cudaStream_t s) {
+  const WalkItem<ASSEMBLE> item{walk_mesh(h, rec), f, {o.A, o.G, o.rhs}, 0};
+  return run_lanes<P, ASSEMBLE>(h, item, row0, row1, s);
+}
+
+template <int P>
+nsi_status launch_step(NsiHandle* h, const FieldView& f, const StepView& o, bool nodal, cudaStream_t s) {
+  if (nodal) {
+    const WalkItem<NODAL> item{walk_mesh(h, nullptr), f, {o.rhs, o.dt_rho, o.mass_rho, o.kmr, o.kmrf}, 0};
+    return run_lanes<P, NODAL>(h, item, 0, h->n, s);
+  }
+  const WalkItem<STEP> item{walk_mesh(h, nullptr), f, {o.A, o.rhs, o.A_static}, 0};
+  return run_lanes<P, STEP>(h, item, 0, h->n, s);
+}
+
+template <int P>
+nsi_status launch_batched(NsiHandle* const* hs, const NsiFields* fs, const NsiOutputs* os, int count,
+                          cudaStream_t s) {
+  static BatchArgs args;  // host staging of the by-value kernel argument
+  static std::mutex mu;
+  std::lock_guard<std::mutex> lock(mu);
+  int warps = MAX_WARPS, W[2] = {1, 1}, L[2] = {0, 0}, S[2] = {0, 0}, item = 0;
+  for (int kind = 0; kind < 2; ++kind) {  // two lanes per row, then four
+    const int H = kind ? 4 : 2, rw = 32 / H;
+    int64_t groups = 0;
+    args.count[kind] = 0;
+    for (int k = 0; k < count; ++k) {
+      const NsiHandle* h = hs[k];
+      if (h->nsub != H) continue;
+      const GatherPlan& pl = h->plan;
+      warps = std::min(warps, pl.warps);
+      W[kind] = std::max(W[kind], pl.w);
+      L[kind] = std::max(L[kind], pl.max_block_entries);
+      S[kind] = std::max(S[kind], pl.max_block_steps);
+      args.item[item++] = WalkItem<ASSEMBLE>{walk_mesh(h, nullptr), fields_of(&fs[k]),
+                                             {os[k].A_val, os[k].G_val, os[k].rhs}, (int)groups};
+      ++args.count[kind];
+      groups += (h->n + rw - 1) / rw;
+      if (groups > INT32_MAX / 2) return fail(NSI_ERR_UNSUPPORTED, "too many rows in a batch");
+    }
+    args.total[kind] = (int)groups;
+  }
+  const int64_t groups = (int64_t)args.total[0] + args.total[1];
+  if (groups == 0) return NSI_OK;
+  const GatherSmem lay2 = group_smem(P, ASSEMBLE, 2, W[0], L[0], S[0]);
+  const GatherSmem lay4 = group_smem(P, ASSEMBLE, 4, W[1], L[1], S[1]);
+  if (!lay2.group_fits() || !lay4.group_fits())  // (each mesh's fits, and so do the maxima of W and L)
+    return fail(NSI_ERR_UNSUPPORTED, "batched meshes need more shared memory than a group has");
+  const size_t bytes = std::max(args.count[0] ? lay2.total() : 0, args.count[1] ? lay4.total() : 0);
+  while (warps > 1 && bytes * warps > SMEM_MAX) --warps;
+  if (bytes > SMEM_MAX) return fail(NSI_ERR_UNSUPPORTED, "batched meshes need more shared memory than a block has");
+  static std::once_flag once;
+  static cudaError_t err = cudaSuccess;
+  nsi_status st = allow_smem(batched_kernel<P>, once, err);
+  if (st) return st;
+  batched_pack_kernel<P><<<(args.total[0] + 7) / 8 + (args.total[1] + 15) / 16, 128, 0, s>>>(args);
+  if ((st = check_launch("batched_pack_kernel"))) return st;
+  int64_t grid = 0;
+  if ((st = resident_grid(batched_kernel<P>, warps, bytes * warps, groups, &grid))) return st;
+  batched_kernel<P><<<grid, 32 * warps, bytes * warps, s>>>(args, GroupLay(lay2), GroupLay(lay4));
+  return check_launch("batched_kernel");
+}
+
+#define NSI_INSTANTIATE(P)                                                                                          \
+  template nsi_status launch_pack<P>(NsiHandle*, const FieldView&, void*, cudaStream_t);                            \
+  template nsi_status launch_gather<P>(NsiHandle*, const FieldView&, const OutView&, int64_t, int64_t, void*,       \
+                                       cudaStream_t);                                                               \
+  template nsi_status launch_step<P>(NsiHandle*, const FieldView&, const StepView&, bool, cudaStream_t);            \
+  template nsi_status launch_batched<P>(NsiHandle* const*, const NsiFields*, const NsiOutputs*, int, cudaStream_t);
+NSI_INSTANTIATE(NSI_FP64)
+NSI_INSTANTIATE(NSI_MIXED_F32_ACC64)
+NSI_INSTANTIATE(NSI_MIXED_F32_ACC32)
+#undef NSI_INSTANTIATE
+
+int gather_kernel_regs(int precision) {
+  cudaFuncAttributes a{};
+  cudaError_t e;
+  if (precision == NSI_FP64) e = cudaFuncGetAttributes(&a, gather_persistent_kernel<NSI_FP64, 2, ASSEMBLE, false>);
+  else if (precision == NSI_MIXED_F32_ACC64)
+    e = cudaFuncGetAttributes(&a, gather_persistent_kernel<NSI_MIXED_F32_ACC64, 2, ASSEMBLE, false>);
+  else e = cudaFuncGetAttributes(&a, gather_persistent_kernel<NSI_MIXED_F32_ACC32, 2, ASSEMBLE, false>);
+  return e == cudaSuccess ? a.numRegs : 96;
+}
+
+}  // namespace nsi

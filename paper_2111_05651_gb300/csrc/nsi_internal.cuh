@@ -79,46 +79,60 @@ struct alignas(32) D4 {
 };
 
 struct GatherPlan {
-  int rows_per_block = 0;     // threads per block = rows per block
-  int max_block_entries = 0;  // max over blocks of the CSR entries of the block's rows
-  int max_block_steps = 0;    // max over blocks of the walk steps of the block's rows
-  int w = 0;                  // slots per row of the layout (>= the longest row the kernels take, and
-                              // large enough that every block's entries fit R * w)
-  int64_t n_blocks = 0;
+  int rows_per_block = 0;     // the plan's name: 32, 64, 96 or 128
+  int warps = 0;              // warps per block, each with row groups of its own
+  int max_block_entries = 0;  // max over the groups of the CSR entries of a group's rows
+  int max_block_steps = 0;    // max over the groups of the walk bytes of a group's rows
+  int w = 0;                  // slots per row (>= the off-diagonal entries of the longest row the kernels
+                              // take, and large enough that every group's entries fit its staging)
 };
+// a mesh of fewer rows has four lanes per row in the row gather, others two
+// (measured equal at about 30 000 rows for the assembly and at 10 000 for the
+// time step)
+constexpr int64_t SMALL_MESH_ROWS = 10000;
+constexpr int SMEM_MAX = 200 * 1024;  // shared memory of one block
 
 // diag_pos value of a row the row gather leaves out ("long row": more than
 // 32 entries, or a star whose walk does not encode): the kernels give it no
 // elements and zero its slice; long_rows_kernel computes it afterwards
 constexpr uint8_t DIAG_LONG = 0xff;
 
-// Shared-memory layout of one row-gather block: R rows (one per thread), W
-// slots per row (the longest row of the mesh), L CSR entries and S walk
-// steps.  Slot q of row t lives at index q * R + t ("thread-interleaved"), so
-// the lanes of a warp touch consecutive records whichever slot each lane
-// uses: the element loop is free of shared-memory bank conflicts.
+// Shared-memory layout of one warp's group of the row gather: R rows, W slots
+// per row (the off-diagonal entries of the longest row of the mesh), H lanes
+// per row, L CSR entries and S walk bytes.  Slot q of row t lives at index
+// q * R + t ("row-interleaved"), so the lanes of a warp touch consecutive
+// records whichever slot each row uses: the element loop is free of
+// shared-memory bank conflicts.
 //   nb0   T[4] per slot: edge vector d = x_j - x_i and u_x of the neighbour
 //   nb1   T[2] per slot: u_y, u_z
-//   acc   accumulators per slot (ab bytes): A and the three sums of c_i
-//   col   int32 per CSR entry, read only while the records are gathered: it
-//         shares nb1's bytes (nb1 is written after a barrier)
-//   walk  one byte per step (copied as aligned 4-byte words, so S + 8 bytes)
-//   stat  (time-step kernels only) the block's slice of A_static
-// After the element loop, nb0 is reused to stage the finished values in CSR
-// order for the coalesced write-out.
+//   acc   H planes of accumulators per slot (ab bytes each): A and the three
+//         sums of c_i
+//   walk  the walk bytes (copied as aligned 4-byte words, so S + 8 bytes)
+//   stat  (step layouts) the rows' slice of A_static
+//   info  the next group's row bounds and diagonal positions
+// After the element loop, nb0 and nb1 are reused to stage the finished values
+// in CSR order for the coalesced write-out (4 T per entry), and past them for
+// the next group's column indices.
 // Used identically by the host (launch size) and the kernel (carving).
 struct GatherSmem {
   int R, W, L, S, tb, ab, ob, cr;  // ob: bytes of an output value; cr: components staged per write-out round
   int xs;                          // bytes per CSR entry of the time step's static slice (0: none)
+  int H = 1;                       // accumulator planes
   __host__ __device__ static size_t up16(size_t x) { return (x + 15) & ~size_t(15); }
   __host__ __device__ size_t N() const { return (size_t)R * W; }
   __host__ __device__ size_t nb0() const { return 0; }
   __host__ __device__ size_t nb1() const { return up16(nb0() + (size_t)4 * tb * N()); }
   __host__ __device__ size_t acc() const { return up16(nb1() + (size_t)2 * tb * N()); }
   __host__ __device__ size_t col() const { return nb1(); }  // (L <= N: 4 L bytes fit in nb1)
-  __host__ __device__ size_t walk() const { return up16(acc() + (size_t)ab * N()); }
+  __host__ __device__ size_t walk() const { return up16(acc() + (size_t)ab * H * N()); }
   __host__ __device__ size_t stat() const { return up16(walk() + (size_t)S + 8); }
-  __host__ __device__ size_t total() const { return up16(stat() + (size_t)xs * L); }
+  // the rows' bounds and diagonal positions
+  __host__ __device__ size_t info() const { return up16(stat() + (size_t)xs * L); }
+  // (a multiple of 32: the next warp's nb0 holds 32-byte aligned FP64 vectors)
+  __host__ __device__ size_t total() const { return (info() + 8 * (size_t)(R + 1) + R + 31) & ~size_t(31); }
+  // the column indices of the next group's entries, past the staged entries (4 T each)
+  __host__ __device__ size_t cols() const { return up16(nb0() + (size_t)4 * tb * L); }
+  __host__ __device__ bool group_fits() const { return cols() + (size_t)4 * L <= acc(); }
   // the write-out stages cr components of the block's L entries in nb0
   __host__ __device__ size_t stage_bytes() const { return (size_t)cr * L * ob; }
   __host__ __device__ bool stage_fits() const { return stage_bytes() <= nb1() - nb0(); }
@@ -170,7 +184,8 @@ struct NsiHandle {
   // row-gather map: every row's element walk (one byte per step)
   int32_t* walk_ptr = nullptr;  // [n+1]
   uint8_t* walk = nullptr;      // [walk_ptr[n] + 8]
-  uint8_t* diag_pos = nullptr;  // [n] position of the diagonal inside its row (rows <= 32 entries)
+  int nsub = 2;                 // sub-walks per row
+  uint8_t* diag_pos = nullptr;  // [n + 32] position of the diagonal inside its row (rows <= 32 entries)
   unsigned long long* elem_pos = nullptr;  // [E] element-position map (rows <= 32 entries), or null
   // edge-fan map (one word per CSR entry) and its block partition of the rows
   bool fan_ok = false;
@@ -179,7 +194,6 @@ struct NsiHandle {
   int64_t fan_blocks = 0;
   bool use_fan = false;         // row-gather mode runs the edge-fan kernel
   bool atomic_agg = false;      // atomic mode runs the warp-aggregated atomics (else one atomic per value)
-  bool persistent = false;      // row-gather mode runs the persistent grid (set by create: mixed64)
   int64_t long_rows = 0;        // rows the row gather leaves out, recomputed by long_rows_kernel
   int32_t* long_list = nullptr;  // [long_rows] their node ids
   int32_t* long_ptr = nullptr;   // [long_rows + 1] into long_inc

@@ -4,21 +4,8 @@
 //                   perform_assembly_in_global_system of Listing 1 fused),
 //                   scatter by global atomics or, colour by colour, by plain
 //                   read-add-write (deterministic)
-//   gather_kernel   one CSR row per thread: the row's owner walks every
-//                   element around its node (the element walk built at
-//                   create), accumulates the row privately and the block
-//                   writes its contiguous slice of A, G and rhs once,
-//                   coalesced (no atomics, no zeroing, deterministic)
-//   gather_persistent_kernel  the same as a persistent grid (a CTA's next
-//                   block of rows starts its copies under the current
-//                   block's write-out)
 //   fan_kernel      one CSR entry per thread, walking the ring of elements
 //                   around its edge (autotuning candidate)
-//   batched_kernel  the row gather over many meshes in one persistent launch
-//                   (their node records packed by one batched_pack_kernel)
-//   step_kernel     one time step with cached geometry (A_static + C(u),
-//                   rhs), or the paper's per-node outputs
-//   step_persistent_kernel  the same as a persistent grid (mixed32)
 //   vjp_kernel      adjoint of R(u, mu) = A(u) u - b, element per thread
 //   residual_kernel R(u, mu) without the matrix (both with an exact
 //                   companion for badly shaped elements in double)
@@ -33,6 +20,7 @@
 //   gather_values_kernel, add_values_kernel  pack / add the interface-row
 //                   values of the element-partition exchange
 //
+// The row gather, the time step and the batched launch are in nsi_gather.cu.
 // Formulas: see the element-arithmetic comment in nsi_internal.cuh.
 #include <algorithm>
 #include <cstdio>
@@ -40,213 +28,9 @@
 #include <mutex>
 #include <vector>
 
-#include "nsi_internal.cuh"
+#include "nsi_device.cuh"
 
 namespace nsi {
-
-// ------------------------------------------------------------ views ------
-struct MeshView {
-  int64_t n, E, nnz;
-  const int32_t* __restrict__ row_ptr;
-  const int32_t* __restrict__ col_idx;
-  const int4* __restrict__ lnods;
-  const int32_t* __restrict__ walk_ptr;
-  const uint8_t* __restrict__ walk;
-  const uint8_t* __restrict__ diag_pos;
-  const D4* __restrict__ xyz64;
-  const float4* __restrict__ xyz_hi;
-  const float4* __restrict__ xyz_lo;
-  const void* __restrict__ rec;
-  const uint32_t* __restrict__ fan;
-  const int32_t* __restrict__ fan_blk;
-  unsigned* err;
-};
-
-// Physical constants of the element formulas, precomputed on the host in
-// double (the float copies are rounded once): rho/120 (convection), mu/6
-// (viscous) and rho/(24 dt) (lumped mass).
-struct FieldView {
-  const void* u[3];
-  const void* un[3];
-  double kc, kmu, kmass;
-  float kcf, kmuf, kmassf;
-};
-
-template <typename T>
-__device__ __forceinline__ T kc_of(const FieldView& f) {
-  if constexpr (sizeof(T) == 8) return f.kc;
-  else return f.kcf;
-}
-template <typename T>
-__device__ __forceinline__ T kmu_of(const FieldView& f) {
-  if constexpr (sizeof(T) == 8) return f.kmu;
-  else return f.kmuf;
-}
-template <typename T>
-__device__ __forceinline__ T kmass_of(const FieldView& f) {
-  if constexpr (sizeof(T) == 8) return f.kmass;
-  else return f.kmassf;
-}
-
-struct OutView {
-  void* A;
-  void* G;
-  void* rhs;
-};
-
-static MeshView view_of(const NsiHandle* h) {
-  MeshView m;
-  m.n = h->n;
-  m.E = h->E;
-  m.nnz = h->nnz;
-  m.row_ptr = h->row_ptr;
-  m.col_idx = h->col_idx;
-  m.lnods = h->lnods;
-  m.walk_ptr = h->walk_ptr;
-  m.walk = h->walk;
-  m.diag_pos = h->diag_pos;
-  m.xyz64 = h->xyz64;
-  m.xyz_hi = h->xyz_hi;
-  m.xyz_lo = h->xyz_lo;
-  m.rec = h->rec;
-  m.fan = h->fan;
-  m.fan_blk = h->fan_blk;
-  m.err = h->err;
-  return m;
-}
-
-static FieldView fields_of(const NsiFields* f) {
-  FieldView v;
-  for (int k = 0; k < 3; ++k) {
-    v.u[k] = f->u[k];
-    v.un[k] = f->u_n[k] ? f->u_n[k] : f->u[k];
-  }
-  v.kc = f->rho / 120.0;
-  v.kmu = f->mu / 6.0;
-  v.kmass = f->rho / (24.0 * f->dt);
-  v.kcf = (float)v.kc;
-  v.kmuf = (float)v.kmu;
-  v.kmassf = (float)v.kmass;
-  return v;
-}
-
-// precision traits: compute type T, output type Out
-template <int P>
-struct Prec;
-template <>
-struct Prec<NSI_FP64> {
-  using T = double;
-  using Out = double;
-};
-template <>
-struct Prec<NSI_MIXED_F32_ACC64> {
-  using T = float;
-  using Out = double;
-};
-template <>
-struct Prec<NSI_MIXED_F32_ACC32> {
-  using T = float;
-  using Out = float;
-};
-
-template <typename T>
-__device__ __forceinline__ T rcp(T x);
-template <>
-__device__ __forceinline__ float rcp<float>(float x) {
-  return __frcp_rn(x);
-}
-template <>
-__device__ __forceinline__ double rcp<double>(double x) {
-  return 1.0 / x;
-}
-
-// node coordinates: exact double, or a float hi/lo pair whose difference
-// gives edge vectors to ~2^-48 relative before the float arithmetic starts
-template <int P>
-struct NodeX;
-template <>
-struct NodeX<NSI_FP64> {
-  V3<double> x;
-  __device__ __forceinline__ void load(const MeshView& m, int64_t v) {
-    D4 p = m.xyz64[v];
-    x = {p.x, p.y, p.z};
-  }
-  __device__ __forceinline__ V3<double> minus(const NodeX& o) const { return sub(x, o.x); }
-};
-template <int P>
-struct NodeX {
-  V3<float> hi, lo;
-  __device__ __forceinline__ void load(const MeshView& m, int64_t v) {
-    float4 a = __ldg(m.xyz_hi + v);
-    float4 b = __ldg(m.xyz_lo + v);
-    hi = {a.x, a.y, a.z};
-    lo = {b.x, b.y, b.z};
-  }
-  __device__ __forceinline__ V3<float> minus(const NodeX& o) const { return add(sub(hi, o.hi), sub(lo, o.lo)); }
-};
-
-template <typename T>
-__device__ __forceinline__ V3<T> load_vec(const void* const* comp, int64_t v) {
-  return {__ldg(static_cast<const T*>(comp[0]) + v), __ldg(static_cast<const T*>(comp[1]) + v),
-          __ldg(static_cast<const T*>(comp[2]) + v)};
-}
-
-// asynchronous global -> shared copies (cp.async): many gathers in flight per
-// thread without holding registers
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-// wait until at most the most recent committed group is still in flight
-__device__ __forceinline__ void cp_async_wait_prior() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
-
-// ---------------------------------------------------------- node records ---
-// One record per node, rebuilt every call from the handle's coordinates and
-// the caller's velocities, so that the row-gather kernel fetches a neighbour
-// with one 32-byte (mixed) or 64-byte (FP64) request instead of five:
-//   mixed: {hx, hy, hz, ux} {uy, uz, lo_xy, lo_z}, lo_* the top 16 bits of
-//          the float low parts (coordinates kept to ~2^-32 relative)
-//   FP64:  {x, y, z, 0} {ux, uy, uz, 0} as doubles
-template <int P>
-__device__ __forceinline__ void pack_node(const MeshView& m, const FieldView& f, void* __restrict__ rec, int64_t i) {
-  if constexpr (P == NSI_FP64) {
-    const D4 x = m.xyz64[i];
-    const V3<double> u = load_vec<double>(f.u, i);
-    D4* r = static_cast<D4*>(rec) + 2 * i;
-    r[0] = D4{x.x, x.y, x.z, 0.0};
-    r[1] = D4{u.x, u.y, u.z, 0.0};
-  } else {
-    const float4 hi = __ldg(m.xyz_hi + i);
-    const float4 lo = __ldg(m.xyz_lo + i);
-    const V3<float> u = load_vec<float>(f.u, i);
-    uint4* r = static_cast<uint4*>(rec) + 2 * i;
-    r[0] = make_uint4(__float_as_uint(hi.x), __float_as_uint(hi.y), __float_as_uint(hi.z), __float_as_uint(u.x));
-    r[1] = make_uint4(__float_as_uint(u.y), __float_as_uint(u.z),
-                      (__float_as_uint(lo.x) >> 16) | (__float_as_uint(lo.y) & 0xffff0000u),
-                      __float_as_uint(lo.z) & 0xffff0000u);
-  }
-}
-
-template <int P>
-__global__ void __launch_bounds__(256) pack_kernel(MeshView m, FieldView f, void* __restrict__ rec) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i < m.n) pack_node<P>(m, f, rec, i);
-}
-
-__device__ __forceinline__ V3<float> record_lo(float w6, float w7) {
-  const unsigned a = __float_as_uint(w6), b = __float_as_uint(w7);
-  return {__uint_as_float(a << 16), __uint_as_float(a & 0xffff0000u), __uint_as_float(b & 0xffff0000u)};
-}
 
 // ------------------------------------------------ element-centric kernel ---
 template <typename T, typename Out>
@@ -444,1070 +228,6 @@ __global__ void __launch_bounds__(256) elem_kernel(MeshView m, FieldView f, OutV
 #pragma unroll
       for (int k = 0; k < 3; ++k) add_out<T, Out>(R + k * m.n + vv[a], r3[k], false);
     }
-  }
-}
-
-// ---------------------------------------------------- row-gather kernel ---
-// Register accumulator of one output value: plain T, or a compensated float
-// pair (TwoSum) for the mixed mode with double output.
-template <int P>
-struct Acc {
-  using T = typename Prec<P>::T;
-  T v;
-  __device__ __forceinline__ void zero() { v = T(0); }
-  __device__ __forceinline__ void add(T x) { v += x; }
-};
-template <>
-struct Acc<NSI_MIXED_F32_ACC64> {
-  float hi, lo;
-  __device__ __forceinline__ void zero() { hi = lo = 0.0f; }
-  __device__ __forceinline__ void add(float x) {
-    float s, e;
-    two_sum(hi, x, s, e);
-    hi = s;
-    lo += e;
-  }
-};
-
-__device__ __forceinline__ void store_acc(double* p, const Acc<NSI_FP64>& a) { *p = a.v; }
-__device__ __forceinline__ void store_acc(float* p, const Acc<NSI_MIXED_F32_ACC32>& a) { *p = a.v; }
-// The double nearest hi + lo for a renormalised float pair (|lo| <= ulp(hi) /
-// 2) with a finite hi, without branches: the double of |hi| from its bits, lo
-// (with hi's sign taken out) added as an integer k of the double's units in
-// the last place (|k| <= 2^28), hi's sign set last.  When |hi| is a power of
-// two and the sum lies below it, k counts the half-size units of the binade
-// below.  Zero gives zero; a tiny |hi| (below 2^-75, where the scale of k would
-// leave the float range) is handled at 2^100 times its size, the exponent
-// taken back in the result.  Infinite and NaN values are the callers' (a test
-// for them here costs the write-out loop several percent).
-__device__ __forceinline__ double normalised_pair_double(float hi, float lo) {
-  const unsigned u0 = __float_as_uint(hi);
-  const bool tiny = ((u0 >> 23) & 0xffu) < 52u;
-  const float sc = tiny ? 0x1p100f : 1.0f;
-  const float h2 = hi * sc, l2 = lo * sc;  // exact
-  const unsigned uh = __float_as_uint(h2);
-  const unsigned eh = (uh >> 23) & 0xffu;
-  const float ls = __uint_as_float(__float_as_uint(l2) ^ (uh & 0x80000000u));
-  const unsigned below = ((uh << 9) == 0u && ls < 0.0f) ? 1u : 0u;
-  const int k = __float2int_rn(ls * __uint_as_float((306u + below - eh) << 23));
-  const unsigned long long mag =
-      ((unsigned long long)(uh & 0x7fffffffu) << 29) + ((tiny ? 796ull : 896ull) << 52);
-  const unsigned long long r = (mag + (unsigned long long)(long long)k) | ((unsigned long long)(uh & 0x80000000u) << 32);
-  return __longlong_as_double((u0 << 1) == 0u ? (long long)((unsigned long long)(u0 & 0x80000000u) << 32)
-                                              : (long long)r);
-}
-// an infinite or NaN accumulator (hi) as a double of the same class
-__device__ __forceinline__ double nonfinite_double(float hi) { return __longlong_as_double(f32_to_f64_bits(hi)); }
-// true if the exponent bits of x are all ones (infinite or NaN)
-__device__ __forceinline__ bool nonfinite_bits(float x) { return (__float_as_uint(x) | 0x807fffffu) == 0xffffffffu; }
-// true for an infinite, NaN or subnormal float (the cases float_double leaves out)
-__device__ __forceinline__ bool special_float(float x) {
-  const unsigned e = __float_as_uint(x) & 0x7f800000u;
-  return e == 0x7f800000u || (e == 0u && (__float_as_uint(x) & 0x007fffffu) != 0u);
-}
-// the double equal to a normal or zero float, from its bit pattern: the
-// exponent rebiased (+896), the 23 mantissa bits moved to the top of the
-// double's 52; the sign kept.  A subnormal float (below 2^-126 in magnitude)
-// gives a signed zero; infinite and NaN floats are not handled (the values
-// converted this way are the pressure-gradient sums, functions of the
-// coordinates a handle validates, far inside the float range for any mesh
-// whose float element arithmetic is meaningful).
-__device__ __forceinline__ double float_double(float x) {
-  const unsigned u = __float_as_uint(x);
-  const unsigned a = u & 0x7fffffffu;
-  const unsigned hi = (a < 0x00800000u ? 0u : (a >> 3) + (896u << 20)) | (u & 0x80000000u);
-  return __hiloint2double((int)hi, a < 0x00800000u ? 0 : (int)(u << 29));
-}
-// the double nearest hi + lo of a pair with a finite hi: renormalised first
-// (Fast2Sum)
-__device__ __forceinline__ double pair_double(float hi, float lo) {
-  const float s = hi + lo;
-  const float l = lo - (s - hi);
-  return normalised_pair_double(s, l);
-}
-__device__ __forceinline__ void store_acc(double* p, const Acc<NSI_MIXED_F32_ACC64>& a) {
-  *p = nonfinite_bits(a.hi) ? nonfinite_double(a.hi) : pair_double(a.hi, a.lo);
-}
-
-template <typename T>
-struct alignas(4 * sizeof(T)) T4 {
-  T x, y, z, w;
-};
-template <typename T>
-struct alignas(2 * sizeof(T)) T2 {
-  T x, y;
-};
-
-// Accumulators of the block's slots in shared memory: the A value and the
-// pressure-gradient values (sums of -c_i / 24) of each entry.  A slot is only
-// touched by the thread owning its row until the final write-out, so no
-// atomics are needed.  add3() updates three DISTINCT slots (the three other
-// nodes of one element sit at three different positions of the row), so all
-// three loads are issued before the stores.
-template <int P>
-struct AccSmem;
-// paired float arithmetic (one instruction for two lanes of a float2, each
-// rounded like its scalar counterpart); a - b is formed as b * (-1) + a with a
-// single rounding
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
-// error-free sum of pairs (TwoSum lane by lane): h + x = s + e exactly; s
-// replaces h and e is added to the error term l
-__device__ __forceinline__ void two_sum2(float2& h, float2& l, float2 x) {
-  const float2 s = add2(h, x);
-  const float2 bb = sub2(s, h);
-  const float2 e = add2(sub2(h, sub2(s, bb)), sub2(x, bb));
-  h = s;
-  l = add2(l, e);
-}
-
-// Float slots hold (G_x, G_y, G_z, A): the two halves are
-// the pairs (G_x, G_y) and (G_z, A) of the paired updates.
-template <>
-struct AccSmem<NSI_MIXED_F32_ACC32> {
-  float4* __restrict__ a;
-  __device__ __forceinline__ AccSmem(unsigned char* p, size_t) : a(reinterpret_cast<float4*>(p)) {}
-  __device__ __forceinline__ void zero(int k) { a[k] = make_float4(0.f, 0.f, 0.f, 0.f); }
-  struct Slot {
-    float2 g, r;  // (G_x, G_y), (G_z, A)
-  };
-  __device__ __forceinline__ Slot load1(int k) const {
-    const float4 v = a[k];
-    return {make_float2(v.x, v.y), make_float2(v.z, v.w)};
-  }
-  __device__ __forceinline__ void store1(int k, const Slot& v) { a[k] = make_float4(v.g.x, v.g.y, v.r.x, v.r.y); }
-  static __device__ __forceinline__ void add(Slot& s, float2 gxy, float2 gz_a) {
-    s.g = add2(s.g, gxy);
-    s.r = add2(s.r, gz_a);
-  }
-  // sums over the row's slots t, t + R, ... (len of them), the diagonal's
-  // included: it is still zero here (zeroed with the others; the walk only
-  // ever adds zeros to it), so no test is needed (r[0]: A, r[1..3]: G_x..G_z)
-  __device__ __forceinline__ void row_sums(int t, int R, int len, Acc<NSI_MIXED_F32_ACC32>* r) const {
-#pragma unroll 4
-    for (int q = 0, k = t; q < len; ++q, k += R) {
-      const float4 v = a[k];
-      r[0].add(v.w); r[1].add(v.x); r[2].add(v.y); r[3].add(v.z);
-    }
-  }
-  __device__ __forceinline__ void set(int k, const Acc<NSI_MIXED_F32_ACC32>* r) {
-    a[k] = make_float4(r[1].v, r[2].v, r[3].v, r[0].v);
-  }
-  // finished values (A, G_x, G_y, G_z) of slot k
-  __device__ __forceinline__ T4<float> values(int k) const {
-    const float4 v = a[k];
-    return {v.w, v.x, v.y, v.z};
-  }
-};
-// mixed64: float slots (G_x, G_y, G_z, A) as mixed32.  An off-diagonal entry
-// sums the ~5 element terms of its edge (float products), so its float sum
-// carries a few roundings of those terms; the cancellation is in the
-// diagonal, the lumped mass minus the row's other entries, which row_sums
-// forms as a compensated sum (TwoSum over the row's entries, about 48
-// significant bits).  The diagonal's error term stays in a register of the
-// row's thread (dlo) until the write-out converts the pair to double.
-template <>
-struct AccSmem<NSI_MIXED_F32_ACC64> {
-  float4* __restrict__ hi;  // (G_x, G_y, G_z, A)
-  float dlo = 0.f;          // error term of this thread's diagonal A (set())
-  __device__ __forceinline__ AccSmem(unsigned char* p, size_t) : hi(reinterpret_cast<float4*>(p)) {}
-  __device__ __forceinline__ void zero(int k) { hi[k] = make_float4(0.f, 0.f, 0.f, 0.f); }
-  struct Slot {
-    float2 g, r;  // (G_x, G_y), (G_z, A)
-  };
-  __device__ __forceinline__ Slot load1(int k) const {
-    const float4 h = hi[k];
-    return {make_float2(h.x, h.y), make_float2(h.z, h.w)};
-  }
-  __device__ __forceinline__ void store1(int k, const Slot& v) { hi[k] = make_float4(v.g.x, v.g.y, v.r.x, v.r.y); }
-  static __device__ __forceinline__ void add(Slot& s, float2 gxy, float2 gz_a) {
-    s.g = add2(s.g, gxy);
-    s.r = add2(s.r, gz_a);
-  }
-  // sums over the row's slots, the diagonal's included (still zero): A
-  // compensated, G plain (r[0]: A, r[1..3]: G_x..G_z with zero error terms)
-  __device__ __forceinline__ void row_sums(int t, int R, int len, Acc<NSI_MIXED_F32_ACC64>* r) const {
-    float2 g = make_float2(0.f, 0.f), za = g;
-    float al = 0.f;
-#pragma unroll 4
-    for (int q = 0, k = t; q < len; ++q, k += R) {
-      const float4 h = hi[k];
-      g = add2(g, make_float2(h.x, h.y));
-      const float2 t2 = add2(za, make_float2(h.z, h.w));
-      const float bb = t2.y - za.y;
-      al += (za.y - (t2.y - bb)) + (h.w - bb);
-      za = t2;
-    }
-    r[0].hi = za.y; r[0].lo = al;
-    r[1].hi = g.x; r[1].lo = 0.f;
-    r[2].hi = g.y; r[2].lo = 0.f;
-    r[3].hi = za.x; r[3].lo = 0.f;
-  }
-  // the diagonal: A's leading part and G in the slot, A's error term kept
-  __device__ __forceinline__ void set(int k, const Acc<NSI_MIXED_F32_ACC64>* r) {
-    hi[k] = make_float4(r[1].hi, r[2].hi, r[3].hi, r[0].hi);
-    dlo = r[0].lo;
-  }
-};
-template <>
-struct AccSmem<NSI_FP64> {
-  T2<double>* __restrict__ a0;  // A, G_x
-  T2<double>* __restrict__ a1;  // G_y, G_z
-  __device__ __forceinline__ AccSmem(unsigned char* p, size_t N)
-      : a0(reinterpret_cast<T2<double>*>(p)), a1(reinterpret_cast<T2<double>*>(p) + N) {}
-  __device__ __forceinline__ void zero(int k) {
-    a0[k] = {0.0, 0.0};
-    a1[k] = {0.0, 0.0};
-  }
-  struct Slot {
-    T2<double> x, y;  // (A, G_x), (G_y, G_z)
-  };
-  __device__ __forceinline__ Slot load1(int k) const { return {a0[k], a1[k]}; }
-  __device__ __forceinline__ void store1(int k, const Slot& v) {
-    a0[k] = v.x;
-    a1[k] = v.y;
-  }
-  static __device__ __forceinline__ void update1(Slot& s, double A, double gx, double gy, double gz) {
-    s.x.x += A; s.x.y += gx; s.y.x += gy; s.y.y += gz;
-  }
-  __device__ __forceinline__ void row_sums(int t, int R, int len, Acc<NSI_FP64>* r) const {
-#pragma unroll 4
-    for (int q = 0, k = t; q < len; ++q, k += R) {
-      const T2<double> x = a0[k], y = a1[k];
-      r[0].add(x.x); r[1].add(x.y); r[2].add(y.x); r[3].add(y.y);
-    }
-  }
-  __device__ __forceinline__ void set(int k, const Acc<NSI_FP64>* r) {
-    a0[k] = {r[0].v, r[1].v};
-    a1[k] = {r[2].v, r[3].v};
-  }
-  __device__ __forceinline__ T4<double> values(int k) const {
-    const T2<double> x = a0[k], y = a1[k];
-    return {x.x, x.y, y.x, y.y};
-  }
-};
-
-// where the second half of a neighbour's record lands before the edge vectors
-// are formed: inside the slot's accumulators, which are zeroed right after
-template <int P>
-__device__ __forceinline__ void* staged_half(unsigned char* smem, const GatherSmem& lay, int k, int part) {
-  if constexpr (P == NSI_FP64) return reinterpret_cast<T2<double>*>(smem + lay.acc()) + (size_t)part * lay.N() + k;
-  else return reinterpret_cast<float4*>(smem + lay.acc()) + k;
-}
-
-// reciprocal of det: the float path uses the fast approximate division
-// (about 1 ulp); the double path refines the hardware's approximate double
-// reciprocal (rcp.approx.ftz.f64, relative error at most 2^-20 over 4 M
-// normal inputs measured on GB300) by two Newton-Raphson steps for 1/x,
-// r <- r + r (1 - x r), each of which squares the relative error (2^-40,
-// then below the double's rounding): four FMAs instead of the IEEE
-// division's longer sequence on GB300's slow FP64 pipe (3.18 -> 3.15 ms at
-// the 100^3 cube).  det is a normal number here (the mesh is validated at
-// create).
-__device__ __forceinline__ float rcp_fast(float x) { return __fdividef(1.0f, x); }
-__device__ __forceinline__ double rcp_fast(double x) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-#pragma unroll
-  for (int it = 0; it < 2; ++it) r = fma(r, fma(-x, r, 1.0), r);
-  return r;
-}
-
-// The element walk of one row (the element loop of phase 2), node i as the
-// origin.  A window of two neighbours (p, q) stays in registers with their
-// edge vectors, velocities and accumulators; every step brings one node c in
-// from shared memory, evaluates the element (i, p, q, c) if the step says so,
-// then writes back the accumulator of the node that leaves the window; c
-// always becomes q, and p keeps its node or takes q's (one register move of
-// a node per step instead of two selects).  With
-// c_p = d_q x d_c, c_q = d_c x d_p, c_c = d_p x d_q (cofactors of the
-// Jacobian, calculate_cartesian_derivatives, for the order (p, q, c)),
-// det = d_p . c_p and c_i = -(c_p + c_q + c_c), the element adds
-//   A(i,x) += w . c_x  (x = p, q, c),  w = rho/120 (2 u_i + u_p + u_q + u_c) + mu/(6 det) c_i
-// (FP64: the staged velocities already carry the factor rho/120)
-// -c_i / 24 (= -|T| grad N_i / 4, the element's G(i, x)) to the three
-// pressure-gradient values and det to the lumped mass sum (scaled after the
-// walk).  For the order (p, q, c) an odd permutation of the
-// element's own, det and every cofactor change sign, w does not, so every
-// contribution is multiplied by -1.  c_c is carried from the previous step:
-// after q leaves, the window (p, c) has d_p x d_c = -c_q; after p leaves,
-// (q, c) has d_q x d_c = c_p; m holds c_q or c_p and c_c = -sg m with sg = 1
-// or -1.
-template <typename T, typename Slot>
-struct WalkNode {
-  int k;  // shared-memory slot
-  V3<T> d, u;
-  Slot v;
-};
-
-template <int P>
-__device__ __forceinline__ WalkNode<typename Prec<P>::T, typename AccSmem<P>::Slot> walk_load(
-    int k, const T4<typename Prec<P>::T>* __restrict__ nb0, const T2<typename Prec<P>::T>* __restrict__ nb1,
-    const AccSmem<P>& acc) {
-  using T = typename Prec<P>::T;
-  const T4<T> a = nb0[k];
-  const T2<T> b = nb1[k];
-  return {k, {a.x, a.y, a.z}, {a.w, b.x, b.y}, acc.load1(k)};
-}
-
-template <int P, bool DEBUG>
-__device__ __forceinline__ void walk_row(const uint8_t* __restrict__ st, int nsteps, int len,
-                                         const T4<typename Prec<P>::T>* __restrict__ nb0,
-                                         const T2<typename Prec<P>::T>* __restrict__ nb1, AccSmem<P>& acc, int t,
-                                         int R, const V3<typename Prec<P>::T>& u2i, typename Prec<P>::T kc,
-                                         typename Prec<P>::T kmu, Acc<P>& detsum, unsigned* err) {
-  using T = typename Prec<P>::T;
-  using Node = WalkNode<T, typename AccSmem<P>::Slot>;
-  constexpr T kg = T(-1.0 / 24.0);  // the pressure-gradient sums are accumulated scaled
-  if (nsteps <= 0) return;
-  if (DEBUG) {
-    bool ok = nsteps >= 3 && !(st[0] & WALK_ELEM) && !(st[1] & WALK_ELEM);
-    for (int s = 0; s < nsteps; ++s) ok &= (int)(st[s] & WALK_POS) < len;
-    if (!ok) {
-      atomicOr(err, ERR_STAR);
-      return;
-    }
-  }
-  if (nsteps < 3) return;  // (every walk of a row with elements has at least 3 steps)
-  // a row's walk starts with two steps that only fill the window (the
-  // encoder begins the first path that way): their nodes are loaded directly,
-  // with the cofactor the first element carries, c_c = d_p x d_q
-  Node p = walk_load<P>((int)(st[0] & WALK_POS) * R + t, nb0, nb1, acc);
-  Node n0 = walk_load<P>((int)(st[1] & WALK_POS) * R + t, nb0, nb1, acc);
-  V3<T> m = cross(p.d, n0.d);
-  T sg = T(-1);  // c_c = -sg m
-  unsigned w = st[2];
-  Node n1 = walk_load<P>((int)(w & WALK_POS) * R + t, nb0, nb1, acc);
-  Node n2;
-  // One step: the element (i, p, q, c); the next step's node is loaded into
-  // nx (in flight while the element is evaluated; never one of p, q, c: the
-  // walk is encoded that way; the last step reloads its own node, unused).
-  // Afterwards the window is (p, c): p keeps its node or takes q's.
-  auto step = [&](Node& q, Node& c, Node& nx, int s) {
-    const unsigned wn = st[s + 1 < nsteps ? s + 1 : s];
-    nx = walk_load<P>((int)(wn & WALK_POS) * R + t, nb0, nb1, acc);
-    const V3<T> cp = cross(q.d, c.d), cq = cross(c.d, p.d);
-    const bool elem = (w & WALK_ELEM) != 0u;
-    if constexpr (P == NSI_FP64) {
-      if (elem) {  // (steps that only fill the window come first in a row: warp-uniform)
-        const T det = dot(p.d, cp);
-        const V3<T> ci{fma(sg, m.x, -(cp.x + cq.x)), fma(sg, m.y, -(cp.y + cq.y)), fma(sg, m.z, -(cp.z + cq.z))};
-        const T kv = kmu * rcp_fast(det);
-        const V3<T> w3{(u2i.x + p.u.x + q.u.x + c.u.x) + kv * ci.x, (u2i.y + p.u.y + q.u.y + c.u.y) + kv * ci.y,
-                       (u2i.z + p.u.z + q.u.z + c.u.z) + kv * ci.z};
-        const bool neg = (w & WALK_NEG) != 0u;  // orientation
-        const T f = neg ? T(-1) : T(1), fg = neg ? -kg : kg;
-        const T gx = fg * ci.x, gy = fg * ci.y, gz = fg * ci.z;
-        AccSmem<P>::update1(p.v, f * dot(w3, cp), gx, gy, gz);
-        AccSmem<P>::update1(q.v, f * dot(w3, cq), gx, gy, gz);
-        AccSmem<P>::update1(c.v, -f * sg * dot(w3, m), gx, gy, gz);
-        detsum.add(f * det);
-      }
-    } else {
-      // branch-free: a step that only fills the window adds zeros
-      const float det = dot(p.d, cp);
-      const V3<float> ci{fmaf(sg, m.x, -(cp.x + cq.x)), fmaf(sg, m.y, -(cp.y + cq.y)), fmaf(sg, m.z, -(cp.z + cq.z))};
-      const float kv = kmu * rcp_fast(elem ? det : 1.0f);
-      const V3<float> w3{kc * (u2i.x + p.u.x + q.u.x + c.u.x) + kv * ci.x,
-                         kc * (u2i.y + p.u.y + q.u.y + c.u.y) + kv * ci.y,
-                         kc * (u2i.z + p.u.z + q.u.z + c.u.z) + kv * ci.z};
-      const bool neg = (w & WALK_NEG) != 0u;
-      const float f = elem ? (neg ? -1.0f : 1.0f) : 0.0f;  // orientation, or 0
-      const float fg = elem ? (neg ? -kg : kg) : 0.0f;
-      const float2 gg = make_float2(fg, fg), ff = make_float2(fg, f);
-      const float2 gxy = __fmul2_rn(make_float2(ci.x, ci.y), gg);
-      AccSmem<P>::add(p.v, gxy, __fmul2_rn(make_float2(ci.z, dot(w3, cp)), ff));
-      AccSmem<P>::add(q.v, gxy, __fmul2_rn(make_float2(ci.z, dot(w3, cq)), ff));
-      AccSmem<P>::add(c.v, gxy, __fmul2_rn(make_float2(ci.z, dot(w3, m)), make_float2(fg, -f * sg)));
-      detsum.add(f * det);
-    }
-    const bool evq = (w & WALK_EVQ) != 0u;
-    const Node& lv = evq ? q : p;  // the node that leaves the window
-    acc.store1(lv.k, lv.v);
-    if (!evq) p = q;
-    m = evq ? cq : cp;
-    sg = evq ? T(1) : T(-1);
-    w = wn;
-  };
-  // The nodes q, c and the one in flight rotate through n0, n1, n2: three
-  // steps per iteration bring them back to their places, so the newest node
-  // never moves between registers (only p's update depends on the walk).
-  int s = 2;
-  for (; s + 3 <= nsteps; s += 3) {
-    step(n0, n1, n2, s);
-    step(n1, n2, n0, s + 1);
-    step(n2, n0, n1, s + 2);
-  }
-  if (s < nsteps) {
-    step(n0, n1, n2, s);
-    if (s + 1 < nsteps) {
-      step(n1, n2, n0, s + 1);
-      acc.store1(n2.k, n2.v);
-    } else {
-      acc.store1(n1.k, n1.v);
-    }
-  } else {
-    acc.store1(n0.k, n0.v);
-  }
-  acc.store1(p.k, p.v);
-}
-
-// Per-thread view of one block of rows [r0, r0 + blockDim.x) of one mesh.
-template <typename T>
-struct BlockRows {
-  int R, t, nrows, L, len, lb, s0, s1, dp;
-  int64_t i;
-  int32_t base;
-  V3<T> uni;
-  int zl;  // a long row's entries (its slice is zeroed in the write-out; 0 for the others)
-};
-
-// Phase 0 of a block: its bounds and the row's scalars (plain loads, in
-// flight until first used), then the asynchronous copies of the block's
-// column indices (into nb1) and walk steps.
-template <typename T>
-struct Phase0 {
-  int64_t r0;
-  int nrows, L, S;
-  int32_t base, sbase, rs, re, s0, s1;
-  int dp, zl;
-  V3<T> uni;
-};
-
-template <int P>
-__device__ __forceinline__ Phase0<typename Prec<P>::T> load_phase0(const MeshView& m, const FieldView& f, int64_t r0) {
-  using T = typename Prec<P>::T;
-  Phase0<T> p;
-  const int R = blockDim.x;
-  const int t = threadIdx.x;
-  const int64_t r_end = min(r0 + (int64_t)R, m.n);
-  p.r0 = r0;
-  p.nrows = (int)(r_end - r0);
-  p.base = m.row_ptr[r0];
-  p.L = m.row_ptr[r_end] - p.base;
-  p.sbase = m.walk_ptr[r0];
-  p.S = m.walk_ptr[r_end] - p.sbase;
-  p.rs = p.re = p.s0 = p.s1 = 0;
-  p.dp = p.zl = 0;
-  p.uni = V3<T>{T(0), T(0), T(0)};
-  const int soff = p.sbase & 3;  // walk bytes are copied as aligned 4-byte words
-  if (t < p.nrows) {
-    const int64_t i = r0 + t;
-    p.rs = m.row_ptr[i];
-    p.re = m.row_ptr[i + 1];
-    p.s0 = m.walk_ptr[i] - p.sbase + soff;
-    p.s1 = m.walk_ptr[i + 1] - p.sbase + soff;
-    p.dp = m.diag_pos[i];
-    p.uni = load_vec<T>(f.un, i);
-    if (p.dp == DIAG_LONG) {  // left to long_rows_kernel: no elements, a zeroed slice
-      p.zl = p.re - p.rs;
-      p.re = p.rs;
-      p.s1 = p.s0;
-      p.dp = 0;
-    }
-  }
-  return p;
-}
-
-template <bool DEBUG, typename T>
-__device__ __forceinline__ void issue_phase0(const MeshView& m, unsigned char* smem, const GatherSmem& lay,
-                                             const Phase0<T>& p) {
-  const int R = blockDim.x;
-  const int t = threadIdx.x;
-  if (DEBUG && (p.L > lay.L || p.S > lay.S || R != lay.R)) return;  // reported by stage_records
-  int32_t* col = reinterpret_cast<int32_t*>(smem + lay.col());
-  uint8_t* walk = smem + lay.walk();
-  for (int k = t; k < p.L; k += R) cp_async4(&col[k], m.col_idx + p.base + k);
-  const int soff = p.sbase & 3;
-  const uint32_t* src = reinterpret_cast<const uint32_t*>(m.walk + (p.sbase - soff));
-  const int words = (p.S + soff + 3) >> 2;
-  for (int k = t; k < words; k += R) cp_async4(reinterpret_cast<uint32_t*>(walk) + k, src + k);
-}
-
-// Phase 1 of a block whose phase-0 copies are in flight: every neighbour's
-// record (calculate_transients for the row, asynchronous copies all in
-// flight at once), turned into edge vectors d = x_j - x_i (the row's own
-// record, its diagonal slot, gives the origin) and velocities in nb0/nb1
-// (FP64: scaled by kc = rho/120, the convection weight, once per slot instead
-// of once per element step: 3.09 -> 3.02 ms at the 100^3 cube; the float
-// walks keep the product in the step, 2% faster there); the accumulators
-// zeroed.  Returns false (block-uniform) if the block does not
-// fit the layout.
-template <int P, bool DEBUG, typename Accum>
-__device__ __forceinline__ bool stage_records(const MeshView& m, unsigned char* smem, const GatherSmem& lay,
-                                              Accum& acc, const Phase0<typename Prec<P>::T>& p,
-                                              BlockRows<typename Prec<P>::T>& b, typename Prec<P>::T kc) {
-  using T = typename Prec<P>::T;
-  const int R = blockDim.x;
-  const int t = threadIdx.x;
-  if (DEBUG && (p.L > lay.L || p.S > lay.S || R != lay.R)) {
-    if (t == 0) atomicOr(m.err, ERR_STAR);
-    return false;
-  }
-  T4<T>* __restrict__ nb0 = reinterpret_cast<T4<T>*>(smem + lay.nb0());
-  T2<T>* __restrict__ nb1 = reinterpret_cast<T2<T>*>(smem + lay.nb1());
-  const int32_t* col = reinterpret_cast<const int32_t*>(smem + lay.col());
-  cp_async_wait_all();
-  __syncthreads();
-
-  const int len = p.re - p.rs;
-  const int lb = p.rs - p.base;
-  if (t < p.nrows) {
-    const unsigned char* recs = static_cast<const unsigned char*>(m.rec);
-    constexpr int RB = P == NSI_FP64 ? 64 : 32;
-    for (int q = 0, k = t; q < len; ++q, k += R) {
-      const int j = col[lb + q];
-      if (DEBUG && (j < 0 || j >= m.n)) {
-        atomicOr(m.err, ERR_BAD_INDEX);
-        continue;
-      }
-      const unsigned char* r = recs + (size_t)j * RB;
-      if constexpr (P == NSI_FP64) {
-        cp_async16(&nb0[k], r);
-        cp_async16(reinterpret_cast<char*>(&nb0[k]) + 16, r + 16);
-        cp_async16(staged_half<P>(smem, lay, k, 0), r + 32);
-        cp_async16(staged_half<P>(smem, lay, k, 1), r + 48);
-      } else {
-        cp_async16(&nb0[k], r);
-        cp_async16(staged_half<P>(smem, lay, k, 0), r + 16);
-      }
-    }
-  }
-  // every row's column indices have been read: nb1, which holds them, may now
-  // be written
-  __syncthreads();
-  if (t < p.nrows) {
-    cp_async_wait_all();
-    if (len > 0) {
-      const int kd = p.dp * R + t;
-      if constexpr (P == NSI_FP64) {
-        const T4<T> hi = nb0[kd];
-        const V3<T> xi{hi.x, hi.y, hi.z};
-        for (int q = 0, k = t; q < len; ++q, k += R) {
-          const T4<T> h = nb0[k];
-          const T2<T> ua = *static_cast<T2<T>*>(staged_half<P>(smem, lay, k, 0));
-          const T2<T> ub = *static_cast<T2<T>*>(staged_half<P>(smem, lay, k, 1));
-          nb0[k] = T4<T>{h.x - xi.x, h.y - xi.y, h.z - xi.z, kc * ua.x};
-          nb1[k] = T2<T>{kc * ua.y, kc * ub.x};
-          acc.zero(k);
-        }
-      } else {
-        const T4<T> hi = nb0[kd];
-        const float4 si = *static_cast<float4*>(staged_half<P>(smem, lay, kd, 0));
-        const V3<float> xh{hi.x, hi.y, hi.z};
-        const V3<float> xl = record_lo(si.z, si.w);
-        for (int q = 0, k = t; q < len; ++q, k += R) {
-          const T4<T> h = nb0[k];
-          const float4 sv = *static_cast<float4*>(staged_half<P>(smem, lay, k, 0));
-          const V3<float> d = add(sub(V3<float>{h.x, h.y, h.z}, xh), sub(record_lo(sv.z, sv.w), xl));
-          nb0[k] = T4<T>{d.x, d.y, d.z, h.w};
-          nb1[k] = T2<T>{sv.x, sv.y};
-          acc.zero(k);
-        }
-      }
-    }
-  }
-  b = BlockRows<T>{R, t, p.nrows, p.L, len, lb, p.s0, p.s1, p.dp, p.r0 + t, p.base, p.uni, p.zl};
-  return true;
-}
-
-// Phases 0 and 1 of a row-gather block, shared by the full assembly and the
-// time-step kernels.
-template <int P, bool DEBUG, typename Accum>
-__device__ __forceinline__ bool stage_block(const MeshView& m, const FieldView& f, int64_t r0, unsigned char* smem,
-                                            const GatherSmem& lay, Accum& acc, BlockRows<typename Prec<P>::T>& b) {
-  const Phase0<typename Prec<P>::T> p = load_phase0<P>(m, f, r0);
-  issue_phase0<DEBUG>(m, smem, lay, p);
-  return stage_records<P, DEBUG>(m, smem, lay, acc, p, b, kc_of<typename Prec<P>::T>(f));
-}
-
-// phase 2 of a staged block: every element of each row's star, the diagonal
-// and the RHS; ends with a barrier (nb1 and the walk bytes are free after it)
-template <int P, bool DEBUG>
-__device__ __forceinline__ void gather_compute(const MeshView& m, const FieldView& f, const OutView& o,
-                                               unsigned char* smem, const GatherSmem& lay, AccSmem<P>& acc,
-                                               const BlockRows<typename Prec<P>::T>& b) {
-  using T = typename Prec<P>::T;
-  using Out = typename Prec<P>::Out;
-  const int R = b.R, t = b.t, nrows = b.nrows, len = b.len, s0 = b.s0, s1 = b.s1, dp = b.dp;
-  const int64_t i = b.i;
-  const V3<T> uni = b.uni;
-  const T4<T>* __restrict__ nb0 = reinterpret_cast<const T4<T>*>(smem + lay.nb0());
-  const T2<T>* __restrict__ nb1 = reinterpret_cast<const T2<T>*>(smem + lay.nb1());
-  const uint8_t* walk = smem + lay.walk();
-  const T kmu = kmu_of<T>(f);
-  const T kc = kc_of<T>(f);
-  const T kmass = kmass_of<T>(f);
-  Acc<P> detsum;
-  detsum.zero();
-  if (t < nrows) {
-    // phase 2: every element of the row's star, accumulated privately
-    if (len > 0) {
-      if (DEBUG && dp >= len) atomicOr(m.err, ERR_STAR);
-      const int kd = dp * R + t;
-      const T4<T> di = nb0[kd];
-      const T2<T> ei = nb1[kd];
-      const V3<T> u2i{di.w + di.w, ei.x + ei.x, ei.y + ei.y};
-      walk_row<P, DEBUG>(walk + s0, s1 - s0, len, nb0, nb1, acc, t, R, u2i, kc, kmu, detsum, m.err);
-      // diagonal from the partition of unity (sum_b grad N_b = 0, exact):
-      //   A(i,i) = lumped mass - sum_{j != i} A(i,j)   (convection + viscous parts)
-      //   G(i,i) = 1/3 sum_{j != i} G(i,j)            (each element adds c_i to three
-      //                                                 off-diagonal entries and the diagonal)
-      Acc<P> rsum[4];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) rsum[c].zero();
-      acc.row_sums(t, R, len, rsum);  // (the diagonal slot is still zero)
-      Acc<P> dg[4];
-      if constexpr (P == NSI_MIXED_F32_ACC64) {
-        const float p = kmass * detsum.hi;  // kmass * (hi + lo), product error kept
-        dg[0].hi = p;
-        dg[0].lo = fmaf(kmass, detsum.hi, -p) + kmass * detsum.lo;
-        dg[0].add(-rsum[0].hi);
-        dg[0].lo -= rsum[0].lo;
-#pragma unroll
-        for (int c = 1; c < 4; ++c) {  // G: plain float
-          dg[c].hi = rsum[c].hi * (1.0f / 3.0f);
-          dg[c].lo = 0.f;
-        }
-      } else {
-        dg[0].v = kmass * detsum.v - rsum[0].v;
-#pragma unroll
-        for (int c = 1; c < 4; ++c) dg[c].v = rsum[c].v * (T(1) / T(3));
-      }
-      if (!DEBUG || dp < len) acc.set(kd, dg);
-    }
-    // lumped RHS: (sum_e rho |T_e| / (4 dt)) u^n_i
-    const T unk[3] = {uni.x, uni.y, uni.z};
-    Out* Rh = static_cast<Out*>(o.rhs);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      Acc<P> r;
-      const T c = kmass * unk[k];
-      if constexpr (P == NSI_MIXED_F32_ACC64) {
-        const float p = detsum.hi * c;
-        r.hi = p;
-        r.lo = fmaf(detsum.hi, c, -p) + detsum.lo * c;
-      } else {
-        r.v = detsum.v * c;
-      }
-      store_acc(Rh + k * m.n + i, r);
-    }
-  }
-  __syncthreads();
-}
-
-// phase 3 of a block: its contiguous slice of A and G (uses nb0 and acc only)
-template <int P>
-__device__ __forceinline__ void gather_writeout(const MeshView& m, const OutView& o, unsigned char* smem,
-                                                const GatherSmem& lay, AccSmem<P>& acc,
-                                                const BlockRows<typename Prec<P>::T>& b) {
-  using T = typename Prec<P>::T;
-  using Out = typename Prec<P>::Out;
-  const int R = b.R, t = b.t, nrows = b.nrows, L = b.L, len = b.len, lb = b.lb;
-  const int32_t base = b.base;
-  // phase 3: the block's contiguous slice of A and G.  Every thread moves its
-  // own row's finished values into CSR order (nb0 reused as staging), then the
-  // block streams the slice out coalesced.
-  Out* A = static_cast<Out*>(o.A);
-  Out* G = static_cast<Out*>(o.G);
-  Out* stage = reinterpret_cast<Out*>(smem + lay.nb0());
-  Out* dst[4] = {A + base, G + base, G + m.nnz + base, G + 2 * m.nnz + base};
-  if constexpr (sizeof(Out) == sizeof(T4<T>) / 4 || P == NSI_FP64) {
-    // room for all four components at once
-    if (t < nrows) {
-#pragma unroll 4
-      for (int q = 0, k = t; q < len; ++q, k += R) {
-        const T4<Out> v = acc.values(k);
-        stage[lb + q] = v.x;
-        stage[L + lb + q] = v.y;
-        stage[2 * L + lb + q] = v.z;
-        stage[3 * L + lb + q] = v.w;
-      }
-      for (int q = 0; q < b.zl; ++q)  // a long row: its slice zeroed here, computed later
-        stage[lb + q] = stage[L + lb + q] = stage[2 * L + lb + q] = stage[3 * L + lb + q] = Out(0);
-    }
-    __syncthreads();
-    for (int k = t; k < L; k += R) {
-      dst[0][k] = stage[k];
-      dst[1][k] = stage[L + k];
-      dst[2][k] = stage[2 * L + k];
-      dst[3][k] = stage[3 * L + k];
-    }
-  } else {
-    // mixed64: one staging round.  Every thread stages its own row's float
-    // values in CSR order -- A and G_x, G_y in nb0, G_z in the half of nb1
-    // that the next block's column indices (copied in under this write-out by
-    // the persistent grid) leave free -- then the block converts them to
-    // double exactly and streams them out coalesced (the conversions spread
-    // evenly over the threads); an infinite, NaN or subnormal A is converted
-    // again by a rare pass.  Last, each row's thread overwrites its diagonal
-    // with the double of its compensated pair (leading part in the slot, error
-    // term in dlo).
-    float* sa = reinterpret_cast<float*>(smem + lay.nb0());
-    float* gx = sa + L;
-    float* gy = gx + L;
-    float* gz = reinterpret_cast<float*>(smem + lay.nb1()) + lay.N();
-    if (t < nrows) {
-#pragma unroll 4
-      for (int q = 0, k = t; q < len; ++q, k += R) {
-        const float4 h = acc.hi[k];
-        sa[lb + q] = h.w;
-        gx[lb + q] = h.x;
-        gy[lb + q] = h.y;
-        gz[lb + q] = h.z;
-      }
-      for (int q = 0; q < b.zl; ++q) {  // a long row: its slice zeroed here, computed later
-        sa[lb + q] = 0.f;
-        gx[lb + q] = gy[lb + q] = gz[lb + q] = 0.f;
-      }
-    }
-    __syncthreads();
-    bool slow = false;
-    for (int k = t; k < L; k += R) {
-      const float a = sa[k];
-      slow |= special_float(a);
-      dst[0][k] = float_double(a);
-      dst[1][k] = float_double(gx[k]);
-      dst[2][k] = float_double(gy[k]);
-      dst[3][k] = float_double(gz[k]);
-    }
-    if (__syncthreads_or(slow)) {  // block-uniform and rare
-      for (int k = t; k < L; k += R) {
-        const float a = sa[k];
-        if (special_float(a)) dst[0][k] = nonfinite_bits(a) ? nonfinite_double(a) : (double)a;
-      }
-      __syncthreads();
-    }
-    if (t < nrows && len > 0) {
-      const float hd = acc.hi[b.dp * R + t].w;
-      dst[0][lb + b.dp] = nonfinite_bits(hd) ? nonfinite_double(hd) : pair_double(hd, acc.dlo);
-    }
-  }
-}
-
-// one block of rows [r0, r0 + blockDim.x) of one mesh
-template <int P, bool DEBUG>
-__device__ __forceinline__ void gather_rows(const MeshView& m, const FieldView& f, const OutView& o, int64_t r0,
-                                            unsigned char* smem, const GatherSmem& lay) {
-  AccSmem<P> acc(smem + lay.acc(), lay.N());
-  BlockRows<typename Prec<P>::T> b;
-  if (!stage_block<P, DEBUG>(m, f, r0, smem, lay, acc, b)) return;
-  gather_compute<P, DEBUG>(m, f, o, smem, lay, acc, b);
-  gather_writeout<P>(m, o, smem, lay, acc, b);
-}
-
-// ------------------------------------------- cached-geometry time step ---
-// Over time steps on a fixed mesh with fixed rho, mu and dt, the viscous
-// part, the lumped mass and the pressure gradient of the assembly do not
-// change; only the convection C(u) and the RHS do.  The step kernel forms
-//   A = A_static + C(u),  C(i,x) = sum over the star of i of w_e . c_x,
-//   w_e = rho/120 (2 u_i + u_p + u_q + u_c)
-// and the lumped RHS, where A_static is the A of a full assembly at u = 0
-// (the viscous part and the lumped mass).  C has zero row sums (the shape
-// gradients of an element sum to zero), so C(i,i) = -sum_{j != i} C(i,j).  G
-// is not touched.  The nodal variant forms the paper's per-node outputs
-// instead (perform_assembly_in_global_system): rhsid, dt_rho = sum_e
-// rho|T|/(4 dt) and mass_rho = sum_e rho|T|/4.  Both follow the element walk
-// of the full assembly, with one accumulator per slot (none for the nodal
-// outputs).
-
-// A-only accumulator slots, at the stride of the staged record halves (16
-// bytes, FP64 two planes of 16): a slot's bytes first receive its record's
-// second half, then its accumulator.
-template <int P>
-struct AccA;
-template <>
-struct AccA<NSI_MIXED_F32_ACC32> {
-  float4* __restrict__ a;
-  using Slot = float;
-  __device__ __forceinline__ AccA(unsigned char* p) : a(reinterpret_cast<float4*>(p)) {}
-  __device__ __forceinline__ void zero(int k) { a[k].x = 0.f; }
-  __device__ __forceinline__ Slot load1(int k) const { return a[k].x; }
-  __device__ __forceinline__ void store1(int k, Slot v) { a[k].x = v; }
-  static __device__ __forceinline__ void add(Slot& s, float x) { s += x; }
-  __device__ __forceinline__ void row_sum(int t, int R, int len, Acc<NSI_MIXED_F32_ACC32>& r) const {
-#pragma unroll 4
-    for (int q = 0, k = t; q < len; ++q, k += R) r.add(a[k].x);
-  }
-  __device__ __forceinline__ void set(int k, const Acc<NSI_MIXED_F32_ACC32>& r) { a[k].x = r.v; }
-};
-// mixed64: an off-diagonal entry of C(u) sums the few element terms of its
-// edge in plain float (its error term stays zero); the diagonal, minus the
-// row's other entries, is the compensated row sum (set() stores the pair).
-template <>
-struct AccA<NSI_MIXED_F32_ACC64> {
-  float4* __restrict__ a;
-  using Slot = float2;  // leading part, error term
-  __device__ __forceinline__ AccA(unsigned char* p) : a(reinterpret_cast<float4*>(p)) {}
-  __device__ __forceinline__ void zero(int k) { a[k].x = a[k].y = 0.f; }
-  __device__ __forceinline__ Slot load1(int k) const {
-    const float4 v = a[k];
-    return make_float2(v.x, v.y);
-  }
-  __device__ __forceinline__ void store1(int k, Slot v) { reinterpret_cast<float2*>(a + k)[0] = v; }
-  static __device__ __forceinline__ void add(Slot& s, float x) { s.x += x; }
-  __device__ __forceinline__ void row_sum(int t, int R, int len, Acc<NSI_MIXED_F32_ACC64>& r) const {
-#pragma unroll 4
-    for (int q = 0, k = t; q < len; ++q, k += R) {
-      const float4 v = a[k];
-      r.add(v.x);
-      r.lo += v.y;
-    }
-  }
-  __device__ __forceinline__ void set(int k, const Acc<NSI_MIXED_F32_ACC64>& r) {
-    reinterpret_cast<float2*>(a + k)[0] = make_float2(r.hi, r.lo);
-  }
-};
-template <>
-struct AccA<NSI_FP64> {
-  T2<double>* __restrict__ a;  // plane 0 of the staged halves
-  using Slot = double;
-  __device__ __forceinline__ AccA(unsigned char* p) : a(reinterpret_cast<T2<double>*>(p)) {}
-  __device__ __forceinline__ void zero(int k) { a[k].x = 0.0; }
-  __device__ __forceinline__ Slot load1(int k) const { return a[k].x; }
-  __device__ __forceinline__ void store1(int k, Slot v) { a[k].x = v; }
-  static __device__ __forceinline__ void add(Slot& s, double x) { s += x; }
-  __device__ __forceinline__ void row_sum(int t, int R, int len, Acc<NSI_FP64>& r) const {
-#pragma unroll 4
-    for (int q = 0, k = t; q < len; ++q, k += R) r.add(a[k].x);
-  }
-  __device__ __forceinline__ void set(int k, const Acc<NSI_FP64>& r) { a[k].x = r.v; }
-};
-
-// The element walk of the time step: det for the lumped sums and, unless
-// NODAL, the convection w . c_x into the window's accumulators.  Same window,
-// orientation and carried cofactor as walk_row.
-template <int P, bool NODAL, bool DEBUG>
-__device__ __forceinline__ void walk_step(const uint8_t* __restrict__ st, int nsteps, int len,
-                                          const T4<typename Prec<P>::T>* __restrict__ nb0,
-                                          const T2<typename Prec<P>::T>* __restrict__ nb1, AccA<P>& acc, int t,
-                                          int R, const V3<typename Prec<P>::T>& u2i, typename Prec<P>::T kc,
-                                          Acc<P>& detsum, unsigned* err) {
-  using T = typename Prec<P>::T;
-  using Node = WalkNode<T, typename AccA<P>::Slot>;
-  if (nsteps <= 0) return;
-  if (DEBUG) {
-    bool ok = nsteps >= 3 && !(st[0] & WALK_ELEM) && !(st[1] & WALK_ELEM);
-    for (int s = 0; s < nsteps; ++s) ok &= (int)(st[s] & WALK_POS) < len;
-    if (!ok) {
-      atomicOr(err, ERR_STAR);
-      return;
-    }
-  }
-  if (nsteps < 3) return;  // (every walk of a row with elements has at least 3 steps)
-  auto load = [&](int k) {
-    const T4<T> a = nb0[k];
-    Node nd;
-    nd.k = k;
-    nd.d = V3<T>{a.x, a.y, a.z};
-    if constexpr (!NODAL) {
-      const T2<T> b = nb1[k];
-      nd.u = V3<T>{a.w, b.x, b.y};
-      nd.v = acc.load1(k);
-    }
-    return nd;
-  };
-  // as walk_row: the two filling steps' nodes loaded directly
-  Node p = load((int)(st[0] & WALK_POS) * R + t);
-  Node q = load((int)(st[1] & WALK_POS) * R + t);
-  V3<T> m = cross(p.d, q.d);
-  T sg = T(-1);  // c_c = -sg m
-  unsigned w = st[2];
-  Node c = load((int)(w & WALK_POS) * R + t);
-#pragma unroll 2
-  for (int s = 2; s < nsteps; ++s) {
-    const unsigned wn = st[min(s + 1, nsteps - 1)];
-    const Node cn = load((int)(wn & WALK_POS) * R + t);
-    const V3<T> cp = cross(q.d, c.d), cq = cross(c.d, p.d);
-    const bool elem = (w & WALK_ELEM) != 0u;
-    const T f = elem ? ((w & WALK_NEG) ? T(-1) : T(1)) : T(0);  // orientation, or 0
-    detsum.add(f * dot(p.d, cp));
-    if constexpr (!NODAL) {
-      const V3<T> s3{u2i.x + p.u.x + q.u.x + c.u.x, u2i.y + p.u.y + q.u.y + c.u.y, u2i.z + p.u.z + q.u.z + c.u.z};
-      const V3<T> w3 = P == NSI_FP64 ? s3 : V3<T>{kc * s3.x, kc * s3.y, kc * s3.z};
-      AccA<P>::add(p.v, f * dot(w3, cp));
-      AccA<P>::add(q.v, f * dot(w3, cq));
-      AccA<P>::add(c.v, -f * sg * dot(w3, m));
-    }
-    // as walk_row: the newest node always enters q
-    if (w & WALK_EVQ) {
-      if constexpr (!NODAL) acc.store1(q.k, q.v);
-      m = cq;
-      sg = T(1);
-    } else {
-      if constexpr (!NODAL) acc.store1(p.k, p.v);
-      p = q;
-      m = cp;
-      sg = T(-1);
-    }
-    q = c;
-    c = cn;
-    w = wn;
-  }
-  if constexpr (!NODAL) {
-    acc.store1(p.k, p.v);
-    acc.store1(q.k, q.v);
-  }
-}
-
-// outputs of the time-step kernels; kmr = rho/24 (the density mass per det)
-struct StepView {
-  const void* A_static;
-  void* A;
-  void* rhs;
-  void* dt_rho;
-  void* mass_rho;
-  double kmr;
-  float kmrf;
-};
-
-template <typename T, int P>
-__device__ __forceinline__ Acc<P> scaled_sum(const Acc<P>& s, T c) {
-  Acc<P> r;
-  if constexpr (P == NSI_MIXED_F32_ACC64) {
-    const float p = s.hi * c;  // c * (hi + lo), product error kept
-    r.hi = p;
-    r.lo = fmaf(s.hi, c, -p) + s.lo * c;
-  } else {
-    r.v = s.v * c;
-  }
-  return r;
-}
-
-// one staged block of the time step; `between` runs once the walk is done
-// (nb1 and the walk bytes are free) and commits a group of asynchronous
-// copies (the persistent grid's next phase 0, or none)
-template <int P, bool NODAL, bool DEBUG, typename Hook>
-__device__ __forceinline__ void step_block(const MeshView& m, const FieldView& f, const StepView& o,
-                                           unsigned char* smem, const GatherSmem& lay, AccA<P>& acc,
-                                           const BlockRows<typename Prec<P>::T>& b, const Hook& between) {
-  using T = typename Prec<P>::T;
-  using Out = typename Prec<P>::Out;
-  const int R = b.R, t = b.t;
-  const T4<T>* __restrict__ nb0 = reinterpret_cast<const T4<T>*>(smem + lay.nb0());
-  const T2<T>* __restrict__ nb1 = reinterpret_cast<const T2<T>*>(smem + lay.nb1());
-  const T kc = kc_of<T>(f);
-  const T kmass = kmass_of<T>(f);
-  Out* stat = reinterpret_cast<Out*>(smem + lay.stat());
-  if constexpr (!NODAL) {
-    // the block's slice of A_static, in flight during the walk
-    const Out* As = static_cast<const Out*>(o.A_static) + b.base;
-    for (int k = t; k < b.L; k += R) {
-      if constexpr (sizeof(Out) == 8) cp_async8(stat + k, As + k);
-      else cp_async4(stat + k, As + k);
-    }
-    cp_async_commit();
-  }
-  Acc<P> detsum;
-  detsum.zero();
-  if (t < b.nrows) {
-    const int kd = b.dp * R + t;
-    if (b.len > 0) {
-      if (DEBUG && b.dp >= b.len) atomicOr(m.err, ERR_STAR);
-      const T4<T> di = nb0[kd];
-      const T2<T> ei = nb1[kd];
-      const V3<T> u2i{di.w + di.w, ei.x + ei.x, ei.y + ei.y};
-      walk_step<P, NODAL, DEBUG>(smem + lay.walk() + b.s0, b.s1 - b.s0, b.len, nb0, nb1, acc, t, R, u2i, kc,
-                                 detsum, m.err);
-      if constexpr (!NODAL) {  // C(i,i) = -sum_{j != i} C(i,j)
-        Acc<P> rsum;
-        rsum.zero();
-        acc.row_sum(t, R, b.len, rsum);  // (the diagonal slot is still zero)
-        Acc<P> dg;
-        if constexpr (P == NSI_MIXED_F32_ACC64) {
-          dg.hi = -rsum.hi;
-          dg.lo = -rsum.lo;
-        } else {
-          dg.v = -rsum.v;
-        }
-        if (!DEBUG || b.dp < b.len) acc.set(kd, dg);
-      }
-    }
-    // lumped RHS: (sum_e rho |T_e| / (4 dt)) u^n_i
-    const T unk[3] = {b.uni.x, b.uni.y, b.uni.z};
-    Out* Rh = static_cast<Out*>(o.rhs);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) store_acc(Rh + k * m.n + b.i, scaled_sum<T, P>(detsum, kmass * unk[k]));
-    if constexpr (NODAL) {
-      store_acc(static_cast<Out*>(o.dt_rho) + b.i, scaled_sum<T, P>(detsum, kmass));
-      store_acc(static_cast<Out*>(o.mass_rho) + b.i, scaled_sum<T, P>(detsum, (T)(sizeof(T) == 8 ? o.kmr : o.kmrf)));
-    }
-  }
-  __syncthreads();
-  between();
-  if constexpr (!NODAL) {
-    // the block's contiguous slice of A: staged in CSR order, then
-    // A = A_static + C streamed out coalesced
-    Out* A = static_cast<Out*>(o.A) + b.base;
-    cp_async_wait_prior();  // the slice of A_static (the group before `between`'s)
-    if constexpr (P == NSI_MIXED_F32_ACC64) {
-      float2* stage = reinterpret_cast<float2*>(smem + lay.nb0());
-      bool nonfinite = false;  // as in the assembly's write-out
-      if (t < b.nrows) {
-        for (int q = 0; q < b.len; ++q) {
-          const float2 v = acc.load1(q * R + t);
-          stage[b.lb + q] = v;
-          nonfinite |= nonfinite_bits(v.x);
-        }
-        // a long row: A_static kept here (C = 0), the convection added later
-        for (int q = 0; q < b.zl; ++q) stage[b.lb + q] = make_float2(0.f, 0.f);
-      }
-      const bool fix = __syncthreads_or(nonfinite);
-#pragma unroll 2
-      for (int k = t; k < b.L; k += R) A[k] = stat[k] + pair_double(stage[k].x, stage[k].y);
-      if (fix)
-        for (int k = t; k < b.L; k += R)
-          if (nonfinite_bits(stage[k].x)) A[k] = stat[k] + nonfinite_double(stage[k].x);
-    } else {
-      Out* stage = reinterpret_cast<Out*>(smem + lay.nb0());
-      if (t < b.nrows) {
-        for (int q = 0; q < b.len; ++q) stage[b.lb + q] = acc.load1(q * R + t);
-        for (int q = 0; q < b.zl; ++q) stage[b.lb + q] = Out(0);  // a long row (as above)
-      }
-      __syncthreads();
-#pragma unroll 2
-      for (int k = t; k < b.L; k += R) A[k] = stat[k] + stage[k];
-    }
-  }
-}
-
-template <int P, bool NODAL, bool DEBUG>
-__global__ void __launch_bounds__(128) step_kernel(MeshView m, FieldView f, StepView o, GatherSmem lay) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  AccA<P> acc(smem_raw + lay.acc());
-  BlockRows<typename Prec<P>::T> b;
-  if (!stage_block<P, DEBUG>(m, f, (int64_t)blockIdx.x * blockDim.x, smem_raw, lay, acc, b)) return;
-  step_block<P, NODAL, DEBUG>(m, f, o, smem_raw, lay, acc, b, []() { cp_async_commit(); });
-}
-
-// the time step as a persistent grid: a CTA's next block starts its phase-0
-// copies (column indices into nb1, walk bytes) under the current block's
-// write-out, as in gather_persistent_kernel
-template <int P, bool NODAL, bool DEBUG>
-__global__ void __launch_bounds__(128) step_persistent_kernel(MeshView m, FieldView f, StepView o, GatherSmem lay,
-                                                              int64_t nblocks) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  using T = typename Prec<P>::T;
-  int64_t blk = blockIdx.x;
-  if (blk >= nblocks) return;
-  const int R = blockDim.x;
-  AccA<P> acc(smem_raw + lay.acc());
-  Phase0<T> p = load_phase0<P>(m, f, blk * R);
-  issue_phase0<DEBUG>(m, smem_raw, lay, p);
-  while (true) {
-    BlockRows<T> b;
-    if (!stage_records<P, DEBUG>(m, smem_raw, lay, acc, p, b, kc_of<T>(f))) return;
-    const int64_t nxt = blk + gridDim.x;
-    const bool more = nxt < nblocks;  // block-uniform
-    Phase0<T> pn = p;
-    if (more) pn = load_phase0<P>(m, f, nxt * R);
-    step_block<P, NODAL, DEBUG>(m, f, o, smem_raw, lay, acc, b, [&]() {
-      if (more) issue_phase0<DEBUG>(m, smem_raw, lay, pn);
-      cp_async_commit();
-    });
-    if (!more) return;
-    blk = nxt;
-    p = pn;
   }
 }
 
@@ -1744,6 +464,14 @@ __global__ void __launch_bounds__(64) long_rows_kernel(MeshView m, FieldView f, 
     static_cast<Out*>(mass_rho)[i] = (Out)(kmr * detsum);
   }
 }
+
+// asynchronous global -> shared copies (cp.async): many gathers in flight per
+// thread without holding registers
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
 // ------------------------------------------------------ edge-fan kernel ---
 // One thread per CSR entry (i, j) of a block of whole rows.  An off-diagonal
@@ -2609,115 +1337,18 @@ __global__ void __launch_bounds__(64) stab_rows_kernel(MeshView m, FieldView f, 
   Rh[2 * m.n + i] = (Out)(f.kmass * detsum * un.z);
 }
 
-template <int P, bool DEBUG>
-__global__ void __launch_bounds__(128) gather_kernel(MeshView m, FieldView f, OutView o, GatherSmem lay,
-                                                     int64_t block0) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  gather_rows<P, DEBUG>(m, f, o, (block0 + blockIdx.x) * blockDim.x, smem_raw, lay);
-}
-
-// The row gather as a persistent grid (one CTA per resident block slot): a
-// CTA's next block of rows loads its bounds and row scalars while the current
-// block walks, and copies its column indices and walk steps (into nb1 and the
-// walk region, free after the walk) while the current block writes out.
-template <int P, bool DEBUG>
-__global__ void __launch_bounds__(128) gather_persistent_kernel(MeshView m, FieldView f, OutView o, GatherSmem lay,
-                                                                int64_t nblocks) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  using T = typename Prec<P>::T;
-  int64_t blk = blockIdx.x;
-  if (blk >= nblocks) return;
-  const int R = blockDim.x;
-  AccSmem<P> acc(smem_raw + lay.acc(), lay.N());
-  Phase0<T> p = load_phase0<P>(m, f, blk * R);
-  issue_phase0<DEBUG>(m, smem_raw, lay, p);
-  while (true) {
-    BlockRows<T> b;
-    if (!stage_records<P, DEBUG>(m, smem_raw, lay, acc, p, b, kc_of<T>(f))) return;
-    const int64_t nxt = blk + gridDim.x;
-    const bool more = nxt < nblocks;  // block-uniform
-    Phase0<T> pn = p;
-    if (more) pn = load_phase0<P>(m, f, nxt * R);
-    gather_compute<P, DEBUG>(m, f, o, smem_raw, lay, acc, b);
-    if (more) issue_phase0<DEBUG>(m, smem_raw, lay, pn);
-    gather_writeout<P>(m, o, smem_raw, lay, acc, b);
-    if (!more) return;
-    blk = nxt;
-    p = pn;
-  }
-}
-
-// ------------------------------------------------------ batched kernel ---
+// --------------------------------------------- batched edge-fan kernel ---
 struct BatchItem {
   MeshView m;
   FieldView f;
   OutView o;
-  int64_t block0;  // first global block of this mesh
+  int64_t block0;  // first global fan block of this mesh
 };
 struct BatchArgs {
   int32_t count;
   int64_t total_blocks;
   BatchItem item[NSI_MAX_BATCH];
 };
-
-// the item (mesh) of global block b: the last item with block0 <= b
-__device__ __forceinline__ const BatchItem& batch_item(const BatchArgs& args, int64_t b) {
-  int lo = 0, hi = args.count - 1;
-  while (lo < hi) {
-    int mid = (lo + hi + 1) >> 1;
-    if (args.item[mid].block0 <= b) lo = mid;
-    else hi = mid - 1;
-  }
-  return args.item[lo];
-}
-
-// the node records of every mesh of a batch in one launch: block b packs the
-// nodes of the batch's row block b (the row gather's blocks of R rows)
-template <int P>
-__global__ void __launch_bounds__(128) batched_pack_kernel(const __grid_constant__ BatchArgs args) {
-  const BatchItem& it = batch_item(args, blockIdx.x);
-  const int64_t i = (blockIdx.x - it.block0) * (int64_t)blockDim.x + threadIdx.x;
-  if (i < it.m.n) pack_node<P>(it.m, it.f, const_cast<void*>(it.m.rec), i);
-}
-
-template <int P>
-__global__ void __launch_bounds__(128) batched_kernel(const __grid_constant__ BatchArgs args, GatherSmem lay) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  if constexpr (P == NSI_MIXED_F32_ACC64) {
-    // as gather_persistent_kernel: the next block's phase 0 runs under the
-    // current block's write-out (the next block may belong to another mesh)
-    using T = typename Prec<P>::T;
-    int64_t b = blockIdx.x;
-    if (b >= args.total_blocks) return;
-    const int R = blockDim.x;
-    AccSmem<P> acc(smem_raw + lay.acc(), lay.N());
-    const BatchItem* it = &batch_item(args, b);
-    Phase0<T> p = load_phase0<P>(it->m, it->f, (b - it->block0) * R);
-    issue_phase0<false>(it->m, smem_raw, lay, p);
-    while (true) {
-      BlockRows<T> rows;
-      stage_records<P, false>(it->m, smem_raw, lay, acc, p, rows, kc_of<T>(it->f));
-      const int64_t nxt = b + gridDim.x;
-      const bool more = nxt < args.total_blocks;  // block-uniform
-      const BatchItem* itn = more ? &batch_item(args, nxt) : it;
-      Phase0<T> pn = p;
-      if (more) pn = load_phase0<P>(itn->m, itn->f, (nxt - itn->block0) * R);
-      gather_compute<P, false>(it->m, it->f, it->o, smem_raw, lay, acc, rows);
-      if (more) issue_phase0<false>(itn->m, smem_raw, lay, pn);
-      gather_writeout<P>(it->m, it->o, smem_raw, lay, acc, rows);
-      if (!more) return;
-      b = nxt;
-      it = itn;
-      p = pn;
-    }
-  } else {
-    for (int64_t b = blockIdx.x; b < args.total_blocks; b += gridDim.x) {
-      const BatchItem& it = batch_item(args, b);
-      gather_rows<P, false>(it.m, it.f, it.o, (b - it.block0) * blockDim.x, smem_raw, lay);
-      __syncthreads();  // the next block reuses the shared records
-    }
-  }
-}
 
 // many meshes, edge-fan variant: a persistent grid strides over the fan
 // blocks of all meshes (item.block0 counts fan blocks here)
@@ -3003,34 +1634,12 @@ __global__ void __launch_bounds__(256) add_values_kernel(CompPtrs dst, int ncomp
 }
 
 // ----------------------------------------------------------- launchers ---
-static nsi_status check_launch(const char* what) {
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return cuda_fail(e, what);
-  return NSI_OK;
-}
-
 template <int P>
 static nsi_status zero_outputs(const NsiHandle* h, const OutView& o, cudaStream_t s) {
   using Out = typename Prec<P>::Out;
   NSI_CUDA(cudaMemsetAsync(o.A, 0, sizeof(Out) * h->nnz, s));
   NSI_CUDA(cudaMemsetAsync(o.G, 0, sizeof(Out) * 3 * h->nnz, s));
   NSI_CUDA(cudaMemsetAsync(o.rhs, 0, sizeof(Out) * 3 * h->n, s));
-  return NSI_OK;
-}
-
-template <int P, bool DEBUG>
-static nsi_status set_gather_smem() {
-  static std::once_flag once;
-  static cudaError_t err = cudaSuccess;
-  std::call_once(once, [] {
-    err = cudaFuncSetAttribute(gather_kernel<P, DEBUG>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    if (err == cudaSuccess)
-      err = cudaFuncSetAttribute(gather_persistent_kernel<P, DEBUG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 200 * 1024);
-    if (err == cudaSuccess)
-      err = cudaFuncSetAttribute(batched_kernel<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-  });
-  if (err != cudaSuccess) return cuda_fail(err, "cudaFuncSetAttribute(gather smem)");
   return NSI_OK;
 }
 
@@ -3126,9 +1735,8 @@ static nsi_status assemble_core_p(NsiHandle* h, const FieldView& f, const OutVie
   }
   // row gather
   if (!h->gather_ok) return fail(NSI_ERR_UNSUPPORTED, "row-gather mode not available for this mesh");
-  nsi_status st = h->debug ? set_gather_smem<P, true>() : set_gather_smem<P, false>();
+  nsi_status st = launch_pack<P>(h, f, rec, s);
   if (st) return st;
-  pack_kernel<P><<<(h->n + 255) / 256, 256, 0, s>>>(m, f, const_cast<void*>(m.rec));
   if (h->use_fan) {
     const size_t fsm = FanSmem<P>::total(FAN_BLOCK);
     if (h->ev_start) NSI_CUDA(cudaEventRecord(h->ev_start, s));
@@ -3137,29 +1745,7 @@ static nsi_status assemble_core_p(NsiHandle* h, const FieldView& f, const OutVie
     if (h->ev_stop) NSI_CUDA(cudaEventRecord(h->ev_stop, s));
     return check_launch("fan_kernel");
   }
-  const int R = h->plan.rows_per_block;
-  const GatherSmem lay = gather_smem(P, R, h->plan.w, h->plan.max_block_entries, h->plan.max_block_steps);
-  const size_t smem = lay.total();
-  if (h->persistent) {
-    int per_sm = 0, sms = 0, dev = 0;
-    NSI_CUDA(cudaGetDevice(&dev));
-    NSI_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    if (h->debug)
-      NSI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gather_persistent_kernel<P, true>, R, smem));
-    else
-      NSI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gather_persistent_kernel<P, false>, R, smem));
-    const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(h->plan.n_blocks, (int64_t)std::max(1, per_sm) * sms));
-    if (h->ev_start) NSI_CUDA(cudaEventRecord(h->ev_start, s));
-    if (h->debug) gather_persistent_kernel<P, true><<<grid, R, smem, s>>>(m, f, o, lay, h->plan.n_blocks);
-    else gather_persistent_kernel<P, false><<<grid, R, smem, s>>>(m, f, o, lay, h->plan.n_blocks);
-    if (h->ev_stop) NSI_CUDA(cudaEventRecord(h->ev_stop, s));
-    return check_launch("gather_persistent_kernel");
-  }
-  if (h->ev_start) NSI_CUDA(cudaEventRecord(h->ev_start, s));
-  if (h->debug) gather_kernel<P, true><<<h->plan.n_blocks, R, smem, s>>>(m, f, o, lay, 0);
-  else gather_kernel<P, false><<<h->plan.n_blocks, R, smem, s>>>(m, f, o, lay, 0);
-  if (h->ev_stop) NSI_CUDA(cudaEventRecord(h->ev_stop, s));
-  return check_launch("gather_kernel");
+  return launch_gather<P>(h, f, o, 0, h->n, rec, s);
 }
 
 template <int P>
@@ -3205,56 +1791,12 @@ static nsi_status assemble_dispatch(NsiHandle* h, const NsiFields* f, const NsiO
   }
 }
 
-// the time-step kernels (convective step, nodal outputs): pack, then one
-// step_kernel launch with the handle's rows per block
-template <int P, bool NODAL, bool DEBUG>
-static nsi_status set_step_smem() {
-  static std::once_flag once;
-  static cudaError_t err = cudaSuccess;
-  std::call_once(once, [] {
-    err = cudaFuncSetAttribute(step_kernel<P, NODAL, DEBUG>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    if (err == cudaSuccess)
-      err = cudaFuncSetAttribute(step_persistent_kernel<P, NODAL, DEBUG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 200 * 1024);
-  });
-  if (err != cudaSuccess) return cuda_fail(err, "cudaFuncSetAttribute(step smem)");
-  return NSI_OK;
-}
-
+// the time step and the nodal outputs: the node records, the row gather, then
+// the rows that it leaves out
 template <int P, bool NODAL>
 static nsi_status step_p(NsiHandle* h, const FieldView& f, const StepView& o, cudaStream_t s) {
-  const MeshView m = view_of(h);
-  nsi_status st = h->debug ? set_step_smem<P, NODAL, true>() : set_step_smem<P, NODAL, false>();
-  if (st) return st;
-  const int R = h->plan.rows_per_block;
-  const GatherSmem lay = gather_smem(P, R, h->plan.w, h->plan.max_block_entries, h->plan.max_block_steps, true);
-  const size_t smem = lay.total();
-  if (smem > 200 * 1024) return fail(NSI_ERR_UNSUPPORTED, "the time-step layout needs more shared memory than a block has");
-  pack_kernel<P><<<(h->n + 255) / 256, 256, 0, s>>>(m, f, h->rec);
-  if constexpr (P == NSI_MIXED_F32_ACC32) {
-    // the persistent grid measured faster for mixed32 only (0.235 against
-    // 0.250 ms at the 100^3 cube; mixed64 0.321 against 0.291, FP64 2.38
-    // against 2.17)
-    int per_sm = 0, sms = 0, dev = 0;
-    NSI_CUDA(cudaGetDevice(&dev));
-    NSI_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    if (h->debug)
-      NSI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step_persistent_kernel<P, NODAL, true>, R, smem));
-    else
-      NSI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step_persistent_kernel<P, NODAL, false>, R, smem));
-    const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(h->plan.n_blocks, (int64_t)std::max(1, per_sm) * sms));
-    if (h->ev_start) NSI_CUDA(cudaEventRecord(h->ev_start, s));
-    if (h->debug) step_persistent_kernel<P, NODAL, true><<<grid, R, smem, s>>>(m, f, o, lay, h->plan.n_blocks);
-    else step_persistent_kernel<P, NODAL, false><<<grid, R, smem, s>>>(m, f, o, lay, h->plan.n_blocks);
-    if (h->ev_stop) NSI_CUDA(cudaEventRecord(h->ev_stop, s));
-    st = check_launch("step_persistent_kernel");
-  } else {
-    if (h->ev_start) NSI_CUDA(cudaEventRecord(h->ev_start, s));
-    if (h->debug) step_kernel<P, NODAL, true><<<h->plan.n_blocks, R, smem, s>>>(m, f, o, lay);
-    else step_kernel<P, NODAL, false><<<h->plan.n_blocks, R, smem, s>>>(m, f, o, lay);
-    if (h->ev_stop) NSI_CUDA(cudaEventRecord(h->ev_stop, s));
-    st = check_launch("step_kernel");
-  }
+  nsi_status st = launch_pack<P>(h, f, nullptr, s);
+  if (!st) st = launch_step<P>(h, f, o, NODAL, s);
   if (st) return st;
   st = fix_exact_rows<P>(h, f, NODAL ? 2 : 1, nullptr, nullptr, o.rhs, o.dt_rho, o.mass_rho, o.kmr, s);
   if (st) return st;
@@ -3299,86 +1841,35 @@ static nsi_status batched_p(NsiHandle* const* hs, const NsiFields* fs, const Nsi
 template <int P>
 static nsi_status batched_core_p(NsiHandle* const* hs, const NsiFields* fs, const NsiOutputs* os, int count,
                                  cudaStream_t s) {
+  bool all_fan = true;
+  for (int k = 0; k < count; ++k) all_fan &= hs[k]->use_fan;
+  if (!all_fan) return launch_batched<P>(hs, fs, os, count, s);
   static BatchArgs args;  // host staging of the by-value kernel argument
   static std::mutex mu;
   std::lock_guard<std::mutex> lock(mu);
   args.count = count;
-  bool all_fan = true;
-  for (int k = 0; k < count; ++k) all_fan &= hs[k]->use_fan;
-  if (all_fan) {
-    int64_t fblocks = 0;
-    for (int k = 0; k < count; ++k) {
-      args.item[k].m = view_of(hs[k]);
-      args.item[k].f = fields_of(&fs[k]);
-      args.item[k].o = OutView{os[k].A_val, os[k].G_val, os[k].rhs};
-      args.item[k].block0 = fblocks;
-      fblocks += hs[k]->fan_blocks;
-    }
-    args.total_blocks = fblocks;
-    if (fblocks == 0) return NSI_OK;
-    for (int k = 0; k < count; ++k)
-      pack_kernel<P><<<(hs[k]->n + 255) / 256, 256, 0, s>>>(args.item[k].m, args.item[k].f, hs[k]->rec);
-    const size_t fsm = FanSmem<P>::total(FAN_BLOCK);
-    int per_sm = 0, sms = 0, dev = 0;
-    NSI_CUDA(cudaGetDevice(&dev));
-    NSI_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    NSI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batched_fan_kernel<P>, FAN_BLOCK, fsm));
-    const int64_t grid = std::min<int64_t>(fblocks, (int64_t)std::max(1, per_sm) * sms);
-    batched_fan_kernel<P><<<grid, FAN_BLOCK, fsm, s>>>(args);
-    return check_launch("batched_fan_kernel");
-  }
-  // one block size for the whole batch: the largest one, no larger than any
-  // mesh's own choice, that every mesh has planned (the per-block maxima of
-  // the shared-memory layout are those of that size: blocks of different
-  // sizes do not nest)
-  int Rmin = 1 << 30, R = 0, max_entries = 0, max_steps = 0, max_row = 1;
-  for (int k = 0; k < count; ++k) Rmin = std::min(Rmin, hs[k]->plan.rows_per_block);
-  const GatherPlan* use[NSI_MAX_BATCH] = {};
-  for (int cand : {128, 96, 64, 32}) {
-    if (cand > Rmin) continue;
-    bool all = true;
-    for (int k = 0; k < count && all; ++k) {
-      use[k] = nullptr;
-      for (int j = 0; j < hs[k]->n_plans; ++j)
-        if (hs[k]->plans[j].rows_per_block == cand) use[k] = &hs[k]->plans[j];
-      all = use[k] != nullptr;
-    }
-    if (all) {
-      R = cand;
-      break;
-    }
-  }
-  if (R == 0) return fail(NSI_ERR_UNSUPPORTED, "no block size is planned for every mesh of the batch");
-  int64_t blocks = 0;
+  int64_t fblocks = 0;
   for (int k = 0; k < count; ++k) {
-    const NsiHandle* h = hs[k];
-    max_entries = std::max(max_entries, use[k]->max_block_entries);
-    max_steps = std::max(max_steps, use[k]->max_block_steps);
-    max_row = std::max(max_row, use[k]->w);
-    args.item[k].m = view_of(h);
+    args.item[k].m = view_of(hs[k]);
     args.item[k].f = fields_of(&fs[k]);
     args.item[k].o = OutView{os[k].A_val, os[k].G_val, os[k].rhs};
-    args.item[k].block0 = blocks;
-    blocks += (h->n + R - 1) / R;
+    args.item[k].block0 = fblocks;
+    fblocks += hs[k]->fan_blocks;
   }
-  args.total_blocks = blocks;
-  if (blocks == 0) return NSI_OK;
-  batched_pack_kernel<P><<<blocks, R, 0, s>>>(args);
-  nsi_status st = check_launch("batched_pack_kernel");
-  if (st) return st;
-  st = set_gather_smem<P, false>();
-  if (st) return st;
-  const GatherSmem lay = gather_smem(P, R, max_row, max_entries, max_steps);
-  const size_t smem = lay.total();
-  if (smem > 200 * 1024 || !lay.stage_fits())
-    return fail(NSI_ERR_UNSUPPORTED, "batched meshes need more shared memory than a block has");
+  args.total_blocks = fblocks;
+  if (fblocks == 0) return NSI_OK;
+  for (int k = 0; k < count; ++k) {
+    nsi_status st = launch_pack<P>(hs[k], args.item[k].f, nullptr, s);
+    if (st) return st;
+  }
+  const size_t fsm = FanSmem<P>::total(FAN_BLOCK);
   int per_sm = 0, sms = 0, dev = 0;
   NSI_CUDA(cudaGetDevice(&dev));
   NSI_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  NSI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batched_kernel<P>, R, smem));
-  const int64_t grid = std::min<int64_t>(blocks, (int64_t)std::max(1, per_sm) * sms);
-  batched_kernel<P><<<grid, R, smem, s>>>(args, lay);
-  return check_launch("batched_kernel");
+  NSI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batched_fan_kernel<P>, FAN_BLOCK, fsm));
+  const int64_t grid = std::min<int64_t>(fblocks, (int64_t)std::max(1, per_sm) * sms);
+  batched_fan_kernel<P><<<grid, FAN_BLOCK, fsm, s>>>(args);
+  return check_launch("batched_fan_kernel");
 }
 
 template <int P>
@@ -3407,15 +1898,6 @@ static nsi_status residual_p(NsiHandle* h, const FieldView& f, void* r, cudaStre
   if (st || h->n_bad == 0) return st;
   residual_exact_kernel<P><<<(h->n_bad + 63) / 64, 64, 0, s>>>(view_of(h), f, r, h->bad_list, h->n_bad);
   return check_launch("residual_exact_kernel");
-}
-
-int gather_kernel_regs(int precision) {
-  cudaFuncAttributes a{};
-  cudaError_t e;
-  if (precision == NSI_FP64) e = cudaFuncGetAttributes(&a, gather_kernel<NSI_FP64, false>);
-  else if (precision == NSI_MIXED_F32_ACC64) e = cudaFuncGetAttributes(&a, gather_kernel<NSI_MIXED_F32_ACC64, false>);
-  else e = cudaFuncGetAttributes(&a, gather_kernel<NSI_MIXED_F32_ACC32, false>);
-  return e == cudaSuccess ? a.numRegs : 96;
 }
 
 // ------------------------------------------------ allocation-free variant ---
@@ -3473,16 +1955,12 @@ static nsi_status host_chunked_p(NsiHandle* h, const NsiFields* fd, const NsiOut
   if (!h->copy_stream) NSI_CUDA(cudaStreamCreateWithFlags(&h->copy_stream, cudaStreamNonBlocking));
   for (cudaEvent_t& e : h->chunk_ev)
     if (!e) NSI_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-  nsi_status st = h->debug ? set_gather_smem<P, true>() : set_gather_smem<P, false>();
-  if (st) return st;
-  const MeshView m = view_of(h);
   const FieldView fv = fields_of(fd);
   const OutView ov{od->A_val, od->G_val, od->rhs};
-  const int R = h->plan.rows_per_block;
-  const GatherSmem lay = gather_smem(P, R, h->plan.w, h->plan.max_block_entries, h->plan.max_block_steps);
-  const size_t smem = lay.total();
-  pack_kernel<P><<<(h->n + 255) / 256, 256, 0, s>>>(m, fv, h->rec);
-  const int64_t nb = h->plan.n_blocks;
+  const int R = 32;
+  nsi_status st = launch_pack<P>(h, fv, nullptr, s);
+  if (st) return st;
+  const int64_t nb = (h->n + R - 1) / R;
   const int chunks = (int)std::min<int64_t>(C, nb);
   const Out* dA = static_cast<const Out*>(od->A_val);
   const Out* dG = static_cast<const Out*>(od->G_val);
@@ -3500,13 +1978,11 @@ static nsi_status host_chunked_p(NsiHandle* h, const NsiFields* fd, const NsiOut
   for (int c = 0; c < chunks; ++c) {
     const int64_t b0 = bound(c), b1 = c + 1 == chunks ? nb : bound(c + 1);
     if (b1 <= b0) continue;
-    if (h->debug) gather_kernel<P, true><<<b1 - b0, R, smem, s>>>(m, fv, ov, lay, b0);
-    else gather_kernel<P, false><<<b1 - b0, R, smem, s>>>(m, fv, ov, lay, b0);
-    st = check_launch("gather_kernel (host chunk)");
+    const int64_t r0 = b0 * R, r1 = std::min<int64_t>(h->n, b1 * R);
+    st = launch_gather<P>(h, fv, ov, r0, r1, nullptr, s);
     if (st) return st;
     NSI_CUDA(cudaEventRecord(h->chunk_ev[c], s));
     NSI_CUDA(cudaStreamWaitEvent(h->copy_stream, h->chunk_ev[c], 0));
-    const int64_t r0 = b0 * R, r1 = std::min<int64_t>(h->n, b1 * R);
     const int64_t e0 = h->row_ptr_host[r0], e1 = h->row_ptr_host[r1];
     const size_t eb = sizeof(Out) * (size_t)(e1 - e0), rb = sizeof(Out) * (size_t)(r1 - r0);
     // A's slice, then the three components of G and of rhs (equal slices at a
@@ -3545,7 +2021,7 @@ static nsi_status stabilized_p(NsiHandle* h, const FieldView& f, const StabConst
   nsi_status st = h->debug ? set_star_smem<P, true>() : set_star_smem<P, false>();
   if (st) return st;
   MeshView m = view_of(h);
-  pack_kernel<P><<<(h->n + 255) / 256, 256, 0, s>>>(m, f, const_cast<void*>(m.rec));
+  if ((st = launch_pack<P>(h, f, nullptr, s))) return st;
   const size_t smem = StarSmem<P>::bytes() * STAR_WARPS;
   const int64_t grid = (h->n_star_tasks + STAR_WARPS - 1) / STAR_WARPS;
   if (h->ev_start) NSI_CUDA(cudaEventRecord(h->ev_start, s));

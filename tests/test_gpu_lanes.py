@@ -1,0 +1,53 @@
+"""The row gather at the edges of its lane rule: meshes around the row count
+where four lanes per row become two, and one whose groups are more than the
+resident warps (every warp takes several), against the oracle; a batch that
+mixes both kinds against the single calls, bit for bit."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import meshgen
+import oracle
+from tests._common import errors, vec_scaled_err
+
+nsi = pytest.importorskip("paper_2111_05651_gb300")
+pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a GPU")]
+TOL = {"fp64": 1e-12, "mixed64": 1e-5, "mixed32": 1e-5}  # the library's stated bars
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed64", "mixed32"])
+@pytest.mark.parametrize("N", [20, 21, 36])  # 9,261, 10,648 and 50,653 rows
+def test_lanes_match_oracle(precision, N):
+    mesh, u = meshgen.config_mesh(N=N, jitter=0.15, numbering="random", seed=300 + N)
+    asm = nsi.Assembler(mesh.coord, mesh.lnods, precision=precision)
+    ut = torch.as_tensor(u.T.copy())
+    uo = u if precision == "fp64" else u.astype(np.float32).astype(np.float64)
+    rp, _, oA, oG, orhs = oracle.assemble(mesh.coord, mesh.lnods, uo, None, 1.0, 1e-3, 1e-2)
+    A, G, rhs = asm.assemble(ut, rho=1.0, mu=1e-3, dt=1e-2)
+    got = [t.double().cpu().numpy() for t in (A, G, rhs)]
+    assert max(errors(rp, *got, oA, oG, orhs).values()) <= TOL[precision]
+    A_static, _ = asm.static_part(rho=1.0, mu=1e-3, dt=1e-2)
+    A2, rhs2 = asm.assemble_convective(ut, A_static, rho=1.0, mu=1e-3, dt=1e-2)
+    got = [A2.double().cpu().numpy(), oG, rhs2.double().cpu().numpy()]
+    assert max(errors(rp, *got, oA, oG, orhs).values()) <= TOL[precision]
+    alias = A_static.clone()
+    asm.assemble_convective(ut, alias, rho=1.0, mu=1e-3, dt=1e-2, out=(alias, rhs2))
+    assert torch.equal(alias, A2)
+    onr, ondt, onm = oracle.nodal(mesh.coord, mesh.lnods, uo, 1.0, 1e-2)
+    r3, dtr, mr = (t.double().cpu().numpy() for t in asm.nodal(ut, rho=1.0, dt=1e-2))
+    assert max([vec_scaled_err(dtr, ondt), vec_scaled_err(mr, onm)] +
+               [vec_scaled_err(r3[k], onr[k]) for k in range(3)]) <= TOL[precision]
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed64", "mixed32"])
+def test_batch_of_both_kinds_equals_single(precision):
+    asms, us = [], []
+    for N in (3, 36, 20, 22):
+        mesh, u = meshgen.config_mesh(N=N, jitter=0.15, numbering="natural", seed=310 + N)
+        asms.append(nsi.Assembler(mesh.coord, mesh.lnods, precision=precision))
+        us.append(torch.as_tensor(u.T.copy()))
+    single = [[t.clone() for t in a.assemble(v)] for a, v in zip(asms, us)]
+    for s, b in zip(single, nsi.assemble_batched(asms, us)):
+        for x, y in zip(s, b):
+            assert torch.equal(x, y)
