@@ -191,7 +191,7 @@ typedef struct {
     int32_t long_rows;      /* rows the row gather leaves out -- more than 32 entries (its walk
                                steps hold five bits of row position), or a star its walk
                                encoder could not cover -- computed after every row-gather
-                               assembly or time step by one thread per row, in double; the rest
+                               assembly or time step by one block per row, in double; the rest
                                of the mesh stays on the row gather */
     int32_t fan_ok;         /* 1: the mesh has an edge-fan map (rows of at most 16 entries, the
                                ring of elements around every edge at most 7 nodes, no long

@@ -432,7 +432,7 @@ static nsi_status build(NsiHandle* h, const NsiMesh* m, cudaStream_t s) {
 
   // 4. row-gather map (positions of the other three nodes in the row).  Rows
   //    of more than 32 entries (five bits of row position) are "long rows":
-  //    the row gather leaves them out and long_rows_kernel computes them.
+  //    the row gather leaves them out and rows64_kernel computes them.
   h->gather_ok = inc_ptr[n] <= INT32_MAX;
   std::vector<uint16_t> star;
   std::vector<uint8_t> diag(n, 0);
@@ -739,9 +739,17 @@ static nsi_status build(NsiHandle* h, const NsiMesh* m, cudaStream_t s) {
         bad_list.push_back((int32_t)e);
       }
     }
+    // first the rows with a walk, then the rest
+    auto walks = [&](int64_t i) { return h->gather_ok && !is_long[i]; };
     for (int64_t i = 0; i < n; ++i)
-      if (flag[i] && row_len[i] <= STAR_MAX_ROW) exact_list.push_back((int32_t)i);
+      if (flag[i] && row_len[i] <= STAR_MAX_ROW && walks(i)) {
+        exact_list.push_back((int32_t)i);
+        h->exact_slots = std::max(h->exact_slots, (int)row_len[i] - 1);
+      }
     h->exact_rows = (int64_t)exact_list.size();
+    for (int64_t i = 0; i < n; ++i)
+      if (flag[i] && row_len[i] <= STAR_MAX_ROW && !walks(i)) exact_list.push_back((int32_t)i);
+    h->exact_rest = (int64_t)exact_list.size() - h->exact_rows;
     // every listed row's incident elements (element * 4 + local index of the node)
     exact_ptr.assign(exact_list.size() + 1, 0);
     for (size_t r = 0; r < exact_list.size(); ++r) {
@@ -749,7 +757,7 @@ static nsi_status build(NsiHandle* h, const NsiMesh* m, cudaStream_t s) {
       for (int64_t t = inc_ptr[i]; t < inc_ptr[i + 1]; ++t) exact_inc.push_back((uint32_t)inc[t]);
       exact_ptr[r + 1] = (int32_t)exact_inc.size();
     }
-    if (E > (int64_t)(UINT32_MAX >> 2)) h->exact_rows = 0;  // not encodable: keep the float results
+    if (E > (int64_t)(UINT32_MAX >> 2)) h->exact_rows = h->exact_rest = 0;  // not encodable: keep the float results
   }
 
   // 7c. long rows: every incident element of each (element * 4 + local index)
@@ -767,6 +775,10 @@ static nsi_status build(NsiHandle* h, const NsiMesh* m, cudaStream_t s) {
     if (!long_list.empty() && (E > (int64_t)(UINT32_MAX >> 2) || long_inc.size() > (size_t)INT32_MAX))
       h->gather_ok = false;
     h->long_rows = h->gather_ok ? (int64_t)long_list.size() : 0;
+    if (!h->gather_ok) {  // no walks after all
+      h->exact_rest += h->exact_rows;
+      h->exact_rows = 0;
+    }
   }
 
   // 8. upload
@@ -806,7 +818,7 @@ static nsi_status build(NsiHandle* h, const NsiMesh* m, cudaStream_t s) {
     if ((st = dev_upload(h, &h->bad_list, bad_list.data(), bad_list.size(), s))) return st;
     if ((st = dev_upload(h, &h->bad_mask, mask.data(), mask.size(), s))) return st;
   }
-  if (h->exact_rows > 0) {
+  if (h->exact_rows + h->exact_rest > 0) {
     if ((st = dev_upload(h, &h->exact_list, exact_list.data(), exact_list.size(), s))) return st;
     if ((st = dev_upload(h, &h->exact_ptr, exact_ptr.data(), exact_ptr.size(), s))) return st;
     if ((st = dev_upload(h, &h->exact_inc, exact_inc.data(), exact_inc.size(), s))) return st;
@@ -943,7 +955,7 @@ nsi_status nsi_info(const NsiHandle* h, NsiInfo* info) {
   info->rows_per_block = h->use_fan ? -1 : h->plan.rows_per_block;
   info->n_plans = h->n_plans;
   info->persistent = h->use_fan ? 0 : 1;
-  info->exact_rows = (int32_t)std::min<int64_t>(h->exact_rows, INT32_MAX);
+  info->exact_rows = (int32_t)std::min<int64_t>(h->exact_rows + h->exact_rest, INT32_MAX);
   info->long_rows = (int32_t)std::min<int64_t>(h->long_rows, INT32_MAX);
   info->fan_ok = h->fan_ok ? 1 : 0;
   return NSI_OK;

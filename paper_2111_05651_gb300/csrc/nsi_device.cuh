@@ -105,6 +105,14 @@ inline FieldView fields_of(const NsiFields* f) {
   return v;
 }
 
+// outputs of the kernels that compute listed rows in double: A, G (assembly),
+// A with A_static (time step), rhs, dt_rho and mass_rho (nodal outputs)
+struct RowOut {
+  const void* A_static;
+  void *A, *G, *rhs, *dt_rho, *mass_rho;
+  double kmr;
+};
+
 // precision traits: compute type T, output type Out
 template <int P>
 struct Prec;
@@ -324,6 +332,10 @@ nsi_status launch_gather(NsiHandle* h, const FieldView& f, const OutView& o, int
                          cudaStream_t s);
 template <int P>
 nsi_status launch_step(NsiHandle* h, const FieldView& f, const StepView& o, bool nodal, cudaStream_t s);
+// the handle's rows of badly shaped elements that have a walk, in double (mixed
+// modes), by mode: 0 the assembly, 1 the time step, 2 the nodal outputs
+template <int P>
+nsi_status launch_exact_rows(NsiHandle* h, const FieldView& f, int mode, const RowOut& o, cudaStream_t s);
 template <int P>
 nsi_status launch_batched(NsiHandle* const* hs, const NsiFields* fs, const NsiOutputs* os, int count, cudaStream_t s);
 

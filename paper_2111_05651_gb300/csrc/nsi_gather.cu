@@ -416,7 +416,7 @@ __device__ __forceinline__ GroupRow read_row(const unsigned char* info, int t) {
   return r;
 }
 // slots of a row: its off-diagonal entries (none for a long row, which
-// long_rows_kernel computes)
+// rows64_kernel computes)
 __device__ __forceinline__ int row_slots(const GroupRow& r) {
   return r.dp == DIAG_LONG ? 0 : max(0, r.re - r.rs - 1);
 }
@@ -859,6 +859,122 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, P == NSI_FP64 ? 2 : 4)
                                 smem_raw + w * lay.total, lay);
 }
 
+// ------------------------------------------------ badly shaped elements ---
+// Rows listed at create (mixed modes: the rows of the nodes of an element with
+// |d1||d2||d3| > EXACT_RATIO |det|) are recomputed after the assembly in double
+// from the handle's coordinates (leading + residual float parts) and the given
+// velocities, and their entries overwritten: a float determinant of such an
+// element would carry about that ratio times the float rounding of its edge
+// vectors.  The lanes of a warp walk 32 / H listed rows as in the group loop
+// (the walk bytes read from memory, the entries written row by row): the FP64
+// pipe, the bound here, issues a warp's instruction at the same cost whether or
+// not its lanes are active, so rows side by side fill it best (a 14x40x70 pipe,
+// 14,905 of its 39,831 rows listed: 66 us, of which the pipe is busy 45).  MODE 0: A, G and rhs; 1: rhs only (the time
+// step: the convection does not involve the determinant); 2: rhs, dt_rho and
+// mass_rho.
+template <int P, int H, int MODE>
+__global__ void __launch_bounds__(32) exact_rows_kernel(WalkMesh m, FieldView f, RowOut o, GroupLay lay,
+                                                        const int32_t* __restrict__ rows, int64_t count) {
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  using Out = typename Prec<P>::Out;
+  constexpr int RW = 32 / H, WMODE = MODE == 0 ? ASSEMBLE : NODAL;
+  using S = Slots<NSI_FP64, WMODE>;
+  constexpr unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31, t = lane & (RW - 1), h = lane / RW;
+  const int64_t r = (int64_t)blockIdx.x * RW + t;
+  unsigned char* smem = smem_raw;
+  const bool valid = r < count;
+  const int64_t i = valid ? rows[r] : 0;
+  const int32_t rs = m.row_ptr[i];
+  const int ns = valid ? m.row_ptr[i + 1] - rs - 1 : 0, dp = m.diag_pos[i];
+  auto coord = [&](int64_t j) {
+    const float4 a = __ldg(m.xyz_hi + j), b = __ldg(m.xyz_lo + j);
+    return V3<double>{(double)a.x + (double)b.x, (double)a.y + (double)b.y, (double)a.z + (double)b.z};
+  };
+  auto slots = [&](int p) { return S(smem + lay.acc + p * lay.plane, lay.N); };
+  T4<double>* nb0 = reinterpret_cast<T4<double>*>(smem) + t;
+  T2<double>* nb1 = reinterpret_cast<T2<double>*>(smem + lay.nb1) + t;
+  const V3<double> xi = coord(i);
+  V3<double> u2i{0.0, 0.0, 0.0};
+  if constexpr (MODE == 0) {
+    const V3<float> ui = load_vec<float>(f.u, i);
+    u2i = V3<double>{2.0 * f.kc * ui.x, 2.0 * f.kc * ui.y, 2.0 * f.kc * ui.z};
+  }
+  for (int s = h; s < ns; s += H) {
+    const int64_t j = m.col_idx[rs + slot_pos(s, dp)];
+    const V3<double> d = sub(coord(j), xi);
+    if constexpr (MODE == 0) {
+      const V3<float> u = load_vec<float>(f.u, j);
+      nb0[s * RW] = T4<double>{d.x, d.y, d.z, f.kc * u.x};
+      nb1[s * RW] = T2<double>{f.kc * u.y, f.kc * u.z};
+      for (int p = 0; p < H; ++p) slots(p).store(s * RW + t, S::zero_value());
+    } else {
+      nb0[s * RW] = T4<double>{d.x, d.y, d.z, 0.0};
+    }
+  }
+  __syncwarp();
+  Acc<NSI_FP64> det;
+  det.zero();
+  if (ns > 0) {
+    const uint8_t* st = m.walk + m.walk_ptr[i];
+    int b = H;
+    for (int k = 0; k < h; ++k) b += st[k];
+    S acc = slots(h);
+    if constexpr (MODE == 0) {
+      acc.a0 += t;
+      acc.a1 += t;
+    }
+    walk_lane<NSI_FP64, RW, WMODE>(st + b, st[h], nb0, nb1, acc, u2i, f.kmu, det);
+  }
+  __syncwarp();
+#pragma unroll
+  for (int off = RW; off < 32; off <<= 1) det.v += __shfl_xor_sync(FULL, det.v, off);
+  if constexpr (MODE == 0) {
+    Out* A = static_cast<Out*>(o.A) + rs;
+    Out* G = static_cast<Out*>(o.G) + rs;
+    double ra = 0.0, gx = 0.0, gy = 0.0, gz = 0.0;
+    for (int s = h; s < ns; s += H) {
+      typename S::V v = slots(0).load(s * RW + t);
+#pragma unroll
+      for (int p = 1; p < H; ++p) v = S::sum(v, slots(p).load(s * RW + t));
+      ra += v.x.x;
+      gx += v.x.y;
+      gy += v.y.x;
+      gz += v.y.y;
+      const int q = slot_pos(s, dp);
+      A[q] = (Out)v.x.x;
+      G[q] = (Out)v.x.y;
+      G[m.nnz + q] = (Out)v.y.x;
+      G[2 * m.nnz + q] = (Out)v.y.y;
+    }
+#pragma unroll
+    for (int off = RW; off < 32; off <<= 1) {
+      ra += __shfl_xor_sync(FULL, ra, off);
+      gx += __shfl_xor_sync(FULL, gx, off);
+      gy += __shfl_xor_sync(FULL, gy, off);
+      gz += __shfl_xor_sync(FULL, gz, off);
+    }
+    if (h == 0 && ns > 0) {  // the diagonal from the partition of unity, as in the group loop
+      A[dp] = (Out)(f.kmass * det.v - ra);
+      G[dp] = (Out)(gx / 3.0);
+      G[m.nnz + dp] = (Out)(gy / 3.0);
+      G[2 * m.nnz + dp] = (Out)(gz / 3.0);
+    }
+  }
+  if (valid && h == 0) {
+    const V3<float> un = load_vec<float>(f.un, i);
+    const double mass = f.kmass * det.v;
+    Out* Rh = static_cast<Out*>(o.rhs);
+    Rh[i] = (Out)(mass * un.x);
+    Rh[m.n + i] = (Out)(mass * un.y);
+    Rh[2 * m.n + i] = (Out)(mass * un.z);
+    if constexpr (MODE == 2) {
+      static_cast<Out*>(o.dt_rho)[i] = (Out)mass;
+      static_cast<Out*>(o.mass_rho)[i] = (Out)(o.kmr * det.v);
+    }
+  }
+}
+
 // ------------------------------------------------------ batched kernel ---
 // The meshes with two lanes per row first, then those with four: a warp takes
 // its share of the first's groups, then of the second's, so that every mesh is
@@ -999,6 +1115,21 @@ nsi_status run_lanes(NsiHandle* h, const WalkItem<MODE>& item, int64_t row0, int
   }
 }
 
+template <int P, int H>
+nsi_status exact_rows_h(NsiHandle* h, const FieldView& f, int mode, const RowOut& o, cudaStream_t s) {
+  const auto kernel = mode == 0   ? exact_rows_kernel<P, H, 0>
+                      : mode == 1 ? exact_rows_kernel<P, H, 1>
+                                  : exact_rows_kernel<P, H, 2>;
+  static std::once_flag once[3];
+  static cudaError_t err[3] = {};
+  nsi_status st = allow_smem(kernel, once[mode], err[mode]);
+  if (st) return st;
+  const int64_t warps = (h->exact_rows * H + 31) / 32;
+  const GatherSmem lay = group_smem(NSI_FP64, mode == 0 ? ASSEMBLE : NODAL, H, h->exact_slots, 0, 0);
+  kernel<<<warps, 32, lay.total(), s>>>(walk_mesh(h, nullptr), f, o, GroupLay(lay), h->exact_list, h->exact_rows);
+  return check_launch("exact_rows_kernel");
+}
+
 }  // namespace
 
 template <int P>
@@ -1071,6 +1202,15 @@ nsi_status launch_batched(NsiHandle* const* hs, const NsiFields* fs, const NsiOu
   batched_kernel<P><<<grid, 32 * warps, bytes * warps, s>>>(args, GroupLay(lay2), GroupLay(lay4));
   return check_launch("batched_kernel");
 }
+
+template <int P>
+nsi_status launch_exact_rows(NsiHandle* h, const FieldView& f, int mode, const RowOut& o, cudaStream_t s) {
+  return h->nsub == 2 ? exact_rows_h<P, 2>(h, f, mode, o, s) : exact_rows_h<P, 4>(h, f, mode, o, s);
+}
+template nsi_status launch_exact_rows<NSI_MIXED_F32_ACC64>(NsiHandle*, const FieldView&, int, const RowOut&,
+                                                            cudaStream_t);
+template nsi_status launch_exact_rows<NSI_MIXED_F32_ACC32>(NsiHandle*, const FieldView&, int, const RowOut&,
+                                                            cudaStream_t);
 
 #define NSI_INSTANTIATE(P)                                                                                          \
   template nsi_status launch_pack<P>(NsiHandle*, const FieldView&, void*, cudaStream_t);                            \

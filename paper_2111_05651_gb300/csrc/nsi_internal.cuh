@@ -94,7 +94,7 @@ constexpr int SMEM_MAX = 200 * 1024;  // shared memory of one block
 
 // diag_pos value of a row the row gather leaves out ("long row": more than
 // 32 entries, or a star whose walk does not encode): the kernels give it no
-// elements and zero its slice; long_rows_kernel computes it afterwards
+// elements and zero its slice; rows64_kernel computes it afterwards
 constexpr uint8_t DIAG_LONG = 0xff;
 
 // Shared-memory layout of one warp's group of the row gather: R rows, W slots
@@ -194,16 +194,20 @@ struct NsiHandle {
   int64_t fan_blocks = 0;
   bool use_fan = false;         // row-gather mode runs the edge-fan kernel
   bool atomic_agg = false;      // atomic mode runs the warp-aggregated atomics (else one atomic per value)
-  int64_t long_rows = 0;        // rows the row gather leaves out, recomputed by long_rows_kernel
+  int64_t long_rows = 0;        // rows the row gather leaves out, recomputed by rows64_kernel
   int32_t* long_list = nullptr;  // [long_rows] their node ids
   int32_t* long_ptr = nullptr;   // [long_rows + 1] into long_inc
   uint32_t* long_inc = nullptr;  // element * 4 + local index of the row's node
   int64_t n_bad = 0;            // mixed modes: badly shaped elements (the adjoint and residual take them in double)
   int32_t* bad_list = nullptr;  // [n_bad] their ids
   uint32_t* bad_mask = nullptr; // [ceil(E / 32)] one bit per element, or null when there are none
-  int64_t exact_rows = 0;       // mixed modes: rows recomputed in double (badly shaped elements)
-  int32_t* exact_list = nullptr;  // [exact_rows] their node ids
-  int32_t* exact_ptr = nullptr;   // [exact_rows + 1] into exact_inc
+  // mixed modes: the rows of badly shaped elements, recomputed in double: first
+  // those with a walk (exact_rows of them, at most exact_slots off-diagonal
+  // entries), then the rest (exact_rest)
+  int64_t exact_rows = 0, exact_rest = 0;
+  int exact_slots = 0;
+  int32_t* exact_list = nullptr;  // [exact_rows + exact_rest] their node ids
+  int32_t* exact_ptr = nullptr;   // [exact_rows + exact_rest + 1] into exact_inc
   uint32_t* exact_inc = nullptr;  // element * 4 + local index of the row's node
   // the stabilised block's row kernel: every row's star as row positions of
   // each element's other three nodes (five bits each, the row's node and the

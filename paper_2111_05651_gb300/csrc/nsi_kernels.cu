@@ -9,9 +9,8 @@
 //   vjp_kernel      adjoint of R(u, mu) = A(u) u - b, element per thread
 //   residual_kernel R(u, mu) without the matrix (both with an exact
 //                   companion for badly shaped elements in double)
-//   exact_rows_kernel, long_rows_kernel  rows recomputed or computed per
-//                   thread in double: the mixed modes' rows of badly shaped
-//                   elements, and rows beyond the walk (more than 32 entries)
+//   rows64_kernel   rows without a walk (more than 32 entries, for instance)
+//                   in double, one block per row
 //   stab_star_kernel  the stabilised velocity block (3x3 per CSR entry): one
 //                   warp per row or pair of rows, each element evaluated
 //                   once per row, entry sums from shared memory
@@ -231,237 +230,175 @@ __global__ void __launch_bounds__(256) elem_kernel(MeshView m, FieldView f, OutV
   }
 }
 
-// ------------------------------------------------ badly shaped elements ---
-// Rows listed at create (mixed modes: the rows of the nodes of an element with
-// |d1||d2||d3| > EXACT_RATIO |det|) are recomputed after the assembly with
-// every element of their star evaluated in double from the coordinates
-// (leading + residual float parts) and velocities, and their entries
-// overwritten: a float determinant of such an element would carry about that
-// ratio times the float rounding of its edge vectors.  One thread per row,
-// its sums in a local array.  MODE 0: A, G and rhs; 1: rhs only (the time
-// step: the convection does not involve the determinant); 2: rhs, dt_rho and
-// mass_rho.
-template <int P, int MODE>
-__global__ void __launch_bounds__(64) exact_rows_kernel(MeshView m, FieldView f, void* A, void* G, void* rhs,
-                                                        void* dt_rho, void* mass_rho, double kmr, const int32_t* rows,
-                                                        const int32_t* ptr, const uint32_t* inc, int64_t count) {
-  using Out = typename Prec<P>::Out;
-  const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (r >= count) return;
-  const int64_t i = rows[r];
-  const int32_t rs = m.row_ptr[i], len = m.row_ptr[i + 1] - rs;
-  if (len > STAR_MAX_ROW) return;
-  const int32_t* cols = m.col_idx + rs;
-  auto coord = [&](int64_t j) {
+// the element's coordinates, velocities and weights in double (the handle's
+// copy of the coordinates: double, or the float hi + lo pair)
+template <int P>
+__device__ __forceinline__ V3<double> coord64(const MeshView& m, int64_t j) {
+  if constexpr (P == NSI_FP64) {
+    const D4 x = m.xyz64[j];
+    return V3<double>{x.x, x.y, x.z};
+  } else {
     const float4 h = m.xyz_hi[j], l = m.xyz_lo[j];
     return V3<double>{(double)h.x + (double)l.x, (double)h.y + (double)l.y, (double)h.z + (double)l.z};
-  };
-  auto vel = [&](int64_t j) {
-    const V3<float> u = load_vec<float>(f.u, j);
-    return V3<double>{u.x, u.y, u.z};
-  };
-  // even permutations of (0,1,2,3) that bring vertex a to the front
-  const int EVEN[4][3] = {{1, 2, 3}, {0, 3, 2}, {3, 0, 1}, {2, 1, 0}};
-  double acc[STAR_MAX_ROW][4];
-  for (int q = 0; q < len; ++q) acc[q][0] = acc[q][1] = acc[q][2] = acc[q][3] = 0.0;
-  const V3<double> xi = coord(i), ui = vel(i);
-  double detsum = 0.0;
-  int dpos = 0;
-  for (int q = 0; q < len; ++q)
-    if (cols[q] == i) dpos = q;
-  for (int32_t t = ptr[r]; t < ptr[r + 1]; ++t) {
-    const int64_t e = inc[t] >> 2;
-    const int a = (int)(inc[t] & 3u);
-    const int4 v4 = m.lnods[e];
-    const int v[4] = {v4.x, v4.y, v4.z, v4.w};
-    int pos[3];
-    V3<double> d[3], u[3];
-    for (int b = 0; b < 3; ++b) {
-      const int j = v[EVEN[a][b]];
-      int lo = 0, hi = len - 1;  // position of j in the row (columns ascending)
-      while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (cols[mid] < j) lo = mid + 1;
-        else hi = mid;
-      }
-      pos[b] = lo;
-      d[b] = sub(coord(j), xi);
-      u[b] = vel(j);
-    }
-    const V3<double> c[3] = {cross(d[1], d[2]), cross(d[2], d[0]), cross(d[0], d[1])};
-    const double det = dot(d[0], c[0]);
-    const V3<double> ci{-(c[0].x + c[1].x + c[2].x), -(c[0].y + c[1].y + c[2].y), -(c[0].z + c[1].z + c[2].z)};
-    const double kv = f.kmu / det;
-    const V3<double> w3{f.kc * (2.0 * ui.x + u[0].x + u[1].x + u[2].x) + kv * ci.x,
-                        f.kc * (2.0 * ui.y + u[0].y + u[1].y + u[2].y) + kv * ci.y,
-                        f.kc * (2.0 * ui.z + u[0].z + u[1].z + u[2].z) + kv * ci.z};
-    for (int b = 0; b < 3; ++b) {
-      acc[pos[b]][0] += dot(w3, c[b]);
-      acc[pos[b]][1] += ci.x;
-      acc[pos[b]][2] += ci.y;
-      acc[pos[b]][3] += ci.z;
-    }
-    detsum += det;
-  }
-  // lumped RHS and nodal sums
-  const V3<double> un = [&] {
-    if constexpr (P == NSI_FP64) return load_vec<double>(f.un, i);
-    else {
-      const V3<float> w = load_vec<float>(f.un, i);
-      return V3<double>{w.x, w.y, w.z};
-    }
-  }();
-  Out* Rh = static_cast<Out*>(rhs);
-  Rh[i] = (Out)(f.kmass * detsum * un.x);
-  Rh[m.n + i] = (Out)(f.kmass * detsum * un.y);
-  Rh[2 * m.n + i] = (Out)(f.kmass * detsum * un.z);
-  if constexpr (MODE == 2) {
-    static_cast<Out*>(dt_rho)[i] = (Out)(f.kmass * detsum);
-    static_cast<Out*>(mass_rho)[i] = (Out)(kmr * detsum);
-  }
-  if constexpr (MODE == 0) {
-    // diagonal from the partition of unity, as in the row gather
-    double s[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int q = 0; q < len; ++q)
-      if (q != dpos)
-        for (int k = 0; k < 4; ++k) s[k] += acc[q][k];
-    acc[dpos][0] = f.kmass * detsum - s[0];
-    for (int k = 1; k < 4; ++k) acc[dpos][k] = s[k] / 3.0;
-    Out* Ao = static_cast<Out*>(A) + rs;
-    Out* Go = static_cast<Out*>(G) + rs;
-    for (int q = 0; q < len; ++q) {
-      Ao[q] = (Out)acc[q][0];
-      for (int d = 0; d < 3; ++d) Go[d * m.nnz + q] = (Out)(-acc[q][d + 1] / 24.0);
-    }
   }
 }
+template <typename T>
+__device__ __forceinline__ V3<double> vec64(const void* const* comp, int64_t j) {
+  const V3<T> v = load_vec<T>(comp, j);
+  return V3<double>{(double)v.x, (double)v.y, (double)v.z};
+}
 
-// ---------------------------------------------------------- long rows ---
-// Rows the row gather leaves out (more than 32 entries, whose row positions
-// do not fit the walk's five bits, or a star the walk encoder could not
-// cover), computed after the kernels by one thread per row, in double (the
-// coordinates of the handle's copy, the velocities as given): every
-// off-diagonal entry (i, j) sums the contributions of the row's elements that
-// contain j, w . c_j and -c_i / 24 (with i first and the element's other
-// nodes in an even order, so that det > 0); the diagonal follows from the
-// partition of unity as in the row gather, A(i,i) = lumped mass - sum_{j != i}
-// A(i,j) and G(i,i) = 1/3 sum_{j != i} G(i,j).  MODE 0: A, G and rhs; 1: the
-// time step, A = A_static + C(u) (A may alias A_static: each entry is read
-// before it is written, by this thread) and rhs; 2: rhs, dt_rho and
-// mass_rho.  The row's elements are scanned once per entry: the rows are few.
+// ------------------------------------------------- rows without a walk ---
+// Listed rows computed in double, one block per row: the rows the row gather
+// leaves out (more than 32 entries, whose row positions do not fit the walk's
+// five bits, or a star the walk encoder could not cover) and, of the rows of
+// badly shaped elements, those without a walk.  In chunks of a block's threads
+// every thread evaluates one element of the row (the row's node i first, the
+// others in an even order, so that det > 0; its nodes' row positions by binary
+// search) into shared memory and marks it in its entries' bit masks, then every
+// entry's thread adds, in element order, the contributions w . c_j and
+// -c_i / 24 of its marked elements; rows of more entries than threads take the
+// elements again for every tile of entries.  The
+// diagonal follows from the partition of unity as in the row gather,
+// A(i,i) = lumped mass - sum_{j != i} A(i,j) and G(i,i) = 1/3 sum_{j != i}
+// G(i,j).  MODE 0: A, G and rhs; 1: the time step, A = A_static + C(u) (A may
+// alias A_static: each entry is read before it is written, by its thread) and
+// rhs, or with no A (rows of badly shaped elements: the convection does not
+// involve the determinant) rhs alone; 2: rhs, dt_rho and mass_rho.
+// The rows are few and their serial work is what counts: the 71 rows of a
+// pipe's axis (83 entries, 240 elements) take 36 us; with the entries scanning
+// all elements instead of their marked ones 54; with one thread per row the
+// whole assembly of the pipe took 7.2 ms.
+constexpr int ROW_THREADS = 128;
 template <int P, int MODE>
-__global__ void __launch_bounds__(64) long_rows_kernel(MeshView m, FieldView f, const void* A_static, void* A,
-                                                       void* G, void* rhs, void* dt_rho, void* mass_rho, double kmr,
-                                                       const int32_t* rows, const int32_t* ptr, const uint32_t* inc,
-                                                       int64_t count) {
+__global__ void __launch_bounds__(ROW_THREADS) rows64_kernel(MeshView m, FieldView f, RowOut o,
+                                                             const int32_t* __restrict__ rows,
+                                                             const int32_t* __restrict__ ptr,
+                                                             const uint32_t* __restrict__ inc) {
   using Out = typename Prec<P>::Out;
-  const int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (r >= count) return;
-  const int64_t i = rows[r];
+  constexpr int B = ROW_THREADS;
+  __shared__ double ea[B][3], ec[B][3], red[5][B / 32];
+  __shared__ int ep[B][3];
+  __shared__ unsigned mask[B][B / 32];  // per entry of the tile: the chunk's elements that hold it
+  __shared__ int32_t near[4 * B];       // the row's columns, or the first of them
+  const int tid = threadIdx.x;
+  const int64_t r = blockIdx.x, i = rows[r];
   const int32_t rs = m.row_ptr[i], len = m.row_ptr[i + 1] - rs;
   const int32_t* cols = m.col_idx + rs;
-  auto coord = [&](int64_t j) {
-    if constexpr (P == NSI_FP64) {
-      const D4 x = m.xyz64[j];
-      return V3<double>{x.x, x.y, x.z};
-    } else {
-      const float4 h = m.xyz_hi[j], l = m.xyz_lo[j];
-      return V3<double>{(double)h.x + (double)l.x, (double)h.y + (double)l.y, (double)h.z + (double)l.z};
-    }
-  };
-  auto vel = [&](const void* const* comp, int64_t j) {
-    if constexpr (P == NSI_FP64) return load_vec<double>(comp, j);
-    else {
-      const V3<float> w = load_vec<float>(comp, j);
-      return V3<double>{w.x, w.y, w.z};
-    }
-  };
+  const int32_t t0 = ptr[r], nel = ptr[r + 1] - t0;
+  auto vel = [&](const void* const* comp, int64_t j) { return vec64<typename Prec<P>::T>(comp, j); };
   // even permutations of (0,1,2,3) that bring vertex a to the front
   const int EVEN[4][3] = {{1, 2, 3}, {0, 3, 2}, {3, 0, 1}, {2, 1, 0}};
-  const V3<double> xi = coord(i), ui = vel(f.u, i);
-  // one element of the row: its other nodes in even order, their edge vectors
-  // from node i, cofactors c[0..2] = det(J) grad N of those nodes, c_i, det
-  struct El {
-    int v[3];
-    V3<double> c[3], ci;
-    double det;
-    V3<double> w;  // rho/120 (2 u_i + sum of the others) + (MODE 0) mu/(6 det) c_i
-  };
-  auto element = [&](int32_t t) {
-    El el;
-    const int64_t e = inc[t] >> 2;
-    const int a = (int)(inc[t] & 3u);
-    const int4 v4 = m.lnods[e];
-    const int v[4] = {v4.x, v4.y, v4.z, v4.w};
-    V3<double> d[3], us{2.0 * ui.x, 2.0 * ui.y, 2.0 * ui.z};
-    for (int b = 0; b < 3; ++b) {
-      el.v[b] = v[EVEN[a][b]];
-      d[b] = sub(coord(el.v[b]), xi);
-      us = add(us, vel(f.u, el.v[b]));
+  const V3<double> xi = coord64<P>(m, i), ui = vel(f.u, i);
+  // of this thread: the determinants of its elements, its entries' sums for the diagonal
+  double det = 0.0, sa = 0.0, sg[3] = {0.0, 0.0, 0.0};
+  const bool entries = MODE == 0 || (MODE == 1 && o.A);
+  if (entries)
+    for (int q = tid; q < min(len, 4 * B); q += B) near[q] = cols[q];
+  // position of column j in the row (columns ascending)
+  auto position = [&](int32_t j) {
+    int lo = 0, hi = len - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if ((mid < 4 * B ? near[mid] : cols[mid]) < j) lo = mid + 1;
+      else hi = mid;
     }
-    el.c[0] = cross(d[1], d[2]);
-    el.c[1] = cross(d[2], d[0]);
-    el.c[2] = cross(d[0], d[1]);
-    el.det = dot(d[0], el.c[0]);
-    el.ci = V3<double>{-(el.c[0].x + el.c[1].x + el.c[2].x), -(el.c[0].y + el.c[1].y + el.c[2].y),
-                       -(el.c[0].z + el.c[1].z + el.c[2].z)};
-    const double kv = MODE == 0 ? f.kmu / el.det : 0.0;
-    el.w = V3<double>{f.kc * us.x + kv * el.ci.x, f.kc * us.y + kv * el.ci.y, f.kc * us.z + kv * el.ci.z};
-    return el;
+    return lo;
   };
-  double detsum = 0.0;
-  for (int32_t t = ptr[r]; t < ptr[r + 1]; ++t) detsum += element(t).det;
-  if constexpr (MODE != 2) {
-    Out* Ao = static_cast<Out*>(A) + rs;
-    const Out* As = MODE == 1 ? static_cast<const Out*>(A_static) + rs : nullptr;
-    Out* Go = MODE == 0 ? static_cast<Out*>(G) + rs : nullptr;
-    double sa = 0.0, sg[3] = {0.0, 0.0, 0.0};
-    int dpos = 0;
-    for (int q = 0; q < len; ++q) {
-      const int32_t j = cols[q];
-      if (j == i) {
-        dpos = q;
-        continue;
+  for (int q0 = 0; q0 == 0 || (entries && q0 < len); q0 += B) {
+    const int q = q0 + tid;
+    const bool mine = entries && q < len && cols[q] != i;
+    double a = 0.0, g[3] = {0.0, 0.0, 0.0};
+    for (int c0 = 0; c0 < nel; c0 += B) {
+      __syncthreads();  // the previous chunk is used up
+      if (entries) {
+        for (int w = 0; w < B / 32; ++w) mask[tid][w] = 0u;
+        __syncthreads();
       }
-      double a = 0.0, g[3] = {0.0, 0.0, 0.0};
-      for (int32_t t = ptr[r]; t < ptr[r + 1]; ++t) {
-        const int4 v4 = m.lnods[inc[t] >> 2];
-        if (v4.x != j && v4.y != j && v4.z != j && v4.w != j) continue;
-        const El el = element(t);
-        const int b = el.v[0] == j ? 0 : el.v[1] == j ? 1 : 2;
-        a += dot(el.w, el.c[b]);
-        g[0] += el.ci.x;
-        g[1] += el.ci.y;
-        g[2] += el.ci.z;
+      if (c0 + tid < nel) {
+        const uint32_t w = inc[t0 + c0 + tid];
+        const int4 v4 = m.lnods[w >> 2];
+        const int v[4] = {v4.x, v4.y, v4.z, v4.w};
+        int nb[3];
+        V3<double> d[3], us{2.0 * ui.x, 2.0 * ui.y, 2.0 * ui.z};
+        for (int b = 0; b < 3; ++b) {
+          nb[b] = v[EVEN[w & 3u][b]];
+          d[b] = sub(coord64<P>(m, nb[b]), xi);
+        }
+        const V3<double> c[3] = {cross(d[1], d[2]), cross(d[2], d[0]), cross(d[0], d[1])};
+        const double dt = dot(d[0], c[0]);
+        if (q0 == 0) det += dt;
+        if (entries) {
+          const V3<double> ci{-(c[0].x + c[1].x + c[2].x), -(c[0].y + c[1].y + c[2].y), -(c[0].z + c[1].z + c[2].z)};
+          for (int b = 0; b < 3; ++b) us = add(us, vel(f.u, nb[b]));
+          const double kv = MODE == 0 ? f.kmu / dt : 0.0;
+          const V3<double> w3{f.kc * us.x + kv * ci.x, f.kc * us.y + kv * ci.y, f.kc * us.z + kv * ci.z};
+          for (int b = 0; b < 3; ++b) {
+            ea[tid][b] = dot(w3, c[b]);
+            ep[tid][b] = position(nb[b]);
+            const int e = ep[tid][b] - q0;
+            if (e >= 0 && e < B) atomicOr(&mask[e][tid >> 5], 1u << (tid & 31));
+          }
+          ec[tid][0] = ci.x;
+          ec[tid][1] = ci.y;
+          ec[tid][2] = ci.z;
+        }
       }
+      __syncthreads();
+      if (mine) {
+        for (int w = 0; w < B / 32; ++w)
+          for (unsigned bits = mask[tid][w]; bits; bits &= bits - 1) {
+            const int e = 32 * w + __ffs(bits) - 1;
+            a += ea[e][ep[e][0] == q ? 0 : ep[e][1] == q ? 1 : 2];
+            if constexpr (MODE == 0)
+              for (int d = 0; d < 3; ++d) g[d] += ec[e][d];
+          }
+      }
+    }
+    if (mine) {
       sa += a;
       if constexpr (MODE == 0) {
-        Ao[q] = (Out)a;
+        static_cast<Out*>(o.A)[rs + q] = (Out)a;
         for (int d = 0; d < 3; ++d) {
-          Go[d * m.nnz + q] = (Out)(-g[d] / 24.0);
+          static_cast<Out*>(o.G)[d * m.nnz + rs + q] = (Out)(-g[d] / 24.0);
           sg[d] += g[d];
         }
-      } else {
-        Ao[q] = (Out)((double)As[q] + a);
+      } else if constexpr (MODE == 1) {
+        static_cast<Out*>(o.A)[rs + q] = (Out)((double)static_cast<const Out*>(o.A_static)[rs + q] + a);
       }
     }
-    if (len > 0) {
-      if constexpr (MODE == 0) {
-        Ao[dpos] = (Out)(f.kmass * detsum - sa);
-        for (int d = 0; d < 3; ++d) Go[d * m.nnz + dpos] = (Out)(-sg[d] / 72.0);
-      } else {
-        Ao[dpos] = (Out)((double)As[dpos] - sa);
-      }
+  }
+  // the row's totals: a tree over each warp, then the warps in order
+  double tot[5] = {det, sa, sg[0], sg[1], sg[2]};
+  for (int k = 0; k < 5; ++k) {
+    for (int off = 16; off > 0; off >>= 1) tot[k] += __shfl_xor_sync(0xffffffffu, tot[k], off);
+    if ((tid & 31) == 0) red[k][tid >> 5] = tot[k];
+  }
+  __syncthreads();
+  if (tid != 0) return;
+  for (int k = 0; k < 5; ++k) {
+    tot[k] = 0.0;
+    for (int w = 0; w < B / 32; ++w) tot[k] += red[k][w];
+  }
+  if (entries && len > 0) {
+    const int lo = position((int32_t)i);
+    Out* A = static_cast<Out*>(o.A) + rs + lo;
+    if constexpr (MODE == 0) {
+      *A = (Out)(f.kmass * tot[0] - tot[1]);
+      for (int d = 0; d < 3; ++d) static_cast<Out*>(o.G)[d * m.nnz + rs + lo] = (Out)(-tot[2 + d] / 72.0);
+    } else {
+      *A = (Out)((double)static_cast<const Out*>(o.A_static)[rs + lo] - tot[1]);
     }
   }
   const V3<double> un = vel(f.un, i);
-  Out* Rh = static_cast<Out*>(rhs);
-  Rh[i] = (Out)(f.kmass * detsum * un.x);
-  Rh[m.n + i] = (Out)(f.kmass * detsum * un.y);
-  Rh[2 * m.n + i] = (Out)(f.kmass * detsum * un.z);
+  const double mass = f.kmass * tot[0];
+  Out* Rh = static_cast<Out*>(o.rhs);
+  Rh[i] = (Out)(mass * un.x);
+  Rh[m.n + i] = (Out)(mass * un.y);
+  Rh[2 * m.n + i] = (Out)(mass * un.z);
   if constexpr (MODE == 2) {
-    static_cast<Out*>(dt_rho)[i] = (Out)(f.kmass * detsum);
-    static_cast<Out*>(mass_rho)[i] = (Out)(kmr * detsum);
+    static_cast<Out*>(o.dt_rho)[i] = (Out)mass;
+    static_cast<Out*>(o.mass_rho)[i] = (Out)(o.kmr * tot[0]);
   }
 }
 
@@ -1431,24 +1368,6 @@ __device__ __forceinline__ bool marked(const uint32_t* __restrict__ mask, int64_
   return mask && ((mask[e >> 5] >> (e & 31)) & 1u);
 }
 
-// the element's coordinates, velocities and weights in double (the handle's
-// copy of the coordinates: double, or the float hi + lo pair)
-template <int P>
-__device__ __forceinline__ V3<double> coord64(const MeshView& m, int64_t j) {
-  if constexpr (P == NSI_FP64) {
-    const D4 x = m.xyz64[j];
-    return V3<double>{x.x, x.y, x.z};
-  } else {
-    const float4 h = m.xyz_hi[j], l = m.xyz_lo[j];
-    return V3<double>{(double)h.x + (double)l.x, (double)h.y + (double)l.y, (double)h.z + (double)l.z};
-  }
-}
-template <typename T>
-__device__ __forceinline__ V3<double> vec64(const void* const* comp, int64_t j) {
-  const V3<T> v = load_vec<T>(comp, j);
-  return V3<double>{(double)v.x, (double)v.y, (double)v.z};
-}
-
 // The adjoint, one element per thread, in the handle's arithmetic; the
 // elements marked in `skip` (badly shaped, mixed modes) are left to
 // vjp_exact_kernel.
@@ -1643,54 +1562,46 @@ static nsi_status zero_outputs(const NsiHandle* h, const OutView& o, cudaStream_
   return NSI_OK;
 }
 
-// after an assembly or time step in a mixed mode: the rows listed at create
-// for badly shaped elements, recomputed in double (nothing if there are none)
+// listed rows by one block each
 template <int P>
-static nsi_status fix_exact_rows(NsiHandle* h, const FieldView& f, int mode, void* A, void* G, void* rhs,
-                                 void* dt_rho, void* mass_rho, double kmr, cudaStream_t s) {
-  if constexpr (P == NSI_FP64) {
-    return NSI_OK;
-  } else {
-    if (h->exact_rows == 0) return NSI_OK;
-    const MeshView m = view_of(h);
-    const int blk = 64;
-    const int64_t grid = (h->exact_rows + blk - 1) / blk;
-    if (mode == 0)
-      exact_rows_kernel<P, 0><<<grid, blk, 0, s>>>(m, f, A, G, rhs, dt_rho, mass_rho, kmr, h->exact_list,
-                                                  h->exact_ptr, h->exact_inc, h->exact_rows);
-    else if (mode == 1)
-      exact_rows_kernel<P, 1><<<grid, blk, 0, s>>>(m, f, A, G, rhs, dt_rho, mass_rho, kmr, h->exact_list,
-                                                  h->exact_ptr, h->exact_inc, h->exact_rows);
-    else
-      exact_rows_kernel<P, 2><<<grid, blk, 0, s>>>(m, f, A, G, rhs, dt_rho, mass_rho, kmr, h->exact_list,
-                                                  h->exact_ptr, h->exact_inc, h->exact_rows);
-    return check_launch("exact_rows_kernel");
+static nsi_status launch_rows64(NsiHandle* h, const FieldView& f, int mode, const RowOut& o, const int32_t* rows,
+                                const int32_t* ptr, const uint32_t* inc, int64_t count, cudaStream_t s) {
+  const MeshView m = view_of(h);
+  if (mode == 0) rows64_kernel<P, 0><<<count, ROW_THREADS, 0, s>>>(m, f, o, rows, ptr, inc);
+  else if (mode == 1) rows64_kernel<P, 1><<<count, ROW_THREADS, 0, s>>>(m, f, o, rows, ptr, inc);
+  else rows64_kernel<P, 2><<<count, ROW_THREADS, 0, s>>>(m, f, o, rows, ptr, inc);
+  return check_launch("rows64_kernel");
+}
+
+// after an assembly or time step in a mixed mode: the rows listed at create
+// for badly shaped elements, recomputed in double (nothing if there are none);
+// the time step's A does not depend on the determinant and stays
+template <int P>
+static nsi_status fix_exact_rows(NsiHandle* h, const FieldView& f, int mode, const RowOut& out, cudaStream_t s) {
+  if constexpr (P != NSI_FP64) {
+    RowOut o = out;
+    if (mode == 1) o.A = nullptr;
+    if (h->exact_rows > 0) {
+      nsi_status st = launch_exact_rows<P>(h, f, mode, o, s);
+      if (st) return st;
+    }
+    if (h->exact_rest > 0)
+      return launch_rows64<P>(h, f, mode, o, h->exact_list + h->exact_rows, h->exact_ptr + h->exact_rows,
+                              h->exact_inc, h->exact_rest, s);
   }
+  return NSI_OK;
+}
+
+// after any row-gather assembly or time step: the long rows (nothing if there
+// are none)
+template <int P>
+static nsi_status fix_long_rows(NsiHandle* h, const FieldView& f, int mode, const RowOut& o, cudaStream_t s) {
+  if (h->long_rows == 0) return NSI_OK;
+  return launch_rows64<P>(h, f, mode, o, h->long_list, h->long_ptr, h->long_inc, h->long_rows, s);
 }
 
 // `rec` (nullptr: the handle's buffer) receives the row gather's per-call
 // node records
-// after any row-gather assembly or time step: the long rows (nothing if
-// there are none)
-template <int P>
-static nsi_status fix_long_rows(NsiHandle* h, const FieldView& f, int mode, const void* A_static, void* A, void* G,
-                                void* rhs, void* dt_rho, void* mass_rho, double kmr, cudaStream_t s) {
-  if (h->long_rows == 0) return NSI_OK;
-  const MeshView m = view_of(h);
-  const int blk = 64;
-  const int64_t grid = (h->long_rows + blk - 1) / blk;
-  if (mode == 0)
-    long_rows_kernel<P, 0><<<grid, blk, 0, s>>>(m, f, A_static, A, G, rhs, dt_rho, mass_rho, kmr, h->long_list,
-                                               h->long_ptr, h->long_inc, h->long_rows);
-  else if (mode == 1)
-    long_rows_kernel<P, 1><<<grid, blk, 0, s>>>(m, f, A_static, A, G, rhs, dt_rho, mass_rho, kmr, h->long_list,
-                                               h->long_ptr, h->long_inc, h->long_rows);
-  else
-    long_rows_kernel<P, 2><<<grid, blk, 0, s>>>(m, f, A_static, A, G, rhs, dt_rho, mass_rho, kmr, h->long_list,
-                                               h->long_ptr, h->long_inc, h->long_rows);
-  return check_launch("long_rows_kernel");
-}
-
 template <int P>
 static nsi_status assemble_core_p(NsiHandle* h, const FieldView& f, const OutView& o, int mode, cudaStream_t s,
                                   void* rec = nullptr) {
@@ -1752,9 +1663,10 @@ template <int P>
 static nsi_status assemble_p(NsiHandle* h, const FieldView& f, const OutView& o, int mode, cudaStream_t s) {
   nsi_status st = assemble_core_p<P>(h, f, o, mode, s);
   if (st) return st;
-  st = fix_exact_rows<P>(h, f, 0, o.A, o.G, o.rhs, nullptr, nullptr, 0.0, s);
+  const RowOut ro{nullptr, o.A, o.G, o.rhs, nullptr, nullptr, 0.0};
+  st = fix_exact_rows<P>(h, f, 0, ro, s);
   if (st || mode != NSI_SCATTER_GATHER) return st;
-  return fix_long_rows<P>(h, f, 0, nullptr, o.A, o.G, o.rhs, nullptr, nullptr, 0.0, s);
+  return fix_long_rows<P>(h, f, 0, ro, s);
 }
 
 static nsi_status check_call(const NsiHandle* h, const NsiFields* f, const NsiOutputs* o) {
@@ -1798,9 +1710,10 @@ static nsi_status step_p(NsiHandle* h, const FieldView& f, const StepView& o, cu
   nsi_status st = launch_pack<P>(h, f, nullptr, s);
   if (!st) st = launch_step<P>(h, f, o, NODAL, s);
   if (st) return st;
-  st = fix_exact_rows<P>(h, f, NODAL ? 2 : 1, nullptr, nullptr, o.rhs, o.dt_rho, o.mass_rho, o.kmr, s);
+  const RowOut ro{o.A_static, o.A, nullptr, o.rhs, o.dt_rho, o.mass_rho, o.kmr};
+  st = fix_exact_rows<P>(h, f, NODAL ? 2 : 1, ro, s);
   if (st) return st;
-  return fix_long_rows<P>(h, f, NODAL ? 2 : 1, o.A_static, o.A, nullptr, o.rhs, o.dt_rho, o.mass_rho, o.kmr, s);
+  return fix_long_rows<P>(h, f, NODAL ? 2 : 1, ro, s);
 }
 
 static nsi_status step_dispatch(NsiHandle* h, const NsiFields* f, const StepView& o, bool nodal, cudaStream_t s) {
@@ -1829,11 +1742,9 @@ static nsi_status batched_p(NsiHandle* const* hs, const NsiFields* fs, const Nsi
                             cudaStream_t s) {
   nsi_status st = batched_core_p<P>(hs, fs, os, count, s);
   for (int k = 0; k < count && !st; ++k) {
-    st = fix_exact_rows<P>(hs[k], fields_of(&fs[k]), 0, os[k].A_val, os[k].G_val, os[k].rhs, nullptr, nullptr, 0.0,
-                           s);
-    if (!st)
-      st = fix_long_rows<P>(hs[k], fields_of(&fs[k]), 0, nullptr, os[k].A_val, os[k].G_val, os[k].rhs, nullptr,
-                            nullptr, 0.0, s);
+    const RowOut ro{nullptr, os[k].A_val, os[k].G_val, os[k].rhs, nullptr, nullptr, 0.0};
+    st = fix_exact_rows<P>(hs[k], fields_of(&fs[k]), 0, ro, s);
+    if (!st) st = fix_long_rows<P>(hs[k], fields_of(&fs[k]), 0, ro, s);
   }
   return st;
 }
@@ -1934,9 +1845,10 @@ static nsi_status assemble_noalloc_p(NsiHandle* h, const FieldView& f, const Out
                                      cudaStream_t s) {
   nsi_status st = assemble_core_p<P>(h, f, o, NSI_SCATTER_GATHER, s, scratch);
   if (st) return st;
-  st = fix_exact_rows<P>(h, f, 0, o.A, o.G, o.rhs, nullptr, nullptr, 0.0, s);
+  const RowOut ro{nullptr, o.A, o.G, o.rhs, nullptr, nullptr, 0.0};
+  st = fix_exact_rows<P>(h, f, 0, ro, s);
   if (st) return st;
-  return fix_long_rows<P>(h, f, 0, nullptr, o.A, o.G, o.rhs, nullptr, nullptr, 0.0, s);
+  return fix_long_rows<P>(h, f, 0, ro, s);
 }
 
 }  // namespace nsi
@@ -2039,9 +1951,10 @@ static nsi_status stabilized_p(NsiHandle* h, const FieldView& f, const StabConst
                                                                  h->long_inc, h->long_rows);
     if ((st = check_launch("stab_rows_kernel (long rows)"))) return st;
   }
-  if (P == NSI_FP64 || h->exact_rows == 0) return NSI_OK;
-  stab_rows_kernel<P><<<(h->exact_rows + 63) / 64, 64, 0, s>>>(m, f, sc, Auu, G, rhs, h->exact_list, h->exact_ptr,
-                                                                h->exact_inc, h->exact_rows);
+  const int64_t exact = h->exact_rows + h->exact_rest;
+  if (P == NSI_FP64 || exact == 0) return NSI_OK;
+  stab_rows_kernel<P><<<(exact + 63) / 64, 64, 0, s>>>(m, f, sc, Auu, G, rhs, h->exact_list, h->exact_ptr,
+                                                       h->exact_inc, exact);
   return check_launch("stab_rows_kernel (exact rows)");
 }
 
@@ -2309,7 +2222,7 @@ nsi_status nsi_assemble_host(NsiHandle* h, const NsiFields* f, const NsiOutputs*
   }
   char* ob = base + ((u_bytes + 255) / 256) * 256;
   NsiOutputs od{ob, ob + osz * h->nnz, ob + osz * 4 * h->nnz};
-  if (resolve_mode(h, NSI_SCATTER_AUTO) == NSI_SCATTER_GATHER && !h->use_fan && h->n > 0 && h->exact_rows == 0 &&
+  if (resolve_mode(h, NSI_SCATTER_AUTO) == NSI_SCATTER_GATHER && !h->use_fan && h->n > 0 && h->exact_rows + h->exact_rest == 0 &&
       h->long_rows == 0) {
     int dev = 0;
     cudaGetDevice(&dev);

@@ -51,3 +51,46 @@ def test_batch_of_both_kinds_equals_single(precision):
     for s, b in zip(single, nsi.assemble_batched(asms, us)):
         for x, y in zip(s, b):
             assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("precision", ["mixed64", "mixed32"])
+@pytest.mark.parametrize("N", [1, 7, 22])  # four lanes per row (8 and 512 rows), two (12,167)
+def test_flat_cube_rows_in_double(precision, N):
+    """A cube 40 times flatter than wide: every element is badly shaped, every
+    row is recomputed in double, so mixed64 is as exact as its inputs (the
+    coordinates are kept as float pairs, 2^-48 of the domain against flat edges
+    of 1/(40 N)) and mixed32 as its float outputs."""
+    mesh, u = meshgen.config_mesh(N=N, jitter=0.1, numbering="random", seed=320 + N)
+    coord = mesh.coord * np.array([1.0, 1.0, 1.0 / 40])
+    asm = nsi.Assembler(coord, mesh.lnods, precision=precision)
+    assert asm.info().exact_rows == mesh.n_nodes
+    tol = 1e-10 if precision == "mixed64" else 3e-7
+    ut = torch.as_tensor(u.T.copy())
+    uo = u.astype(np.float32).astype(np.float64)
+    rp, _, oA, oG, orhs = oracle.assemble(coord, mesh.lnods, uo, None, 1.0, 1e-3, 1e-2)
+    got = [t.double().cpu().numpy() for t in asm.assemble(ut, rho=1.0, mu=1e-3, dt=1e-2)]
+    assert max(errors(rp, *got, oA, oG, orhs).values()) <= tol
+    A_static, _ = asm.static_part(rho=1.0, mu=1e-3, dt=1e-2)
+    A2, rhs2 = asm.assemble_convective(ut, A_static, rho=1.0, mu=1e-3, dt=1e-2)
+    got = [A2.double().cpu().numpy(), oG, rhs2.double().cpu().numpy()]
+    assert max(errors(rp, *got, oA, oG, orhs).values()) <= 1e-5
+    onr, ondt, onm = oracle.nodal(coord, mesh.lnods, uo, 1.0, 1e-2)
+    r3, dtr, mr = (t.double().cpu().numpy() for t in asm.nodal(ut, rho=1.0, dt=1e-2))
+    assert max([vec_scaled_err(dtr, ondt), vec_scaled_err(mr, onm)] +
+               [vec_scaled_err(r3[k], onr[k]) for k in range(3)]) <= tol
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed64", "mixed32"])
+def test_row_of_more_entries_than_a_block_has_threads(precision):
+    mesh, u = meshgen.delaunay_hub(8, 200, seed=330)
+    asm = nsi.Assembler(mesh.coord, mesh.lnods, precision=precision)
+    assert asm.max_row > 128 and asm.info().long_rows > 0
+    ut = torch.as_tensor(u.T.copy())
+    uo = u if precision == "fp64" else u.astype(np.float32).astype(np.float64)
+    rp, _, oA, oG, orhs = oracle.assemble(mesh.coord, mesh.lnods, uo, None, 1.0, 1e-3, 1e-2)
+    got = [t.double().cpu().numpy() for t in asm.assemble(ut, rho=1.0, mu=1e-3, dt=1e-2)]
+    assert max(errors(rp, *got, oA, oG, orhs).values()) <= TOL[precision]
+    A_static, _ = asm.static_part(rho=1.0, mu=1e-3, dt=1e-2)
+    A2, rhs2 = asm.assemble_convective(ut, A_static, rho=1.0, mu=1e-3, dt=1e-2)
+    got = [A2.double().cpu().numpy(), oG, rhs2.double().cpu().numpy()]
+    assert max(errors(rp, *got, oA, oG, orhs).values()) <= TOL[precision]
