@@ -17,6 +17,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 import threading
 
 from . import _build
@@ -119,6 +120,8 @@ def library_path() -> str:
 def load_library(build: bool = True):
     """Load (building first if needed) the CUDA library; raises if it cannot be built."""
     global _lib
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             path = _build.build() if build else _build.LIB
@@ -242,20 +245,35 @@ def nsi_device_status(h, stream=None):
 
 
 # --------------------------------------------------------------- torch layer --
+_torch_module = None
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
 
 
 def _stream_ptr(stream):
-    torch = _torch()
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+        torch = _torch()
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream
 
 
 def _ptr(t):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None else None
+    return t.data_ptr() if t is not None else None
+
+
+# the bytes of an NsiFields (u[3], u_n[3], rho, mu, dt) and of an NsiOutputs
+_FIELDS, _OUTPUTS = struct.Struct("@6P3d"), struct.Struct("@3P")
+assert _FIELDS.size == ctypes.sizeof(NsiFields) and _OUTPUTS.size == ctypes.sizeof(NsiOutputs)
+
+
+def _outputs(A, G, rhs):
+    return NsiOutputs.from_buffer_copy(_OUTPUTS.pack(A.data_ptr(), G.data_ptr(), rhs.data_ptr()))
 
 
 class Assembler:
@@ -290,6 +308,7 @@ class Assembler:
         opts = NsiOptions(self.precision, self.scatter, 0, int(bool(debug_checks)))
         with torch.cuda.device(self.device):
             self.handle = nsi_assemble_create(mesh, opts, _stream_ptr(stream))
+            self._index = torch.cuda.current_device()
         info = nsi_info(self.handle)
         self.scatter = info.scatter  # the handle's default mode, resolved by the library
         self.n, self.E, self.nnz = info.n_nodes, info.n_elems, info.nnz
@@ -319,6 +338,21 @@ class Assembler:
         return self._pattern
 
     # ------------------------------------------------------------- marshal
+    def _is_ready(self, u):
+        """True for a [3, n] tensor that the library can read in place: its
+        component pointers are then base + k * n values."""
+        return (type(u) is _torch().Tensor and u.dtype is self.vel_dtype and u.is_cuda and
+                u.get_device() == self._index and u.dim() == 2 and u.shape[0] == 3 and u.shape[1] == self.n and
+                u.is_contiguous())
+
+    def _vel_ptrs(self, u):
+        """(pointers of the three components, what keeps them alive)."""
+        if self._is_ready(u):
+            p, step = u.data_ptr(), self.n * u.element_size()
+            return (p, p + step, p + 2 * step), u
+        comps = self._vel(u)
+        return tuple(c.data_ptr() for c in comps), comps
+
     def _vel(self, u):
         torch = _torch()
         if isinstance(u, (tuple, list)):
@@ -336,14 +370,11 @@ class Assembler:
         return out
 
     def fields(self, u, u_n=None, rho=1.0, mu=1e-3, dt=1e-2):
-        comps = self._vel(u)
-        ncomps = self._vel(u_n) if u_n is not None else None
-        f = NsiFields()
-        for k in range(3):
-            f.u[k] = comps[k].data_ptr()
-            f.u_n[k] = ncomps[k].data_ptr() if ncomps is not None else None
-        f.rho, f.mu, f.dt = float(rho), float(mu), float(dt)
-        return f, (comps, ncomps)
+        # one struct from bytes: a field-by-field ctypes structure and three
+        # slices per velocity took two thirds of a small call
+        pu, keep = self._vel_ptrs(u)
+        pn, keep_n = self._vel_ptrs(u_n) if u_n is not None else ((0, 0, 0), None)
+        return NsiFields.from_buffer_copy(_FIELDS.pack(*pu, *pn, float(rho), float(mu), float(dt))), (keep, keep_n)
 
     def empty_outputs(self):
         torch = _torch()
@@ -357,7 +388,7 @@ class Assembler:
         """Assemble (A, G, rhs) for nodal velocity u ([3, n], [n, 3] or 3 tensors)."""
         f, keep = self.fields(u, u_n, rho, mu, dt)
         A, G, rhs = out if out is not None else self.empty_outputs()
-        o = NsiOutputs(A.data_ptr(), G.data_ptr(), rhs.data_ptr())
+        o = _outputs(A, G, rhs)
         mode = self.scatter if scatter is None else (SCATTERS[scatter] if isinstance(scatter, str) else scatter)
         nsi_assemble_mode(self.handle, f, o, mode, _stream_ptr(stream))
         return A, G, rhs
@@ -433,7 +464,7 @@ class Assembler:
         """(grad_u [3, n], grad_mu) of sum(w * R(u, mu))."""
         torch = _torch()
         f, keep = self.fields(u, None, rho, mu, dt)
-        wc = torch.stack(self._vel(w)).contiguous()
+        wc = w if self._is_ready(w) else torch.stack(self._vel(w)).contiguous()
         gu = torch.empty(3, self.n, dtype=self.vel_dtype, device=self.device)
         gmu = torch.empty(1, dtype=torch.float64, device=self.device)
         nsi_assemble_vjp(self.handle, f, _ptr(wc), _ptr(gu), _ptr(gmu), _stream_ptr(stream))
@@ -537,7 +568,7 @@ def assemble_batched(assemblers, us, rho=1.0, mu=1e-3, dt=1e-2, outs=None, strea
         fields.append(f)
         keep.append(kp)
         A, G, rhs = outs[k] if outs is not None else asm.empty_outputs()
-        outputs.append(NsiOutputs(A.data_ptr(), G.data_ptr(), rhs.data_ptr()))
+        outputs.append(_outputs(A, G, rhs))
         results.append((A, G, rhs))
     nsi_assemble_batched([a.handle for a in assemblers], fields, outputs, _stream_ptr(stream))
     return results

@@ -1072,14 +1072,20 @@ nsi_status allow_smem(K kernel, std::once_flag& once, cudaError_t& err) {
 }
 
 // blocks of a persistent launch: as many as are resident at once, no more
-// than the groups need
+// than the groups need.  `resident` keeps the first number for a launch shape
+// (0: not asked for yet; the device's answer takes longer than a small launch).
 template <typename K>
-nsi_status resident_grid(K kernel, int warps, size_t smem, int64_t groups, int64_t* grid) {
-  int per_sm = 0, sms = 0, dev = 0;
-  NSI_CUDA(cudaGetDevice(&dev));
-  NSI_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  NSI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 32 * warps, smem));
-  *grid = std::max<int64_t>(1, std::min<int64_t>((groups + warps - 1) / warps, (int64_t)std::max(1, per_sm) * sms));
+nsi_status resident_grid(K kernel, int warps, size_t smem, int64_t groups, std::atomic<int>* resident, int64_t* grid) {
+  int at_once = resident ? resident->load(std::memory_order_relaxed) : 0;
+  if (at_once == 0) {
+    int per_sm = 0, sms = 0, dev = 0;
+    NSI_CUDA(cudaGetDevice(&dev));
+    NSI_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    NSI_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, 32 * warps, smem));
+    at_once = std::max(1, per_sm) * sms;
+    if (resident) resident->store(at_once, std::memory_order_relaxed);
+  }
+  *grid = std::max<int64_t>(1, std::min<int64_t>((groups + warps - 1) / warps, at_once));
   return NSI_OK;
 }
 
@@ -1096,7 +1102,7 @@ nsi_status run_groups(NsiHandle* h, const WalkItem<MODE>& item, int64_t row0, in
   const size_t smem = lay.total() * pl.warps;
   const int64_t g0 = row0 / RW, g1 = (row1 + RW - 1) / RW;
   int64_t grid = 0;
-  if ((st = resident_grid(kernel, pl.warps, smem, g1 - g0, &grid))) return st;
+  if ((st = resident_grid(kernel, pl.warps, smem, g1 - g0, &h->resident[MODE][pl.warps - 1], &grid))) return st;
   if (h->ev_start) NSI_CUDA(cudaEventRecord(h->ev_start, s));
   kernel<<<grid, 32 * pl.warps, smem, s>>>(item, GroupLay(lay), (int)g0, (int)g1);
   if (h->ev_stop) NSI_CUDA(cudaEventRecord(h->ev_stop, s));
@@ -1198,7 +1204,7 @@ nsi_status launch_batched(NsiHandle* const* hs, const NsiFields* fs, const NsiOu
   batched_pack_kernel<P><<<(args.total[0] + 7) / 8 + (args.total[1] + 15) / 16, 128, 0, s>>>(args);
   if ((st = check_launch("batched_pack_kernel"))) return st;
   int64_t grid = 0;
-  if ((st = resident_grid(batched_kernel<P>, warps, bytes * warps, groups, &grid))) return st;
+  if ((st = resident_grid(batched_kernel<P>, warps, bytes * warps, groups, nullptr, &grid))) return st;
   batched_kernel<P><<<grid, 32 * warps, bytes * warps, s>>>(args, GroupLay(lay2), GroupLay(lay4));
   return check_launch("batched_kernel");
 }

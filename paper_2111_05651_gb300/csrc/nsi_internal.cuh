@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <string>
 #include <vector>
 
@@ -222,6 +223,7 @@ struct NsiHandle {
   nsi::GatherPlan plan;         // the launch plan in use
   nsi::GatherPlan plans[4];     // every rows-per-block candidate that fits shared memory
   int n_plans = 0;
+  std::atomic<int> resident[3][4] = {};  // row gather by mode and warps per block: blocks resident at once (0: not known)
   // coordinates: double4 for FP64, float4 hi + float4 lo for the mixed modes
   nsi::D4* xyz64 = nullptr;
   float4* xyz_hi = nullptr;
