@@ -64,6 +64,16 @@ struct NodeRec {
         : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
         : "l"(r));
   }
+  // the record's words from the node's own data, without a packed record
+  template <typename Mesh>
+  __device__ __forceinline__ void gather(const Mesh& m, const FieldView& f, int64_t j) {
+    const uint4 hi = __ldg(reinterpret_cast<const uint4*>(m.xyz_hi + j));
+    const uint4 lo = __ldg(reinterpret_cast<const uint4*>(m.xyz_lo + j));
+    const V3<float> u = load_vec<float>(f.u, j);
+    a = make_uint4(hi.x, hi.y, hi.z, __float_as_uint(u.x));
+    b = make_uint4(__float_as_uint(u.y), __float_as_uint(u.z), (lo.x >> 16) | (lo.y & 0xffff0000u),
+                   lo.z & 0xffff0000u);
+  }
   // edge vector from node o to this one
   __device__ __forceinline__ V3<float> minus(const NodeRec& o) const {
     const V3<float> h{__uint_as_float(a.x) - __uint_as_float(o.a.x), __uint_as_float(a.y) - __uint_as_float(o.a.y),
@@ -83,6 +93,13 @@ struct NodeRec<NSI_FP64> {
     [[maybe_unused]] double pad;
     asm("ld.global.nc.L1::no_allocate.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(x), "=d"(y), "=d"(z), "=d"(pad) : "l"(r));
     asm("ld.global.nc.L1::no_allocate.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(ux), "=d"(uy), "=d"(uz), "=d"(pad) : "l"(r + 4));
+  }
+  template <typename Mesh>
+  __device__ __forceinline__ void gather(const Mesh& m, const FieldView& f, int64_t j) {
+    const D4 p = m.xyz64[j];
+    const V3<double> u = load_vec<double>(f.u, j);
+    x = p.x, y = p.y, z = p.z;
+    ux = u.x, uy = u.y, uz = u.z;
   }
   __device__ __forceinline__ V3<double> minus(const NodeRec& o) const { return {x - o.x, y - o.y, z - o.z}; }
   __device__ __forceinline__ V3<double> vel() const { return {ux, uy, uz}; }
@@ -461,7 +478,10 @@ __device__ __forceinline__ void merge_lanes(Acc<P>& a, int off) {
 // The next group's row bounds are copied under the current walk, its walk
 // bytes and column indices under the merge, and its records are loaded under
 // the write-out.
-template <int P, int H, int MODE, bool DEBUG, typename Source>
+// DIRECT: the nodes' coordinates and velocities are read where they are (five
+// loads a node) instead of from packed records (one), which saves a small mesh
+// the packing launch; the values are the same.
+template <int P, int H, int MODE, bool DEBUG, bool DIRECT, typename Source>
 __device__ __forceinline__ void group_loop(const Source& src, int g, int stride, int g_end, unsigned char* smem,
                                            const GroupLay& lay) {
   using T = typename Prec<P>::T;
@@ -488,10 +508,15 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
   struct Recs {
     NodeRec<P> me, r[UT];
   };
-  auto load_recs = [&](Recs& v, const WalkMesh& m, const GroupRow& r, const int32_t* col, int64_t i, int s0) {
+  auto load_recs = [&](Recs& v, const WalkItem<MODE>& of, const GroupRow& r, const int32_t* col, int64_t i, int s0) {
+    const WalkMesh& m = of.m;
     const int ns = row_slots(r);
     const int64_t self = min(i, m.n - 1);
-    if (s0 == h) v.me.load(m.rec, self);
+    auto load = [&](NodeRec<P>& to, int64_t j) {
+      if constexpr (DIRECT) to.gather(m, of.f, j);
+      else to.load(m.rec, j);
+    };
+    if (s0 == h) load(v.me, self);
 #pragma unroll
     for (int c = 0; c < UT; ++c) {
       const int s = s0 + c * H;
@@ -500,20 +525,20 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
         atomicOr(m.err, ERR_BAD_INDEX);
         k = self;
       }
-      v.r[c].load(m.rec, k);
+      load(v.r[c], k);
     }
   };
   // the group's slots: edge vectors from the row's node, velocities, zeroed
   // sums; 2 rho/120 u_i of the row's own node
   V3<T> u2i;
-  auto put = [&](Recs& v, const WalkMesh& m, const FieldView& f, const GroupRow& r, int64_t i) {
-    const T kc = kc_of<T>(f), kc2 = kc + kc;
+  auto put = [&](Recs& v, const WalkItem<MODE>& of, const GroupRow& r, int64_t i) {
+    const T kc = kc_of<T>(of.f), kc2 = kc + kc;
     const V3<T> ui = v.me.vel();
     u2i = V3<T>{mul_rn(kc2, ui.x), mul_rn(kc2, ui.y), mul_rn(kc2, ui.z)};
     const int ns = DEBUG ? min(row_slots(r), lay.W) : row_slots(r);
 #pragma unroll 1
     for (int s0 = h; s0 < ns; s0 += UT * H) {
-      if (s0 != h) load_recs(v, m, r, m.col_idx + r.rs, i, s0);
+      if (s0 != h) load_recs(v, of, r, of.m.col_idx + r.rs, i, s0);
 #pragma unroll
       for (int c = 0; c < UT; ++c) {
         if (s0 + c * H >= ns) break;
@@ -557,9 +582,10 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
     cp_async_wait_all();
     __syncwarp();
     Recs v;
-    load_recs(v, m, row, cols_of(m, row, base, end), r0 + t, h);
+    if constexpr (!DIRECT) wait_for_records();
+    load_recs(v, src.item(at), row, cols_of(m, row, base, end), r0 + t, h);
     __syncwarp();
-    put(v, m, src.item(at).f, row, r0 + t);
+    put(v, src.item(at), row, r0 + t);
   }
   while (true) {
     const WalkMesh& m = src.item(at).m;
@@ -760,8 +786,8 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
     // the next group's records, in flight during the write-out
     Recs v{};
     if (more) {
-      const WalkMesh& mn = src.item(atn).m;
-      load_recs(v, mn, rown, cols_of(mn, rown, basen, endn), (int64_t)(gn - src.item(atn).group0) * RW + t, h);
+      load_recs(v, src.item(atn), rown, cols_of(src.item(atn).m, rown, basen, endn),
+                (int64_t)(gn - src.item(atn).group0) * RW + t, h);
     }
 
     // 3. the group's contiguous slice of the outputs
@@ -830,7 +856,7 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
     if (!more) return;
     __syncwarp();  // the next group reuses the staging
     refresh();
-    put(v, src.item(atn).m, src.item(atn).f, rown, (int64_t)(gn - src.item(atn).group0) * RW + t);
+    put(v, src.item(atn), rown, (int64_t)(gn - src.item(atn).group0) * RW + t);
     g = gn;
     at = atn;
     row = rown;
@@ -855,7 +881,7 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, P == NSI_FP64 ? 2 : 4)
     gather_persistent_kernel(const __grid_constant__ WalkItem<MODE> item, GroupLay lay, int g0, int g_end) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int warps = blockDim.x >> 5, w = threadIdx.x >> 5;
-  group_loop<P, H, MODE, DEBUG>(OneMesh<MODE>{item}, g0 + (int)blockIdx.x * warps + w, (int)gridDim.x * warps, g_end,
+  group_loop<P, H, MODE, DEBUG, H == 4>(OneMesh<MODE>{item}, g0 + (int)blockIdx.x * warps + w, (int)gridDim.x * warps, g_end,
                                 smem_raw + w * lay.total, lay);
 }
 
@@ -1009,11 +1035,11 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, P == NSI_FP64 ? 2 : 4)
   const int warps = blockDim.x >> 5, w = threadIdx.x >> 5;
   const int all = (int)gridDim.x * warps, me = (int)blockIdx.x * warps + w;
   unsigned char* smem = smem_raw + w * max(lay2.total, lay4.total);
-  group_loop<P, 2, ASSEMBLE, false>(BatchMesh{args, 0, args.count[0]}, me, all, args.total[0], smem, lay2);
+  group_loop<P, 2, ASSEMBLE, false, false>(BatchMesh{args, 0, args.count[0]}, me, all, args.total[0], smem, lay2);
   __syncwarp();
   // (the warps with one group less of the first kind begin the second)
   const int start = me - args.total[0] % all;
-  group_loop<P, 4, ASSEMBLE, false>(BatchMesh{args, args.count[0], args.count[1]}, start < 0 ? start + all : start, all,
+  group_loop<P, 4, ASSEMBLE, false, false>(BatchMesh{args, args.count[0], args.count[1]}, start < 0 ? start + all : start, all,
                                     args.total[1], smem, lay4);
 }
 
@@ -1104,7 +1130,10 @@ nsi_status run_groups(NsiHandle* h, const WalkItem<MODE>& item, int64_t row0, in
   int64_t grid = 0;
   if ((st = resident_grid(kernel, pl.warps, smem, g1 - g0, &h->resident[MODE][pl.warps - 1], &grid))) return st;
   if (h->ev_start) NSI_CUDA(cudaEventRecord(h->ev_start, s));
-  kernel<<<grid, 32 * pl.warps, smem, s>>>(item, GroupLay(lay), (int)g0, (int)g1);
+  if constexpr (H == 4)
+    kernel<<<grid, 32 * pl.warps, smem, s>>>(item, GroupLay(lay), (int)g0, (int)g1);
+  else
+    NSI_CUDA(launch_early(kernel, grid, 32 * pl.warps, smem, s, item, GroupLay(lay), (int)g0, (int)g1));
   if (h->ev_stop) NSI_CUDA(cudaEventRecord(h->ev_stop, s));
   return check_launch("gather_persistent_kernel");
 }
@@ -1205,7 +1234,7 @@ nsi_status launch_batched(NsiHandle* const* hs, const NsiFields* fs, const NsiOu
   if ((st = check_launch("batched_pack_kernel"))) return st;
   int64_t grid = 0;
   if ((st = resident_grid(batched_kernel<P>, warps, bytes * warps, groups, nullptr, &grid))) return st;
-  batched_kernel<P><<<grid, 32 * warps, bytes * warps, s>>>(args, GroupLay(lay2), GroupLay(lay4));
+  NSI_CUDA(launch_early(batched_kernel<P>, grid, 32 * warps, bytes * warps, s, args, GroupLay(lay2), GroupLay(lay4)));
   return check_launch("batched_kernel");
 }
 

@@ -186,6 +186,7 @@ struct NsiHandle {
   int32_t* walk_ptr = nullptr;  // [n+1]
   uint8_t* walk = nullptr;      // [walk_ptr[n] + 8]
   int nsub = 2;                 // sub-walks per row
+  bool packs() const { return nsub == 2; }  // the row gather reads packed node records (else the nodes' own data)
   uint8_t* diag_pos = nullptr;  // [n + 32] position of the diagonal inside its row (rows <= 32 entries)
   unsigned long long* elem_pos = nullptr;  // [E] element-position map (rows <= 32 entries), or null
   // edge-fan map (one word per CSR entry) and its block partition of the rows

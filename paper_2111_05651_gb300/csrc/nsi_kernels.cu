@@ -1646,7 +1646,7 @@ static nsi_status assemble_core_p(NsiHandle* h, const FieldView& f, const OutVie
   }
   // row gather
   if (!h->gather_ok) return fail(NSI_ERR_UNSUPPORTED, "row-gather mode not available for this mesh");
-  nsi_status st = launch_pack<P>(h, f, rec, s);
+  nsi_status st = h->use_fan || h->packs() ? launch_pack<P>(h, f, rec, s) : NSI_OK;
   if (st) return st;
   if (h->use_fan) {
     const size_t fsm = FanSmem<P>::total(FAN_BLOCK);
@@ -1707,7 +1707,7 @@ static nsi_status assemble_dispatch(NsiHandle* h, const NsiFields* f, const NsiO
 // the rows that it leaves out
 template <int P, bool NODAL>
 static nsi_status step_p(NsiHandle* h, const FieldView& f, const StepView& o, cudaStream_t s) {
-  nsi_status st = launch_pack<P>(h, f, nullptr, s);
+  nsi_status st = h->packs() ? launch_pack<P>(h, f, nullptr, s) : NSI_OK;
   if (!st) st = launch_step<P>(h, f, o, NODAL, s);
   if (st) return st;
   const RowOut ro{o.A_static, o.A, nullptr, o.rhs, o.dt_rho, o.mass_rho, o.kmr};
@@ -1870,7 +1870,7 @@ static nsi_status host_chunked_p(NsiHandle* h, const NsiFields* fd, const NsiOut
   const FieldView fv = fields_of(fd);
   const OutView ov{od->A_val, od->G_val, od->rhs};
   const int R = 32;
-  nsi_status st = launch_pack<P>(h, fv, nullptr, s);
+  nsi_status st = h->packs() ? launch_pack<P>(h, fv, nullptr, s) : NSI_OK;
   if (st) return st;
   const int64_t nb = (h->n + R - 1) / R;
   const int chunks = (int)std::min<int64_t>(C, nb);
