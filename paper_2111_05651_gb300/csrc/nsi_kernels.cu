@@ -805,19 +805,22 @@ __device__ __forceinline__ void tau_lengths(double det, double s2, double& h, do
   sh = sqrt(s2) * h;
 }
 
-// Shared memory of one warp of the stabilised row kernel: entry records
-// (component-major [6][32]: edge vector from the row's node, velocity), then
-// element records for a chunk of 64 elements (element-major, five T4 each:
-// (c_i, mu/(6 det)), (c_1, A+S to node 1), (c_2, ..), (c_3, ..),
-// (tau2/(6 det), det, -, -)), then per entry three 64-bit masks of the
-// chunk's elements holding the entry as their first, second or third node.
+// Shared memory of one warp of the stabilised row kernel: entry records (edge
+// vector from the row's node and u_x in a T4, u_y and u_z in a T2), then element
+// records for a chunk of 64 elements, field by field: (c_i, mu/(6 det)),
+// (c_1, A+S to node 1), (c_2, ..), (c_3, ..), tau2/(6 det); then per entry three
+// 64-bit masks of the chunk's elements holding the entry as their first, second
+// or third node.  The entries' reads of the element records are scattered and
+// are what the kernel's shared memory is busy with most, so they are two T4 and
+// one T per element and entry, and det stays with the lane that evaluated it.
 template <int P>
 struct StarSmem {
   using T = typename Prec<P>::T;
   static constexpr int CHUNK = 64;
   static constexpr size_t ent() { return 0; }
   static constexpr size_t el() { return sizeof(T) * 6 * 32; }
-  static constexpr size_t mask() { return el() + sizeof(T4<T>) * 5 * CHUNK; }
+  static constexpr size_t kd() { return el() + sizeof(T4<T>) * 4 * CHUNK; }
+  static constexpr size_t mask() { return kd() + sizeof(T) * CHUNK; }
   static constexpr size_t bytes() { return mask() + sizeof(unsigned) * 6 * 32; }
 };
 constexpr int STAR_WARPS = 4;  // warps (tasks) per block
@@ -835,15 +838,13 @@ constexpr int STAR_WARPS = 4;  // warps (tasks) per block
 //     and the contributions (w + v) . c_k to its three entries; its record
 //     goes to shared memory and its bit into those entries' masks.
 //  3. Each off-diagonal entry lane adds, in element order, the records of its
-//     masked elements: A + S, K += kv c_k x c_i + kd c_i x c_k, G's c_i sum and
-//     det for the lumped mass.
-//  4. A butterfly over the row's lanes gives every lane the row totals (FP64:
-//     K and G summed in shared memory instead); the diagonal block is the
-//     lumped mass times I minus the off-diagonal blocks' sum.
+//     masked elements: A + S, K += kv c_k x c_i + kd c_i x c_k and G's c_i sum.
+//  4. The row's lanes 0-13 add up one value each over the row's entries, in
+//     shared memory; the diagonal block is the lumped mass times I minus the
+//     off-diagonal blocks' sum.
 //  5. Every lane writes its own entry (the row's slice of each output array
-//     is contiguous); the diagonal block's three compensated diagonal values
-//     and the right-hand side are written by the row's lanes 0-5 (mixed32:
-//     by the diagonal lane).
+//     is contiguous); the diagonal's twelve values and the right-hand side are
+//     written by the row's lanes 0-14, one each.
 // Each element is evaluated once per row of its star (four times per tet).
 // Long rows (more than 32 entries, or a star the row-gather encoder could
 // not cover) are single-row tasks this kernel skips.
@@ -851,7 +852,7 @@ template <int P, bool DEBUG>
 __global__ void __launch_bounds__(32 * STAR_WARPS, P == NSI_FP64 ? 1 : 6) stab_star_kernel(
     MeshView m, FieldView f, StabConst sc, const int4* __restrict__ tasks, int64_t ntasks,
     const uint16_t* __restrict__ star_word, void* Auu, void* Gv, void* rhs) {
-  extern __shared__ __align__(16) unsigned char smem[];
+  extern __shared__ __align__(128) unsigned char smem[];
   using T = typename Prec<P>::T;
   using Out = typename Prec<P>::Out;
   constexpr unsigned FULL = 0xffffffffu;
@@ -860,8 +861,10 @@ __global__ void __launch_bounds__(32 * STAR_WARPS, P == NSI_FP64 ? 1 : 6) stab_s
   const int64_t task = (int64_t)blockIdx.x * STAR_WARPS + (threadIdx.x >> 5);
   if (task >= ntasks) return;  // warp-uniform
   unsigned char* ws = smem + (threadIdx.x >> 5) * StarSmem<P>::bytes();
-  T* er = reinterpret_cast<T*>(ws + StarSmem<P>::ent());
+  T4<T>* er = reinterpret_cast<T4<T>*>(ws + StarSmem<P>::ent());
+  T2<T>* eu = reinterpret_cast<T2<T>*>(er + 32);
   T4<T>* el = reinterpret_cast<T4<T>*>(ws + StarSmem<P>::el());
+  T* ekd = reinterpret_cast<T*>(ws + StarSmem<P>::kd());
   unsigned* mk = reinterpret_cast<unsigned*>(ws + StarSmem<P>::mask());  // [3 nodes][2 words][32 lanes]
 
   // the task's rows, CSR and star bounds and diagonal positions in one
@@ -893,6 +896,7 @@ __global__ void __launch_bounds__(32 * STAR_WARPS, P == NSI_FP64 ? 1 : 6) stab_s
   // 1. entry records
   {
     const int j = has ? m.col_idx[rs + q] : 0;
+    wait_for_records();
     if (DEBUG && has && (j < 0 || j >= m.n)) atomicOr(m.err, ERR_BAD_INDEX);
     const int dl = seg * width + (len > 0 ? dp : 0);  // the diagonal's lane
     V3<T> d, u;
@@ -924,12 +928,8 @@ __global__ void __launch_bounds__(32 * STAR_WARPS, P == NSI_FP64 ? 1 : 6) stab_s
       d = add(sub(hj, hi), sub(lj, li));
       u = {__uint_as_float(a.w), __uint_as_float(b.x), __uint_as_float(b.y)};
     }
-    er[0 * 32 + lane] = d.x;
-    er[1 * 32 + lane] = d.y;
-    er[2 * 32 + lane] = d.z;
-    er[3 * 32 + lane] = u.x;
-    er[4 * 32 + lane] = u.y;
-    er[5 * 32 + lane] = u.z;
+    er[lane] = T4<T>{d.x, d.y, d.z, u.x};
+    eu[lane] = T2<T>{u.y, u.z};
   }
   __syncwarp();
 
@@ -938,7 +938,7 @@ __global__ void __launch_bounds__(32 * STAR_WARPS, P == NSI_FP64 ? 1 : 6) stab_s
   const int len0 = __shfl_sync(FULL, len, 0), len1 = __shfl_sync(FULL, len, 16);
   // an entry's sums (the few elements of its edge) in plain T; the row
   // totals below are compensated in mixed64
-  T sA = T(0), sD = T(0);
+  T sA = T(0), dA = T(0), dB = T(0);  // dA, dB: det of this lane's elements of the task's rows
   T K[9], G[3] = {T(0), T(0), T(0)};
 #pragma unroll
   for (int c = 0; c < 9; ++c) K[c] = T(0);
@@ -961,9 +961,17 @@ __global__ void __launch_bounds__(32 * STAR_WARPS, P == NSI_FP64 ? 1 : 6) stab_s
           atomicOr(m.err, ERR_STAR);  // the element is left out
           continue;
         }
-        auto rd = [&](int l, int c) { return V3<T>{er[c * 32 + l], er[(c + 1) * 32 + l], er[(c + 2) * 32 + l]}; };
-        const V3<T> d1 = rd(eb + pa, 0), d2 = rd(eb + pb, 0), d3 = rd(eb + pc, 0);
-        const V3<T> u1 = rd(eb + pa, 3), u2 = rd(eb + pb, 3), u3 = rd(eb + pc, 3), ui = rd(eb + edp, 3);
+        V3<T> d1, d2, d3, di, u1, u2, u3, ui;
+        auto rd = [&](int l, V3<T>& d, V3<T>& u) {
+          const T4<T> a = er[l];
+          const T2<T> b = eu[l];
+          d = {a.x, a.y, a.z};
+          u = {a.w, b.x, b.y};
+        };
+        rd(eb + pa, d1, u1);
+        rd(eb + pb, d2, u2);
+        rd(eb + pc, d3, u3);
+        rd(eb + edp, di, ui);
         const V3<T> c1 = cross(d2, d3), c2 = cross(d3, d1), c3 = cross(d1, d2);
         const T det = dot(d1, c1);
         const V3<T> ci{-(c1.x + c2.x + c3.x), -(c1.y + c2.y + c3.y), -(c1.z + c2.z + c3.z)};
@@ -981,12 +989,14 @@ __global__ void __launch_bounds__(32 * STAR_WARPS, P == NSI_FP64 ? 1 : 6) stab_s
         wv.x = kc * (ui.x + us.x) + kv * ci.x + (as * us.x + ai * ui.x + a1 * u1.x + a2 * u2.x + a3 * u3.x);
         wv.y = kc * (ui.y + us.y) + kv * ci.y + (as * us.y + ai * ui.y + a1 * u1.y + a2 * u2.y + a3 * u3.y);
         wv.z = kc * (ui.z + us.z) + kv * ci.z + (as * us.z + ai * ui.z + a1 * u1.z + a2 * u2.z + a3 * u3.z);
-        T4<T>* r = el + 5 * slot;
+        T4<T>* r = el + slot;
         r[0] = T4<T>{ci.x, ci.y, ci.z, kv};
-        r[1] = T4<T>{c1.x, c1.y, c1.z, dot(wv, c1)};
-        r[2] = T4<T>{c2.x, c2.y, c2.z, dot(wv, c2)};
-        r[3] = T4<T>{c3.x, c3.y, c3.z, dot(wv, c3)};
-        r[4] = T4<T>{kd, det, T(0), T(0)};
+        r[CH] = T4<T>{c1.x, c1.y, c1.z, dot(wv, c1)};
+        r[2 * CH] = T4<T>{c2.x, c2.y, c2.z, dot(wv, c2)};
+        r[3 * CH] = T4<T>{c3.x, c3.y, c3.z, dot(wv, c3)};
+        ekd[slot] = kd;
+        if (es) dB += det;
+        else dA += det;
         const unsigned bit = 1u << lane;
         atomicOr(&mk[(0 * 2 + half) * 32 + eb + pa], bit);
         atomicOr(&mk[(1 * 2 + half) * 32 + eb + pb], bit);
@@ -1002,11 +1012,9 @@ __global__ void __launch_bounds__(32 * STAR_WARPS, P == NSI_FP64 ? 1 : 6) stab_s
         const int e = __ffsll((long long)bits) - 1;
         bits &= bits - 1;
         const int k = ((m1 >> e) & 1ull) ? 2 : ((m2 >> e) & 1ull) ? 3 : 1;
-        const T4<T>* r = el + 5 * e;
-        const T4<T> r0v = r[0], rk = r[k], r4 = r[4];
+        const T4<T> r0v = el[e], rk = el[k * CH + e];
         sA += rk.w;
-        sD += r4.y;
-        const T kv = r0v.w, kd = r4.x;
+        const T kv = r0v.w, kd = ekd[e];
         const T ri[3] = {r0v.x, r0v.y, r0v.z}, c[3] = {rk.x, rk.y, rk.z};
 #pragma unroll
         for (int a = 0; a < 3; ++a)
@@ -1021,145 +1029,80 @@ __global__ void __launch_bounds__(32 * STAR_WARPS, P == NSI_FP64 ? 1 : 6) stab_s
     __syncwarp();
   }
 
-  // 4. row totals (lanes without an off-diagonal entry hold zeros).  The
-  // merge adds the error terms first (a commutative sum), so both lanes of a
-  // butterfly pair, and in the end every lane of the row, hold bitwise the
-  // same totals.
-  auto merge_sym = [](Acc<P>& a, const Acc<P>& b) {
+  // 4. row totals: every lane's sums (a lane without an off-diagonal entry has
+  // zeros) to shared memory (the element records' space, free now), where the
+  // row's lanes 0-13 each add one value up over the row's entries (mixed64:
+  // compensated); A's and det's go to all of the row's lanes
+  constexpr int NV = 14, ST = 15;  // K, G, A + S, det; an odd stride: no bank conflicts
+  T* red = reinterpret_cast<T*>(el);
+#pragma unroll
+  for (int c = 0; c < 9; ++c) red[lane * ST + c] = K[c];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) red[lane * ST + 9 + c] = G[c];
+  red[lane * ST + 12] = sA;
+  {  // two rows of 16 lanes: a row's elements are on all 32
+    const T a = dA + __shfl_xor_sync(FULL, dA, 16), b = dB + __shfl_xor_sync(FULL, dB, 16);
+    red[lane * ST + 13] = nrow == 2 ? (seg ? b : a) : dA;
+  }
+  __syncwarp();
+  Acc<P> tot;
+  tot.zero();
+  if (q < NV)
+    for (int r = 0; r < width; ++r) tot.add(red[(seg * width + r) * ST + q]);
+  auto from = [&](int l) {
+    Acc<P> a;
     if constexpr (P == NSI_MIXED_F32_ACC64) {
-      a.lo += b.lo;
-      a.add(b.hi);
+      a.hi = __shfl_sync(FULL, tot.hi, seg * width + l);
+      a.lo = __shfl_sync(FULL, tot.lo, seg * width + l);
     } else {
-      a.v += b.v;
+      a.v = __shfl_sync(FULL, tot.v, seg * width + l);
     }
+    return a;
   };
-  Acc<P> tA, tD;
-  tA.zero();
-  tD.zero();
-  tA.add(sA);
-  tD.add(sD);
-  T tK[9], tG[3];
-#pragma unroll
-  for (int c = 0; c < 9; ++c) tK[c] = K[c];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) tG[c] = G[c];
-  for (int o = 1; o < width; o <<= 1) {
-    Acc<P> xA, xD;
-    if constexpr (P == NSI_MIXED_F32_ACC64) {
-      xA.hi = __shfl_xor_sync(FULL, tA.hi, o);
-      xA.lo = __shfl_xor_sync(FULL, tA.lo, o);
-      xD.hi = __shfl_xor_sync(FULL, tD.hi, o);
-      xD.lo = __shfl_xor_sync(FULL, tD.lo, o);
-    } else {
-      xA.v = __shfl_xor_sync(FULL, tA.v, o);
-      xD.v = __shfl_xor_sync(FULL, tD.v, o);
-    }
-    merge_sym(tA, xA);
-    merge_sym(tD, xD);
-    if constexpr (P != NSI_FP64) {
-#pragma unroll
-      for (int c = 0; c < 9; ++c) tK[c] += __shfl_xor_sync(FULL, tK[c], o);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) tG[c] += __shfl_xor_sync(FULL, tG[c], o);
-    }
-  }
-  if constexpr (P == NSI_FP64) {
-    // K and G totals in FP64 (a shuffled double is two shuffles): each lane's
-    // values to shared memory (the element records' space, free now), the
-    // row's lanes 0-11 each sum one value over the row's entries in lane
-    // order, then every lane reads the totals
-    T* red = reinterpret_cast<T*>(el);  // [32 lanes][13], then [2 rows][12] totals
-    T* tot = red + 32 * 13;
-#pragma unroll
-    for (int c = 0; c < 9; ++c) red[lane * 13 + c] = K[c];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) red[lane * 13 + 9 + c] = G[c];
-    __syncwarp();
-    if (q < 12) {
-      T sum = T(0);
-      for (int r = 0; r < len; ++r) sum += red[(seg * width + r) * 13 + q];
-      tot[seg * 12 + q] = sum;
-    }
-    __syncwarp();
-#pragma unroll
-    for (int c = 0; c < 9; ++c) tK[c] = tot[seg * 12 + c];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) tG[c] = tot[seg * 12 + 9 + c];
-  }
+  const Acc<P> tA = from(12), tD = from(13);
 
-  // 5. write-out: every lane its own entry.  mixed64 and FP64: the row's six
-  // compensated values (the diagonal components of the diagonal block and
-  // the right-hand side) by the row's lanes 0-5, one each, from the totals
-  // every lane holds (the diagonal lane alone took them in turn: 2% of the
-  // kernel in mixed64); mixed32, whose values are plain floats, keeps them on
-  // the diagonal lane (the spread costs it 2%).
+  // 5. write-out: every lane its own entry; then the row's lanes 0-11 the
+  // components of the diagonal block and of the diagonal's G (the totals they
+  // hold), lanes 12-14 the right-hand side: each one value, in one store
   Out* A = static_cast<Out*>(Auu);
   Out* Go = static_cast<Out*>(Gv);
   Out* Rh = static_cast<Out*>(rhs);
-  if constexpr (P == NSI_MIXED_F32_ACC32) {
-    if (has) {
-      const int64_t g = (int64_t)rs + q;
-      if (q == dp) {
-        const Acc<P> mass = acc_scale<P>(acc_third<P>(tD), kmass);
+  if (has && q != dp) {
+    const int64_t g = (int64_t)rs + q;
 #pragma unroll
-        for (int c = 0; c < 9; ++c) A[c * m.nnz + g] = c % 4 == 0 ? mass.v - tA.v - tK[c] : -tK[c];
+    for (int c = 0; c < 9; ++c) A[c * m.nnz + g] = (Out)(c % 4 == 0 ? sA + K[c] : K[c]);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) Go[c * m.nnz + g] = tG[c] * (kg / T(3));
-        const V3<T> un = load_vec<T>(f.un, i);
-        Rh[i] = mass.v * un.x;
-        Rh[m.n + i] = mass.v * un.y;
-        Rh[2 * m.n + i] = mass.v * un.z;
-      } else {
-#pragma unroll
-        for (int c = 0; c < 9; ++c) A[c * m.nnz + g] = c % 4 == 0 ? sA + K[c] : K[c];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) Go[c * m.nnz + g] = G[c] * kg;
-      }
-    } else if (q == 0 && len == 0) {  // a node in no element: zero right-hand side
-      Rh[i] = 0.0f;
-      Rh[m.n + i] = 0.0f;
-      Rh[2 * m.n + i] = 0.0f;
-    }
-  } else {
-    if (has) {
-      const int64_t g = (int64_t)rs + q;
-      if (q == dp) {
-#pragma unroll
-        for (int c = 0; c < 9; ++c)
-          if (c % 4 != 0) A[c * m.nnz + g] = (Out)(-tK[c]);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) Go[c * m.nnz + g] = (Out)(tG[c] * (kg / T(3)));
-      } else {
-#pragma unroll
-        for (int c = 0; c < 9; ++c) {
-          A[c * m.nnz + g] = (Out)(c % 4 == 0 ? sA + K[c] : K[c]);
-        }
-#pragma unroll
-        for (int c = 0; c < 3; ++c) Go[c * m.nnz + g] = (Out)(G[c] * kg);
-      }
-    }
-    if (len > 0 && q < 6) {  // (a row's lanes number 16 or 32)
-      const Acc<P> mass = acc_scale<P>(acc_third<P>(tD), kmass);
-      if (q < 3) {  // A(i,i)[c][c] = lumped mass - sum of the row's off-diagonal A - sum of K[c][c]
-        Acc<P> x = mass;
+    for (int c = 0; c < 3; ++c) Go[c * m.nnz + g] = (Out)(G[c] * kg);
+  }
+  if (len > 0 && q < 15) {  // (a row's lanes number 16 or 32)
+    const Acc<P> mass = acc_scale<P>(tD, kmass);
+    Acc<P> x;
+    Out* at;
+    if (q < 12) {  // A(i,i)[a][b] = delta_ab (lumped mass - sum of the row's A + S) - sum of K[a][b]; G(i,i) = G's / 3
+      x = acc_scale<P>(tot, q < 9 ? T(-1) : kg / T(3));
+      if (q < 9 && q % 4 == 0) {
+        Acc<P> y = mass;
         if constexpr (P == NSI_MIXED_F32_ACC64) {
-          x.add(-tA.hi);
-          x.lo -= tA.lo;
+          y.add(-tA.hi);
+          y.lo -= tA.lo;
+          y.add(x.hi);
+          y.lo += x.lo;
         } else {
-          x.v = mass.v - tA.v;
+          y.v = (mass.v - tA.v) + x.v;
         }
-        x.add(-(q == 0 ? tK[0] : q == 1 ? tK[4] : tK[8]));
-        store_acc(A + 4 * q * m.nnz + rs + dp, x);
-      } else {  // rhs[k][i] = lumped mass * u^n_k
-        const int k = q - 3;
-        const T* un = static_cast<const T*>(k == 0 ? f.un[0] : k == 1 ? f.un[1] : f.un[2]);
-        store_acc(Rh + k * m.n + i, acc_scale<P>(mass, __ldg(un + i)));
+        x = y;
       }
-    } else if (q == 0 && len == 0) {  // a node in no element: zero right-hand side
-      Rh[i] = Out(0);
-      Rh[m.n + i] = Out(0);
-      Rh[2 * m.n + i] = Out(0);
+      at = (q < 9 ? A + q * m.nnz : Go + (q - 9) * m.nnz) + rs + dp;
+    } else {  // rhs[k][i] = lumped mass * u^n_k
+      const T* un = static_cast<const T*>(q == 12 ? f.un[0] : q == 13 ? f.un[1] : f.un[2]);
+      x = acc_scale<P>(mass, __ldg(un + i));
+      at = Rh + (q - 12) * m.n + i;
     }
+    store_acc(at, x);
+  } else if (q == 0 && len == 0) {  // a node in no element: zero right-hand side
+    Rh[i] = Out(0);
+    Rh[m.n + i] = Out(0);
+    Rh[2 * m.n + i] = Out(0);
   }
 }
 
@@ -1959,12 +1902,9 @@ static nsi_status stabilized_p(NsiHandle* h, const FieldView& f, const StabConst
   const size_t smem = StarSmem<P>::bytes() * STAR_WARPS;
   const int64_t grid = (h->n_star_tasks + STAR_WARPS - 1) / STAR_WARPS;
   if (h->ev_start) NSI_CUDA(cudaEventRecord(h->ev_start, s));
-  if (h->debug)
-    stab_star_kernel<P, true><<<grid, 32 * STAR_WARPS, smem, s>>>(m, f, sc, h->star_task, h->n_star_tasks,
-                                                                   h->star_word, Auu, G, rhs);
-  else
-    stab_star_kernel<P, false><<<grid, 32 * STAR_WARPS, smem, s>>>(m, f, sc, h->star_task, h->n_star_tasks,
-                                                                    h->star_word, Auu, G, rhs);
+  const auto kernel = h->debug ? stab_star_kernel<P, true> : stab_star_kernel<P, false>;
+  NSI_CUDA(launch_early(kernel, grid, 32 * STAR_WARPS, smem, s, m, f, sc, (const int4*)h->star_task, h->n_star_tasks,
+                        (const uint16_t*)h->star_word, Auu, G, rhs));
   if (h->ev_stop) NSI_CUDA(cudaEventRecord(h->ev_stop, s));
   st = check_launch("stab_star_kernel");
   if (st) return st;
