@@ -259,11 +259,6 @@ __device__ __forceinline__ double normalised_pair_double(float hi, float lo) {
 __device__ __forceinline__ double nonfinite_double(float hi) { return __longlong_as_double(f32_to_f64_bits(hi)); }
 // true if the exponent bits of x are all ones (infinite or NaN)
 __device__ __forceinline__ bool nonfinite_bits(float x) { return (__float_as_uint(x) | 0x807fffffu) == 0xffffffffu; }
-// true for an infinite, NaN or subnormal float (the cases float_double leaves out)
-__device__ __forceinline__ bool special_float(float x) {
-  const unsigned e = __float_as_uint(x) & 0x7f800000u;
-  return e == 0x7f800000u || (e == 0u && (__float_as_uint(x) & 0x007fffffu) != 0u);
-}
 // the double equal to a normal or zero float, from its bit pattern: the
 // exponent rebiased (+896), the 23 mantissa bits moved to the top of the
 // double's 52; the sign kept (an arithmetic shift leaves it in the top bit).  A

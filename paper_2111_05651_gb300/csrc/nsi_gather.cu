@@ -196,9 +196,6 @@ struct Slots<P, ASSEMBLE> {
   }
   __device__ __forceinline__ void store(int k, const V& v) { a[k] = make_float4(v.g.x, v.g.y, v.r.x, v.r.y); }
   static __device__ __forceinline__ V sum(const V& x, const V& y) { return {add2(x.g, y.g), add2(x.r, y.r)}; }
-  static __device__ __forceinline__ V pick(bool c, const V& x, const V& y) {
-    return {make_float2(c ? x.g.x : y.g.x, c ? x.g.y : y.g.y), make_float2(c ? x.r.x : y.r.x, c ? x.r.y : y.r.y)};
-  }
 };
 template <>
 struct Slots<NSI_FP64, ASSEMBLE> {
@@ -217,9 +214,6 @@ struct Slots<NSI_FP64, ASSEMBLE> {
   static __device__ __forceinline__ V sum(const V& x, const V& y) {
     return {{x.x.x + y.x.x, x.x.y + y.x.y}, {x.y.x + y.y.x, x.y.y + y.y.y}};
   }
-  static __device__ __forceinline__ V pick(bool c, const V& x, const V& y) {
-    return {{c ? x.x.x : y.x.x, c ? x.x.y : y.x.y}, {c ? x.y.x : y.y.x, c ? x.y.y : y.y.y}};
-  }
 };
 template <int P>
 struct Slots<P, STEP> {
@@ -230,7 +224,6 @@ struct Slots<P, STEP> {
   __device__ __forceinline__ V load(int k) const { return a[k]; }
   __device__ __forceinline__ void store(int k, V v) { a[k] = v; }
   static __device__ __forceinline__ V sum(V x, V y) { return x + y; }
-  static __device__ __forceinline__ V pick(bool c, V x, V y) { return c ? x : y; }
 };
 template <int P>
 struct Slots<P, NODAL> {
@@ -240,7 +233,6 @@ struct Slots<P, NODAL> {
   __device__ __forceinline__ V load(int) const { return {}; }
   __device__ __forceinline__ void store(int, V) {}
   static __device__ __forceinline__ V sum(V, V) { return {}; }
-  static __device__ __forceinline__ V pick(bool, V, V) { return {}; }
 };
 
 // One lane's sub-walk of one row, node i as the origin: segments of
@@ -351,7 +343,8 @@ __device__ __forceinline__ void walk_lane(const uint8_t* __restrict__ st, int nb
           c.a = fma(neg ? T(1) : T(-1), dot_fma(w3, M), c.a);
         }
         M = V3<T>{evq ? cq.x : -cp.x, evq ? cq.y : -cp.y, evq ? cq.z : -cp.z};
-        acc.store(evq ? q.k : p.k, Slots<P, MODE>::pick(evq, q.a, p.a));
+        if (evq) acc.store(q.k, q.a);
+        else acc.store(p.k, p.a);
       }
       if (!evq) {
         p = q;
@@ -682,7 +675,7 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
       T4<T>* stage = reinterpret_cast<T4<T>*>(smem);
       // the planes' sums of the lane's slots and their entries
       auto each = [&](auto&& use) {
-#pragma unroll 1
+#pragma unroll 2
         for (int s = h; s < (fits ? ns : 0); s += H) {
           typename S::V v = slots(0).load(s * RW + t);
 #pragma unroll
@@ -802,23 +795,16 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
         for (int k = lane; k < (fits ? L : 0); k += 32) put(k, stage[k]);
       };
       if constexpr (P == NSI_MIXED_F32_ACC64) {
-        // converted to double exactly from the bits; an infinite, NaN or
-        // subnormal A again by a rare second pass, then every diagonal by the
-        // double nearest its compensated pair
-        bool slow = false;
+        // converted to double exactly, A by the FP64 pipe's conversion and G from
+        // the bits (all four either way cost 2% more: the pipe's rate, or the
+        // instructions), then every diagonal by the double nearest its
+        // compensated pair
         write([&](int k, const T4<T>& v) {
-          slow |= special_float(v.x);
-          __stcs(A + k, float_double(v.x));
+          __stcs(A + k, (double)v.x);
           __stcs(G + k, float_double(v.y));
           __stcs(G1 + k, float_double(v.z));
           __stcs(G2 + k, float_double(v.w));
         });
-        if (__any_sync(FULL, slow)) {
-          for (int k = lane; k < L; k += 32) {
-            const float a = stage[k].x;
-            if (special_float(a)) A[k] = nonfinite_bits(a) ? nonfinite_double(a) : (double)a;
-          }
-        }
         __syncwarp();
         if (fits && h == 0 && len > 0)
           A[lb + row.dp] = nonfinite_bits(dhi) ? nonfinite_double(dhi) : pair_double(dhi, dlo);
@@ -834,13 +820,9 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
       const T* stage = reinterpret_cast<const T*>(smem);
       const Out* As = static_cast<const Out*>(o.A_static) + base;
       Out* A = static_cast<Out*>(o.A) + base;
-      auto value = [&](int k) -> Out {  // C(u) of entry k in the output type
-        const T c = stage[k];
-        if constexpr (P == NSI_MIXED_F32_ACC64)
-          return special_float(c) ? (nonfinite_bits(c) ? nonfinite_double(c) : (double)c) : float_double(c);
-        else
-          return c;
-      };
+      // C(u) of entry k in the output type (mixed64: by the FP64 pipe's
+      // conversion, 80.5 us for an 81x70x66 time step against 87.7 from the bits)
+      auto value = [&](int k) { return (Out)stage[k]; };
       if (fits) {
 #pragma unroll
         for (int c = 0; c < NS; ++c)
