@@ -1283,9 +1283,12 @@ __device__ __forceinline__ V3<C> axpy(C a, const V3<C>& x, const V3<C>& y) {
 //   sum_a w_a A_e[a][m] = (rho/120 M + mu/(6 det) Q) c_m + rho det/(24 dt) w_m,
 // and the grad_mu term is the sum of Q's and Gu's products entry by entry: 300
 // operations per element instead of 380 with every A_e[a][m].
-template <typename C>
-__device__ __forceinline__ C vjp_element(const V3<C>& d1, const V3<C>& d2, const V3<C>& d3, const V3<C> (&u)[4],
-                                         const V3<C> (&w)[4], C kc, C kmu, C kmass, V3<C> (&g)[4]) {
+// In double only: the float kernel is bound by its atomic adds, not by its
+// operations, and keeps the sums over the entries (below).
+__device__ __forceinline__ double vjp_element(const V3<double>& d1, const V3<double>& d2, const V3<double>& d3,
+                                              const V3<double> (&u)[4], const V3<double> (&w)[4], double kc,
+                                              double kmu, double kmass, V3<double> (&g)[4]) {
+  using C = double;
   V3<C> c[4];
   c[1] = cross(d2, d3);
   c[2] = cross(d3, d1);
@@ -1323,6 +1326,58 @@ __device__ __forceinline__ C vjp_element(const V3<C>& d1, const V3<C>& d2, const
   }
   return s * (C)(1.0 / 6.0) * rdet;
 }
+__device__ __forceinline__ float vjp_element(const V3<float>& d1, const V3<float>& d2, const V3<float>& d3,
+                                             const V3<float> (&u)[4], const V3<float> (&w)[4], float kc, float kmu,
+                                             float kmass, V3<float> (&g)[4]) {
+  using C = float;
+  V3<C> c[4];
+  c[1] = cross(d2, d3);
+  c[2] = cross(d3, d1);
+  c[3] = cross(d1, d2);
+  const C det = dot(d1, c[1]);
+  c[0] = {-(c[1].x + c[2].x + c[3].x), -(c[1].y + c[2].y + c[3].y), -(c[1].z + c[2].z + c[3].z)};
+  const V3<C> S = add(add(u[0], u[1]), add(u[2], u[3]));
+  const V3<C> Ws = add(add(w[0], w[1]), add(w[2], w[3]));
+  const C kv = kmu * rcp(det);
+  const C km = det * kmass;
+  V3<C> Gu[3];
+  const C uk[4][3] = {{u[0].x, u[0].y, u[0].z}, {u[1].x, u[1].y, u[1].z}, {u[2].x, u[2].y, u[2].z},
+                      {u[3].x, u[3].y, u[3].z}};
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    Gu[k] = {C(0), C(0), C(0)};
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      Gu[k].x += uk[b][k] * c[b].x;
+      Gu[k].y += uk[b][k] * c[b].y;
+      Gu[k].z += uk[b][k] * c[b].z;
+    }
+  }
+#pragma unroll
+  for (int mm = 0; mm < 4; ++mm) {
+    V3<C> acc = {C(0), C(0), C(0)};
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      C Aam = kc * dot(add(S, u[a]), c[mm]) + kv * dot(c[a], c[mm]);
+      if (a == mm) Aam += km;
+      acc.x += w[a].x * Aam;
+      acc.y += w[a].y * Aam;
+      acc.z += w[a].z * Aam;
+    }
+    const C wk[3] = {Ws.x + w[mm].x, Ws.y + w[mm].y, Ws.z + w[mm].z};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      acc.x += kc * wk[k] * Gu[k].x;
+      acc.y += kc * wk[k] * Gu[k].y;
+      acc.z += kc * wk[k] * Gu[k].z;
+    }
+    g[mm] = acc;
+  }
+  C s = C(0);
+#pragma unroll
+  for (int a = 0; a < 4; ++a) s += w[a].x * dot(c[a], Gu[0]) + w[a].y * dot(c[a], Gu[1]) + w[a].z * dot(c[a], Gu[2]);
+  return s * (C)(1.0 / 6.0) * rcp(det);
+}
 
 // true if element e is marked in the bit mask of badly shaped elements
 __device__ __forceinline__ bool marked(const uint32_t* __restrict__ mask, int64_t e) {
@@ -1351,7 +1406,7 @@ __global__ void __launch_bounds__(256) vjp_kernel(MeshView m, FieldView f, const
       u[a] = load_vec<T>(f.u, v[a]);
       w[a] = {W[v[a]], W[m.n + v[a]], W[2 * m.n + v[a]]};
     }
-    my_mu = vjp_element<T>(X[1].minus(X[0]), X[2].minus(X[0]), X[3].minus(X[0]), u, w, kc_of<T>(f), kmu_of<T>(f),
+    my_mu = vjp_element(X[1].minus(X[0]), X[2].minus(X[0]), X[3].minus(X[0]), u, w, kc_of<T>(f), kmu_of<T>(f),
                            kmass_of<T>(f), g);
     T* gp = static_cast<T*>(gu);
 #pragma unroll
@@ -1393,7 +1448,7 @@ __global__ void __launch_bounds__(64) vjp_exact_kernel(MeshView m, FieldView f, 
     u[a] = vec64<T>(f.u, v[a]);
     w[a] = vec64<T>(wc, v[a]);
   }
-  const double mu = vjp_element<double>(sub(X[1], X[0]), sub(X[2], X[0]), sub(X[3], X[0]), u, w, f.kc, f.kmu, f.kmass, g);
+  const double mu = vjp_element(sub(X[1], X[0]), sub(X[2], X[0]), sub(X[3], X[0]), u, w, f.kc, f.kmu, f.kmass, g);
   T* gp = static_cast<T*>(gu);
   for (int mm = 0; mm < 4; ++mm) {
     atomicAdd(gp + v[mm], (T)g[mm].x);
