@@ -309,14 +309,17 @@ __device__ __forceinline__ double rcp_fast(double x) {
   return r;
 }
 
-// Programmatic dependent launch, for a kernel that reads the records of the
-// packing launch directly before it: its blocks may start as the packing's
-// blocks end, do what does not need the records (row bounds, column indices,
-// walk bytes), and wait here for the packing to complete.  (Letting them start
-// with the packing's first blocks instead takes the SMs from it: a batch of 16
-// meshes 90.1 us, without early launches 84.2, as it is 84.1; a 47x61x38 box in
-// mixed32 33.0, 36.3, 33.1; a time step of 81x70x66 96.8, 94.6, 92.5.)
-__device__ __forceinline__ void wait_for_records() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Programmatic dependent launch: a kernel launched by launch_early may start
+// as the blocks of the launch directly before it end, and calls
+// wait_for_previous before it reads what that launch writes, or writes what it
+// may write too; the wait ends when that launch, and so every one before it, is
+// complete.  Used by the kernels that read the packing's node records, which
+// first fetch row bounds, column indices and walk bytes, and by those that
+// overwrite listed rows.  (Letting them start with the packing's first blocks
+// takes the SMs from it: a batch of 16 meshes 90.1 us, without early launches
+// 84.2, as it is 84.1; a 47x61x38 box in mixed32 33.0, 36.3, 33.1; a time step
+// of 81x70x66 96.8, 94.6, 92.5.)
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 template <typename... Params, typename... Args>
 cudaError_t launch_early(void (*kernel)(Params...), int64_t grid, int block, size_t smem, cudaStream_t s,
                          const Args&... args) {

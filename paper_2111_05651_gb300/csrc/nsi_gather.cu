@@ -575,7 +575,7 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
     cp_async_wait_all();
     __syncwarp();
     Recs v;
-    if constexpr (!DIRECT) wait_for_records();
+    if constexpr (!DIRECT) wait_for_previous();
     load_recs(v, src.item(at), row, cols_of(m, row, base, end), r0 + t, h);
     __syncwarp();
     put(v, src.item(at), row, r0 + t);
@@ -935,6 +935,7 @@ __global__ void __launch_bounds__(32) exact_rows_kernel(WalkMesh m, FieldView f,
     walk_lane<NSI_FP64, RW, WMODE>(st + b, st[h], nb0, nb1, acc, u2i, f.kmu, det);
   }
   __syncwarp();
+  wait_for_previous();  // (the rows' first values come from an earlier launch)
 #pragma unroll
   for (int off = RW; off < 32; off <<= 1) det.v += __shfl_xor_sync(FULL, det.v, off);
   if constexpr (MODE == 0) {
@@ -1143,7 +1144,8 @@ nsi_status exact_rows_h(NsiHandle* h, const FieldView& f, int mode, const RowOut
   if (st) return st;
   const int64_t warps = (h->exact_rows * H + 31) / 32;
   const GatherSmem lay = group_smem(NSI_FP64, mode == 0 ? ASSEMBLE : NODAL, H, h->exact_slots, 0, 0);
-  kernel<<<warps, 32, lay.total(), s>>>(walk_mesh(h, nullptr), f, o, GroupLay(lay), h->exact_list, h->exact_rows);
+  NSI_CUDA(launch_early(kernel, warps, 32, lay.total(), s, walk_mesh(h, nullptr), f, o, GroupLay(lay),
+                        (const int32_t*)h->exact_list, h->exact_rows));
   return check_launch("exact_rows_kernel");
 }
 

@@ -268,11 +268,12 @@ __device__ __forceinline__ V3<double> vec64(const void* const* comp, int64_t j) 
 // alias A_static: each entry is read before it is written, by its thread) and
 // rhs, or with no A (rows of badly shaped elements: the convection does not
 // involve the determinant) rhs alone; 2: rhs, dt_rho and mass_rho.
-// The rows are few and their serial work is what counts: the 71 rows of a
-// pipe's axis (83 entries, 240 elements) take 36 us; with the entries scanning
-// all elements instead of their marked ones 54; with one thread per row the
-// whole assembly of the pipe took 7.2 ms.
-constexpr int ROW_THREADS = 128;
+// The rows are few and their serial work is what counts: the assembly of a
+// pipe with 71 of them (the axis: 83 entries, 240 elements) takes 106 us with
+// 256 threads a block, 111 with 128, 138 with 64; 14 us more with the entries
+// scanning all elements instead of their marked ones; with one thread per row
+// (and one per row of a badly shaped element) it took 7.2 ms.
+constexpr int ROW_THREADS = 256;
 template <int P, int MODE>
 __global__ void __launch_bounds__(ROW_THREADS) rows64_kernel(MeshView m, FieldView f, RowOut o,
                                                              const int32_t* __restrict__ rows,
@@ -334,7 +335,7 @@ __global__ void __launch_bounds__(ROW_THREADS) rows64_kernel(MeshView m, FieldVi
         if (entries) {
           const V3<double> ci{-(c[0].x + c[1].x + c[2].x), -(c[0].y + c[1].y + c[2].y), -(c[0].z + c[1].z + c[2].z)};
           for (int b = 0; b < 3; ++b) us = add(us, vel(f.u, nb[b]));
-          const double kv = MODE == 0 ? f.kmu / dt : 0.0;
+          const double kv = MODE == 0 ? f.kmu * rcp_fast(dt) : 0.0;
           const V3<double> w3{f.kc * us.x + kv * ci.x, f.kc * us.y + kv * ci.y, f.kc * us.z + kv * ci.z};
           for (int b = 0; b < 3; ++b) {
             ea[tid][b] = dot(w3, c[b]);
@@ -358,6 +359,7 @@ __global__ void __launch_bounds__(ROW_THREADS) rows64_kernel(MeshView m, FieldVi
           }
       }
     }
+    wait_for_previous();  // (the rows' first values come from the launch before)
     if (mine) {
       sa += a;
       if constexpr (MODE == 0) {
@@ -896,7 +898,7 @@ __global__ void __launch_bounds__(32 * STAR_WARPS, P == NSI_FP64 ? 1 : 6) stab_s
   // 1. entry records
   {
     const int j = has ? m.col_idx[rs + q] : 0;
-    wait_for_records();
+    wait_for_previous();
     if (DEBUG && has && (j < 0 || j >= m.n)) atomicOr(m.err, ERR_BAD_INDEX);
     const int dl = seg * width + (len > 0 ? dp : 0);  // the diagonal's lane
     V3<T> d, u;
@@ -1586,38 +1588,32 @@ static nsi_status zero_outputs(const NsiHandle* h, const OutView& o, cudaStream_
 template <int P>
 static nsi_status launch_rows64(NsiHandle* h, const FieldView& f, int mode, const RowOut& o, const int32_t* rows,
                                 const int32_t* ptr, const uint32_t* inc, int64_t count, cudaStream_t s) {
-  const MeshView m = view_of(h);
-  if (mode == 0) rows64_kernel<P, 0><<<count, ROW_THREADS, 0, s>>>(m, f, o, rows, ptr, inc);
-  else if (mode == 1) rows64_kernel<P, 1><<<count, ROW_THREADS, 0, s>>>(m, f, o, rows, ptr, inc);
-  else rows64_kernel<P, 2><<<count, ROW_THREADS, 0, s>>>(m, f, o, rows, ptr, inc);
+  const auto kernel = mode == 0 ? rows64_kernel<P, 0> : mode == 1 ? rows64_kernel<P, 1> : rows64_kernel<P, 2>;
+  NSI_CUDA(launch_early(kernel, count, ROW_THREADS, 0, s, view_of(h), f, o, rows, ptr, inc));
   return check_launch("rows64_kernel");
 }
 
-// after an assembly or time step in a mixed mode: the rows listed at create
-// for badly shaped elements, recomputed in double (nothing if there are none);
-// the time step's A does not depend on the determinant and stays
+// After an assembly, time step or nodal outputs: the long rows (after a row
+// gather), and in a mixed mode the rows listed at create for badly shaped
+// elements, recomputed in double (nothing if there are none; the time step's A
+// does not depend on the determinant and stays).  (Run side by side, the few
+// rows of the first kind wait for the FP64 pipe that the others fill: a pipe's
+// assembly 121 us, one after the other 112.)
 template <int P>
-static nsi_status fix_exact_rows(NsiHandle* h, const FieldView& f, int mode, const RowOut& out, cudaStream_t s) {
+static nsi_status fix_rows(NsiHandle* h, const FieldView& f, int mode, const RowOut& out, bool gathered,
+                           cudaStream_t s) {
+  nsi_status st = NSI_OK;
+  if (gathered && h->long_rows > 0)
+    st = launch_rows64<P>(h, f, mode, out, h->long_list, h->long_ptr, h->long_inc, h->long_rows, s);
   if constexpr (P != NSI_FP64) {
     RowOut o = out;
     if (mode == 1) o.A = nullptr;
-    if (h->exact_rows > 0) {
-      nsi_status st = launch_exact_rows<P>(h, f, mode, o, s);
-      if (st) return st;
-    }
-    if (h->exact_rest > 0)
-      return launch_rows64<P>(h, f, mode, o, h->exact_list + h->exact_rows, h->exact_ptr + h->exact_rows,
-                              h->exact_inc, h->exact_rest, s);
+    if (!st && h->exact_rest > 0)
+      st = launch_rows64<P>(h, f, mode, o, h->exact_list + h->exact_rows, h->exact_ptr + h->exact_rows, h->exact_inc,
+                            h->exact_rest, s);
+    if (!st && h->exact_rows > 0) st = launch_exact_rows<P>(h, f, mode, o, s);
   }
-  return NSI_OK;
-}
-
-// after any row-gather assembly or time step: the long rows (nothing if there
-// are none)
-template <int P>
-static nsi_status fix_long_rows(NsiHandle* h, const FieldView& f, int mode, const RowOut& o, cudaStream_t s) {
-  if (h->long_rows == 0) return NSI_OK;
-  return launch_rows64<P>(h, f, mode, o, h->long_list, h->long_ptr, h->long_inc, h->long_rows, s);
+  return st;
 }
 
 // `rec` (nullptr: the handle's buffer) receives the row gather's per-call
@@ -1684,9 +1680,7 @@ static nsi_status assemble_p(NsiHandle* h, const FieldView& f, const OutView& o,
   nsi_status st = assemble_core_p<P>(h, f, o, mode, s);
   if (st) return st;
   const RowOut ro{nullptr, o.A, o.G, o.rhs, nullptr, nullptr, 0.0};
-  st = fix_exact_rows<P>(h, f, 0, ro, s);
-  if (st || mode != NSI_SCATTER_GATHER) return st;
-  return fix_long_rows<P>(h, f, 0, ro, s);
+  return fix_rows<P>(h, f, 0, ro, mode == NSI_SCATTER_GATHER, s);
 }
 
 static nsi_status check_call(const NsiHandle* h, const NsiFields* f, const NsiOutputs* o) {
@@ -1731,9 +1725,7 @@ static nsi_status step_p(NsiHandle* h, const FieldView& f, const StepView& o, cu
   if (!st) st = launch_step<P>(h, f, o, NODAL, s);
   if (st) return st;
   const RowOut ro{o.A_static, o.A, nullptr, o.rhs, o.dt_rho, o.mass_rho, o.kmr};
-  st = fix_exact_rows<P>(h, f, NODAL ? 2 : 1, ro, s);
-  if (st) return st;
-  return fix_long_rows<P>(h, f, NODAL ? 2 : 1, ro, s);
+  return fix_rows<P>(h, f, NODAL ? 2 : 1, ro, true, s);
 }
 
 static nsi_status step_dispatch(NsiHandle* h, const NsiFields* f, const StepView& o, bool nodal, cudaStream_t s) {
@@ -1763,8 +1755,7 @@ static nsi_status batched_p(NsiHandle* const* hs, const NsiFields* fs, const Nsi
   nsi_status st = batched_core_p<P>(hs, fs, os, count, s);
   for (int k = 0; k < count && !st; ++k) {
     const RowOut ro{nullptr, os[k].A_val, os[k].G_val, os[k].rhs, nullptr, nullptr, 0.0};
-    st = fix_exact_rows<P>(hs[k], fields_of(&fs[k]), 0, ro, s);
-    if (!st) st = fix_long_rows<P>(hs[k], fields_of(&fs[k]), 0, ro, s);
+    st = fix_rows<P>(hs[k], fields_of(&fs[k]), 0, ro, true, s);
   }
   return st;
 }
@@ -1866,9 +1857,7 @@ static nsi_status assemble_noalloc_p(NsiHandle* h, const FieldView& f, const Out
   nsi_status st = assemble_core_p<P>(h, f, o, NSI_SCATTER_GATHER, s, scratch);
   if (st) return st;
   const RowOut ro{nullptr, o.A, o.G, o.rhs, nullptr, nullptr, 0.0};
-  st = fix_exact_rows<P>(h, f, 0, ro, s);
-  if (st) return st;
-  return fix_long_rows<P>(h, f, 0, ro, s);
+  return fix_rows<P>(h, f, 0, ro, true, s);
 }
 
 }  // namespace nsi

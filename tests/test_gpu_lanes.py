@@ -82,9 +82,9 @@ def test_flat_cube_rows_in_double(precision, N):
 
 @pytest.mark.parametrize("precision", ["fp64", "mixed64", "mixed32"])
 def test_row_of_more_entries_than_a_block_has_threads(precision):
-    mesh, u = meshgen.delaunay_hub(8, 200, seed=330)
+    mesh, u = meshgen.delaunay_hub(8, 300, seed=330)
     asm = nsi.Assembler(mesh.coord, mesh.lnods, precision=precision)
-    assert asm.max_row > 128 and asm.info().long_rows > 0
+    assert asm.max_row > 256 and asm.info().long_rows > 0
     ut = torch.as_tensor(u.T.copy())
     uo = u if precision == "fp64" else u.astype(np.float32).astype(np.float64)
     rp, _, oA, oG, orhs = oracle.assemble(mesh.coord, mesh.lnods, uo, None, 1.0, 1e-3, 1e-2)
