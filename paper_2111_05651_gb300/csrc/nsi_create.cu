@@ -489,7 +489,7 @@ static nsi_status build(NsiHandle* h, const NsiMesh* m, cudaStream_t s) {
 
   // 4a. every row's sub-walks (the order and steps of the kernel's element
   // loops), one per lane of the row
-  h->nsub = n >= SMALL_MESH_ROWS ? 2 : 4;
+  h->nsub = n < SMALL_MESH_ROWS ? 4 : h->precision == NSI_FP64 && n >= LARGE_FP64_ROWS ? 1 : 2;
   std::vector<int32_t> walk_ptr;
   std::vector<uint8_t> walk;
   if (h->gather_ok) {

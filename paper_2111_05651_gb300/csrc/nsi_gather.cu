@@ -25,15 +25,19 @@
 // and 269 -> 235 in natural node order, mixed32 228 -> 226, time step 275 ->
 // 229, nodal outputs 216 -> 126; 47x61x38 mixed32 39.6 -> 31.4).  The records
 // bypass L1 (allocating there cost 439 us: 115 KB of sectors in flight per SM
-// through the 28 KB that shared memory leaves).  What is left in random order is
-// the rate of scattered 32-byte requests (40 us against natural order; loading
-// still earlier changes nothing), then issue: 67 M warp instructions at the
-// 70^3 cube, 53% of the slots used.  FP64 is bound by the FP64 pipe.
+// through the 28 KB that shared memory leaves).  What is left is the shared
+// memory's data path (72% busy: 695 wavefronts of a group's 16 rows) and issue
+// (61%), and in random node order the rate of scattered 32-byte requests (40 us
+// against natural order; loading still earlier changes nothing).
 //
 // A small mesh has four lanes per row: its groups do not fill the chip, so the
-// chain is the time (8^3 cube in FP64: 66 us with one lane, 29 with four; 20^3
+// chain is the time (8^3 cube in FP64: 66 us with one lane, 27 with four; 20^3
 // mixed64 13.8 with one, 12.5 with two, 10.9 with four; at 30 000 rows two and
-// four are equal, and at 100^3 four cost 374 us).
+// four are equal, and at 100^3 four cost 374 us).  FP64 is bound by the FP64
+// pipe (one warp instruction in 18 cycles, 97-100% busy): a large mesh has one
+// lane per row, which saves the merge's additions (74 000 rows: 257 us with one
+// lane, 244 with two, whose smaller groups fill the last round better; 166 000:
+// 511 and 525; 100^3: 2977 and 3057, before all this 3023).
 #include <algorithm>
 #include <mutex>
 
@@ -112,6 +116,7 @@ struct NodeRec<NSI_FP64> {
 // operands of the instructions that use them and take no registers.
 struct GroupLay {
   int nb1, acc, plane, walk, info, cols, total, N, W, L, S;
+  GroupLay() = default;
   explicit GroupLay(const GatherSmem& g)
       : nb1((int)g.nb1()), acc((int)g.acc()), plane((int)(g.ab * g.N())), walk((int)g.walk()), info((int)g.info()),
         cols((int)g.cols()), total((int)g.total()), N((int)g.N()), W(g.W),
@@ -290,6 +295,7 @@ __device__ __forceinline__ void walk_lane(const uint8_t* __restrict__ st, int nb
     s += 2 + cnt;
     Node p = load(f1), n0 = load(f2);
     V3<T> M{};
+    bool flip = false;  // FP64: c_c is M, not -M
     if constexpr (MODE != NODAL) {
       M = cross_fma(n0.d, p.d);
       p.v = add(u2i, p.v);
@@ -312,7 +318,13 @@ __device__ __forceinline__ void walk_lane(const uint8_t* __restrict__ st, int nb
         const V3<T> cq = cross_fma(c.d, p.d);
         V3<T> w3{p.v.x + q.v.x + c.v.x, p.v.y + q.v.y + c.v.y, p.v.z + q.v.z + c.v.z};
         if constexpr (MODE == ASSEMBLE) {
-          const V3<T> ci{M.x - (cp.x + cq.x), M.y - (cp.y + cq.y), M.z - (cp.z + cq.z)};
+          V3<T> ci;
+          if constexpr (P == NSI_FP64) {
+            const T sg = flip ? T(-1) : T(1);
+            ci = V3<T>{fma(sg, M.x, -(cp.x + cq.x)), fma(sg, M.y, -(cp.y + cq.y)), fma(sg, M.z, -(cp.z + cq.z))};
+          } else {
+            ci = V3<T>{M.x - (cp.x + cq.x), M.y - (cp.y + cq.y), M.z - (cp.z + cq.z)};
+          }
           const T kv = mul_rn(kmu, rcp_fast(det));
           w3 = V3<T>{fma(kv, ci.x, w3.x), fma(kv, ci.y, w3.y), fma(kv, ci.z, w3.z)};
           const T fg = neg ? -kg : kg;
@@ -326,7 +338,7 @@ __device__ __forceinline__ void walk_lane(const uint8_t* __restrict__ st, int nb
             };
             upd(p.a, f, ap);
             upd(q.a, f, aq);
-            upd(c.a, neg ? T(1) : T(-1), ac);
+            upd(c.a, neg != flip ? T(1) : T(-1), ac);
           } else {
             const float2 gg = make_float2(fg, fg), cxy = make_float2(ci.x, ci.y);
             auto upd = [&](typename Slots<P, MODE>::V& a, float fs, float v) {
@@ -340,9 +352,14 @@ __device__ __forceinline__ void walk_lane(const uint8_t* __restrict__ st, int nb
         } else {
           p.a = fma(f, dot_fma(w3, cp), p.a);
           q.a = fma(f, dot_fma(w3, cq), q.a);
-          c.a = fma(neg ? T(1) : T(-1), dot_fma(w3, M), c.a);
+          c.a = fma(neg != flip ? T(1) : T(-1), dot_fma(w3, M), c.a);
         }
-        M = V3<T>{evq ? cq.x : -cp.x, evq ? cq.y : -cp.y, evq ? cq.z : -cp.z};
+        if constexpr (P == NSI_FP64) {  // (a negated double is an operation of the FP64 pipe, its bound)
+          M = V3<T>{evq ? cq.x : cp.x, evq ? cq.y : cp.y, evq ? cq.z : cp.z};
+          flip = !evq;
+        } else {
+          M = V3<T>{evq ? cq.x : -cp.x, evq ? cq.y : -cp.y, evq ? cq.z : -cp.z};
+        }
         if (evq) acc.store(q.k, q.a);
         else acc.store(p.k, p.a);
       }
@@ -407,10 +424,10 @@ struct GroupRow {
 template <int RW>
 __device__ __forceinline__ void copy_rows(const WalkMesh& m, unsigned char* info, int64_t r0, int lane) {
   int32_t* b = reinterpret_cast<int32_t*>(info);
-  if (lane <= RW) {
-    const int64_t i = min(r0 + lane, m.n);
-    cp_async4(b + lane, m.row_ptr + i);
-    cp_async4(b + RW + 1 + lane, m.walk_ptr + i);
+  for (int k = lane; k <= RW; k += 32) {
+    const int64_t i = min(r0 + k, m.n);
+    cp_async4(b + k, m.row_ptr + i);
+    cp_async4(b + RW + 1 + k, m.walk_ptr + i);
   }
   if (lane < RW / 4) cp_async4(b + 2 * (RW + 1) + lane, m.diag_pos + r0 + 4 * lane);  // (padded past n)
 }
@@ -491,7 +508,7 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
   // one lane's accumulators
   auto slots = [&](int p) { return Slots<P, MODE>(smem + lay.acc + p * lay.plane, lay.N); };
 
-  constexpr int UT = P == NSI_FP64 ? 4 : 16 / H;  // records of a lane in flight
+  constexpr int UT = P == NSI_FP64 || H == 1 ? 4 : 16 / H;  // records of a lane in flight
 
   auto copy_cols = [&](const WalkMesh& m, int32_t c0, int32_t c1) {
     if (DEBUG && c1 - c0 > lay.L) return;  // reported below
@@ -789,7 +806,8 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
       const T4<T>* stage = reinterpret_cast<const T4<T>*>(smem);
       Out* A = static_cast<Out*>(o.A) + base;
       Out *G = static_cast<Out*>(o.G) + base, *G1 = G + m.nnz, *G2 = G1 + m.nnz;
-      // (streaming stores: the outputs leave L2 before the records do)
+      // (mixed64 by streaming stores: the outputs leave L2 before the records do,
+      // 271 against 279 us at 100^3 in random order; mixed32 236 against 226)
       auto write = [&](auto&& put) {
 #pragma unroll 1
         for (int k = lane; k < (fits ? L : 0); k += 32) put(k, stage[k]);
@@ -810,10 +828,10 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
           A[lb + row.dp] = nonfinite_bits(dhi) ? nonfinite_double(dhi) : pair_double(dhi, dlo);
       } else {
         write([&](int k, const T4<T>& v) {
-          __stcs(A + k, v.x);
-          __stcs(G + k, v.y);
-          __stcs(G1 + k, v.z);
-          __stcs(G2 + k, v.w);
+          A[k] = v.x;
+          G[k] = v.y;
+          G1[k] = v.z;
+          G2[k] = v.w;
         });
       }
     } else if constexpr (MODE == STEP) {
@@ -985,15 +1003,21 @@ __global__ void __launch_bounds__(32) exact_rows_kernel(WalkMesh m, FieldView f,
 }
 
 // ------------------------------------------------------ batched kernel ---
-// The meshes with two lanes per row first, then those with four: a warp takes
-// its share of the first's groups, then of the second's, so that every mesh is
-// assembled as by its own launch.
+// The meshes with one lane per row first, then those with two, then those with
+// four: a warp takes its share of the first's groups, then of the next's, so
+// that every mesh is assembled as by its own launch.
+constexpr int KINDS = 3;
+__host__ __device__ constexpr int kind_lanes(int kind) { return 1 << kind; }
 struct BatchArgs {
-  int32_t count[2];  // meshes
-  int32_t total[2];  // row groups
+  int32_t count[KINDS];  // meshes
+  int32_t total[KINDS];  // row groups
   WalkItem<ASSEMBLE> item[NSI_MAX_BATCH];
 };
-static_assert(sizeof(BatchArgs) + 2 * sizeof(GroupLay) <= 32764, "kernel parameters");
+struct BatchLays {
+  GroupLay kind[KINDS];
+  int stride;  // bytes of a warp's shared memory
+};
+static_assert(sizeof(BatchArgs) + sizeof(BatchLays) <= 32764, "kernel parameters");
 
 struct BatchMesh {
   const BatchArgs& args;
@@ -1013,17 +1037,28 @@ struct BatchMesh {
 
 template <int P>
 __global__ void __launch_bounds__(32 * MAX_WARPS, P == NSI_FP64 ? 2 : 4)
-    batched_kernel(const __grid_constant__ BatchArgs args, GroupLay lay2, GroupLay lay4) {
+    batched_kernel(const __grid_constant__ BatchArgs args, const __grid_constant__ BatchLays lays) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int warps = blockDim.x >> 5, w = threadIdx.x >> 5;
-  const int all = (int)gridDim.x * warps, me = (int)blockIdx.x * warps + w;
-  unsigned char* smem = smem_raw + w * max(lay2.total, lay4.total);
-  group_loop<P, 2, ASSEMBLE, false, false>(BatchMesh{args, 0, args.count[0]}, me, all, args.total[0], smem, lay2);
-  __syncwarp();
-  // (the warps with one group less of the first kind begin the second)
-  const int start = me - args.total[0] % all;
-  group_loop<P, 4, ASSEMBLE, false, false>(BatchMesh{args, args.count[0], args.count[1]}, start < 0 ? start + all : start, all,
-                                    args.total[1], smem, lay4);
+  const int all = (int)gridDim.x * warps;
+  unsigned char* smem = smem_raw + w * lays.stride;
+  int me = (int)blockIdx.x * warps + w;
+  // (the warps with one group less of a kind begin the next kind's)
+  auto next = [&](int kind) {
+    __syncwarp();
+    me -= args.total[kind] % all;
+    if (me < 0) me += all;
+  };
+  if constexpr (P == NSI_FP64) {
+    group_loop<P, 1, ASSEMBLE, false, false>(BatchMesh{args, 0, args.count[0]}, me, all, args.total[0], smem,
+                                             lays.kind[0]);
+    next(0);
+  }
+  group_loop<P, 2, ASSEMBLE, false, false>(BatchMesh{args, args.count[0], args.count[1]}, me, all, args.total[1], smem,
+                                           lays.kind[1]);
+  next(1);
+  group_loop<P, 4, ASSEMBLE, false, false>(BatchMesh{args, args.count[0] + args.count[1], args.count[2]}, me, all,
+                                           args.total[2], smem, lays.kind[2]);
 }
 
 template <int P>
@@ -1033,15 +1068,20 @@ __global__ void __launch_bounds__(256) pack_kernel(WalkMesh m, FieldView f) {
 }
 
 // the node records of every mesh of a batch in one launch: a block packs the
-// rows of 8 consecutive groups of 16, or of 16 of 8
+// 128 rows of consecutive groups of one kind
 template <int P>
 __global__ void __launch_bounds__(128) batched_pack_kernel(const __grid_constant__ BatchArgs args) {
-  const int blocks2 = (args.total[0] + 7) / 8;
-  const int kind = (int)blockIdx.x < blocks2 ? 0 : 1;
-  const int rw = kind ? 8 : 16;
-  const int g = ((int)blockIdx.x - kind * blocks2) * (128 / rw) + (int)threadIdx.x / rw;
+  int block = (int)blockIdx.x, kind = 0, first = 0;
+  for (; kind < KINDS - 1; ++kind) {
+    const int groups = 4 * kind_lanes(kind), blocks = (args.total[kind] + groups - 1) / groups;
+    if (block < blocks) break;
+    block -= blocks;
+    first += args.count[kind];
+  }
+  const int rw = 32 / kind_lanes(kind);
+  const int g = block * (128 / rw) + (int)threadIdx.x / rw;
   if (g >= args.total[kind]) return;
-  const BatchMesh src{args, kind * args.count[0], args.count[kind]};
+  const BatchMesh src{args, first, args.count[kind]};
   const WalkItem<ASSEMBLE>& it = src.item(src.find(g));
   const int64_t i = (int64_t)(g - it.group0) * rw + threadIdx.x % rw;
   if (i < it.m.n) pack_node<P>(it.m, it.f, it.m.rec, i);
@@ -1124,6 +1164,11 @@ nsi_status run_groups(NsiHandle* h, const WalkItem<MODE>& item, int64_t row0, in
 template <int P, int MODE>
 nsi_status run_lanes(NsiHandle* h, const WalkItem<MODE>& item, int64_t row0, int64_t row1, cudaStream_t s) {
   switch (h->nsub) {
+    case 1:
+      if constexpr (P == NSI_FP64)
+        return h->debug ? run_groups<P, 1, MODE, true>(h, item, row0, row1, s)
+                        : run_groups<P, 1, MODE, false>(h, item, row0, row1, s);
+      return fail(NSI_ERR_UNSUPPORTED, "one lane per row in FP64 only");
     case 2:
       return h->debug ? run_groups<P, 2, MODE, true>(h, item, row0, row1, s)
                       : run_groups<P, 2, MODE, false>(h, item, row0, row1, s);
@@ -1180,9 +1225,13 @@ nsi_status launch_batched(NsiHandle* const* hs, const NsiFields* fs, const NsiOu
   static BatchArgs args;  // host staging of the by-value kernel argument
   static std::mutex mu;
   std::lock_guard<std::mutex> lock(mu);
-  int warps = MAX_WARPS, W[2] = {1, 1}, L[2] = {0, 0}, S[2] = {0, 0}, item = 0;
-  for (int kind = 0; kind < 2; ++kind) {  // two lanes per row, then four
-    const int H = kind ? 4 : 2, rw = 32 / H;
+  int warps = MAX_WARPS, item = 0;
+  int64_t all = 0, pack_blocks = 0;
+  size_t bytes = 0;
+  BatchLays lays;
+  for (int kind = 0; kind < KINDS; ++kind) {
+    const int H = kind_lanes(kind), rw = 32 / H;
+    int W = 1, L = 0, S = 0;
     int64_t groups = 0;
     args.count[kind] = 0;
     for (int k = 0; k < count; ++k) {
@@ -1190,9 +1239,9 @@ nsi_status launch_batched(NsiHandle* const* hs, const NsiFields* fs, const NsiOu
       if (h->nsub != H) continue;
       const GatherPlan& pl = h->plan;
       warps = std::min(warps, pl.warps);
-      W[kind] = std::max(W[kind], pl.w);
-      L[kind] = std::max(L[kind], pl.max_block_entries);
-      S[kind] = std::max(S[kind], pl.max_block_steps);
+      W = std::max(W, pl.w);
+      L = std::max(L, pl.max_block_entries);
+      S = std::max(S, pl.max_block_steps);
       args.item[item++] = WalkItem<ASSEMBLE>{walk_mesh(h, nullptr), fields_of(&fs[k]),
                                              {os[k].A_val, os[k].G_val, os[k].rhs}, (int)groups};
       ++args.count[kind];
@@ -1200,25 +1249,27 @@ nsi_status launch_batched(NsiHandle* const* hs, const NsiFields* fs, const NsiOu
       if (groups > INT32_MAX / 2) return fail(NSI_ERR_UNSUPPORTED, "too many rows in a batch");
     }
     args.total[kind] = (int)groups;
+    all += groups;
+    pack_blocks += (groups + 4 * H - 1) / (4 * H);
+    const GatherSmem lay = group_smem(P, ASSEMBLE, H, W, L, S);
+    if (!lay.group_fits())  // (each mesh's fits, and so do the maxima of W and L)
+      return fail(NSI_ERR_UNSUPPORTED, "batched meshes need more shared memory than a group has");
+    if (args.count[kind]) bytes = std::max(bytes, lay.total());
+    lays.kind[kind] = GroupLay(lay);
   }
-  const int64_t groups = (int64_t)args.total[0] + args.total[1];
-  if (groups == 0) return NSI_OK;
-  const GatherSmem lay2 = group_smem(P, ASSEMBLE, 2, W[0], L[0], S[0]);
-  const GatherSmem lay4 = group_smem(P, ASSEMBLE, 4, W[1], L[1], S[1]);
-  if (!lay2.group_fits() || !lay4.group_fits())  // (each mesh's fits, and so do the maxima of W and L)
-    return fail(NSI_ERR_UNSUPPORTED, "batched meshes need more shared memory than a group has");
-  const size_t bytes = std::max(args.count[0] ? lay2.total() : 0, args.count[1] ? lay4.total() : 0);
+  if (all == 0) return NSI_OK;
   while (warps > 1 && bytes * warps > SMEM_MAX) --warps;
   if (bytes > SMEM_MAX) return fail(NSI_ERR_UNSUPPORTED, "batched meshes need more shared memory than a block has");
+  lays.stride = (int)bytes;
   static std::once_flag once;
   static cudaError_t err = cudaSuccess;
   nsi_status st = allow_smem(batched_kernel<P>, once, err);
   if (st) return st;
-  batched_pack_kernel<P><<<(args.total[0] + 7) / 8 + (args.total[1] + 15) / 16, 128, 0, s>>>(args);
+  batched_pack_kernel<P><<<pack_blocks, 128, 0, s>>>(args);
   if ((st = check_launch("batched_pack_kernel"))) return st;
   int64_t grid = 0;
-  if ((st = resident_grid(batched_kernel<P>, warps, bytes * warps, groups, nullptr, &grid))) return st;
-  NSI_CUDA(launch_early(batched_kernel<P>, grid, 32 * warps, bytes * warps, s, args, GroupLay(lay2), GroupLay(lay4)));
+  if ((st = resident_grid(batched_kernel<P>, warps, bytes * warps, all, nullptr, &grid))) return st;
+  NSI_CUDA(launch_early(batched_kernel<P>, grid, 32 * warps, bytes * warps, s, args, lays));
   return check_launch("batched_kernel");
 }
 

@@ -91,6 +91,8 @@ struct GatherPlan {
 // (measured equal at about 30 000 rows for the assembly and at 10 000 for the
 // time step)
 constexpr int64_t SMALL_MESH_ROWS = 10000;
+// from here on FP64 has one lane per row (two are faster at 74 000, one at 166 000)
+constexpr int64_t LARGE_FP64_ROWS = 120000;
 constexpr int SMEM_MAX = 200 * 1024;  // shared memory of one block
 
 // diag_pos value of a row the row gather leaves out ("long row": more than
@@ -186,7 +188,7 @@ struct NsiHandle {
   int32_t* walk_ptr = nullptr;  // [n+1]
   uint8_t* walk = nullptr;      // [walk_ptr[n] + 8]
   int nsub = 2;                 // sub-walks per row
-  bool packs() const { return nsub == 2; }  // the row gather reads packed node records (else the nodes' own data)
+  bool packs() const { return nsub != 4; }  // the row gather reads packed node records (else the nodes' own data)
   uint8_t* diag_pos = nullptr;  // [n + 32] position of the diagonal inside its row (rows <= 32 entries)
   unsigned long long* elem_pos = nullptr;  // [E] element-position map (rows <= 32 entries), or null
   // edge-fan map (one word per CSR entry) and its block partition of the rows

@@ -1,5 +1,5 @@
 """The row gather at the edges of its lane rule: meshes around the row count
-where four lanes per row become two, and one whose groups are more than the
+where four lanes per row become two (and, in FP64, two one), and one whose groups are more than the
 resident warps (every warp takes several), against the oracle; a batch that
 mixes both kinds against the single calls, bit for bit."""
 import numpy as np
@@ -16,8 +16,8 @@ pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not torch.cuda.is_available(),
 TOL = {"fp64": 1e-12, "mixed64": 1e-5, "mixed32": 1e-5}  # the library's stated bars
 
 
-@pytest.mark.parametrize("precision", ["fp64", "mixed64", "mixed32"])
-@pytest.mark.parametrize("N", [20, 21, 36])  # 9,261, 10,648 and 50,653 rows
+@pytest.mark.parametrize("precision,N", [(p, N) for p in ("fp64", "mixed64", "mixed32") for N in (20, 21, 36)] +
+                         [("fp64", 49)])  # 9,261, 10,648, 50,653 and (one lane in FP64) 125,000 rows
 def test_lanes_match_oracle(precision, N):
     mesh, u = meshgen.config_mesh(N=N, jitter=0.15, numbering="random", seed=300 + N)
     asm = nsi.Assembler(mesh.coord, mesh.lnods, precision=precision)
@@ -43,7 +43,7 @@ def test_lanes_match_oracle(precision, N):
 @pytest.mark.parametrize("precision", ["fp64", "mixed64", "mixed32"])
 def test_batch_of_both_kinds_equals_single(precision):
     asms, us = [], []
-    for N in (3, 36, 20, 22):
+    for N in (3, 36, 20, 49, 22):
         mesh, u = meshgen.config_mesh(N=N, jitter=0.15, numbering="natural", seed=310 + N)
         asms.append(nsi.Assembler(mesh.coord, mesh.lnods, precision=precision))
         us.append(torch.as_tensor(u.T.copy()))
