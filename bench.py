@@ -484,7 +484,7 @@ def run_gpu(args, world, rank, local):
     main = results[main_prec]
     ms_max = allreduce_max(main["ms"], world)
     value = world * E / (ms_max * 1e-3)
-    gather_name = "fan_kernel" if args.fan else ("gather_persistent_kernel" if main["persistent"] else "gather_kernel")
+    gather_name = "fan_kernel" if args.fan else "gather_persistent_kernel"
     kernel = {"gather": gather_name, "atomic": "elem_kernel",
               "color": "elem_kernel"}[main["mode"]]
     bytes_alg = algorithmic_bytes(E, n, main["nnz"], main_prec)
@@ -862,7 +862,7 @@ def run_step(args, world, rank, local):
                                      "l2": "flushed (256 MiB write) before every timed step"},
                           "roofline": {"bound": "hbm", "achieved": m["achieved_gbs"], "peak": peak, "unit": "GB/s",
                                        "frac": m["achieved_gbs"] / peak,
-                                       "traffic": read_traffic("step_kernel", "cube100", "mixed64"), "kernel": "step_kernel",
+                                       "traffic": read_traffic("gather_persistent_kernel:step", "cube100", "mixed64"), "kernel": "gather_persistent_kernel",
                                        "algorithmic_bytes": m["algorithmic_bytes"], "kernel_ms": m["kernel_ms"],
                                        "peak_source": src},
                           "clocks": m.pop("clocks", None), "gpu_launches": args.steps * 2,  # pack + step kernel

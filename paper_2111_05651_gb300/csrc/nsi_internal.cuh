@@ -87,7 +87,7 @@ struct GatherPlan {
   int w = 0;                  // slots per row (>= the off-diagonal entries of the longest row the kernels
                               // take, and large enough that every group's entries fit its staging)
 };
-// a mesh of fewer rows has four lanes per row in the row gather, others two
+// a mesh of fewer rows has four lanes per row in the row gather, others two or one
 // (measured equal at about 30 000 rows for the assembly and at 10 000 for the
 // time step)
 constexpr int64_t SMALL_MESH_ROWS = 10000;
