@@ -21,13 +21,13 @@
 // and a second set of accumulators (13 KB, 16 warps) behind chains of 12, and
 // the neighbours' records come as one 256-bit load each, in registers under the
 // previous group's write-out, instead of two 16-byte copies through shared
-// memory (100^3 cube, us, one lane per row -> two: mixed64 277 -> 271 in random
-// and 269 -> 235 in natural node order, mixed32 228 -> 226, time step 275 ->
-// 229, nodal outputs 216 -> 126; 47x61x38 mixed32 39.6 -> 31.4).  The records
+// memory (100^3 cube, us, one lane per row -> two: mixed64 277 -> 266 in random
+// and 269 -> 226 in natural node order, mixed32 228 -> 226, time step 275 ->
+// 198, nodal outputs 216 -> 126; 47x61x38 mixed32 39.6 -> 31.4).  The records
 // bypass L1 (allocating there cost 439 us: 115 KB of sectors in flight per SM
 // through the 28 KB that shared memory leaves).  What is left is the shared
-// memory's data path (72% busy: 695 wavefronts of a group's 16 rows) and issue
-// (61%), and in random node order the rate of scattered 32-byte requests (40 us
+// memory's data path (75% busy: 740 wavefronts of a group's 16 rows) and issue
+// (about 60%), and in random node order the rate of scattered 32-byte requests (40 us
 // against natural order; loading still earlier changes nothing).
 //
 // A small mesh has four lanes per row: its groups do not fill the chip, so the
@@ -895,7 +895,8 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, P == NSI_FP64 ? 2 : 4)
 // (the walk bytes read from memory, the entries written row by row): the FP64
 // pipe, the bound here, issues a warp's instruction at the same cost whether or
 // not its lanes are active, so rows side by side fill it best (a 14x40x70 pipe,
-// 14,905 of its 39,831 rows listed: 66 us, of which the pipe is busy 45).  MODE 0: A, G and rhs; 1: rhs only (the time
+// 14,905 of its 39,831 rows listed: 66 us, of which the pipe is busy 45).
+// MODE 0: A, G and rhs; 1: rhs only (the time
 // step: the convection does not involve the determinant); 2: rhs, dt_rho and
 // mass_rho.
 template <int P, int H, int MODE>

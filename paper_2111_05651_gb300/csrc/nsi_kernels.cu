@@ -850,6 +850,10 @@ constexpr int STAR_WARPS = 4;  // warps (tasks) per block
 // Each element is evaluated once per row of its star (four times per tet).
 // Long rows (more than 32 entries, or a star the row-gather encoder could
 // not cover) are single-row tasks this kernel skips.
+// Bound by issue, at six blocks per SM (registers; five 233 us per call of a
+// 64x57x60 box in mixed64, seven 206, six 205).  With the totals by shuffles of
+// every lane, the diagonal's values by its own lane and det in the records the
+// call took 222 us, and the kernel at 100^3 944 instead of 890.
 template <int P, bool DEBUG>
 __global__ void __launch_bounds__(32 * STAR_WARPS, P == NSI_FP64 ? 1 : 6) stab_star_kernel(
     MeshView m, FieldView f, StabConst sc, const int4* __restrict__ tasks, int64_t ntasks,
@@ -1285,8 +1289,10 @@ __device__ __forceinline__ V3<C> axpy(C a, const V3<C>& x, const V3<C>& y) {
 //   sum_a w_a A_e[a][m] = (rho/120 M + mu/(6 det) Q) c_m + rho det/(24 dt) w_m,
 // and the grad_mu term is the sum of Q's and Gu's products entry by entry: 300
 // operations per element instead of 380 with every A_e[a][m].
-// In double only: the float kernel is bound by its atomic adds, not by its
-// operations, and keeps the sums over the entries (below).
+// In double only, where the FP64 pipe is the bound (84-88% busy; residual and
+// adjoint of 166,320 tets 184 us, 243 with every entry in both): the float
+// kernel is bound by its atomic adds (31 us for 750,000 tets either way), not
+// by its operations, and keeps the sums over the entries (below).
 __device__ __forceinline__ double vjp_element(const V3<double>& d1, const V3<double>& d2, const V3<double>& d3,
                                               const V3<double> (&u)[4], const V3<double> (&w)[4], double kc,
                                               double kmu, double kmass, V3<double> (&g)[4]) {
