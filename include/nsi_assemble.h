@@ -98,7 +98,7 @@ typedef enum {
     NSI_SCATTER_AUTO = 0,     /* library choice (row gather when available) */
     NSI_SCATTER_COLOR = 1,    /* element colouring, plain read-add-write, deterministic */
     NSI_SCATTER_ATOMIC = 2,   /* one element per thread, global atomic adds */
-    NSI_SCATTER_GATHER = 3    /* one CSR row per thread, gathers its elements, writes once;
+    NSI_SCATTER_GATHER = 3    /* one to four lanes per CSR row, gathers its elements, writes once;
                                  deterministic (rows of more than 32 entries by a second,
                                  per-row kernel: NsiInfo.long_rows) */
 } nsi_scatter;
