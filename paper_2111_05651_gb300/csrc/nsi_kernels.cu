@@ -1255,89 +1255,19 @@ __global__ void __launch_bounds__(FAN_BLOCK) batched_fan_kernel(const __grid_con
 }
 
 // ----------------------------------------------------------- VJP kernel ---
-// reciprocal of a determinant: IEEE in float; double by rcp_fast (its error is
-// below the double's rounding, and the FP64 pipe bounds the FP64 kernels)
-__device__ __forceinline__ float rcp_det(float x) { return rcp(x); }
-__device__ __forceinline__ double rcp_det(double x) { return rcp_fast(x); }
-
-// row k of sum_b v_b c_b^T over the element's nodes, by the differences to node
-// 0 (sum_b c_b = 0): v = u gives det du_k / dx
-template <typename C>
-__device__ __forceinline__ V3<C> moment(C d1, C d2, C d3, const V3<C> (&c)[4]) {
-  return {d1 * c[1].x + d2 * c[2].x + d3 * c[3].x, d1 * c[1].y + d2 * c[2].y + d3 * c[3].y,
-          d1 * c[1].z + d2 * c[2].z + d3 * c[3].z};
-}
-template <typename C>
-__device__ __forceinline__ void moments(const V3<C> (&v)[4], const V3<C> (&c)[4], V3<C> (&m)[3]) {
-  const V3<C> a = sub(v[1], v[0]), b = sub(v[2], v[0]), d = sub(v[3], v[0]);
-  m[0] = moment(a.x, b.x, d.x, c);
-  m[1] = moment(a.y, b.y, d.y, c);
-  m[2] = moment(a.z, b.z, d.z, c);
-}
-template <typename C>
-__device__ __forceinline__ V3<C> axpy(C a, const V3<C>& x, const V3<C>& y) {
-  return {fma_of(a, x.x, y.x), fma_of(a, x.y, y.y), fma_of(a, x.z, y.z)};
-}
-
 // One element's adjoint terms in arithmetic C (edge vectors d1, d2, d3 from
 // node 0; velocities u and adjoint weights w of the 4 nodes):
-//   g[m] = sum_a w_a A_e[a][m] + rho/120 sum_j (W_j + w_{m,j}) Gu[j]
+//   g[m] = sum_a w_a A_e[a][m] + rho/120 sum_k (W_k + w_{m,k}) Gu[k]
 //   returned: 1/(6 det) sum_{a,k} w_{a,k} c_a . Gu[k]   (the grad_mu term)
-// with W = sum_a w_a and Gu[k] = sum_b u_{b,k} c_b = det grad u_k.  The sum over
-// a is a 3x3 matrix applied to c_m: with S = sum_a u_a and the moments
-// M = W S^T + sum_a w_a u_a^T and Q = sum_a w_a c_a^T,
-//   sum_a w_a A_e[a][m] = (rho/120 M + mu/(6 det) Q) c_m + rho det/(24 dt) w_m,
-// and the grad_mu term is the sum of Q's and Gu's products entry by entry: 300
-// operations per element instead of 380 with every A_e[a][m].
-// In double only, where the FP64 pipe is the bound (84-88% busy; residual and
-// adjoint of 166,320 tets 184 us, 243 with every entry in both): the float
-// kernel is bound by its atomic adds (31 us for 750,000 tets either way), not
-// by its operations, and keeps the sums over the entries (below).
-__device__ __forceinline__ double vjp_element(const V3<double>& d1, const V3<double>& d2, const V3<double>& d3,
-                                              const V3<double> (&u)[4], const V3<double> (&w)[4], double kc,
-                                              double kmu, double kmass, V3<double> (&g)[4]) {
-  using C = double;
-  V3<C> c[4];
-  c[1] = cross(d2, d3);
-  c[2] = cross(d3, d1);
-  c[3] = cross(d1, d2);
-  const C det = dot(d1, c[1]);
-  c[0] = {-(c[1].x + c[2].x + c[3].x), -(c[1].y + c[2].y + c[3].y), -(c[1].z + c[2].z + c[3].z)};
-  const V3<C> S = add(add(u[0], u[1]), add(u[2], u[3]));
-  const V3<C> Ws = add(add(w[0], w[1]), add(w[2], w[3]));
-  const C rdet = rcp_det(det);
-  const C kv = kmu * rdet;
-  const C km = det * kmass;
-  V3<C> Gu[3], Q[3];
-  moments(u, c, Gu);
-  moments(w, c, Q);
-  const C s = dot(Q[0], Gu[0]) + dot(Q[1], Gu[1]) + dot(Q[2], Gu[2]);
-  const C W[3] = {Ws.x, Ws.y, Ws.z};
-  const C wk[4][3] = {{w[0].x, w[0].y, w[0].z}, {w[1].x, w[1].y, w[1].z}, {w[2].x, w[2].y, w[2].z},
-                      {w[3].x, w[3].y, w[3].z}};
-  V3<C> P[3], H[3], T{C(0), C(0), C(0)};  // rho/120 M + mu/(6 det) Q; rho/120 Gu; its part with W
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    V3<C> M = {W[k] * S.x, W[k] * S.y, W[k] * S.z};
-#pragma unroll
-    for (int a = 0; a < 4; ++a) M = axpy(wk[a][k], u[a], M);
-    P[k] = axpy(kv, Q[k], V3<C>{kc * M.x, kc * M.y, kc * M.z});
-    H[k] = {kc * Gu[k].x, kc * Gu[k].y, kc * Gu[k].z};
-    T = axpy(W[k], H[k], T);
-  }
-#pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    V3<C> acc = axpy(km, w[m], T);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) acc = axpy(wk[m][k], H[k], acc);
-    g[m] = {acc.x + dot(P[0], c[m]), acc.y + dot(P[1], c[m]), acc.z + dot(P[2], c[m])};
-  }
-  return s * (C)(1.0 / 6.0) * rdet;
-}
-__device__ __forceinline__ float vjp_element(const V3<float>& d1, const V3<float>& d2, const V3<float>& d3,
-                                             const V3<float> (&u)[4], const V3<float> (&w)[4], float kc, float kmu,
-                                             float kmass, V3<float> (&g)[4]) {
-  using C = float;
+// with W = sum_a w_a and Gu[k][l] = sum_b u_{b,k} c_b[l] = det du^k/dx_l.
+// The viscosity gradient is one sum of terms of both signs over all elements,
+// so a term's rounding shows in it multiplied by the sum's cancellation: the
+// terms keep this form.  (With 3x3 moments, Q = sum_a w_a c_a^T and the term Q . Gu,
+// an FP64 call took 300 operations per element instead of 380, and grad_mu of
+// cancelling weights moved by 1e-14 and more.)
+template <typename C>
+__device__ __forceinline__ C vjp_element(const V3<C>& d1, const V3<C>& d2, const V3<C>& d3, const V3<C> (&u)[4],
+                                         const V3<C> (&w)[4], C kc, C kmu, C kmass, V3<C> (&g)[4]) {
   V3<C> c[4];
   c[1] = cross(d2, d3);
   c[2] = cross(d3, d1);
@@ -1414,7 +1344,7 @@ __global__ void __launch_bounds__(256) vjp_kernel(MeshView m, FieldView f, const
       u[a] = load_vec<T>(f.u, v[a]);
       w[a] = {W[v[a]], W[m.n + v[a]], W[2 * m.n + v[a]]};
     }
-    my_mu = vjp_element(X[1].minus(X[0]), X[2].minus(X[0]), X[3].minus(X[0]), u, w, kc_of<T>(f), kmu_of<T>(f),
+    my_mu = vjp_element<T>(X[1].minus(X[0]), X[2].minus(X[0]), X[3].minus(X[0]), u, w, kc_of<T>(f), kmu_of<T>(f),
                            kmass_of<T>(f), g);
     T* gp = static_cast<T*>(gu);
 #pragma unroll
@@ -1468,6 +1398,30 @@ __global__ void __launch_bounds__(64) vjp_exact_kernel(MeshView m, FieldView f, 
 
 
 // ----------------------------------------------------- residual kernel ---
+// reciprocal of a determinant: IEEE in float; double by rcp_fast (its error is
+// below the double's rounding, and the FP64 pipe bounds the FP64 kernels)
+__device__ __forceinline__ float rcp_det(float x) { return rcp(x); }
+__device__ __forceinline__ double rcp_det(double x) { return rcp_fast(x); }
+
+// row k of sum_b v_b c_b^T over the element's nodes, by the differences to node
+// 0 (sum_b c_b = 0): v = u gives det du_k / dx
+template <typename C>
+__device__ __forceinline__ V3<C> moment(C d1, C d2, C d3, const V3<C> (&c)[4]) {
+  return {d1 * c[1].x + d2 * c[2].x + d3 * c[3].x, d1 * c[1].y + d2 * c[2].y + d3 * c[3].y,
+          d1 * c[1].z + d2 * c[2].z + d3 * c[3].z};
+}
+template <typename C>
+__device__ __forceinline__ void moments(const V3<C> (&v)[4], const V3<C> (&c)[4], V3<C> (&m)[3]) {
+  const V3<C> a = sub(v[1], v[0]), b = sub(v[2], v[0]), d = sub(v[3], v[0]);
+  m[0] = moment(a.x, b.x, d.x, c);
+  m[1] = moment(a.y, b.y, d.y, c);
+  m[2] = moment(a.z, b.z, d.z, c);
+}
+template <typename C>
+__device__ __forceinline__ V3<C> axpy(C a, const V3<C>& x, const V3<C>& y) {
+  return {fma_of(a, x.x, y.x), fma_of(a, x.y, y.y), fma_of(a, x.z, y.z)};
+}
+
 // R[k][v_a] += sum_b A_e[a][b] u_b[k] - rho |T_e| / (4 dt) u^n_a[k]: the
 // residual of the assembled system without forming A (element per thread).  The
 // sum over b is a product with Gu[k] = sum_b u_{b,k} c_b:
