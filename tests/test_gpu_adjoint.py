@@ -43,3 +43,12 @@ def test_grad_mu_of_cancelling_weights(seed):
     w = torch.as_tensor(w0 - alpha * w1).cuda()  # (exact: 20-bit fields, alpha of 20 fraction bits)
     _, gmu = asm.vjp(torch.as_tensor(u).cuda(), w, rho=1.0, mu=1e-3, dt=1e-2)
     assert gmu.item() == float.fromhex(ref)
+
+
+def test_grad_mu_of_one_cluster_repeats():
+    """750 tets, three blocks, whose sums are added in one order: repeats are equal to the bit."""
+    mesh, u = meshgen.config_mesh(N=5, jitter=0.15, numbering="random", seed=51)
+    w = torch.as_tensor(np.random.default_rng(52).standard_normal(u.shape).T.copy()).cuda()
+    asm = nsi.Assembler(mesh.coord, mesh.lnods, precision="fp64")
+    ut = torch.as_tensor(u.T.copy()).cuda()
+    assert len({asm.vjp(ut, w)[1].item() for _ in range(20)}) == 1
