@@ -313,13 +313,42 @@ __device__ __forceinline__ double rcp_fast(double x) {
 // as the blocks of the launch directly before it end, and calls
 // wait_for_previous before it reads what that launch writes, or writes what it
 // may write too; the wait ends when that launch, and so every one before it, is
-// complete.  Used by the kernels that read the packing's node records, which
-// first fetch row bounds, column indices and walk bytes, and by those that
-// overwrite listed rows.  (Letting them start with the packing's first blocks
+// complete.  What that launch writes is not read-only for such a kernel's
+// life: it is never read by .nc loads (or __ldg), and inline loads of it are
+// volatile with a memory clobber, so that they stay after the wait.  Used by the
+// kernels that read the packing's node records, which first fetch row bounds,
+// column indices and walk bytes, and by those that overwrite listed rows.
+// (Letting them start with the packing's first blocks
 // takes the SMs from it: a batch of 16 meshes 90.1 us, without early launches
 // 84.2, as it is 84.1; a 47x61x38 box in mixed32 33.0, 36.3, 33.1; a time step
 // of 81x70x66 96.8, 94.6, 92.5.)
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// 32 bytes of a node record (32-byte aligned) by one 256-bit load.  CACHE:
+// through L1 (the stabilised kernel, whose warps share neighbours), else past it.
+template <bool CACHE>
+__device__ __forceinline__ void load_record(const unsigned* r, uint4& a, uint4& b) {
+  if constexpr (CACHE)
+    asm volatile("ld.global.v8.u32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
+                 : "l"(r)
+                 : "memory");
+  else
+    asm volatile("ld.global.L1::no_allocate.v8.u32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
+                 : "l"(r)
+                 : "memory");
+}
+template <bool CACHE>
+__device__ __forceinline__ void load_record(const double* r, double& x, double& y, double& z) {
+  [[maybe_unused]] double pad;
+  if constexpr (CACHE)
+    asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(x), "=d"(y), "=d"(z), "=d"(pad) : "l"(r) : "memory");
+  else
+    asm volatile("ld.global.L1::no_allocate.v4.f64 {%0, %1, %2, %3}, [%4];"
+                 : "=d"(x), "=d"(y), "=d"(z), "=d"(pad)
+                 : "l"(r)
+                 : "memory");
+}
 template <typename... Params, typename... Args>
 cudaError_t launch_early(void (*kernel)(Params...), int64_t grid, int block, size_t smem, cudaStream_t s,
                          const Args&... args) {

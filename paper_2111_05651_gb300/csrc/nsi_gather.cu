@@ -63,10 +63,7 @@ template <int P>
 struct NodeRec {
   uint4 a, b;
   __device__ __forceinline__ void load(const void* rec, int64_t j) {
-    const unsigned* r = static_cast<const unsigned*>(rec) + 8 * j;
-    asm("ld.global.nc.L1::no_allocate.v8.u32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-        : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
-        : "l"(r));
+    load_record<false>(static_cast<const unsigned*>(rec) + 8 * j, a, b);
   }
   // the record's words from the node's own data, without a packed record
   template <typename Mesh>
@@ -94,9 +91,8 @@ struct NodeRec<NSI_FP64> {
   double x, y, z, ux, uy, uz;
   __device__ __forceinline__ void load(const void* rec, int64_t j) {
     const double* r = static_cast<const double*>(rec) + 8 * j;
-    [[maybe_unused]] double pad;
-    asm("ld.global.nc.L1::no_allocate.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(x), "=d"(y), "=d"(z), "=d"(pad) : "l"(r));
-    asm("ld.global.nc.L1::no_allocate.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(ux), "=d"(uy), "=d"(uz), "=d"(pad) : "l"(r + 4));
+    load_record<false>(r, x, y, z);
+    load_record<false>(r + 4, ux, uy, uz);
   }
   template <typename Mesh>
   __device__ __forceinline__ void gather(const Mesh& m, const FieldView& f, int64_t j) {
@@ -521,22 +517,25 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
   auto load_recs = [&](Recs& v, const WalkItem<MODE>& of, const GroupRow& r, const int32_t* col, int64_t i, int s0) {
     const WalkMesh& m = of.m;
     const int ns = row_slots(r);
-    const int64_t self = min(i, m.n - 1);
+    const int32_t self = (int32_t)min(i, m.n - 1);
     auto load = [&](NodeRec<P>& to, int64_t j) {
       if constexpr (DIRECT) to.gather(m, of.f, j);
       else to.load(m.rec, j);
     };
-    if (s0 == h) load(v.me, self);
+    // (all columns first: the records' loads keep their place among each other)
+    int32_t k[UT];
 #pragma unroll
     for (int c = 0; c < UT; ++c) {
       const int s = s0 + c * H;
-      int64_t k = s < ns ? (int64_t)col[slot_pos(s, r.dp)] : self;  // (past the row: its own, unused)
-      if (DEBUG && (k < 0 || k >= m.n)) {
+      k[c] = s < ns ? col[slot_pos(s, r.dp)] : self;  // (past the row: its own, unused)
+      if (DEBUG && (k[c] < 0 || k[c] >= m.n)) {
         atomicOr(m.err, ERR_BAD_INDEX);
-        k = self;
+        k[c] = self;
       }
-      load(v.r[c], k);
     }
+    if (s0 == h) load(v.me, self);
+#pragma unroll
+    for (int c = 0; c < UT; ++c) load(v.r[c], k[c]);
   };
   // the group's slots: edge vectors from the row's node, velocities, zeroed
   // sums; 2 rho/120 u_i of the row's own node

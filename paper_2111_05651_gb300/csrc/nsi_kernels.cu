@@ -909,26 +909,21 @@ __global__ void __launch_bounds__(32 * STAR_WARPS, P == NSI_FP64 ? 1 : 6) stab_s
     const int dl = seg * width + (len > 0 ? dp : 0);  // the diagonal's lane
     V3<T> d, u;
     if constexpr (P == NSI_FP64) {
-      D4 x{0.0, 0.0, 0.0, 0.0}, v{0.0, 0.0, 0.0, 0.0};
+      V3<double> x{0.0, 0.0, 0.0}, v{0.0, 0.0, 0.0};
       if (has && (!DEBUG || (j >= 0 && j < m.n))) {
-        const D4* r = static_cast<const D4*>(m.rec) + 2 * (int64_t)j;
-        x = r[0];
-        v = r[1];
+        const double* r = static_cast<const double*>(m.rec) + 8 * (int64_t)j;
+        load_record<true>(r, x.x, x.y, x.z);
+        load_record<true>(r + 4, v.x, v.y, v.z);
       }
       const double xi = __shfl_sync(FULL, x.x, dl), yi = __shfl_sync(FULL, x.y, dl), zi = __shfl_sync(FULL, x.z, dl);
       d = {x.x - xi, x.y - yi, x.z - zi};
-      u = {v.x, v.y, v.z};
+      u = v;
     } else {
       uint4 a = make_uint4(0u, 0u, 0u, 0u), b = a;
-      if (has && (!DEBUG || (j >= 0 && j < m.n))) {
-        // the 32-byte record (32-byte aligned; written by the pack kernel, a
-        // separate launch) in one 256-bit load instead of two 128-bit ones:
-        // 0.944 against 0.954 ms mixed64, 0.733 against 0.755 mixed32
-        const unsigned* r = static_cast<const unsigned*>(m.rec) + 8 * (int64_t)j;
-        asm("ld.global.nc.v8.u32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-            : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
-            : "l"(r));
-      }
+      // (one 256-bit load instead of two 128-bit ones: 0.944 against 0.954 ms
+      // mixed64, 0.733 against 0.755 mixed32)
+      if (has && (!DEBUG || (j >= 0 && j < m.n)))
+        load_record<true>(static_cast<const unsigned*>(m.rec) + 8 * (int64_t)j, a, b);
       const V3<float> hj{__uint_as_float(a.x), __uint_as_float(a.y), __uint_as_float(a.z)};
       const V3<float> lj = record_lo(__uint_as_float(b.z), __uint_as_float(b.w));
       const V3<float> hi{__shfl_sync(FULL, hj.x, dl), __shfl_sync(FULL, hj.y, dl), __shfl_sync(FULL, hj.z, dl)};
