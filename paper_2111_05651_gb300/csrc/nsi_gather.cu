@@ -484,10 +484,13 @@ __device__ __forceinline__ void merge_lanes(Acc<P>& a, int off) {
 // The next group's row bounds are copied under the current walk, its walk
 // bytes and column indices under the merge, and its records are loaded under
 // the write-out.
+// LONG: the mesh has groups whose entries, because of a long row among them, are
+// more than the staging holds.  (Kernels of their own: the time step of a mesh
+// without such groups took 88 us instead of 86.)
 // DIRECT: the nodes' coordinates and velocities are read where they are (five
 // loads a node) instead of from packed records (one), which saves a small mesh
 // the packing launch; the values are the same.
-template <int P, int H, int MODE, bool DEBUG, bool DIRECT, typename Source>
+template <int P, int H, int MODE, bool DEBUG, bool DIRECT, bool LONG, typename Source>
 __device__ __forceinline__ void group_loop(const Source& src, int g, int stride, int g_end, unsigned char* smem,
                                            const GroupLay& lay) {
   using T = typename Prec<P>::T;
@@ -507,14 +510,17 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
   constexpr int UT = P == NSI_FP64 || H == 1 ? 4 : 16 / H;  // records of a lane in flight
 
   auto copy_cols = [&](const WalkMesh& m, int32_t c0, int32_t c1) {
-    if (DEBUG && c1 - c0 > lay.L) return;  // reported below
+    if (LONG && c1 - c0 > lay.L) return;  // read where they are
     for (int k = lane; k < c1 - c0; k += 32) cp_async4(reinterpret_cast<int32_t*>(smem + lay.cols) + k, m.col_idx + c0 + k);
   };
-  // a row's record and its first UT slots' per lane, col its column indices
+  // a row's record and its slots' s0, s0 + H, ... (UT per lane); STAGED: by the
+  // column indices in shared memory, where the group's entries from c0 to c1 are
+  // unless they are more than the staging holds
   struct Recs {
     NodeRec<P> me, r[UT];
   };
-  auto load_recs = [&](Recs& v, const WalkItem<MODE>& of, const GroupRow& r, const int32_t* col, int64_t i, int s0) {
+  auto load_recs = [&](Recs& v, const WalkItem<MODE>& of, const GroupRow& r, int32_t c0, int32_t c1, int64_t i, int s0,
+                       bool staged) {
     const WalkMesh& m = of.m;
     const int ns = row_slots(r);
     const int32_t self = (int32_t)min(i, m.n - 1);
@@ -524,15 +530,19 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
     };
     // (all columns first: the records' loads keep their place among each other)
     int32_t k[UT];
+    auto columns = [&](const int32_t* col) {
 #pragma unroll
-    for (int c = 0; c < UT; ++c) {
-      const int s = s0 + c * H;
-      k[c] = s < ns ? col[slot_pos(s, r.dp)] : self;  // (past the row: its own, unused)
-      if (DEBUG && (k[c] < 0 || k[c] >= m.n)) {
-        atomicOr(m.err, ERR_BAD_INDEX);
-        k[c] = self;
+      for (int c = 0; c < UT; ++c) {
+        const int s = s0 + c * H;
+        k[c] = s < ns ? col[slot_pos(s, r.dp)] : self;  // (past the row: its own, unused)
+        if (DEBUG && (k[c] < 0 || k[c] >= m.n)) {
+          atomicOr(m.err, ERR_BAD_INDEX);
+          k[c] = self;
+        }
       }
-    }
+    };
+    if (staged && (!LONG || c1 - c0 <= lay.L)) columns(reinterpret_cast<const int32_t*>(smem + lay.cols) + (r.rs - c0));
+    else columns(m.col_idx + r.rs);
     if (s0 == h) load(v.me, self);
 #pragma unroll
     for (int c = 0; c < UT; ++c) load(v.r[c], k[c]);
@@ -547,7 +557,7 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
     const int ns = DEBUG ? min(row_slots(r), lay.W) : row_slots(r);
 #pragma unroll 1
     for (int s0 = h; s0 < ns; s0 += UT * H) {
-      if (s0 != h) load_recs(v, of, r, of.m.col_idx + r.rs, i, s0);
+      if (s0 != h) load_recs(v, of, r, 0, 0, i, s0, false);
 #pragma unroll
       for (int c = 0; c < UT; ++c) {
         if (s0 + c * H >= ns) break;
@@ -567,12 +577,6 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
         *reinterpret_cast<float4*>(smem + lay.acc + b) = make_float4(0.f, 0.f, 0.f, 0.f);
     __syncwarp();
   };
-  // a group's column indices in shared memory, or in memory where they do not fit (debug)
-  auto cols_of = [&](const WalkMesh& m, const GroupRow& r, int32_t c0, int32_t c1) {
-    return DEBUG && c1 - c0 > lay.L ? m.col_idx + r.rs
-                                    : reinterpret_cast<const int32_t*>(smem + lay.cols) + (r.rs - c0);
-  };
-
   // the first group
   int at = src.find(g);
   GroupRow row;
@@ -592,7 +596,7 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
     __syncwarp();
     Recs v;
     if constexpr (!DIRECT) wait_for_previous();
-    load_recs(v, src.item(at), row, cols_of(m, row, base, end), r0 + t, h);
+    load_recs(v, src.item(at), row, base, end, r0 + t, h, true);
     __syncwarp();
     put(v, src.item(at), row, r0 + t);
   }
@@ -603,10 +607,16 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
     const int64_t i = (int64_t)(g - src.item(at).group0) * RW + t;
     const bool valid = i < m.n;
     const int ns = row_slots(row);
-    const int L = end - base, lb = row.rs - base;
+    // The group's entries are staged as they lie in memory; where a long row
+    // (hundreds of entries, which rows64_kernel computes) makes them more than
+    // the staging holds, every other row in a place of its own.  gb: the row's
+    // first entry in the group's slice, lb: in the staging.
+    const bool dense = !LONG || end - base <= lay.L;  // warp-uniform
+    const int Ld = dense ? end - base : 0, gb = row.rs - base;
+    const int lb = dense ? gb : t * (lay.W + 1);
     bool fits = true;
     if (DEBUG) {
-      fits = L <= lay.L && we - wb <= lay.S && !__any_sync(FULL, ns > lay.W || (ns > 0 && row.dp > ns));
+      fits = we - wb <= lay.S && !__any_sync(FULL, ns > lay.W || (ns > 0 && row.dp > ns));
       if (!fits && lane == 0) atomicOr(m.err, ERR_STAR);
     }
     const T kmass = kmass_of<T>(f);
@@ -667,8 +677,8 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
       const Out* As = static_cast<const Out*>(o.A_static) + base;
 #pragma unroll
       for (int c = 0; c < NS; ++c)
-        if (lane + 32 * c < L) as[c] = As[lane + 32 * c];
-      if (h == 0 && ns > 0) sd = As[lb + row.dp];
+        if (lane + 32 * c < Ld) as[c] = As[lane + 32 * c];
+      if (h == 0 && ns > 0) sd = As[gb + row.dp];
     }
 #pragma unroll
     for (int off = RW; off < 32; off <<= 1) merge_lanes<P>(detsum, off);
@@ -683,7 +693,7 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
     [[maybe_unused]] float dlo = 0.f;  // mixed64: the error term of the diagonal's leading part dhi
     [[maybe_unused]] float dhi = 0.f;
     const int len = !fits || row.dp == DIAG_LONG ? 0 : row.re - row.rs;
-    const int zl = fits && row.dp == DIAG_LONG ? row.re - row.rs : 0;  // a long row's entries
+    const int zl = fits && dense && row.dp == DIAG_LONG ? row.re - row.rs : 0;  // a long row's entries in the staging
     if constexpr (MODE == ASSEMBLE) {
       using S = Slots<P, ASSEMBLE>;
       Acc<P> ra;
@@ -795,8 +805,7 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
     // the next group's records, in flight during the write-out
     Recs v{};
     if (more) {
-      load_recs(v, src.item(atn), rown, cols_of(src.item(atn).m, rown, basen, endn),
-                (int64_t)(gn - src.item(atn).group0) * RW + t, h);
+      load_recs(v, src.item(atn), rown, basen, endn, (int64_t)(gn - src.item(atn).group0) * RW + t, h, true);
     }
 
     // 3. the group's contiguous slice of the outputs
@@ -809,7 +818,12 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
       // 271 against 279 us at 100^3 in random order; mixed32 236 against 226)
       auto write = [&](auto&& put) {
 #pragma unroll 1
-        for (int k = lane; k < (fits ? L : 0); k += 32) put(k, stage[k]);
+        for (int r = 0; r < (dense ? 1 : RW); ++r) {
+          int n = fits ? Ld : 0, to = 0, from = 0;
+          if (!dense) n = __shfl_sync(FULL, len, r), to = __shfl_sync(FULL, gb, r), from = r * (lay.W + 1);
+#pragma unroll 1
+          for (int k = lane; k < n; k += 32) put(to + k, stage[from + k]);
+        }
       };
       if constexpr (P == NSI_MIXED_F32_ACC64) {
         // converted to double exactly, A by the FP64 pipe's conversion and G from
@@ -824,7 +838,7 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
         });
         __syncwarp();
         if (fits && h == 0 && len > 0)
-          A[lb + row.dp] = nonfinite_bits(dhi) ? nonfinite_double(dhi) : pair_double(dhi, dlo);
+          A[gb + row.dp] = nonfinite_bits(dhi) ? nonfinite_double(dhi) : pair_double(dhi, dlo);
       } else {
         write([&](int k, const T4<T>& v) {
           A[k] = v.x;
@@ -843,13 +857,20 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
       if (fits) {
 #pragma unroll
         for (int c = 0; c < NS; ++c)
-          if (lane + 32 * c < L) A[lane + 32 * c] = as[c] + value(lane + 32 * c);
-        for (int k = lane + 32 * NS; k < L; k += 32) A[k] = As[k] + value(k);
+          if (lane + 32 * c < Ld) A[lane + 32 * c] = as[c] + value(lane + 32 * c);
+        for (int k = lane + 32 * NS; k < Ld; k += 32) A[k] = As[k] + value(k);
+      }
+      if (fits && !dense) {  // (a row has no more entries than the warp has lanes)
+#pragma unroll 1
+        for (int r = 0; r < RW; ++r) {
+          const int n = __shfl_sync(FULL, len, r), k = __shfl_sync(FULL, gb, r) + lane;
+          if (lane < n) A[k] = As[k] + value(r * (lay.W + 1) + lane);
+        }
       }
       if constexpr (P == NSI_MIXED_F32_ACC64) {  // the diagonal's sum is a compensated pair
         __syncwarp();
         if (fits && h == 0 && ns > 0)
-          A[lb + row.dp] = sd + (nonfinite_bits(dhi) ? nonfinite_double(dhi) : pair_double(dhi, dlo));
+          A[gb + row.dp] = sd + (nonfinite_bits(dhi) ? nonfinite_double(dhi) : pair_double(dhi, dlo));
       }
     }
     if (!more) return;
@@ -875,13 +896,13 @@ struct OneMesh {
   __device__ __forceinline__ const WalkItem<MODE>& item(int) const { return one; }
 };
 
-template <int P, int H, int MODE, bool DEBUG>
+template <int P, int H, int MODE, bool DEBUG, bool LONG>
 __global__ void __launch_bounds__(32 * MAX_WARPS, P == NSI_FP64 ? 2 : 4)
     gather_persistent_kernel(const __grid_constant__ WalkItem<MODE> item, GroupLay lay, int g0, int g_end) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int warps = blockDim.x >> 5, w = threadIdx.x >> 5;
-  group_loop<P, H, MODE, DEBUG, H == 4>(OneMesh<MODE>{item}, g0 + (int)blockIdx.x * warps + w, (int)gridDim.x * warps, g_end,
-                                smem_raw + w * lay.total, lay);
+  group_loop<P, H, MODE, DEBUG, H == 4, LONG>(OneMesh<MODE>{item}, g0 + (int)blockIdx.x * warps + w,
+                                              (int)gridDim.x * warps, g_end, smem_raw + w * lay.total, lay);
 }
 
 // ------------------------------------------------ badly shaped elements ---
@@ -1035,7 +1056,7 @@ struct BatchMesh {
   __device__ __forceinline__ const WalkItem<ASSEMBLE>& item(int k) const { return args.item[k]; }
 };
 
-template <int P>
+template <int P, bool LONG>
 __global__ void __launch_bounds__(32 * MAX_WARPS, P == NSI_FP64 ? 2 : 4)
     batched_kernel(const __grid_constant__ BatchArgs args, const __grid_constant__ BatchLays lays) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -1050,14 +1071,14 @@ __global__ void __launch_bounds__(32 * MAX_WARPS, P == NSI_FP64 ? 2 : 4)
     if (me < 0) me += all;
   };
   if constexpr (P == NSI_FP64) {
-    group_loop<P, 1, ASSEMBLE, false, false>(BatchMesh{args, 0, args.count[0]}, me, all, args.total[0], smem,
+    group_loop<P, 1, ASSEMBLE, false, false, LONG>(BatchMesh{args, 0, args.count[0]}, me, all, args.total[0], smem,
                                              lays.kind[0]);
     next(0);
   }
-  group_loop<P, 2, ASSEMBLE, false, false>(BatchMesh{args, args.count[0], args.count[1]}, me, all, args.total[1], smem,
+  group_loop<P, 2, ASSEMBLE, false, false, LONG>(BatchMesh{args, args.count[0], args.count[1]}, me, all, args.total[1], smem,
                                            lays.kind[1]);
   next(1);
-  group_loop<P, 4, ASSEMBLE, false, false>(BatchMesh{args, args.count[0] + args.count[1], args.count[2]}, me, all,
+  group_loop<P, 4, ASSEMBLE, false, false, LONG>(BatchMesh{args, args.count[0] + args.count[1], args.count[2]}, me, all,
                                            args.total[2], smem, lays.kind[2]);
 }
 
@@ -1138,11 +1159,11 @@ nsi_status resident_grid(K kernel, int warps, size_t smem, int64_t groups, std::
   return NSI_OK;
 }
 
-template <int P, int H, int MODE, bool DEBUG>
+template <int P, int H, int MODE, bool DEBUG, bool LONG>
 nsi_status run_groups(NsiHandle* h, const WalkItem<MODE>& item, int64_t row0, int64_t row1, cudaStream_t s) {
   static std::once_flag once;
   static cudaError_t err = cudaSuccess;
-  const auto kernel = gather_persistent_kernel<P, H, MODE, DEBUG>;
+  const auto kernel = gather_persistent_kernel<P, H, MODE, DEBUG, LONG>;
   nsi_status st = allow_smem(kernel, once, err);
   if (st) return st;
   constexpr int RW = 32 / H;
@@ -1161,20 +1182,21 @@ nsi_status run_groups(NsiHandle* h, const WalkItem<MODE>& item, int64_t row0, in
   return check_launch("gather_persistent_kernel");
 }
 
+template <int P, int H, int MODE>
+nsi_status run_rows(NsiHandle* h, const WalkItem<MODE>& item, int64_t row0, int64_t row1, cudaStream_t s) {
+  return h->debug             ? run_groups<P, H, MODE, true, true>(h, item, row0, row1, s)
+         : h->plan.long_group ? run_groups<P, H, MODE, false, true>(h, item, row0, row1, s)
+                              : run_groups<P, H, MODE, false, false>(h, item, row0, row1, s);
+}
+
 template <int P, int MODE>
 nsi_status run_lanes(NsiHandle* h, const WalkItem<MODE>& item, int64_t row0, int64_t row1, cudaStream_t s) {
   switch (h->nsub) {
     case 1:
-      if constexpr (P == NSI_FP64)
-        return h->debug ? run_groups<P, 1, MODE, true>(h, item, row0, row1, s)
-                        : run_groups<P, 1, MODE, false>(h, item, row0, row1, s);
+      if constexpr (P == NSI_FP64) return run_rows<P, 1, MODE>(h, item, row0, row1, s);
       return fail(NSI_ERR_UNSUPPORTED, "one lane per row in FP64 only");
-    case 2:
-      return h->debug ? run_groups<P, 2, MODE, true>(h, item, row0, row1, s)
-                      : run_groups<P, 2, MODE, false>(h, item, row0, row1, s);
-    default:
-      return h->debug ? run_groups<P, 4, MODE, true>(h, item, row0, row1, s)
-                      : run_groups<P, 4, MODE, false>(h, item, row0, row1, s);
+    case 2: return run_rows<P, 2, MODE>(h, item, row0, row1, s);
+    default: return run_rows<P, 4, MODE>(h, item, row0, row1, s);
   }
 }
 
@@ -1229,6 +1251,7 @@ nsi_status launch_batched(NsiHandle* const* hs, const NsiFields* fs, const NsiOu
   int64_t all = 0, pack_blocks = 0;
   size_t bytes = 0;
   BatchLays lays;
+  bool long_group = false;
   for (int kind = 0; kind < KINDS; ++kind) {
     const int H = kind_lanes(kind), rw = 32 / H;
     int W = 1, L = 0, S = 0;
@@ -1239,6 +1262,7 @@ nsi_status launch_batched(NsiHandle* const* hs, const NsiFields* fs, const NsiOu
       if (h->nsub != H) continue;
       const GatherPlan& pl = h->plan;
       warps = std::min(warps, pl.warps);
+      long_group |= pl.long_group;
       W = std::max(W, pl.w);
       L = std::max(L, pl.max_block_entries);
       S = std::max(S, pl.max_block_steps);
@@ -1261,15 +1285,16 @@ nsi_status launch_batched(NsiHandle* const* hs, const NsiFields* fs, const NsiOu
   while (warps > 1 && bytes * warps > SMEM_MAX) --warps;
   if (bytes > SMEM_MAX) return fail(NSI_ERR_UNSUPPORTED, "batched meshes need more shared memory than a block has");
   lays.stride = (int)bytes;
-  static std::once_flag once;
-  static cudaError_t err = cudaSuccess;
-  nsi_status st = allow_smem(batched_kernel<P>, once, err);
+  const auto kernel = long_group ? batched_kernel<P, true> : batched_kernel<P, false>;
+  static std::once_flag once[2];
+  static cudaError_t err[2] = {};
+  nsi_status st = allow_smem(kernel, once[long_group], err[long_group]);
   if (st) return st;
   batched_pack_kernel<P><<<pack_blocks, 128, 0, s>>>(args);
   if ((st = check_launch("batched_pack_kernel"))) return st;
   int64_t grid = 0;
-  if ((st = resident_grid(batched_kernel<P>, warps, bytes * warps, all, nullptr, &grid))) return st;
-  NSI_CUDA(launch_early(batched_kernel<P>, grid, 32 * warps, bytes * warps, s, args, lays));
+  if ((st = resident_grid(kernel, warps, bytes * warps, all, nullptr, &grid))) return st;
+  NSI_CUDA(launch_early(kernel, grid, 32 * warps, bytes * warps, s, args, lays));
   return check_launch("batched_kernel");
 }
 
@@ -1296,10 +1321,10 @@ NSI_INSTANTIATE(NSI_MIXED_F32_ACC32)
 int gather_kernel_regs(int precision) {
   cudaFuncAttributes a{};
   cudaError_t e;
-  if (precision == NSI_FP64) e = cudaFuncGetAttributes(&a, gather_persistent_kernel<NSI_FP64, 2, ASSEMBLE, false>);
+  if (precision == NSI_FP64) e = cudaFuncGetAttributes(&a, gather_persistent_kernel<NSI_FP64, 2, ASSEMBLE, false, false>);
   else if (precision == NSI_MIXED_F32_ACC64)
-    e = cudaFuncGetAttributes(&a, gather_persistent_kernel<NSI_MIXED_F32_ACC64, 2, ASSEMBLE, false>);
-  else e = cudaFuncGetAttributes(&a, gather_persistent_kernel<NSI_MIXED_F32_ACC32, 2, ASSEMBLE, false>);
+    e = cudaFuncGetAttributes(&a, gather_persistent_kernel<NSI_MIXED_F32_ACC64, 2, ASSEMBLE, false, false>);
+  else e = cudaFuncGetAttributes(&a, gather_persistent_kernel<NSI_MIXED_F32_ACC32, 2, ASSEMBLE, false, false>);
   return e == cudaSuccess ? a.numRegs : 96;
 }
 

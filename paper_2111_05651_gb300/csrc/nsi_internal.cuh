@@ -82,10 +82,11 @@ struct alignas(32) D4 {
 struct GatherPlan {
   int rows_per_block = 0;     // the plan's name: 32, 64, 96 or 128
   int warps = 0;              // warps per block, each with row groups of its own
-  int max_block_entries = 0;  // max over the groups of the CSR entries of a group's rows
+  int max_block_entries = 0;  // CSR entries that a group's staging holds: w + 1 for each of its rows
   int max_block_steps = 0;    // max over the groups of the walk bytes of a group's rows
   int w = 0;                  // slots per row (>= the off-diagonal entries of the longest row the kernels
-                              // take, and large enough that every group's entries fit its staging)
+                              // take, and large enough for the staging)
+  bool long_group = false;    // a group has more entries, a long row's among them, than its staging holds
 };
 // a mesh of fewer rows has four lanes per row in the row gather, others two or one
 // (measured equal at about 30 000 rows for the assembly and at 10 000 for the
@@ -97,7 +98,8 @@ constexpr int SMEM_MAX = 200 * 1024;  // shared memory of one block
 
 // diag_pos value of a row the row gather leaves out ("long row": more than
 // 32 entries, or a star whose walk does not encode): the kernels give it no
-// elements and zero its slice; rows64_kernel computes it afterwards
+// elements and zero its slice, or leave it out where it is longer than their
+// staging; rows64_kernel computes it afterwards
 constexpr uint8_t DIAG_LONG = 0xff;
 
 // Shared-memory layout of one warp's group of the row gather: R rows, W slots

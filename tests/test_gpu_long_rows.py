@@ -97,3 +97,46 @@ def test_long_rows_batched_noalloc_host(hub, precision):
         assert torch.equal(x, y.cpu())
     for a in asms:
         a.close()
+
+
+# one row of hundreds of entries more than a group's staging: FP64 and mixed
+# below 10,000 rows (four lanes per row) and above (two), with the groups' other
+# rows in places of their own
+@pytest.mark.parametrize("m,k,precision", [(8, 1900, "fp64"), (8, 4300, "mixed64"), (8, 4300, "mixed32"),
+                                           (21, 2900, "fp64"), (21, 4300, "mixed64")])
+def test_row_longer_than_the_staging(m, k, precision):
+    mesh, u = meshgen.delaunay_hub(m=m, k=k, seed=8)
+    asm = nsi.Assembler(mesh.coord, mesh.lnods, precision=precision)
+    assert asm.max_row > k and asm.info().long_rows >= 1 and asm.scatter == nsi.SCATTERS["gather"]
+    assert (mesh.n_nodes < 10000) == (m == 8)
+    ut = torch.as_tensor(u.T.copy())
+    uo = _oracle_u(u, precision)
+    rp, _, oA, oG, orhs = oracle.assemble(mesh.coord, mesh.lnods, uo, None, RHO, MU, DT)
+    out = asm.empty_outputs()
+    for t in out:
+        t.fill_(float("nan"))
+    A, G, rhs = (x.double().cpu().numpy() for x in asm.assemble(ut, out=out))
+    assert max(errors(rp, A, G, rhs, oA, oG, orhs).values()) <= TOL[precision]
+    A_static, _ = asm.static_part()
+    A2, rhs2 = asm.assemble_convective(ut, A_static)
+    assert max(errors(rp, A2.double().cpu().numpy(), oG, rhs2.double().cpu().numpy(), oA, oG,
+                      orhs).values()) <= TOL[precision]
+    asm.assemble_convective(ut, A_static, out=(A_static, rhs2))  # in place
+    assert torch.equal(A_static, A2)
+    onr, ondt, onm = oracle.nodal(mesh.coord, mesh.lnods, uo, RHO, DT)
+    r3, dtr, mr = (x.double().cpu().numpy() for x in asm.nodal(ut))
+    assert max([vec_scaled_err(dtr, ondt), vec_scaled_err(mr, onm)] +
+               [vec_scaled_err(r3[d], onr[d]) for d in range(3)]) <= TOL[precision]
+    cube, uc = meshgen.config_mesh(N=6, jitter=0.15, numbering="random", seed=93)
+    other = nsi.Assembler(cube.coord, cube.lnods, precision=precision)
+    for x, y in zip(out, nsi.assemble_batched([other, asm], [torch.as_tensor(uc.T.copy()), ut])[1]):
+        assert torch.equal(x, y)
+    debug = nsi.Assembler(mesh.coord, mesh.lnods, precision=precision, debug_checks=True)
+    for x, y in zip(out, debug.assemble(ut)):
+        assert torch.equal(x, y)
+    debug.device_status()
+    if k == 1900:
+        _, _, oAuu, oG2, orhs2 = oracle.assemble_stabilized(mesh.coord, mesh.lnods, uo, None, RHO, MU, DT)
+        Auu, G2, rhs2 = (x.double().cpu().numpy() for x in asm.assemble_stabilized(ut))
+        for c in range(9):
+            assert max(errors(rp, Auu[c], G2, rhs2, oAuu[c], oG2, orhs2).values()) <= TOL[precision]
