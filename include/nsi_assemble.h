@@ -179,7 +179,7 @@ typedef struct {
     int32_t rows_per_block; /* row-gather launch shape in use: 32, 64, 96 or 128 for the per-row
                                star kernel (its warps per block: that many rows' worth, at most
                                four), -1 for the edge-fan kernel, 0 if unavailable */
-    int32_t n_plans;        /* row-gather launch shapes available */
+    int32_t n_plans;        /* distinct row-gather launch shapes available */
     int32_t persistent;     /* 1: the row gather runs as a persistent grid of warps (a warp's next
                                group of rows is fetched while the current one is merged and
                                written out), 0: the edge-fan kernel, one CTA per block of rows */

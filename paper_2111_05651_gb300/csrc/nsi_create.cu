@@ -699,6 +699,7 @@ static nsi_status build(NsiHandle* h, const NsiMesh* m, cudaStream_t s) {
       if (!h->gather_ok || g.total() > (size_t)SMEM_MAX) break;
       int warps = std::min(R / RW, 4);
       while (g.total() * warps > (size_t)SMEM_MAX) --warps;
+      if (h->n_plans && warps <= h->plans[h->n_plans - 1].warps) continue;  // the launch of the name before
       const int blocks = (int)std::min<size_t>({smem_sm / (g.total() * warps + 1024), (size_t)32,
                                                 (size_t)(65536 / (32 * warps * regs))});
       GatherPlan cand;
@@ -979,10 +980,12 @@ nsi_status nsi_set_launch(NsiHandle* h, int32_t scatter, int32_t rows_per_block)
     if (!h->fan_ok) return fail(NSI_ERR_UNSUPPORTED, "no edge-fan map for this mesh");
     h->use_fan = true;
   } else if (rows_per_block != 0) {
-    int k = 0;
-    while (k < h->n_plans && h->plans[k].rows_per_block != rows_per_block) ++k;
-    if (k == h->n_plans) return fail(NSI_ERR_UNSUPPORTED, "no launch plan with that many rows per block");
+    if (h->n_plans == 0 || rows_per_block < 32 || rows_per_block > 128 || rows_per_block % 32)
+      return fail(NSI_ERR_UNSUPPORTED, "no launch plan with that many rows per block");
+    int k = h->n_plans - 1;  // a name without a plan of its own is the launch of the name before
+    while (h->plans[k].rows_per_block > rows_per_block) --k;
     h->plan = h->plans[k];
+    h->plan.rows_per_block = rows_per_block;
     h->use_fan = false;
   }
   if (scatter != NSI_SCATTER_AUTO) h->scatter = scatter;

@@ -226,7 +226,7 @@ struct NsiHandle {
   int4* star_task = nullptr;      // [2 n_star_tasks]
   int64_t n_star_tasks = 0;
   nsi::GatherPlan plan;         // the launch plan in use
-  nsi::GatherPlan plans[4];     // every rows-per-block candidate that fits shared memory
+  nsi::GatherPlan plans[4];     // the distinct launches (warps per block, ascending), by the first name of each
   int n_plans = 0;
   std::atomic<int> resident[3][4] = {};  // row gather by mode and warps per block: blocks resident at once (0: not known)
   // coordinates: double4 for FP64, float4 hi + float4 lo for the mixed modes

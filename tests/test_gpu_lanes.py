@@ -94,3 +94,22 @@ def test_row_of_more_entries_than_a_block_has_threads(precision):
     A2, rhs2 = asm.assemble_convective(ut, A_static, rho=1.0, mu=1e-3, dt=1e-2)
     got = [A2.double().cpu().numpy(), oG, rhs2.double().cpu().numpy()]
     assert max(errors(rp, *got, oA, oG, orhs).values()) <= TOL[precision]
+
+
+@pytest.mark.parametrize("precision,N,shapes", [("mixed64", 6, 1), ("mixed64", 22, 2), ("fp64", 6, 1), ("fp64", 49, 4)])
+def test_launch_shapes_are_distinct(precision, N, shapes):
+    """Four lanes per row fill a block of four warps by every name, two have two
+    launches, one lane four; a name that repeats a launch is still accepted."""
+    mesh, u = meshgen.config_mesh(N=N, jitter=0.15, numbering="natural", seed=340 + N)
+    asm = nsi.Assembler(mesh.coord, mesh.lnods, precision=precision)
+    assert asm.info().n_plans == shapes
+    ut = torch.as_tensor(u.T.copy())
+    ref = [t.clone() for t in asm.assemble(ut)]
+    for rows in (128, 32, 96, 64):
+        nsi.nsi_set_launch(asm.handle, nsi.NSI_SCATTER_GATHER, rows)
+        assert asm.info().rows_per_block == rows
+        for x, y in zip(ref, asm.assemble(ut)):
+            assert torch.equal(x, y)
+    for rows in (16, 48, 160):
+        with pytest.raises(RuntimeError):
+            nsi.nsi_set_launch(asm.handle, nsi.NSI_SCATTER_GATHER, rows)
