@@ -828,6 +828,12 @@ struct StarSmem {
   static constexpr size_t bytes() { return mask() + sizeof(unsigned) * 6 * 32; }
 };
 constexpr int STAR_WARPS = 4;  // warps (tasks) per block
+// sum of x[0], x[ST], ..., x[(N - 1) ST] in pairs, neighbours first
+template <int N, int ST, typename T>
+__device__ __forceinline__ T pair_sum(const T* x) {
+  if constexpr (N == 1) return x[0];
+  else return pair_sum<N / 2, ST>(x) + pair_sum<N / 2, ST>(x + N / 2 * ST);
+}
 
 // The stabilised block by rows, one warp per task (one row of up to 32
 // entries, or two consecutive rows of up to 16 on the two half-warps).
@@ -1035,7 +1041,9 @@ __global__ void __launch_bounds__(32 * STAR_WARPS, P == NSI_FP64 ? 1 : 6) stab_s
   // 4. row totals: every lane's sums (a lane without an off-diagonal entry has
   // zeros) to shared memory (the element records' space, free now), where the
   // row's lanes 0-13 each add one value up over the row's entries (mixed64:
-  // compensated); A's and det's go to all of the row's lanes
+  // compensated; else in pairs, neighbours first: one after the other the
+  // diagonal's rounding in mixed32 is a sixth larger); A's and det's go to all of the row's
+  // lanes
   constexpr int NV = 14, ST = 15;  // K, G, A + S, det; an odd stride: no bank conflicts
   T* red = reinterpret_cast<T*>(el);
 #pragma unroll
@@ -1050,8 +1058,15 @@ __global__ void __launch_bounds__(32 * STAR_WARPS, P == NSI_FP64 ? 1 : 6) stab_s
   __syncwarp();
   Acc<P> tot;
   tot.zero();
-  if (q < NV)
-    for (int r = 0; r < width; ++r) tot.add(red[(seg * width + r) * ST + q]);
+  if (q < NV) {
+    const T* x = red + seg * width * ST + q;
+    if constexpr (P == NSI_MIXED_F32_ACC64) {
+      for (int r = 0; r < width; ++r) tot.add(x[r * ST]);
+    } else {
+      tot.v = pair_sum<16, ST>(x);
+      if (width == 32) tot.v += pair_sum<16, ST>(x + 16 * ST);
+    }
+  }
   auto from = [&](int l) {
     Acc<P> a;
     if constexpr (P == NSI_MIXED_F32_ACC64) {

@@ -222,3 +222,19 @@ def test_stabilized_repeated_elements(precision):
     for d in range(3):
         assert row_scaled_err(rp, G[d].double().cpu().numpy(), oG[d]) <= TOL[precision]
         assert vec_scaled_err(rhs[d].double().cpu().numpy(), orhs[d]) <= TOL[precision]
+
+
+@pytest.mark.parametrize("N,seed,mu,bound", [(14, 61, 1e-3, 6.2e-8), (20, 63, 1e-4, 5.9e-8)])
+def test_mixed32_diagonal_sums_in_pairs(N, seed, mu, bound):
+    """rms error of the diagonal blocks' diagonal in mixed32, whose row totals are
+    float sums of up to 14 entries: in pairs 5.7e-8 and 5.5e-8, one entry after
+    the other 6.9e-8 and 6.4e-8 (the kernel's order is fixed, so are these); the
+    bound lies between."""
+    mesh, u = meshgen.config_mesh(N=N, jitter=0.15, numbering="random", seed=seed)
+    asm = nsi.Assembler(mesh.coord, mesh.lnods, precision="mixed32")
+    rp, ci, oAuu, _, _ = oracle.assemble_stabilized(mesh.coord, mesh.lnods, u.astype(np.float32).astype(np.float64),
+                                                    None, 1.0, mu, 1e-2)
+    Auu = asm.assemble_stabilized(torch.as_tensor(u.T.copy()), rho=1.0, mu=mu, dt=1e-2)[0].double().cpu().numpy()
+    diag = np.repeat(np.arange(mesh.n_nodes), np.diff(rp)) == ci
+    got, ref = (x[[0, 4, 8]][:, diag] for x in (Auu, oAuu))
+    assert np.linalg.norm(got - ref) <= bound * np.linalg.norm(ref)
