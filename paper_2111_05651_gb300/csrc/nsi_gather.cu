@@ -246,8 +246,10 @@ struct Slots<P, NODAL> {
 // Jacobian, calculate_cartesian_derivatives, for the order (p, q, c)),
 // det = d_p . c_p and c_i = -(c_p + c_q + c_c), the element adds
 //   A(i,x) += w . c_x  (x = p, q, c),  w = rho/120 (2 u_i + u_p + u_q + u_c) + mu/(6 det) c_i
-// (the staged velocities carry the factor rho/120, p's also the 2 u_i; the time
-// step has no viscous part),
+// (p's velocity carries the 2 u_i; in FP64 the staged velocities carry the
+// factor rho/120 too, which saves its products on the FP64 pipe; in float, where
+// a product per velocity would add its rounding to every term, it is taken in
+// the step; the time step has no viscous part),
 // -c_i / 24 (= -|T| grad N_i / 4, the element's G(i, x)) to the three
 // pressure-gradient sums and det to the lumped mass sum (scaled after the
 // walk).  For the order (p, q, c) an odd permutation of the element's own, det
@@ -266,7 +268,7 @@ template <int P, int RW, int MODE>
 __device__ __forceinline__ void walk_lane(const uint8_t* __restrict__ st, int nbytes,
                                           const T4<typename Prec<P>::T>* nb0, const T2<typename Prec<P>::T>* nb1,
                                           Slots<P, MODE>& acc, const V3<typename Prec<P>::T>& u2i,
-                                          typename Prec<P>::T kmu, Acc<P>& detsum) {
+                                          typename Prec<P>::T kc, typename Prec<P>::T kmu, Acc<P>& detsum) {
   using T = typename Prec<P>::T;
   using Node = WalkNode<P, MODE>;
   constexpr T kg = T(-1.0 / 24.0);  // the pressure-gradient sums are accumulated scaled
@@ -322,7 +324,10 @@ __device__ __forceinline__ void walk_lane(const uint8_t* __restrict__ st, int nb
             ci = V3<T>{M.x - (cp.x + cq.x), M.y - (cp.y + cq.y), M.z - (cp.z + cq.z)};
           }
           const T kv = mul_rn(kmu, rcp_fast(det));
-          w3 = V3<T>{fma(kv, ci.x, w3.x), fma(kv, ci.y, w3.y), fma(kv, ci.z, w3.z)};
+          if constexpr (P == NSI_FP64)
+            w3 = V3<T>{fma(kv, ci.x, w3.x), fma(kv, ci.y, w3.y), fma(kv, ci.z, w3.z)};
+          else
+            w3 = V3<T>{fma(kc, w3.x, mul_rn(kv, ci.x)), fma(kc, w3.y, mul_rn(kv, ci.y)), fma(kc, w3.z, mul_rn(kv, ci.z))};
           const T fg = neg ? -kg : kg;
           const T ap = dot_fma(w3, cp), aq = dot_fma(w3, cq), ac = dot_fma(w3, M);
           if constexpr (P == NSI_FP64) {
@@ -346,9 +351,10 @@ __device__ __forceinline__ void walk_lane(const uint8_t* __restrict__ st, int nb
             upd(c.a, -f, ac);
           }
         } else {
-          p.a = fma(f, dot_fma(w3, cp), p.a);
-          q.a = fma(f, dot_fma(w3, cq), q.a);
-          c.a = fma(neg != flip ? T(1) : T(-1), dot_fma(w3, M), c.a);
+          const T one = P == NSI_FP64 ? T(1) : kc, fk = neg ? -one : one;
+          p.a = fma(fk, dot_fma(w3, cp), p.a);
+          q.a = fma(fk, dot_fma(w3, cq), q.a);
+          c.a = fma(neg != flip ? one : -one, dot_fma(w3, M), c.a);
         }
         if constexpr (P == NSI_FP64) {  // (a negated double is an operation of the FP64 pipe, its bound)
           M = V3<T>{evq ? cq.x : cp.x, evq ? cq.y : cp.y, evq ? cq.z : cp.z};
@@ -548,12 +554,16 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
     for (int c = 0; c < UT; ++c) load(v.r[c], k[c]);
   };
   // the group's slots: edge vectors from the row's node, velocities, zeroed
-  // sums; 2 rho/120 u_i of the row's own node
+  // sums; 2 u_i of the row's own node (FP64: all velocities times rho/120)
   V3<T> u2i;
   auto put = [&](Recs& v, const WalkItem<MODE>& of, const GroupRow& r, int64_t i) {
-    const T kc = kc_of<T>(of.f), kc2 = kc + kc;
-    const V3<T> ui = v.me.vel();
-    u2i = V3<T>{mul_rn(kc2, ui.x), mul_rn(kc2, ui.y), mul_rn(kc2, ui.z)};
+    const T kc = kc_of<T>(of.f);
+    auto scale = [&](const V3<T>& u) {
+      if constexpr (P == NSI_FP64) return V3<T>{mul_rn(kc, u.x), mul_rn(kc, u.y), mul_rn(kc, u.z)};
+      else return u;
+    };
+    const V3<T> ui = scale(v.me.vel());
+    u2i = add(ui, ui);
     const int ns = DEBUG ? min(row_slots(r), lay.W) : row_slots(r);
 #pragma unroll 1
     for (int s0 = h; s0 < ns; s0 += UT * H) {
@@ -566,9 +576,9 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
         if constexpr (MODE == NODAL) {
           nb0()[k] = T4<T>{d.x, d.y, d.z, T(0)};
         } else {
-          const V3<T> u = v.r[c].vel();
-          nb0()[k] = T4<T>{d.x, d.y, d.z, mul_rn(kc, u.x)};
-          nb1()[k] = T2<T>{mul_rn(kc, u.y), mul_rn(kc, u.z)};
+          const V3<T> u = scale(v.r[c].vel());
+          nb0()[k] = T4<T>{d.x, d.y, d.z, u.x};
+          nb1()[k] = T2<T>{u.y, u.z};
         }
       }
     }
@@ -648,7 +658,7 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
         // (each lane finds its bytes first: the row's lanes walk together)
         int b = H;
         for (int k = 0; k < h; ++k) b += st[k];
-        walk_lane<P, RW, MODE>(st + b, st[h], nb0(), nb1(), acc, u2i, kmu_of<T>(f), detsum);
+        walk_lane<P, RW, MODE>(st + b, st[h], nb0(), nb1(), acc, u2i, kc_of<T>(f), kmu_of<T>(f), detsum);
       }
     }
     __syncwarp();
@@ -987,7 +997,7 @@ __global__ void __launch_bounds__(32) exact_rows_kernel(WalkMesh m, FieldView f,
       acc.a0 += t;
       acc.a1 += t;
     }
-    walk_lane<NSI_FP64, RW, WMODE>(st + b, st[h], nb0, nb1, acc, u2i, f.kmu, det);
+    walk_lane<NSI_FP64, RW, WMODE>(st + b, st[h], nb0, nb1, acc, u2i, f.kc, f.kmu, det);
   }
   __syncwarp();
   wait_for_previous();  // (the rows' first values come from an earlier launch)

@@ -137,3 +137,10 @@ def test_row_sums_of_opposite_slots():
     2.45e-7 and 3.09e-7; the bounds are the last's."""
     g, c, _ = _errors_natural("mixed32", "natural", 1e-3)
     assert g <= 2.45e-7 and c <= 3.09e-7
+
+
+def test_velocities_are_not_rounded_before_the_sum():
+    """A's off-diagonal entries where convection leads: 8.44e-8, with every
+    staged velocity multiplied by rho/120 first 8.57e-8; the bound is what the
+    product in the element's step gave with one lane per row."""
+    assert _errors_natural("mixed64", "random", 1e-4)[2] <= 8.51e-8
