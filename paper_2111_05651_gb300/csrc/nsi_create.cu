@@ -684,16 +684,10 @@ static nsi_status build(NsiHandle* h, const NsiMesh* m, cudaStream_t s) {
         mL = std::max<int64_t>(mL, rp64[r1] - rp64[r0]);
         mS = std::max<int64_t>(mS, walk_ptr[r1] - walk_ptr[r0]);
       }
-    // slots per row: the longest row the kernel takes, or more where the
-    // staging would not fit the bytes of nb0 and nb1; entries of long rows
-    // beyond the staging are left out (rows64_kernel computes them)
-    int W = (int)slots;
-    GatherSmem g = gather_smem(h->precision, RW, W, RW * (W + 1), (int)mS);
-    g.H = h->nsub;
-    while (!g.group_fits()) {
-      g.W = ++W;
-      g.L = RW * (W + 1);
-    }
+    // entries of long rows beyond the staging are left out (rows64_kernel
+    // computes them)
+    const int W = group_slots(h->precision, h->nsub, (int)slots);
+    const GatherSmem g = gather_smem(h->precision, ASSEMBLE, h->nsub, W, (int)mS);
     int chosen = -1, best_warps = 0;
     for (int R : {32, 64, 96, 128}) {
       if (!h->gather_ok || g.total() > (size_t)SMEM_MAX) break;
@@ -705,7 +699,6 @@ static nsi_status build(NsiHandle* h, const NsiMesh* m, cudaStream_t s) {
       GatherPlan cand;
       cand.rows_per_block = R;
       cand.warps = warps;
-      cand.max_block_entries = g.L;
       cand.long_group = mL > g.L;
       cand.max_block_steps = (int)mS;
       cand.w = W;

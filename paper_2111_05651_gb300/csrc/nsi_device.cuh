@@ -13,13 +13,11 @@ struct MeshView {
   const int32_t* __restrict__ row_ptr;
   const int32_t* __restrict__ col_idx;
   const int4* __restrict__ lnods;
-  const int32_t* __restrict__ walk_ptr;
-  const uint8_t* __restrict__ walk;
   const uint8_t* __restrict__ diag_pos;
   const D4* __restrict__ xyz64;
   const float4* __restrict__ xyz_hi;
   const float4* __restrict__ xyz_lo;
-  const void* __restrict__ rec;
+  const void* rec;  // (written by the packing, which an early launch may overlap)
   const uint32_t* __restrict__ fan;
   const int32_t* __restrict__ fan_blk;
   unsigned* err;
@@ -77,8 +75,6 @@ inline MeshView view_of(const NsiHandle* h) {
   m.row_ptr = h->row_ptr;
   m.col_idx = h->col_idx;
   m.lnods = h->lnods;
-  m.walk_ptr = h->walk_ptr;
-  m.walk = h->walk;
   m.diag_pos = h->diag_pos;
   m.xyz64 = h->xyz64;
   m.xyz_hi = h->xyz_hi;

@@ -47,7 +47,6 @@ namespace nsi {
 
 namespace {
 
-enum { ASSEMBLE = 0, STEP = 1, NODAL = 2 };
 constexpr int MAX_WARPS = 4;  // warps per block
 
 // --------------------------------------------------------------- copies ---
@@ -1152,15 +1151,6 @@ WalkMesh walk_mesh(const NsiHandle* h, void* rec) {
   return m;
 }
 
-// the shared memory of one warp's group of 32 / H rows
-GatherSmem group_smem(int precision, int mode, int H, int W, int L, int S) {
-  GatherSmem g = gather_smem(precision, 32 / H, W, L, S, mode != ASSEMBLE);
-  g.H = H;
-  g.xs = 0;  // A_static is read in the write-out
-  if (mode != ASSEMBLE) g.ab = mode == STEP ? g.tb : 0;
-  return g;
-}
-
 template <typename K>
 nsi_status allow_smem(K kernel, std::once_flag& once, cudaError_t& err) {
   std::call_once(once, [&] { err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX); });
@@ -1194,7 +1184,7 @@ nsi_status run_groups(NsiHandle* h, const WalkItem<MODE>& item, int64_t row0, in
   if (st) return st;
   constexpr int RW = 32 / H;
   const GatherPlan& pl = h->plan;
-  const GatherSmem lay = group_smem(P, MODE, H, pl.w, pl.max_block_entries, pl.max_block_steps);
+  const GatherSmem lay = gather_smem(P, MODE, H, pl.w, pl.max_block_steps);
   const size_t smem = lay.total() * pl.warps;
   const int64_t g0 = row0 / RW, g1 = (row1 + RW - 1) / RW;
   int64_t grid = 0;
@@ -1236,7 +1226,7 @@ nsi_status exact_rows_h(NsiHandle* h, const FieldView& f, int mode, const RowOut
   nsi_status st = allow_smem(kernel, once[mode], err[mode]);
   if (st) return st;
   const int64_t warps = (h->exact_rows * H + 31) / 32;
-  const GatherSmem lay = group_smem(NSI_FP64, mode == 0 ? ASSEMBLE : NODAL, H, h->exact_slots, 0, 0);
+  const GatherSmem lay = gather_smem(NSI_FP64, mode == 0 ? ASSEMBLE : NODAL, H, h->exact_slots, 0);
   NSI_CUDA(launch_early(kernel, warps, 32, lay.total(), s, walk_mesh(h, nullptr), f, o, GroupLay(lay),
                         (const int32_t*)h->exact_list, h->exact_rows));
   return check_launch("exact_rows_kernel");
@@ -1280,7 +1270,7 @@ nsi_status launch_batched(NsiHandle* const* hs, const NsiFields* fs, const NsiOu
   bool long_group = false;
   for (int kind = 0; kind < KINDS; ++kind) {
     const int H = kind_lanes(kind), rw = 32 / H;
-    int W = 1, L = 0, S = 0;
+    int W = group_slots(P, H, 1), S = 0;
     int64_t groups = 0;
     args.count[kind] = 0;
     for (int k = 0; k < count; ++k) {
@@ -1290,7 +1280,6 @@ nsi_status launch_batched(NsiHandle* const* hs, const NsiFields* fs, const NsiOu
       warps = std::min(warps, pl.warps);
       long_group |= pl.long_group;
       W = std::max(W, pl.w);
-      L = std::max(L, pl.max_block_entries);
       S = std::max(S, pl.max_block_steps);
       args.item[item++] = WalkItem<ASSEMBLE>{walk_mesh(h, nullptr), fields_of(&fs[k]),
                                              {os[k].A_val, os[k].G_val, os[k].rhs}, (int)groups};
@@ -1301,7 +1290,7 @@ nsi_status launch_batched(NsiHandle* const* hs, const NsiFields* fs, const NsiOu
     args.total[kind] = (int)groups;
     all += groups;
     pack_blocks += (groups + 4 * H - 1) / (4 * H);
-    const GatherSmem lay = group_smem(P, ASSEMBLE, H, W, L, S);
+    const GatherSmem lay = gather_smem(P, ASSEMBLE, H, W, S);
     if (!lay.group_fits())  // (each mesh's fits, and so do the maxima of W and L)
       return fail(NSI_ERR_UNSUPPORTED, "batched meshes need more shared memory than a group has");
     if (args.count[kind]) bytes = std::max(bytes, lay.total());

@@ -82,7 +82,6 @@ struct alignas(32) D4 {
 struct GatherPlan {
   int rows_per_block = 0;     // the plan's name: 32, 64, 96 or 128
   int warps = 0;              // warps per block, each with row groups of its own
-  int max_block_entries = 0;  // CSR entries that a group's staging holds: w + 1 for each of its rows
   int max_block_steps = 0;    // max over the groups of the walk bytes of a group's rows
   int w = 0;                  // slots per row (>= the off-diagonal entries of the longest row the kernels
                               // take, and large enough for the staging)
@@ -102,65 +101,60 @@ constexpr int SMEM_MAX = 200 * 1024;  // shared memory of one block
 // staging; rows64_kernel computes it afterwards
 constexpr uint8_t DIAG_LONG = 0xff;
 
+// What a launch of the row gather computes: the assembly, the time step with
+// cached geometry, the nodal outputs.
+enum { ASSEMBLE = 0, STEP = 1, NODAL = 2 };
+
 // Shared-memory layout of one warp's group of the row gather: R rows, W slots
 // per row (the off-diagonal entries of the longest row of the mesh), H lanes
-// per row, L CSR entries and S walk bytes.  Slot q of row t lives at index
-// q * R + t ("row-interleaved"), so the lanes of a warp touch consecutive
+// per row, L entries of staging and S walk bytes.  Slot q of row t lives at
+// index q * R + t ("row-interleaved"), so the lanes of a warp touch consecutive
 // records whichever slot each row uses: the element loop is free of
 // shared-memory bank conflicts.
 //   nb0   T[4] per slot: edge vector d = x_j - x_i and u_x of the neighbour
 //   nb1   T[2] per slot: u_y, u_z
 //   acc   H planes of accumulators per slot (ab bytes each): A and the three
-//         sums of c_i
+//         sums of c_i (time step: A; nodal outputs: none)
 //   walk  the walk bytes (copied as aligned 4-byte words, so S + 8 bytes)
-//   stat  (step layouts) the rows' slice of A_static
 //   info  the next group's row bounds and diagonal positions
 // After the element loop, nb0 and nb1 are reused to stage the finished values
-// in CSR order for the coalesced write-out (4 T per entry), and past them for
-// the next group's column indices.
+// for the coalesced write-out (4 T per entry, in CSR order, or row t's from
+// t * (W + 1) on), and past them for the next group's column indices.
 // Used identically by the host (launch size) and the kernel (carving).
 struct GatherSmem {
-  int R, W, L, S, tb, ab, ob, cr;  // ob: bytes of an output value; cr: components staged per write-out round
-  int xs;                          // bytes per CSR entry of the time step's static slice (0: none)
-  int H = 1;                       // accumulator planes
-  __host__ __device__ static size_t up16(size_t x) { return (x + 15) & ~size_t(15); }
-  __host__ __device__ size_t N() const { return (size_t)R * W; }
-  __host__ __device__ size_t nb0() const { return 0; }
-  __host__ __device__ size_t nb1() const { return up16(nb0() + (size_t)4 * tb * N()); }
-  __host__ __device__ size_t acc() const { return up16(nb1() + (size_t)2 * tb * N()); }
-  __host__ __device__ size_t col() const { return nb1(); }  // (L <= N: 4 L bytes fit in nb1)
-  __host__ __device__ size_t walk() const { return up16(acc() + (size_t)ab * H * N()); }
-  __host__ __device__ size_t stat() const { return up16(walk() + (size_t)S + 8); }
-  // the rows' bounds and diagonal positions
-  __host__ __device__ size_t info() const { return up16(stat() + (size_t)xs * L); }
+  int R, W, L, S, H, tb, ab;
+  static size_t up16(size_t x) { return (x + 15) & ~size_t(15); }
+  size_t N() const { return (size_t)R * W; }
+  size_t nb1() const { return up16((size_t)4 * tb * N()); }
+  size_t acc() const { return up16(nb1() + (size_t)2 * tb * N()); }
+  size_t plane() const { return (size_t)ab * N(); }
+  size_t walk() const { return up16(acc() + plane() * H); }
+  size_t info() const { return up16(walk() + (size_t)S + 8); }
   // (a multiple of 32: the next warp's nb0 holds 32-byte aligned FP64 vectors)
-  __host__ __device__ size_t total() const { return (info() + 8 * (size_t)(R + 1) + R + 31) & ~size_t(31); }
-  // the column indices of the next group's entries, past the staged entries (4 T each)
-  __host__ __device__ size_t cols() const { return up16(nb0() + (size_t)4 * tb * L); }
-  __host__ __device__ bool group_fits() const { return cols() + (size_t)4 * L <= acc(); }
-  // the write-out stages cr components of the block's L entries in nb0
-  __host__ __device__ size_t stage_bytes() const { return (size_t)cr * L * ob; }
-  __host__ __device__ bool stage_fits() const { return stage_bytes() <= nb1() - nb0(); }
+  size_t total() const { return (info() + 8 * (size_t)(R + 1) + R + 31) & ~size_t(31); }
+  // the column indices of the next group's entries, past the staged entries
+  size_t cols() const { return up16((size_t)4 * tb * L); }
+  bool group_fits() const { return cols() + (size_t)4 * L <= acc(); }
 };
 
-// step: the layout of the time-step kernels (one accumulator per slot, at the
-// 16-byte stride of the staged record halves; FP64 two planes of 16)
-__host__ __device__ inline GatherSmem gather_smem(int precision, int R, int W, int L, int S, bool step = false) {
+// the layout of a group of 32 / H rows whose staging holds W + 1 entries of each
+inline GatherSmem gather_smem(int precision, int mode, int H, int W, int S) {
   GatherSmem g;
-  g.R = R;
+  g.R = 32 / H;
   g.W = W;
-  g.L = L;
+  g.L = g.R * (W + 1);
   g.S = S;
+  g.H = H;
   g.tb = precision == NSI_FP64 ? 8 : 4;
-  // accumulator bytes per slot: FP64 (A, G_x, G_y, G_z) doubles; the mixed
-  // modes a float4 (G_x, G_y, G_z, A)
-  g.ab = precision == NSI_FP64 ? 32 : 16;
-  if (step) g.ab = precision == NSI_FP64 ? 32 : 16;
-  g.xs = 0;
-  g.ob = precision == NSI_MIXED_F32_ACC32 ? 4 : 8;
-  g.cr = precision == NSI_MIXED_F32_ACC64 ? 2 : 4;
-  if (step) g.xs = g.ob;  // the block's slice of A_static, copied in before the walk
+  g.ab = mode == ASSEMBLE ? 4 * g.tb : mode == STEP ? g.tb : 0;
   return g;
+}
+// the slots of a mesh whose longest row has `slots` off-diagonal entries: those,
+// or more where the staging would not fit nb0 and nb1
+inline int group_slots(int precision, int H, int slots) {
+  int W = slots;
+  while (!gather_smem(precision, ASSEMBLE, H, W, 0).group_fits()) ++W;
+  return W;
 }
 
 int gather_kernel_regs(int precision);  // registers per thread of the row-gather kernel

@@ -1,10 +1,10 @@
-"""Shared-memory layout of the row-gather kernels (host logic, no GPU).
+"""Shared-memory layout of the row gather (host logic, no GPU).
 
-tests/layout_check.cu includes the library's layout definition and checks,
-over precisions, the assembly and time-step layouts, block sizes and row,
-entry and step counts, that every region is 16-byte aligned, that regions do
-not overlap and that every alias the kernels use fits (column indices in nb1,
-staged record halves in the accumulators, the write-out staging in nb0).
+tests/layout_check.cu includes the library's layout definition and checks, over
+precisions, modes, lanes per row, row lengths and walk bytes, that what the
+launches carve is aligned, does not overlap, and holds what the kernels put in
+it (accumulator planes, staged entries and column indices, walk words, row
+bounds), for one mesh and for a batch's maxima.
 """
 import os
 import shutil
