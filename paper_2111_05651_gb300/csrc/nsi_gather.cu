@@ -31,13 +31,11 @@
 // against natural order; loading still earlier changes nothing).
 //
 // A small mesh has four lanes per row: its groups do not fill the chip, so the
-// chain is the time (8^3 cube in FP64: 66 us with one lane, 27 with four; 20^3
-// mixed64 13.8 with one, 12.5 with two, 10.9 with four; at 30 000 rows two and
-// four are equal, and at 100^3 four cost 374 us).  FP64 is bound by the FP64
-// pipe (one warp instruction in 18 cycles, 97-100% busy): a large mesh has one
-// lane per row, which saves the merge's additions (74 000 rows: 257 us with one
-// lane, 244 with two, whose smaller groups fill the last round better; 166 000:
-// 511 and 525; 100^3: 2977 and 3057, before all this 3023).
+// chain is the time (8^3 cube in FP64: 66 us with one lane, 27 with four; at
+// 100^3 four cost mixed64 374 us).  FP64 is bound by the FP64 pipe (one warp
+// instruction in 18 cycles, 97-100% busy): a large mesh has one lane per row,
+// which saves the merge's additions (100^3: 2977 us, with two 3057, before all
+// this 3023).  SMALL_MESH_ROWS and LARGE_FP64_ROWS have the sizes around the lines.
 #include <algorithm>
 #include <mutex>
 

@@ -87,12 +87,21 @@ struct GatherPlan {
                               // take, and large enough for the staging)
   bool long_group = false;    // a group has more entries, a long row's among them, than its staging holds
 };
-// a mesh of fewer rows has four lanes per row in the row gather, others two or one
-// (measured equal at about 30 000 rows for the assembly and at 10 000 for the
-// time step)
+// A mesh of fewer rows has four lanes per row in the row gather, which then
+// reads the nodes' own data in a single launch; others have two lanes (or one)
+// and a packing launch with the row gather started as it ends.  Assembly, us,
+// two -> four: 2,197 rows mixed64 8.3 -> 6.2, FP64 39 -> 25; 9,261 rows 10.3 ->
+// 8.2 and 41 -> 41; 12,167 rows 10.3 -> 8.3 and 55 -> 59; 15,625 rows 10.3 -> 10.3
+// and 61 -> 70; 19,683 rows 10.3 -> 12.0 and 74 -> 80 (time step and nodal
+// outputs cross at the same sizes): the line is FP64's.
 constexpr int64_t SMALL_MESH_ROWS = 10000;
-// from here on FP64 has one lane per row (two are faster at 74 000, one at 166 000)
-constexpr int64_t LARGE_FP64_ROWS = 120000;
+// From here on FP64 has one lane per row.  Below, two lanes' smaller groups fill
+// the last round better at most sizes; above, the merge's additions weigh more.
+// Assembly, us, one -> two lanes: 68,921 rows 246 -> 232, 79,507 264 -> 274,
+// 91,125 323 -> 299, 103,823 348 -> 337, 110,592 351 -> 356, 125,000 412 -> 403,
+// 148,877 491 -> 474, 166,375 516 -> 526, 185,193 584 -> 581, 205,379 656 -> 643,
+// 226,981 686 -> 704, 287,496 853 -> 884.
+constexpr int64_t LARGE_FP64_ROWS = 215000;
 constexpr int SMEM_MAX = 200 * 1024;  // shared memory of one block
 
 // diag_pos value of a row the row gather leaves out ("long row": more than

@@ -17,7 +17,7 @@ TOL = {"fp64": 1e-12, "mixed64": 1e-5, "mixed32": 1e-5}  # the library's stated 
 
 
 @pytest.mark.parametrize("precision,N", [(p, N) for p in ("fp64", "mixed64", "mixed32") for N in (20, 21, 36)] +
-                         [("fp64", 49)])  # 9,261, 10,648, 50,653 and (one lane in FP64) 125,000 rows
+                         [("fp64", 49), ("fp64", 59)])  # 9,261, 10,648, 50,653, 125,000 and (one lane in FP64) 216,000 rows
 def test_lanes_match_oracle(precision, N):
     mesh, u = meshgen.config_mesh(N=N, jitter=0.15, numbering="random", seed=300 + N)
     asm = nsi.Assembler(mesh.coord, mesh.lnods, precision=precision)
@@ -43,7 +43,7 @@ def test_lanes_match_oracle(precision, N):
 @pytest.mark.parametrize("precision", ["fp64", "mixed64", "mixed32"])
 def test_batch_of_both_kinds_equals_single(precision):
     asms, us = [], []
-    for N in (3, 36, 20, 49, 22):
+    for N in (3, 36, 20, 59, 22):
         mesh, u = meshgen.config_mesh(N=N, jitter=0.15, numbering="natural", seed=310 + N)
         asms.append(nsi.Assembler(mesh.coord, mesh.lnods, precision=precision))
         us.append(torch.as_tensor(u.T.copy()))
@@ -96,7 +96,7 @@ def test_row_of_more_entries_than_a_block_has_threads(precision):
     assert max(errors(rp, *got, oA, oG, orhs).values()) <= TOL[precision]
 
 
-@pytest.mark.parametrize("precision,N,shapes", [("mixed64", 6, 1), ("mixed64", 22, 2), ("fp64", 6, 1), ("fp64", 49, 4)])
+@pytest.mark.parametrize("precision,N,shapes", [("mixed64", 6, 1), ("mixed64", 22, 2), ("fp64", 6, 1), ("fp64", 59, 4)])
 def test_launch_shapes_are_distinct(precision, N, shapes):
     """Four lanes per row fill a block of four warps by every name, two have two
     launches, one lane four; a name that repeats a launch is still accepted."""
