@@ -52,3 +52,22 @@ def test_grad_mu_of_one_cluster_repeats():
     asm = nsi.Assembler(mesh.coord, mesh.lnods, precision="fp64")
     ut = torch.as_tensor(u.T.copy()).cuda()
     assert len({asm.vjp(ut, w)[1].item() for _ in range(20)}) == 1
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed64"])
+def test_vjp_in_a_captured_graph(precision):
+    mesh, u = meshgen.config_mesh(N=9, jitter=0.15, numbering="random", seed=53)
+    asm = nsi.Assembler(mesh.coord, mesh.lnods, precision=precision)
+    ut = torch.as_tensor(u.T.copy()).cuda().to(asm.vel_dtype)
+    w = torch.as_tensor(np.random.default_rng(54).standard_normal(u.shape).T.copy()).cuda().to(asm.vel_dtype)
+    gu, gmu = asm.vjp(ut, w)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        gu2, gmu2 = asm.vjp(ut, w)
+    graph.replay()
+    torch.cuda.synchronize()
+    # (grad_u's and grad_mu's atomic additions have no fixed order)
+    tol = 1e-13 if precision == "fp64" else 1e-5
+    assert (gu2 - gu).abs().max() <= tol * gu.abs().max()
+    assert abs(gmu2.item() - gmu.item()) <= tol * max(abs(gmu.item()), 1.0)
