@@ -490,7 +490,7 @@ static nsi_status build(NsiHandle* h, const NsiMesh* m, cudaStream_t s) {
   // 4a. every row's sub-walks (the order and steps of the kernel's element
   // loops), one per lane of the row
   h->nsub = n < SMALL_MESH_ROWS ? 4 : h->precision == NSI_FP64 && n >= LARGE_FP64_ROWS ? 1 : 2;
-  std::vector<int32_t> walk_ptr;
+  std::vector<uint32_t> walk_ptr;
   std::vector<uint8_t> walk;
   if (h->gather_ok) {
     std::vector<int32_t> wlen(n, 0);
@@ -518,11 +518,11 @@ static nsi_status build(NsiHandle* h, const NsiMesh* m, cudaStream_t s) {
     });
     int64_t total = 0;
     for (int64_t i = 0; i < n; ++i) total += wlen[i];
-    if (bad.load() || total > INT32_MAX - 64) {
+    if (bad.load() || total > (int64_t)UINT32_MAX - 64) {  // (a sub-walk's length and fillings are bytes too)
       h->gather_ok = false;
     } else {
       walk_ptr.assign(n + 1, 0);
-      for (int64_t i = 0; i < n; ++i) walk_ptr[i + 1] = walk_ptr[i] + wlen[i];
+      for (int64_t i = 0; i < n; ++i) walk_ptr[i + 1] = walk_ptr[i] + (uint32_t)wlen[i];
       std::sort(parts.begin(), parts.end(),
                 [](const std::pair<int64_t, std::vector<uint8_t>>& a, const std::pair<int64_t, std::vector<uint8_t>>& b) {
                   return a.first < b.first;

@@ -120,7 +120,7 @@ struct WalkMesh {
   int64_t n, nnz;
   const int32_t* row_ptr;
   const int32_t* col_idx;
-  const int32_t* walk_ptr;
+  const uint32_t* walk_ptr;
   const uint8_t* walk;
   const uint8_t* diag_pos;
   const D4* xyz64;
@@ -415,7 +415,8 @@ __device__ __forceinline__ bool walk_ok(const uint8_t* st, int nbytes, int nsub,
 // ---------------------------------------------------------------- groups ---
 // One row of a group, as each of its lanes sees it.
 struct GroupRow {
-  int32_t rs, re, w0, w1;  // CSR and walk bounds
+  int32_t rs, re;  // CSR bounds
+  uint32_t w0, w1;  // walk bounds
   int dp;
 };
 // the bounds and diagonal positions of rows [r0, r0 + RW) into shared memory
@@ -436,8 +437,8 @@ __device__ __forceinline__ GroupRow read_row(const unsigned char* info, int t) {
   GroupRow r;
   r.rs = b[t];
   r.re = b[t + 1];
-  r.w0 = b[RW + 1 + t];
-  r.w1 = b[RW + 2 + t];
+  r.w0 = (uint32_t)b[RW + 1 + t];
+  r.w1 = (uint32_t)b[RW + 2 + t];
   r.dp = info[8 * (RW + 1) + t];
   return r;
 }
@@ -450,10 +451,10 @@ __device__ __forceinline__ int row_slots(const GroupRow& r) {
 __device__ __forceinline__ int slot_pos(int s, int dp) { return s + (s >= dp ? 1 : 0); }
 
 // the walk bytes of the group's rows into shared memory, as aligned words
-__device__ __forceinline__ void copy_walk(const WalkMesh& m, unsigned char* dst, int32_t w0, int32_t w1, int lane) {
-  const int off = w0 & 3;
+__device__ __forceinline__ void copy_walk(const WalkMesh& m, unsigned char* dst, uint32_t w0, uint32_t w1, int lane) {
+  const uint32_t off = w0 & 3u;
   const uint32_t* src = reinterpret_cast<const uint32_t*>(m.walk + (w0 - off));
-  const int words = (w1 - w0 + off + 3) >> 2;
+  const int words = (int)((w1 - w0 + off + 3) >> 2);
   for (int k = lane; k < words; k += 32) cp_async4(reinterpret_cast<uint32_t*>(dst) + k, src + k);
 }
 
@@ -587,7 +588,8 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
   // the first group
   int at = src.find(g);
   GroupRow row;
-  int32_t wb, we, base, end;
+  int32_t base, end;
+  uint32_t wb, we;
   {
     const WalkMesh& m = src.item(at).m;
     const int64_t r0 = (int64_t)(g - src.item(at).group0) * RW;
@@ -597,7 +599,7 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
     row = read_row<RW>(smem + lay.info, t);
     base = __shfl_sync(FULL, row.rs, 0), end = __shfl_sync(FULL, row.re, RW - 1);
     wb = __shfl_sync(FULL, row.w0, 0), we = __shfl_sync(FULL, row.w1, RW - 1);
-    if (!DEBUG || we - wb <= lay.S) copy_walk(m, smem + lay.walk, wb, we, lane);
+    if (!DEBUG || we - wb <= (uint32_t)lay.S) copy_walk(m, smem + lay.walk, wb, we, lane);
     copy_cols(m, base, end);
     cp_async_wait_all();
     __syncwarp();
@@ -623,7 +625,7 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
     const int lb = dense ? gb : t * (lay.W + 1);
     bool fits = true;
     if (DEBUG) {
-      fits = we - wb <= lay.S && !__any_sync(FULL, ns > lay.W || (ns > 0 && row.dp > ns));
+      fits = we - wb <= (uint32_t)lay.S && !__any_sync(FULL, ns > lay.W || (ns > 0 && row.dp > ns));
       if (!fits && lane == 0) atomicOr(m.err, ERR_STAR);
     }
     const T kmass = kmass_of<T>(f);
@@ -647,8 +649,8 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
       } else if constexpr (MODE != NODAL) {
         acc.a += t;
       }
-      const uint8_t* st = (smem + lay.walk) + (row.w0 - wb) + (wb & 3);
-      const int nb = row.w1 - row.w0;
+      const uint8_t* st = (smem + lay.walk) + (row.w0 - wb) + (wb & 3u);
+      const int nb = (int)(row.w1 - row.w0);
       if (DEBUG && !walk_ok(st, nb, H, ns)) {
         atomicOr(m.err, ERR_STAR);
       } else if (nb > 0) {
@@ -663,7 +665,8 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
     // the next group's walk bytes and column indices
     refresh();
     GroupRow rown = row;
-    int32_t wbn = 0, wen = 0, basen = 0, endn = 0;
+    int32_t basen = 0, endn = 0;
+    uint32_t wbn = 0, wen = 0;
     if (more) {
       cp_async_wait_all();
       __syncwarp();
@@ -671,7 +674,7 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
       rown = read_row<RW>(smem + lay.info, t);
       basen = __shfl_sync(FULL, rown.rs, 0), endn = __shfl_sync(FULL, rown.re, RW - 1);
       wbn = __shfl_sync(FULL, rown.w0, 0), wen = __shfl_sync(FULL, rown.w1, RW - 1);
-      if (!DEBUG || wen - wbn <= lay.S) copy_walk(mn, smem + lay.walk, wbn, wen, lane);
+      if (!DEBUG || wen - wbn <= (uint32_t)lay.S) copy_walk(mn, smem + lay.walk, wbn, wen, lane);
       copy_cols(mn, basen, endn);
     }
     V3<T> un{T(0), T(0), T(0)};

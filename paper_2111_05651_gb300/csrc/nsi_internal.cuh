@@ -190,7 +190,7 @@ struct NsiHandle {
   int32_t* color_elems = nullptr;  // [E] element ids grouped by colour
   std::vector<int64_t> color_off;  // host [n_colors + 1]
   // row-gather map: every row's element walk (one byte per step)
-  int32_t* walk_ptr = nullptr;  // [n+1]
+  uint32_t* walk_ptr = nullptr;  // [n+1]
   uint8_t* walk = nullptr;      // [walk_ptr[n] + 8]
   int nsub = 2;                 // sub-walks per row
   bool packs() const { return nsub != 4; }  // the row gather reads packed node records (else the nodes' own data)
