@@ -840,8 +840,8 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
       const T4<T>* stage = reinterpret_cast<const T4<T>*>(smem);
       Out* A = static_cast<Out*>(o.A) + base;
       Out *G = static_cast<Out*>(o.G) + base, *G1 = G + m.nnz, *G2 = G1 + m.nnz;
-      // (mixed64 by streaming stores: the outputs leave L2 before the records do,
-      // 271 against 279 us at 100^3 in random order; mixed32 236 against 226)
+      // (plain stores: streaming ones took mixed64 275 against 270 us at 100^3 in
+      // random order and 232 against 221 in natural, mixed32 236 against 226)
       auto write = [&](auto&& put) {
 #pragma unroll 1
         for (int r = 0; r < (dense ? 1 : RW); ++r) {
@@ -857,10 +857,10 @@ __device__ __forceinline__ void group_loop(const Source& src, int g, int stride,
         // instructions), then every diagonal by the double nearest its
         // compensated pair
         write([&](int k, const T4<T>& v) {
-          __stcs(A + k, (double)v.x);
-          __stcs(G + k, float_double(v.y));
-          __stcs(G1 + k, float_double(v.z));
-          __stcs(G2 + k, float_double(v.w));
+          A[k] = (double)v.x;
+          G[k] = float_double(v.y);
+          G1[k] = float_double(v.z);
+          G2[k] = float_double(v.w);
         });
         __syncwarp();
         if (fits && h == 0 && len > 0)
