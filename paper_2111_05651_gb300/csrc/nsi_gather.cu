@@ -21,13 +21,13 @@
 // and a second set of accumulators (13 KB, 16 warps) behind chains of 12, and
 // the neighbours' records come as one 256-bit load each, in registers under the
 // previous group's write-out, instead of two 16-byte copies through shared
-// memory (100^3 cube, us, one lane per row -> two: mixed64 277 -> 266 in random
-// and 269 -> 226 in natural node order, mixed32 228 -> 226, time step 275 ->
-// 198, nodal outputs 216 -> 126; 47x61x38 mixed32 39.6 -> 31.4).  The records
-// bypass L1 (allocating there cost 439 us: 115 KB of sectors in flight per SM
+// memory (100^3 cube, us, one lane per row -> two: mixed64 277 -> 270 in random
+// and 269 -> 221 in natural node order, mixed32 228 -> 224, time step 275 ->
+// 195, nodal outputs 216 -> 121; 47x61x38 mixed32 39.6 -> 31.4).  The records
+// bypass L1 (allocating there costs 407 us: 115 KB of sectors in flight per SM
 // through the 28 KB that shared memory leaves).  What is left is the shared
-// memory's data path (75% busy: 740 wavefronts of a group's 16 rows) and issue
-// (about 60%), and in random node order the rate of scattered 32-byte requests (40 us
+// memory's data path (72% busy: 650 wavefronts of a group's 16 rows) and issue
+// (59%), and in random node order the rate of scattered 32-byte requests (50 us
 // against natural order; loading still earlier changes nothing).
 //
 // A small mesh has four lanes per row: its groups do not fill the chip, so the

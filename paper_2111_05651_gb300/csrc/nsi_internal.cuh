@@ -34,8 +34,7 @@ enum : unsigned { ERR_BAD_INDEX = 1u, ERR_NOT_IN_PATTERN = 2u, ERR_STAR = 4u };
 // each), ordered so that (i, j1, j2, j3) is an even permutation of the
 // element's node order (hence a positively oriented tet).  The kernels read
 // the element walk encoded from these words (WALK_* below) and the edge-fan
-// map.  Rows longer than 32 entries cannot be encoded; such meshes do not
-// support the gather mode.
+// map.  Rows longer than 32 entries cannot be encoded: "long rows" (DIAG_LONG).
 constexpr int STAR_BITS = 5;
 constexpr int STAR_MAX_ROW = 1 << STAR_BITS;
 // an element with |d1||d2||d3| > EXACT_RATIO |det| (edge vectors from any of
@@ -129,7 +128,7 @@ enum { ASSEMBLE = 0, STEP = 1, NODAL = 2 };
 // After the element loop, nb0 and nb1 are reused to stage the finished values
 // for the coalesced write-out (4 T per entry, in CSR order, or row t's from
 // t * (W + 1) on), and past them for the next group's column indices.
-// Used identically by the host (launch size) and the kernel (carving).
+// The host sizes launches by it and hands the kernels its offsets.
 struct GatherSmem {
   int R, W, L, S, H, tb, ab;
   static size_t up16(size_t x) { return (x + 15) & ~size_t(15); }
