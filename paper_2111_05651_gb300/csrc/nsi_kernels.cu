@@ -24,6 +24,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -741,7 +742,8 @@ __global__ void __launch_bounds__(FAN_BLOCK) fan_kernel(MeshView m, FieldView f,
 // off-diagonal blocks.
 struct StabConst {
   double ks, k4mu, krh, kr48;  // rho^2 / 120, 4 mu, rho / 2, rho / 48
-  float ksf, k4muf, krhf, kr48f;
+  double kml;                  // what rho / (24 dt) lacks in FieldView::kmass
+  float ksf, k4muf, krhf, kr48f, kmlf;
 };
 
 static StabConst stab_const(const NsiFields* f) {
@@ -750,6 +752,11 @@ static StabConst stab_const(const NsiFields* f) {
   c.k4mu = 4.0 * f->mu;
   c.krh = f->rho / 2.0;
   c.kr48 = f->rho / 48.0;
+  const double k = f->rho / (24.0 * f->dt), d = 24.0 * f->dt;
+  c.kml = (std::fma(-k, d, f->rho) - k * std::fma(24.0, f->dt, -d)) / d;
+  if (!std::isfinite(c.kml)) c.kml = 0.0;
+  c.kmlf = (float)(k - (double)(float)k);
+  if (!std::isfinite(c.kmlf)) c.kmlf = 0.0f;
   c.ksf = (float)c.ks;
   c.k4muf = (float)c.k4mu;
   c.krhf = (float)c.krh;
@@ -759,12 +766,12 @@ static StabConst stab_const(const NsiFields* f) {
 
 template <typename T>
 struct StabK {
-  T ks, k4mu, krh, kr48;
+  T ks, k4mu, krh, kr48, kml;
 };
 template <typename T>
 __device__ __forceinline__ StabK<T> stab_k(const StabConst& c) {
-  if constexpr (sizeof(T) == 8) return StabK<T>{c.ks, c.k4mu, c.krh, c.kr48};
-  else return StabK<T>{c.ksf, c.k4muf, c.krhf, c.kr48f};
+  if constexpr (sizeof(T) == 8) return StabK<T>{c.ks, c.k4mu, c.krh, c.kr48, c.kml};
+  else return StabK<T>{c.ksf, c.k4muf, c.krhf, c.kr48f, c.kmlf};
 }
 __device__ __forceinline__ float cbrt_of(float x) { return cbrtf(x); }
 __device__ __forceinline__ double cbrt_of(double x) { return cbrt(x); }
@@ -1095,7 +1102,11 @@ __global__ void __launch_bounds__(32 * STAR_WARPS, P == NSI_FP64 ? 1 : 6) stab_s
     for (int c = 0; c < 3; ++c) Go[c * m.nnz + g] = (Out)(G[c] * kg);
   }
   if (len > 0 && q < 15) {  // (a row's lanes number 16 or 32)
-    const Acc<P> mass = acc_scale<P>(tD, kmass);
+    // (the factor's own rounding would be the same in every row's mass; mixed32
+    // keeps it, its values are rounded to float once more anyway)
+    Acc<P> mass = acc_scale<P>(tD, kmass);
+    if constexpr (P == NSI_MIXED_F32_ACC64) mass.lo = fmaf(sk.kml, tD.hi, mass.lo);
+    else if constexpr (P == NSI_FP64) mass.v = fma(sk.kml, tD.v, mass.v);
     Acc<P> x;
     Out* at;
     if (q < 12) {  // A(i,i)[a][b] = delta_ab (lumped mass - sum of the row's A + S) - sum of K[a][b]; G(i,i) = G's / 3

@@ -238,3 +238,15 @@ def test_mixed32_diagonal_sums_in_pairs(N, seed, mu, bound):
     diag = np.repeat(np.arange(mesh.n_nodes), np.diff(rp)) == ci
     got, ref = (x[[0, 4, 8]][:, diag] for x in (Auu, oAuu))
     assert np.linalg.norm(got - ref) <= bound * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("dt", [1e-2, 3e-3, 1.7e-2])
+def test_mixed64_mass_carries_no_common_rounding(dt):
+    """The lumped right-hand side in mixed64: rms error 2.2e-8 (the determinants'
+    roundings) whatever rho / (24 dt) rounds to in float; with the factor rounded
+    up to 6e-8 are common to all rows (4.2e-8 in all at dt = 0.01)."""
+    mesh, u = meshgen.config_mesh(N=20, jitter=0.15, numbering="random", seed=62)
+    asm = nsi.Assembler(mesh.coord, mesh.lnods, precision="mixed64")
+    ref = oracle.assemble_stabilized(mesh.coord, mesh.lnods, u.astype(np.float32).astype(np.float64), None, 1.0, 1e-3, dt)[4]
+    got = asm.assemble_stabilized(torch.as_tensor(u.T.copy()), rho=1.0, mu=1e-3, dt=dt)[2].double().cpu().numpy()
+    assert np.linalg.norm(got - ref) <= 3e-8 * np.linalg.norm(ref)
